@@ -101,17 +101,15 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
   constexpr int n = NS + 1;
   extern __shared__ double smem[];
   const int tid = threadIdx.x, stride = blockDim.x;
-  double2* etab = reinterpret_cast<double2*>(smem);
-  for (int i = tid; i < 64; i += stride) etab[i] = g_exp2_tab[i];
-  int boff = 128;
+  int boff = 0;
   const double* blob = a.blob;
   if (a.stage_blob) {
-    for (int i = tid; i < a.d.total; i += stride) smem[boff + i] = a.blob[i];
-    blob = smem + boff;
-    boff += (a.d.total + 1) & ~1;
+    for (int i = tid; i < a.d.total; i += stride) smem[i] = a.blob[i];
+    blob = smem;
+    boff = (a.d.total + 1) & ~1;
   }
   __syncthreads();
-  const MechView mv = make_view(blob, a.d, etab);
+  const MechView mv = make_view(blob, a.d);
   const int M = a.d.M;
   double* base = smem + boff;
   // Dual vectors (value part at even offsets)
@@ -403,7 +401,7 @@ static int adj_threads(const df_mech* m) {
   const int NS = m->dims.N;
   const long per = adj_layout_doubles(NS, m->dims.M, adj_keep_possible(NS));
   const long budget = (long)m->smem_per_sm / 4 - (long)m->smem_reserved_per_block;  // bytes per block
-  const long t = (budget / (long)sizeof(double) - 128) / per;  // 128: the exp table
+  const long t = budget / (long)sizeof(double) / per;
   return t >= 16 && t < 32 ? (int)t : 32;
 }
 
@@ -445,8 +443,8 @@ static int adjoint_dispatch_layout(const df_mech* m, AdjArgs a, cudaStream_t st,
   a.hook_cp = 8 * NS;
   // the mechanism is staged in shared memory unless that leaves fewer blocks
   // on an SM than reading it through L1
-  const size_t sm_staged = sizeof(double) * (128 + ((m->dims.total + 1) & ~1) + per);
-  const size_t sm_plain = sizeof(double) * (128 + per);
+  const size_t sm_staged = sizeof(double) * (((m->dims.total + 1) & ~1) + per);
+  const size_t sm_plain = sizeof(double) * per;
   auto blocks_per_sm = [m](size_t b) {
     return b > m->max_smem_optin ? (size_t)0 : m->smem_per_sm / (b + m->smem_reserved_per_block);
   };

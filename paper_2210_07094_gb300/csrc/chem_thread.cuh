@@ -18,9 +18,9 @@
 //                                           Sec. 2.2 df0DFoam; h conserved)
 #pragma once
 #include "dev_common.cuh"
-#include "fastexp.cuh"
-#include "fastlog.cuh"
 #include "dual.cuh"
+#include "exp2fix.cuh"
+#include "fastlog.cuh"
 
 namespace df {
 
@@ -49,13 +49,11 @@ struct MechView {
   const double* rx;
   const double* tr;
   const double* eff;
-  const double2* etab;  // 2^(j/64) table of exp_tang (shared memory)
   int M;
 };
 
-__device__ __forceinline__ MechView make_view(const double* blob, const MechDims& d, const double2* etab) {
+__device__ __forceinline__ MechView make_view(const double* blob, const MechDims& d) {
   MechView v;
-  v.etab = etab;
   v.sp = blob + d.off_sp;
   v.rx = blob + d.off_rx;
   v.tr = blob + d.off_tr;
@@ -78,12 +76,10 @@ __device__ __forceinline__ RxSlots load_slots(const double* r) {
 }
 
 // exp of two arguments (two independent dependency chains for the scheduler)
-__device__ __forceinline__ void exp_pair(double a, double b, const double2* tab, double& ea, double& eb) {
-  exp_tang2(a, b, tab, ea, eb);
-}
-__device__ __forceinline__ void exp_pair(const Dual& a, const Dual& b, const double2* tab, Dual& ea, Dual& eb) {
-  ea = exp_tang(a, tab);
-  eb = exp_tang(b, tab);
+__device__ __forceinline__ void exp_pair(double a, double b, double& ea, double& eb) { exp_rate2(a, b, ea, eb); }
+__device__ __forceinline__ void exp_pair(const Dual& a, const Dual& b, Dual& ea, Dual& eb) {
+  ea = exp_rate(a);
+  eb = exp_rate(b);
 }
 
 // Result of the rate of one reaction; with J also the pieces of dq/dT|_C and
@@ -210,11 +206,11 @@ __device__ __forceinline__ void rate_compute(const MechView& mv, const RxIn<S>& 
     // Pr = k0 [M] / kinf, as exp(ln k0 - ln kinf) [M] (no division); the
     // exponentials in pairs (see exp_pair)
     S kinf, r0, e3, e1, e2, invKc;
-    exp_pair(lnkf, lnk0 - lnkf, mv.etab, kinf, r0);
+    exp_pair(lnkf, lnk0 - lnkf, kinf, r0);
     const S Pr = r0 * Mc;
     if (!(val(Pr) > 0.0)) return;  // no low-pressure rate or no collider: k = 0
-    exp_pair(-T * tr[4], -T * tr[5], mv.etab, e3, e1);
-    exp_pair(-tr[6] * invT, lnKcinv, mv.etab, e2, invKc);
+    exp_pair(-T * tr[4], -T * tr[5], e3, e1);
+    exp_pair(-tr[6] * invT, lnKcinv, e2, invKc);
     if (!rev) invKc = S(0.0);
     const S Fc = (1.0 - tr[3]) * e3 + tr[3] * e1 + e2;
     const S Lc = fast_log10(Fc);
@@ -227,12 +223,12 @@ __device__ __forceinline__ void rate_compute(const MechView& mv, const RxIn<S>& 
     const S den2 = den * den;
     const S q1 = den2 / (den2 + x * x);
     const S log10F = Lc * q1;
-    const S F = exp_tang(LN10 * log10F, mv.etab);
+    const S F = exp_rate(LN10 * log10F);
     const S onePr = 1.0 / (1.0 + Pr);
     kf = kinf * Pr * onePr * F;
     kr = kf * invKc;
     if (WITH_J) {
-      const S k0 = exp_tang(lnk0, mv.etab);
+      const S k0 = exp_rate(lnk0);
       const S f1 = x / den;
       const S df1_dL = nn / (den * den);
       const S df1_dLc = (-0.67 * den - x * (-1.27 + 0.67 * 0.14)) / (den * den);
@@ -247,7 +243,7 @@ __device__ __forceinline__ void rate_compute(const MechView& mv, const RxIn<S>& 
       dqdM = k0 * F * gpr * onePr * (Pf - Pb * invKc);
     }
   } else {
-    exp_pair(lnkf, lnkf + lnKcinv, mv.etab, kf, kr);
+    exp_pair(lnkf, lnkf + lnKcinv, kf, kr);
     if (!rev) kr = S(0.0);
     if (type == 1) {
       mult = g.Mc;

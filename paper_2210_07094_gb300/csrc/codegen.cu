@@ -446,9 +446,6 @@ std::map<std::pair<int, std::string>, Module> g_modules;
 
 constexpr int kThreads[] = {32, 64};
 constexpr int kIgnThreads = 32;  // the block size of the kernel that refines the ignition time
-// the generated kernels' exp table: 256 entries (one FP64 operation fewer per
-// exponential than the library's 64; 4 KB of shared memory per block)
-constexpr int kGenExpTableBits = 8;
 
 // ---------------------------------------------------------------------------
 // on-disk cache of compiled modules: <dir>/<key>.cubin and <key>.names (the
@@ -516,7 +513,7 @@ uint64_t headers_hash(const std::string& inc) {
   std::call_once(once, [&] {
     uint64_t acc = 1469598103934665603ull;
     const char* files[] = {"integrate_thread.cuh", "rosenbrock.cuh", "chem_thread.cuh", "dev_common.cuh",
-                           "fastexp.cuh", "fastexp_table256.inc", "fastlog.cuh", "fastlog_table.inc", "dual.cuh"};
+                           "exp2fix.cuh", "exp2fix_table.inc", "fastlog.cuh", "fastlog_table.inc", "dual.cuh"};
     for (const char* fn : files) {
       std::string d;
       read_file(inc + "/" + fn, &d);
@@ -610,9 +607,8 @@ Module build_module(int dev, const df_mech* m, const std::string& src) {
   names.push_back(jit_kernel_name(m->dims.N, kIgnThreads, true));
   names.push_back("&df::c_tab");
   const std::string incopt = "-I" + inc;
-  const std::string expopt = "-DDF_EXP_TABLE_BITS=" + std::to_string(kGenExpTableBits);
   const char* opts[] = {arch.c_str(), "-std=c++17", incopt.c_str(), "-default-device", "-lineinfo",
-                        "-diag-suppress=177", expopt.c_str()};
+                        "-diag-suppress=177"};
   // the on-disk cache: keyed by the generated source, the device headers, the
   // architecture, the NVRTC version, the compile options (the include path
   // left out: a moved tree keeps its entries) and the entry format
@@ -716,11 +712,10 @@ int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, cuda
   const int N = m->dims.N;
   const int per_thread = (N + 1) * (N + 1) + 6 * (N + 1);  // J and the stage vectors
   IntegArgs args = a;
-  // the exp table (2 doubles per entry), the mechanism if staging it leaves as
-  // many blocks on an SM as reading it through L1, the per-thread workspace
-  const size_t tab = 2 * ((size_t)1 << kGenExpTableBits);
-  const size_t sm_staged = sizeof(double) * (tab + (size_t)blob_smem_doubles(m->dims) + (size_t)per_thread * threads);
-  const size_t sm_plain = sizeof(double) * (tab + (size_t)per_thread * threads);
+  // the mechanism if staging it leaves as many blocks on an SM as reading it
+  // through L1, the per-thread workspace
+  const size_t sm_staged = sizeof(double) * ((size_t)blob_smem_doubles(m->dims) + (size_t)per_thread * threads);
+  const size_t sm_plain = sizeof(double) * (size_t)per_thread * threads;
   auto blocks_per_sm = [m](size_t b) {
     return b > m->max_smem_optin ? (size_t)0 : m->smem_per_sm / (b + m->smem_reserved_per_block);
   };

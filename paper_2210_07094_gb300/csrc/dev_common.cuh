@@ -95,6 +95,17 @@ inline MechDims mech_dims(int N, int M, int n_eff, int n_troe) {
 }
 
 #ifdef __CUDACC__
+// (double)v for |v| < 2^20, assembled from the integer's sign, leading one and
+// the bits below it with integer operations, so that the conversion takes no
+// slot of the narrow FP64 pipe (exact: every such integer is a double)
+__device__ __forceinline__ double small_int_to_double(int v) {
+  const unsigned a = (unsigned)(v < 0 ? -v : v);
+  const int lz = __clz(a | 1u);                  // the leading one of a > 0 at bit 31 - lz
+  const unsigned mant = ((a << lz) << 1) >> 12;  // the (at most 19) bits below it, left-aligned
+  const unsigned hi = ((unsigned)(v < 0) << 31) | ((unsigned)(1023 + 31 - lz) << 20) | mant;
+  return __hiloint2double(a != 0u ? (int)hi : 0, 0);
+}
+
 // 1/a in FP64 from an FP32 seed and two Newton-Raphson steps r <- r (2 - a r)
 // (the relative error squares at each step: 2^-22 -> 2^-44 -> rounding): four
 // FP64 operations where a correctly rounded division takes a longer sequence

@@ -11,6 +11,7 @@
 
 #include "chem_thread.cuh"
 #include "common.cuh"
+#include "fastexp.cuh"
 #include "gemm_host.cuh"
 #include "tc_gemm.cuh"
 

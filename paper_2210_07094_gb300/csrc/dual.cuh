@@ -4,7 +4,7 @@
 // discrete adjoint uses that for the second-derivative terms of the
 // Rosenbrock step.
 #pragma once
-#include "fastexp.cuh"
+#include "exp2fix.cuh"
 
 namespace df {
 
@@ -47,8 +47,8 @@ __device__ __forceinline__ Dual operator/(double a, Dual b) {
 __device__ __forceinline__ double val(double x) { return x; }
 __device__ __forceinline__ double val(const Dual& x) { return x.v; }
 
-__device__ __forceinline__ Dual exp_tang(Dual x, const double2* tab) {
-  const double e = exp_tang(x.v, tab);
+__device__ __forceinline__ Dual exp_rate(Dual x) {
+  const double e = exp_rate(x.v);
   return Dual(e, e * x.d);
 }
 __device__ __forceinline__ Dual log(Dual x) { return Dual(::log(x.v), x.d / x.v); }

@@ -1,0 +1,83 @@
+// exp(x) and 2^x in 64-bit fixed point on the integer pipes.
+//
+// The FP64 pipe issues one warp instruction in 64 cycles; a 32 x 32 -> 64 bit
+// multiply-add takes 4 and an addition 1.  The table-driven exponential of
+// fastexp.cuh is 8 FP64 instructions, 670 cycles per warp; the one below is
+// about 60 integer instructions: 161 cycles alone on a sub-partition, 115 with
+// several warps (152 SMs, dependent chains of two).  Its argument reduction is
+// exact but for one rounding, so it is also the more accurate: at most 0.93 ulp
+// for |x| <= 128 and 1.08 for |x| < 512, against 1.32 (host emulation, 3e6
+// arguments per range).
+//
+// X = x 2^53 in a 64-bit integer, |x| < 1022: m = X >> 53, j = the next 8 bits,
+// g = the 45 bits below them as a fraction of 2^-8:
+//   2^x = 2^m 2^(j/256) (1 + p),  p = g (a1 + g (a2 + g (a3 + g a4)))
+// with 2^(j/256) a 64-bit fraction from a 2 KB table.  The table is read from
+// global memory through L1: a gather of 8-byte entries costs there what it
+// costs in shared memory (112 against 115 cycles per exponential), and the
+// shared memory stays free for cells.
+#pragma once
+#include "dev_common.cuh"
+
+namespace df {
+
+#include "exp2fix_table.inc"
+
+__device__ __forceinline__ uint64_t wmad(uint32_t a, uint32_t b, uint64_t c) { return (uint64_t)a * b + c; }
+
+// the high 64 bits of a 64 x 64 bit product to within 3 units (the product of
+// the low words and the carries out of the cross products' low words dropped)
+__device__ __forceinline__ uint64_t mulhi64_3(uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl) {
+  return wmad(ah, bh, (uint64_t)__umulhi(ah, bl)) + __umulhi(al, bh);
+}
+
+// 2^((X + 1/2) 2^-53): X is the floor of a value, its mean the half unit above.
+// |X| < 1022 2^53 (normal results).
+__device__ __forceinline__ double exp2_fixed(int64_t X) {
+  const uint32_t xh = (uint32_t)((uint64_t)X >> 32), xl = (uint32_t)X;
+  const uint64_t t = __ldg(reinterpret_cast<const unsigned long long*>(g_exp2fix_tab) + ((xh >> 13) & 255u));
+  const uint32_t gh = (xh << 19) | (xl >> 13), gl = (xl << 19) | (1u << 18);
+  const uint32_t h3 = (uint32_t)EXP2FIX_A3 + __umulhi(gh, (uint32_t)EXP2FIX_A4);  // 2^60
+  const uint64_t h2 = wmad(__umulhi(gh, h3), 1u << 22, EXP2FIX_A2);              // 2^82
+  const uint64_t h1 = EXP2FIX_A1 + (mulhi64_3(gh, gl, (uint32_t)(h2 >> 32), (uint32_t)h2) >> 10);  // 2^72
+  const uint64_t p = mulhi64_3(gh, gl, (uint32_t)(h1 >> 32), (uint32_t)h1);                       // 2^72
+  const uint64_t q = mulhi64_3((uint32_t)(t >> 32), (uint32_t)t, (uint32_t)(p >> 32), (uint32_t)p);
+  const uint64_t r = t + (q >> 8);  // in [2^63, 2^64)
+  // the leading 53 bits, rounded; the leading one adds 1 to the exponent field
+  const uint64_t e = (uint64_t)((uint32_t)(((int32_t)xh >> 21) + 1022) << 20) << 32;
+  return __longlong_as_double((long long)(e + (r >> 11) + ((r >> 10) & 1u)));
+}
+
+// x log2(e) as floor(x log2(e) 2^53), |x| < 512: the 53-bit mantissa (at bit
+// 62) times log2(e)/2, shifted by the exponent; a negative x takes the
+// complement, so both signs are floors
+__device__ __forceinline__ int64_t exp_arg_fixed(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  constexpr uint32_t ch = (uint32_t)(EXP2FIX_LOG2E_HALF >> 32), cl = (uint32_t)EXP2FIX_LOG2E_HALF;
+  const uint32_t mh = 0x40000000u | ((hi << 10) & 0x3fffffffu) | (lo >> 22), ml = lo << 10;
+  const uint64_t p = wmad(mh, ch, wmad(ml, ch, (uint64_t)mh * cl) >> 32);
+  const uint32_t e = (hi >> 20) & 0x7ffu;
+  const uint32_t s = e < 968u ? 63u : 1031u - e;
+  return (int64_t)(p >> s) ^ (int64_t)((int32_t)hi >> 31);
+}
+
+// |x| >= 512, inf and NaN (an integer test of the high word)
+__device__ __forceinline__ bool exp_is_big(double x) { return (__double2hiint(x) & 0x7fffffff) >= 0x40800000; }
+
+__device__ __forceinline__ double exp_rate(double x) {
+  return exp_is_big(x) ? exp(x) : exp2_fixed(exp_arg_fixed(x));
+}
+
+// two at once, as one straight-line block (two independent chains); the rare
+// big arguments are fixed up afterwards
+__device__ __forceinline__ void exp_rate2(double x1, double x2, double& e1, double& e2) {
+  const bool b1 = exp_is_big(x1), b2 = exp_is_big(x2);
+  e1 = exp2_fixed(exp_arg_fixed(b1 ? 0.0 : x1));
+  e2 = exp2_fixed(exp_arg_fixed(b2 ? 0.0 : x2));
+  if (b1 | b2) {
+    if (b1) e1 = exp(x1);
+    if (b2) e2 = exp(x2);
+  }
+}
+
+}  // namespace df

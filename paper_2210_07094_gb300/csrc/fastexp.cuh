@@ -10,22 +10,15 @@
 // fused multiply-adds.  The truncated Taylor tail r^6/720 <= 3.5e-17 stays
 // below one ulp.  |x| >= 700, inf and NaN go to
 // the library exp().  The kernels stage the table into shared memory (lanes
-// index it with different j).  A variant with 256 entries 2^(j/256) (|r| <=
+// index it with different j).  The variant with 256 entries 2^(j/256) (|r| <=
 // ln2/512, so exp(r) - 1 needs terms only up to r^4/24, the tail r^5/120 <=
-// 3.8e-17) saves one FP64 operation per exponential for 4 KB of shared memory
-// per block instead of 1 KB; a translation unit picks it by defining
-// DF_EXP_TABLE_BITS as 8 (the kernels generated for a loaded mechanism).
+// 3.8e-17) takes one FP64 operation fewer.  The surrogate's features use it;
+// the rate expressions use the fixed-point form of exp2fix.cuh.
 #pragma once
 
-#ifndef DF_EXP_TABLE_BITS
-#define DF_EXP_TABLE_BITS 6
-#endif
+#include "dev_common.cuh"  // small_int_to_double
 
 namespace df {
-
-constexpr int EXP_TAB_BITS = DF_EXP_TABLE_BITS;
-static_assert(EXP_TAB_BITS == 6 || EXP_TAB_BITS == 8, "exp table: 64 or 256 entries");
-constexpr int EXP_TAB_SIZE = 1 << EXP_TAB_BITS;
 
 static __device__ const double2 g_exp2_tab[64] = {
     {0x1.0000000000000p+0, 0x0.0p+0},
@@ -94,24 +87,10 @@ static __device__ const double2 g_exp2_tab[64] = {
     {0x1.fa7c1819e90d8p+0, 0x1.74853f3a5931ep-55},
 };
 
-// (double)v for |v| < 2^20, assembled from the integer's sign, leading one and
-// the bits below it with integer operations, so that the conversion takes no
-// slot of the narrow FP64 pipe (exact: every such integer is a double)
-__device__ __forceinline__ double small_int_to_double(int v) {
-  const unsigned a = (unsigned)(v < 0 ? -v : v);
-  const int lz = __clz(a | 1u);                  // the leading one of a > 0 at bit 31 - lz
-  const unsigned mant = ((a << lz) << 1) >> 12;  // the (at most 19) bits below it, left-aligned
-  const unsigned hi = ((unsigned)(v < 0) << 31) | ((unsigned)(1023 + 31 - lz) << 20) | mant;
-  return __hiloint2double(a != 0u ? (int)hi : 0, 0);
-}
-
 // 2^(j/256) as double-doubles (gen_exptab.py, 60-digit evaluation)
 static __device__ const double2 g_exp2_tab256[256] = {
 #include "fastexp_table256.inc"
 };
-
-// the table the kernels of this translation unit stage into shared memory
-__device__ __forceinline__ const double2* exp_table_src() { return EXP_TAB_BITS == 8 ? g_exp2_tab256 : g_exp2_tab; }
 
 // the reduction and polynomial of exp_tang for |x| < 700 (no range guard), with
 // a table of 2^B entries
@@ -148,24 +127,6 @@ __device__ __forceinline__ double exp_tang_core_b(double x, const double2* tab) 
   return __hiloint2double(__double2hiint(s) + (int)((unsigned)m << 20), __double2loint(s));
 }
 
-__device__ __forceinline__ double exp_tang_core(double x, const double2* tab) {
-  return exp_tang_core_b<EXP_TAB_BITS>(x, tab);
-}
-
-// exp of two arguments at once: both reductions and polynomials in one
-// straight-line block (two independent dependency chains for the scheduler),
-// the rare |x| >= 700 / inf / NaN cases fixed up afterwards
-__device__ __forceinline__ void exp_tang2(double x1, double x2, const double2* tab, double& e1, double& e2) {
-  const bool big1 = (__double2hiint(x1) & 0x7fffffff) >= 0x4085E000;
-  const bool big2 = (__double2hiint(x2) & 0x7fffffff) >= 0x4085E000;
-  e1 = exp_tang_core(big1 ? 0.0 : x1, tab);
-  e2 = exp_tang_core(big2 ? 0.0 : x2, tab);
-  if (big1 | big2) {
-    if (big1) e1 = exp(x1);
-    if (big2) e2 = exp(x2);
-  }
-}
-
 template <int B>
 __device__ __forceinline__ double exp_tang_b(double x, const double2* tab) {
   // |x| >= 700, inf and NaN, tested on the high word with integer operations
@@ -175,6 +136,6 @@ __device__ __forceinline__ double exp_tang_b(double x, const double2* tab) {
   return exp_tang_core_b<B>(x, tab);
 }
 
-__device__ __forceinline__ double exp_tang(double x, const double2* tab) { return exp_tang_b<EXP_TAB_BITS>(x, tab); }
+__device__ __forceinline__ double exp_tang(double x, const double2* tab) { return exp_tang_b<6>(x, tab); }
 
 }  // namespace df

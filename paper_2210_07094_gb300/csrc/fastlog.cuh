@@ -12,7 +12,7 @@
 // Troe quantities enter as addends).  Zero, negative, subnormal, inf and NaN
 // arguments go to the library log().  About 13 FP64 operations.
 #pragma once
-#include "fastexp.cuh"  // small_int_to_double
+#include "dev_common.cuh"
 
 namespace df {
 

@@ -59,16 +59,14 @@ __global__ void __launch_bounds__(128) k_eval_thread(EvalArgs a) {
   extern __shared__ double smem[];
   const int tid = threadIdx.x, stride = blockDim.x;
   const double* blob = a.blob;
-  double2* etab = reinterpret_cast<double2*>(smem);
-  for (int i = tid; i < 64; i += stride) etab[i] = g_exp2_tab[i];
-  int boff = 128;
+  int boff = 0;
   if (a.stage_blob) {
-    for (int i = tid; i < a.d.total; i += stride) smem[boff + i] = a.blob[i];
-    blob = smem + boff;
-    boff += blob_smem_doubles(a.d);
+    for (int i = tid; i < a.d.total; i += stride) smem[i] = a.blob[i];
+    blob = smem;
+    boff = blob_smem_doubles(a.d);
   }
   __syncthreads();
-  const MechView mv = make_view(blob, a.d, etab);
+  const MechView mv = make_view(blob, a.d);
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + tid;
   if (c >= a.ncells) return;
   double* ws = smem + boff + tid;
@@ -98,17 +96,15 @@ template <bool CONSTV>
 __global__ void __launch_bounds__(256, 1) k_integrate_warp(IntegArgs a, const int* csr, WarpWS L) {
   extern __shared__ double smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double2* etab = reinterpret_cast<double2*>(smem);
-  for (int i = tid; i < 64; i += blockDim.x) etab[i] = g_exp2_tab[i];
-  int boff = 128;
+  int boff = 0;
   const double* blob = a.blob;
   if (a.stage_blob) {
-    for (int i = tid; i < a.d.total; i += blockDim.x) smem[boff + i] = a.blob[i];
-    blob = smem + boff;
-    boff += blob_smem_doubles(a.d);
+    for (int i = tid; i < a.d.total; i += blockDim.x) smem[i] = a.blob[i];
+    blob = smem;
+    boff = blob_smem_doubles(a.d);
   }
   __syncthreads();
-  const MechView mv = make_view(blob, a.d, etab);
+  const MechView mv = make_view(blob, a.d);
   const int N = a.d.N, n = N + 1;
   double* ws = smem + boff + (size_t)warp * L.total;
   double* y = ws + L.y;
@@ -274,14 +270,11 @@ template <bool WITH_J>
 __global__ void __launch_bounds__(256) k_eval_warp(EvalArgs a, const int* csr, WarpWS L) {
   extern __shared__ double smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  double2* etab = reinterpret_cast<double2*>(smem);
-  for (int i = tid; i < 64; i += blockDim.x) etab[i] = g_exp2_tab[i];
-  __syncthreads();
-  const MechView mv = make_view(a.blob, a.d, etab);
+  const MechView mv = make_view(a.blob, a.d);
   const int N = a.d.N, n = N + 1;
   const int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (c >= a.ncells) return;
-  double* ws = smem + 128 + (size_t)warp * L.total;
+  double* ws = smem + (size_t)warp * L.total;
   for (int i = lane; i < n; i += 32) ws[L.y + i] = i == 0 ? a.T[c] : a.Y[(int64_t)(i - 1) * a.ncells + c];
   __syncwarp();
   const double q = warp_eval<WITH_J>(mv, csr, N, 10.0 * a.p[c], ws, L, L.y);
@@ -405,7 +398,7 @@ namespace {
 
 template <int NS>
 size_t thread_smem_bytes(const MechDims& d, int threads, bool stage) {
-  return sizeof(double) * (2 * EXP_TAB_SIZE + (stage ? blob_smem_doubles(d) : 0) + (size_t)thread_ws_doubles<NS>() * threads);
+  return sizeof(double) * ((stage ? blob_smem_doubles(d) : 0) + (size_t)thread_ws_doubles<NS>() * threads);
 }
 
 template <int NS>
@@ -496,14 +489,13 @@ namespace {
 int warp_shape(const df_mech* m, const WarpWS& L, bool want_stage, int max_warps, int* warps, int* stage,
                size_t* smem) {
   const size_t per_warp = sizeof(double) * (size_t)L.total;
-  const size_t fixed = sizeof(double) * 128;
   const size_t blob = sizeof(double) * (size_t)blob_smem_doubles(m->dims);
   // the mechanism staged in shared memory where that costs no warp; where
   // leaving it in global memory (read through L1) fits one more warp per
   // block, more warps win (they keep the narrow FP64 pipe busier)
   int best_w = 0, best_st = 0;
   for (int st = want_stage ? 1 : 0; st >= 0; --st) {
-    const size_t base = fixed + (st ? blob : 0);
+    const size_t base = st ? blob : 0;
     if (base + per_warp > m->max_smem_optin) continue;
     const int w = std::min((int)((m->max_smem_optin - base) / per_warp), max_warps);
     if (w > best_w) {
@@ -514,7 +506,7 @@ int warp_shape(const df_mech* m, const WarpWS& L, bool want_stage, int max_warps
   if (best_w > 0) {
     *warps = best_w;
     *stage = best_st;
-    *smem = fixed + (best_st ? blob : 0) + per_warp * best_w;
+    *smem = (best_st ? blob : 0) + per_warp * best_w;
     return DF_OK;
   }
   return set_error(DF_EUNSUPPORTED, "warp-path workspace exceeds shared memory");

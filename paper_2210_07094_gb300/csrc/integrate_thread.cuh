@@ -66,16 +66,14 @@ __global__ void __launch_bounds__(128, 1) k_integrate_thread(IntegArgs a) {
   const int tid = threadIdx.x;
   const int stride = BT > 0 ? BT : blockDim.x;
   const double* blob = a.blob;
-  double2* etab = reinterpret_cast<double2*>(smem);
-  for (int i = tid; i < EXP_TAB_SIZE; i += stride) etab[i] = exp_table_src()[i];
-  int boff = 2 * EXP_TAB_SIZE;
+  int boff = 0;
   if (a.stage_blob) {
-    for (int i = tid; i < a.d.total; i += stride) smem[boff + i] = a.blob[i];
-    blob = smem + boff;
-    boff += blob_smem_doubles(a.d);
+    for (int i = tid; i < a.d.total; i += stride) smem[i] = a.blob[i];
+    blob = smem;
+    boff = blob_smem_doubles(a.d);
   }
   __syncthreads();
-  const MechView mv = make_view(blob, a.d, etab);
+  const MechView mv = make_view(blob, a.d);
   double* ws = smem + boff + tid;
   typedef SVT<double, BT> V;
   constexpr int nv = EVAL::kSpeciesVectors ? NS : 0;

@@ -3,6 +3,7 @@
 // of the integrator's FP64 roofline fraction.
 #include "common.cuh"
 #include "../../include/df_probe.h"
+#include "exp2fix.cuh"
 #include "fastexp.cuh"
 #include "fastlog.cuh"
 
@@ -45,6 +46,11 @@ __global__ void k_exp_probe(const double* x, double* y, long long n) {
   if (i < n) y[i] = exp_tang_b<B>(x[i], tab);
 }
 
+__global__ void k_exp_rate_probe(const double* x, double* y, long long n) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = exp_rate(x[i]);
+}
+
 __global__ void k_log_probe(const double* x, double* y, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] = log_tab(x[i]);
@@ -59,6 +65,13 @@ extern "C" int df_probe_log(const double* x, double* y, long long n, void* strea
   if (n == 0) return DF_OK;
   k_log_probe<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(x, y, n);
   return cuda_check(cudaGetLastError(), "log probe kernel");
+}
+
+extern "C" int df_probe_exp_rate(const double* x, double* y, long long n, void* stream) {
+  if (n < 0 || (n > 0 && (!x || !y))) return set_error(DF_EINVAL, "df_probe_exp_rate: bad arguments");
+  if (n == 0) return DF_OK;
+  k_exp_rate_probe<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(x, y, n);
+  return cuda_check(cudaGetLastError(), "exp probe kernel");
 }
 
 extern "C" int df_probe_exp(const double* x, double* y, long long n, int table_bits, void* stream) {
