@@ -42,16 +42,16 @@ FLOP_PER_SUBSTEP = 16531
 TRAFFIC_PER_LAUNCH = 231775232 + 235842048
 # hash of the device sources that kernel is built from, when the two counters
 # above were taken; a different hash at run time marks them stale in the line
-COUNTERS_SOURCES = ("integrate_thread.cuh", "rosenbrock.cuh", "chem_thread.cuh", "dev_common.cuh", "fastexp.cuh",
-                    "fastexp_table256.inc", "fastlog.cuh", "fastlog_table.inc", "codegen.cu")
+COUNTERS_SOURCES = ("integrate_thread.cuh", "rosenbrock.cuh", "chem_thread.cuh", "dev_common.cuh", "exp2fix.cuh",
+                    "exp2fix_table.inc", "log2fix.cuh", "log2fix_table.inc", "codegen.cu")
 COUNTERS_SOURCE_HASH = "1f85abfcfe201580"
 # the same for the 50-species one-warp-per-cell path: FP64 operations per
 # substep from ncu's DP thread-instruction counters of one launch on 8192 cells
 # of the 50-species field (2*DFMA + DADD + DMUL over its substeps), and the
 # hash of the sources of that kernel when they were taken
 FLOP_PER_SUBSTEP_50 = 352115
-COUNTERS50_SOURCES = ("integrate.cu", "chem_warp.cuh", "chem_thread.cuh", "dev_common.cuh", "fastexp.cuh",
-                      "fastlog.cuh", "fastlog_table.inc")
+COUNTERS50_SOURCES = ("integrate.cu", "chem_warp.cuh", "chem_thread.cuh", "dev_common.cuh", "exp2fix.cuh",
+                      "exp2fix_table.inc", "log2fix.cuh", "log2fix_table.inc")
 COUNTERS50_SOURCE_HASH = "b9f7ab353c77172e"
 
 

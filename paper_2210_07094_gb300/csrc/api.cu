@@ -100,9 +100,9 @@ int df_mech_load(const char* path, df_mech** out) {
     m->smem_per_sm = prop.sharedMemPerMultiprocessor;
     m->smem_reserved_per_block = prop.reservedSharedMemPerBlock;
   }
-  if (!rc) rc = cuda_check(cudaMalloc(&m->blob_dev, sizeof(double) * m->dims.total + 8), "cudaMalloc blob");
+  if (!rc) rc = cuda_check(cudaMalloc(&m->blob_dev, sizeof(double) * m->dims.allocated() + 8), "cudaMalloc blob");
   if (!rc)
-    rc = cuda_check(cudaMemcpy(m->blob_dev, m->blob_host.data(), sizeof(double) * m->dims.total,
+    rc = cuda_check(cudaMemcpy(m->blob_dev, m->blob_host.data(), sizeof(double) * m->dims.allocated(),
                                cudaMemcpyHostToDevice),
                     "upload mechanism");
   if (!rc) rc = cuda_check(cudaMalloc(&m->csr_dev, sizeof(int) * m->csr_host.size()), "cudaMalloc csr");

@@ -19,18 +19,17 @@
 #pragma once
 #include "dev_common.cuh"
 #include "dual.cuh"
-#include "exp2fix.cuh"
-#include "fastlog.cuh"
+#include "log2fix.cuh"
 
 namespace df {
 
-// ln and log10 of the rate expressions by the table-driven logarithm (the
+// ln and log10 of the rate expressions by the fixed-point logarithm (the
 // dual-number versions carry the derivative d/x)
-__device__ __forceinline__ double fast_log(double x) { return log_tab(x); }
-__device__ __forceinline__ Dual fast_log(const Dual& x) { return Dual(log_tab(x.v), x.d / x.v); }
-__device__ __forceinline__ double fast_log10(double x) { return log10_tab(x); }
+__device__ __forceinline__ double fast_log(double x) { return log_rate(x); }
+__device__ __forceinline__ Dual fast_log(const Dual& x) { return Dual(log_rate(x.v), x.d / x.v); }
+__device__ __forceinline__ double fast_log10(double x) { return log10_rate(x); }
 __device__ __forceinline__ Dual fast_log10(const Dual& x) {
-  return Dual(log10_tab(x.v), x.d / (x.v * 2.302585092994045684));
+  return Dual(log10_rate(x.v), x.d / (x.v * 2.302585092994045684));
 }
 
 // strided view of a per-thread vector (any scalar type) in shared memory; a
@@ -49,6 +48,7 @@ struct MechView {
   const double* rx;
   const double* tr;
   const double* eff;
+  const long long* fix;  // ln A as fixed-point logarithms (generated evaluation only)
   int M;
 };
 
@@ -58,6 +58,7 @@ __device__ __forceinline__ MechView make_view(const double* blob, const MechDims
   v.rx = blob + d.off_rx;
   v.tr = blob + d.off_tr;
   v.eff = blob + d.off_eff;
+  v.fix = nullptr;
   v.M = d.M;
   return v;
 }
@@ -637,7 +638,7 @@ __device__ __forceinline__ bool lu_factor(SVT<double, ST> A, int* piv) {
         A[p * n + j] = t;
       }
     }
-    const double inv = 1.0 / A[k * n + k];
+    const double inv = rcp_any(A[k * n + k]);
     A[k * n + k] = inv;
     for (int i = k + 1; i < n; ++i) {
       const double l = A[i * n + k] * inv;

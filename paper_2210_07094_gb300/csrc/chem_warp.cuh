@@ -93,7 +93,7 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
   PV C{ws + L.C}, gRT{ws + L.gRT}, hRT{ws + L.hRT};
   double* wdot = ws + L.wdot;  // the g/RT slots, once the rates have read them
   const double T = y[0];
-  const double lnT = log_tab(T);
+  const double lnT = log_rate(T);
   const double invT = rcp_nr(T);
   // thermo and sum Y/W
   double sYW = 0.0;

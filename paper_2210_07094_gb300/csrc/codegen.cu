@@ -6,17 +6,19 @@
 // species vectors (C, wdot, g/RT, h/RT, cp/R) in shared memory, because those
 // indices are only known at run time.  For a loaded mechanism the library can
 // instead emit the evaluation of f and J as straight-line code with the
-// species indices, the reactant / product counts and the reaction types as
-// literals (the numbers -- ln A, beta, Ea/R, efficiencies, Troe parameters,
-// NASA-7 coefficients -- are still read from the blob, so df_mech_set_lnA keeps
-// working), compile it with NVRTC into a module holding the same persistent
-// kernel (integrate_thread.cuh) with that evaluation policy, and launch it
-// through the driver API.  The species vectors then live in registers, no
-// reaction metadata is decoded and no branch depends on the reaction, and the
-// shared memory per thread drops to J and the six stage vectors.  The
-// operations are the mechanism-independent kernel's, in the same order; the
-// two compilations may contract different multiply-adds, so cells agree to
-// rounding.
+// species indices, the reactant / product counts, the reaction types and the
+// mechanism's numbers as literals (ln A is still read from the blob, so
+// df_mech_set_lnA keeps working), compile it with NVRTC into a module holding
+// the same persistent kernel (integrate_thread.cuh) with that evaluation
+// policy, and launch it through the driver API.  The species vectors then live
+// in registers, no reaction metadata is decoded and no branch depends on the
+// reaction, and the shared memory per thread drops to W and one vector.
+//
+// Two evaluations are generated.  gen_fixed forms the exponents of the rate
+// constants in fixed point and is what cells run; gen_eval, the
+// mechanism-independent operations in FP64, takes the states outside the
+// fixed-point range (temperatures, ln A, states that are not finite).  Both
+// agree with the mechanism-independent kernel to rounding.
 //
 // NVRTC is opened at run time (dlopen); the driver entry points come through
 // cudaGetDriverEntryPointByVersion.  If either is missing, the headers cannot
@@ -281,22 +283,571 @@ void emit_eval(std::ostringstream& o, const df_mech* m) {
     << "  return -Hw;\n}\n\n";
 }
 
+// ---------------------------------------------------------------------------
+// the fixed-point evaluation
+// ---------------------------------------------------------------------------
+
+// |c| 2^s, or |c| log2(e) 2^s, as a 64-bit integer and the left shift its use
+// still needs (0 unless the value is too large for 64 bits).  Integer
+// arithmetic only: the same digits on every host.
+void fixed_literal(double c, bool log2e, int s, uint64_t* lit, int* shift) {
+  *lit = 0;
+  *shift = 0;
+  if (c == 0.0) return;
+  int e;
+  const uint64_t m = (uint64_t)std::ldexp(std::frexp(std::fabs(c), &e), 53);  // |c| = m 2^(e - 53)
+  const unsigned __int128 p = log2e ? (unsigned __int128)m * EXP2FIX_LOG2E_HALF : (unsigned __int128)m << 63;
+  int bits = 64;
+  while (bits < 128 && (p >> bits) != 0) ++bits;
+  const int r0 = 116 - e - s;  // |c| (log2 e) 2^s = p 2^-r0
+  int r = std::max(r0, bits - 64);
+  if (r > 126) return;
+  unsigned __int128 v = (p + ((unsigned __int128)1 << (r - 1))) >> r;
+  if ((v >> 64) != 0) {
+    ++r;
+    v = (p + ((unsigned __int128)1 << (r - 1))) >> r;
+  }
+  *lit = (uint64_t)v;
+  *shift = r - r0;
+}
+
+std::string hex64(uint64_t v) {
+  char b[32];
+  snprintf(b, sizeof b, "0x%llxull", (unsigned long long)v);
+  return b;
+}
+
+// "+= c * mono" in units of 2^-53, mono a fixed-point variable of the given scale
+std::string fixed_term(const std::string& dst, double c, bool log2e, const char* mono, int scale) {
+  uint64_t l;
+  int sh;
+  fixed_literal(c, log2e, 117 - scale, &l, &sh);
+  if (l == 0) return "";
+  std::string e = std::string("mul_fixed(") + mono + ", " + hex64(l) + ")";
+  if (sh) e = "(" + e + " << " + std::to_string(sh) + ")";
+  return "    " + dst + (c < 0.0 ? " -= " : " += ") + "(int64_t)" + e + ";\n";
+}
+
+// c log2(e) in units of 2^-53
+std::string fixed_const(double c) {
+  uint64_t l;
+  int sh;
+  fixed_literal(c, true, 53, &l, &sh);
+  return std::string(c < 0.0 ? "-" : "") + "(int64_t)(" + hex64(l) + (sh ? " << " + std::to_string(sh) : "") + ")";
+}
+
+constexpr double kFixTHi = 8000.0;
+
+struct Rx {
+  std::vector<int> r, p;  // species entries
+  std::vector<int> nu;    // net coefficients, by species
+  std::vector<int> spc;   // species of the reaction
+  int type = 0, eff = -1, troe = -1, dnu = 0;
+  bool rev = false;
+  double b = 0, E = 0;
+};
+
+std::vector<Rx> reactions_of(const df_mech* m) {
+  std::vector<Rx> out(m->dims.M);
+  for (int j = 0; j < m->dims.M; ++j) {
+    Rx& x = out[j];
+    const RxMeta mt = meta_of(m, j);
+    const RxSlots sl = slots_of(m, j);
+    for (int i = 0; i < (mt.nrnp & 15); ++i) x.r.push_back(mt.reac[i]);
+    for (int i = 0; i < (mt.nrnp >> 4); ++i) x.p.push_back(mt.prod[i]);
+    x.nu.assign(m->dims.N, 0);
+    for (int k : x.r) x.nu[k] -= 1;
+    for (int k : x.p) x.nu[k] += 1;
+    for (const auto* side : {&x.r, &x.p})
+      for (int k : *side)
+        if (std::find(x.spc.begin(), x.spc.end(), k) == x.spc.end()) x.spc.push_back(k);
+    x.type = mt.flags & 3;
+    x.rev = (mt.flags & 4) != 0;
+    x.eff = sl.eff;
+    x.troe = sl.troe;
+    x.dnu = (int)x.p.size() - (int)x.r.size();
+    x.b = m->blob_host[m->dims.off_rx + RX_REC * j + 1];
+    x.E = m->blob_host[m->dims.off_rx + RX_REC * j + 2];
+  }
+  return out;
+}
+
+// the temperatures the fixed-point evaluation covers: from the lowest one at
+// which every exponent, with any ln A of lnA_fits_fixed, stays within 1000 octaves
+// (sampled every 2% and with 5% to spare); 0 if there is none
+double fixed_T_low(const df_mech* m, const std::vector<Rx>& rx) {
+  const double L2E = 1.4426950408889634;
+  auto sp = [&](int k, int i) { return m->blob_host[m->dims.off_sp + SP_REC * k + i]; };
+  for (double lo : {100.0, 150.0, 200.0, 250.0, 300.0, 400.0}) {
+    double worst = 0.0;
+    for (double T = lo; T < kFixTHi * 1.02; T *= 1.02) {
+      std::vector<double> g(m->dims.N);
+      for (int k = 0; k < m->dims.N; ++k)
+        g[k] = L2E * ((sp(k, 2) - sp(k, 8)) - sp(k, 2) * std::log(T) -
+                      T * (sp(k, 3) / 2 + T * (sp(k, 4) / 6 + T * (sp(k, 5) / 12 + T * sp(k, 6) / 20))) + sp(k, 7) / T);
+      for (const Rx& x : rx) {
+        const double kf = 400.0 + L2E * std::fabs(x.b * std::log(T) - x.E / T);
+        double sg = -x.dnu * L2E * (LOG_PSTD_RU - std::log(T));
+        for (int k : x.spc) sg += x.nu[k] * g[k];
+        worst = std::max({worst, kf, kf + std::fabs(sg)});
+        if (x.type == 2) {
+          const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
+          const double d = L2E * std::fabs(tr[0] + (tr[1] - x.b) * std::log(T) - (tr[2] - x.E) / T);
+          worst = std::max({worst, d, kf + d, std::fabs(sg)});
+        }
+      }
+    }
+    if (worst * 1.05 <= 1000.0) return lo;  // false for NaN and infinity
+  }
+  return 0.0;
+}
+
+// "K C[a] C[b] ..." and, with derivatives, d(K prod C)/dC_l of each distinct
+// species: statements that define `name`p and `name`d<l>
+std::string product_code(const std::string& name, const std::string& K, std::vector<int> e, bool deriv) {
+  std::ostringstream o;
+  auto C = [](int k) { return "C[" + std::to_string(k) + "]"; };
+  auto d = [&](int k) { return name + "d" + std::to_string(k); };
+  if (!deriv) {
+    o << "    const double " << name << "p = " << K;
+    for (int k : e) o << " * " << C(k);
+    o << ";\n";
+    return o.str();
+  }
+  // equal species first
+  if (e.size() == 3 && e[0] != e[1]) {
+    if (e[0] == e[2]) std::swap(e[1], e[2]);
+    else if (e[1] == e[2]) std::swap(e[0], e[2]);
+  }
+  const std::string t = "    const double ";
+  if (e.size() == 1) {
+    o << t << d(e[0]) << " = " << K << ";\n" << t << name << "p = " << K << " * " << C(e[0]) << ";\n";
+  } else if (e.size() == 2) {
+    if (e[0] == e[1]) {
+      o << t << name << "t = " << K << " * " << C(e[0]) << ";\n"
+        << t << d(e[0]) << " = 2.0 * " << name << "t;\n" << t << name << "p = " << name << "t * " << C(e[0]) << ";\n";
+    } else {
+      o << t << d(e[0]) << " = " << K << " * " << C(e[1]) << ";\n" << t << d(e[1]) << " = " << K << " * " << C(e[0])
+        << ";\n" << t << name << "p = " << d(e[1]) << " * " << C(e[1]) << ";\n";
+    }
+  } else if (e[0] == e[1] && e[1] == e[2]) {
+    o << t << name << "t = " << K << " * " << C(e[0]) << " * " << C(e[0]) << ";\n"
+      << t << d(e[0]) << " = 3.0 * " << name << "t;\n" << t << name << "p = " << name << "t * " << C(e[0]) << ";\n";
+  } else if (e[0] == e[1]) {
+    o << t << name << "t = " << K << " * " << C(e[0]) << ";\n"
+      << t << d(e[2]) << " = " << name << "t * " << C(e[0]) << ";\n"
+      << t << d(e[0]) << " = 2.0 * (" << name << "t * " << C(e[2]) << ");\n"
+      << t << name << "p = " << d(e[2]) << " * " << C(e[2]) << ";\n";
+  } else {
+    o << t << name << "t = " << K << " * " << C(e[0]) << ";\n"
+      << t << d(e[2]) << " = " << name << "t * " << C(e[1]) << ";\n"
+      << t << d(e[1]) << " = " << name << "t * " << C(e[2]) << ";\n"
+      << t << d(e[0]) << " = " << K << " * (" << C(e[1]) << " * " << C(e[2]) << ");\n"
+      << t << name << "p = " << d(e[2]) << " * " << C(e[2]) << ";\n";
+  }
+  return o.str();
+}
+
+// The evaluation the generated kernel runs: f and -J, the latter compact over
+// the temperature and the species some reaction changes (the inert ones have
+// zero rows).  The exponents of the rate constants -- ln A + b ln T - E/T, the
+// sums of g_k/RT and the pressure term, all times log2(e) -- are 64-bit
+// fixed-point sums in units of 2^-53 octave: an addition is two integer
+// instructions where an FP64 one occupies the pipe for 64 cycles, a product
+// about a quarter of one, and the result is the argument exp2_fixed wants, more
+// accurate than the rounded FP64 sums it replaces.  Only what multiplies
+// concentrations stays in FP64.  Returns false (nothing written) for states
+// outside the range the fixed-point words cover; the caller then takes gen_eval.
+void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& rx, const std::vector<int>& act,
+                double T_low) {
+  const int N = m->dims.N, NA = (int)act.size();
+  auto sp = [&](int k, int i) { return m->blob_host[m->dims.off_sp + SP_REC * k + i]; };
+  std::vector<int> col(N, -1);  // species -> compact index
+  for (int a = 1; a < NA; ++a) col[act[a] - 1] = a;
+  auto S = [](int k) { return std::to_string(k); };
+  auto W = [&](int a, int b) { return "W[" + std::to_string(a * NA + b) + "]"; };
+  bool any_collider = false, any_inert = false;  // any_inert: a rate depends on an inert species alone
+  std::vector<bool> used(N, false);  // species whose g/RT some reaction needs
+  for (const Rx& x : rx) {
+    any_collider = any_collider || x.type != 0;
+    for (int k : x.spc) {
+      if (x.nu[k] != 0) used[k] = true;
+      if (col[k] < 0) any_inert = true;
+    }
+    for (int l = 0; l < N; ++l)
+      if (x.type != 0 && col[l] < 0 && m->blob_host[m->dims.off_eff + N * x.eff + l] != 1.0) any_inert = true;
+  }
+  o << "template <bool WITH_J, int ST>\n"
+    << "__device__ __forceinline__ bool gen_fixed(const MechView& mv, const double pc, const double (&y)[" << N + 1
+    << "], double (&f)[" << N + 1 << "], SVT<double, ST> W) {\n"
+    << "  constexpr int NS = " << N << ";\n"
+    << "  const double T = y[0];\n"
+    << "  if (!mv.fix[" << m->dims.M << "] || !(T >= " << lit(T_low) << " && T < " << lit(kFixTHi) << ")) return false;\n"
+    << "  double C[NS], cpW[NS];  // cpW: cp_k / (R W_k)\n"
+    << "  double sumYW = 0.0, cpm = 0.0;\n";
+  for (int k = 0; k < N; ++k) {
+    std::vector<double> aw = {sp(k, 2), sp(k, 3), sp(k, 4), sp(k, 5), sp(k, 6)};
+    for (double& v : aw) v *= sp(k, 1);
+    o << "  C[" << k << "] = y[" << 1 + k << "] * " << lit(sp(k, 1)) << ";\n  sumYW += C[" << k << "];\n"
+      << "  cpW[" << k << "] = " << horner(aw, "T") << ";\n  cpm += y[" << 1 + k << "] * cpW[" << k << "];\n";
+  }
+  o << "  if (!rcp_in_range(sumYW) || !rcp_in_range(cpm) || !rcp_in_range(pc)) return false;\n"
+    << "  const double invT = rcp_fast(T), Wbar = rcp_fast(sumYW), invcp = rcp_fast(cpm * RU);\n"
+    << "  const double rho = pc * invT * (Wbar * " << lit(1.0 / RU) << ");\n"
+    << "  const double invrho = rcp_any(rho);\n"
+    << "  // log2 T, 1/T, T and its powers in fixed point\n"
+    << "  const uint64_t L = log2_fixed(T), I = pos_fixed<69>(invT), t1 = pos_fixed<50>(T);\n"
+    << "  const uint64_t t2 = mul_fixed(t1, t1);\n";
+  bool t3 = false, t4 = false;
+  for (int k = 0; k < N; ++k) {
+    t3 = t3 || (used[k] && sp(k, 5) != 0.0);
+    t4 = t4 || (used[k] && sp(k, 6) != 0.0);
+  }
+  if (t3) o << "  const uint64_t t3 = mul_fixed(t2, t1);\n";
+  if (t4) o << "  const uint64_t t4 = mul_fixed(t2, t2);\n";
+  o << "  const int64_t lp = " << fixed_const(LOG_PSTD_RU) << " - (int64_t)(L >> 7);  // log2(p_std / (R T))\n"
+    << "  int64_t G[NS];  // g_k/RT log2(e)\n";
+  for (int k = 0; k < N; ++k) {
+    if (!used[k]) continue;
+    const std::string g = "G[" + S(k) + "]";
+    o << "  {\n    " << g << " = " << fixed_const(sp(k, 2) - sp(k, 8)) << ";\n"
+      << fixed_term(g, -sp(k, 2), false, "L", 60) << fixed_term(g, -0.5 * sp(k, 3), true, "t1", 50)
+      << fixed_term(g, -sp(k, 4) / 6.0, true, "t2", 36) << fixed_term(g, -sp(k, 5) / 12.0, true, "t3", 22)
+      << fixed_term(g, -sp(k, 6) / 20.0, true, "t4", 8) << fixed_term(g, sp(k, 7), true, "I", 69) << "  }\n";
+  }
+  for (int k = 0; k < N; ++k) o << "  C[" << k << "] *= rho;\n";
+  if (any_collider) {
+    o << "  double ctot = C[0];\n";
+    for (int k = 1; k < N; ++k) o << "  ctot += C[" << k << "];\n";
+  }
+  // species enthalpies h/RT of the reacting species; with J also times 1/T
+  o << "  double hRT[NS], hT[NS], w[NS], sM[NS], sN[NS];\n  const double invT2 = invT * invT;\n"
+    << "  (void)hT; (void)sM; (void)sN; (void)invT2;\n";
+  for (int a = 1; a < NA; ++a) {
+    const int k = act[a] - 1;
+    std::vector<double> hs = {sp(k, 2), sp(k, SP_H), sp(k, SP_H + 1), sp(k, SP_H + 2), sp(k, SP_H + 3)};
+    o << "  hRT[" << k << "] = " << horner(hs, "T") << " + " << lit(sp(k, 7)) << " * invT;\n"
+      << "  if (WITH_J) hT[" << k << "] = hRT[" << k << "] * invT;\n";
+  }
+  // accumulators start at zero where their first contribution is conditional
+  // (falloff reactions without a low-pressure rate contribute nothing)
+  std::vector<bool> w_set(N, false), sM_set(N, false), W_set(NA * NA, false);
+  {
+    std::vector<bool> wz(N, true), Wz(NA * NA, true), sMz(N, true);
+    std::vector<bool> seen_w(N, false), seen_W(NA * NA, false), seen_M(N, false);
+    for (const Rx& x : rx) {
+      for (int k : x.spc) {
+        if (x.nu[k] == 0) continue;
+        const int a = col[k];
+        if (!seen_w[k]) wz[k] = x.type == 2;
+        seen_w[k] = true;
+        if (x.type != 0) {
+          if (!seen_M[k]) sMz[k] = x.type == 2;
+          seen_M[k] = true;
+        }
+        std::vector<int> cols = {0};
+        for (int l : x.spc)
+          if (col[l] > 0 && (x.rev || std::find(x.r.begin(), x.r.end(), l) != x.r.end())) cols.push_back(col[l]);
+        for (int c : cols) {
+          if (!seen_W[a * NA + c]) Wz[a * NA + c] = x.type == 2;
+          seen_W[a * NA + c] = true;
+        }
+        if (x.type != 0)
+          for (int l = 0; l < N; ++l)
+            if (m->blob_host[m->dims.off_eff + N * x.eff + l] != 1.0 && col[l] > 0) {
+              const int c = col[l];
+              if (!seen_W[a * NA + c]) Wz[a * NA + c] = true;
+              seen_W[a * NA + c] = true;
+            }
+      }
+    }
+    for (int a = 1; a < NA; ++a) {
+      const int k = act[a] - 1;
+      if (wz[k]) {
+        o << "  w[" << k << "] = 0.0;\n";
+        w_set[k] = true;
+      }
+      if (any_collider && sMz[k]) {
+        o << "  if (WITH_J) sM[" << k << "] = 0.0;\n";
+        sM_set[k] = true;
+      }
+      if (any_inert) o << "  if (WITH_J) sN[" << k << "] = 0.0;\n";
+    }
+    o << "  if (WITH_J) {\n";
+    for (int a = 1; a < NA; ++a)
+      for (int b = 0; b < NA; ++b)
+        if (Wz[a * NA + b]) {
+          o << "    " << W(a, b) << " = 0.0;\n";
+          W_set[a * NA + b] = true;
+        }
+    o << "  }\n";
+  }
+  // the rows take -d w_k/d(...) , species columns pre-scaled by W_k / W_l
+  auto addW = [&](int a, int b, double c, const std::string& v) {
+    std::ostringstream s;
+    const bool set = W_set[a * NA + b];
+    W_set[a * NA + b] = true;
+    s << "      " << W(a, b);
+    if (c == 1.0) s << (set ? " -= " : " = -") << v << ";\n";
+    else if (c == -1.0) s << (set ? " += " : " = ") << v << ";\n";
+    else s << (set ? " -= " : " = -") << lit(c) << " * " << v << ";\n";
+    return s.str();
+  };
+  auto add1 = [&](std::vector<bool>& set, const char* arr, int k, int c, const std::string& v) {
+    std::ostringstream s;
+    s << arr << "[" << k << "]";
+    const bool st = set[k];
+    set[k] = true;
+    if (c == 1) s << (st ? " += " : " = ") << v << ";\n";
+    else if (c == -1) s << (st ? " -= " : " = -") << v << ";\n";
+    else s << (st ? " += " : " = ") << c << ".0 * " << v << ";\n";
+    return s.str();
+  };
+  for (size_t j = 0; j < rx.size(); ++j) {
+    const Rx& x = rx[j];
+    o << "  {  // rate " << j << "\n    int64_t x = mv.fix[" << j << "];\n"
+      << fixed_term("x", x.b, false, "L", 60) << fixed_term("x", -x.E, true, "I", 69);
+    if (x.rev) {
+      std::string sg;
+      for (int k : x.spc)
+        for (int i = 0; i < std::abs(x.nu[k]); ++i) sg += (x.nu[k] > 0 ? " + G[" : " - G[") + S(k) + "]";
+      for (int i = 0; i < std::abs(x.dnu); ++i) sg += x.dnu > 0 ? " - lp" : " + lp";
+      o << "    const int64_t xc = 0" << sg << ";\n";
+    }
+    if (x.type != 0) {
+      o << "    double Mc = ctot;\n";
+      for (int l = 0; l < N; ++l) {
+        const double e = m->blob_host[m->dims.off_eff + N * x.eff + l];
+        if (e != 1.0) o << "    Mc += " << lit(e - 1.0) << " * C[" << l << "];\n";
+      }
+    }
+    // d ln k / dT and d ln K_c / dT
+    std::ostringstream dl;
+    dl << "      const double dk = " << lit(x.b) << " * invT + " << lit(x.E) << " * invT2;\n";
+    std::string dKc = "0.0";
+    for (int k : x.spc)
+      for (int i = 0; i < std::abs(x.nu[k]); ++i) dKc += (x.nu[k] > 0 ? " + hT[" : " - hT[") + S(k) + "]";
+    for (int i = 0; i < std::abs(x.dnu); ++i) dKc += x.dnu > 0 ? " - invT" : " + invT";
+    auto has_dq = [&](int l) {
+      return std::find(x.r.begin(), x.r.end(), l) != x.r.end() ||
+             (x.rev && std::find(x.p.begin(), x.p.end(), l) != x.p.end());
+    };
+    // the Jacobian rows from dq<l>, dqT and, with a collider, dqM
+    auto rows = [&]() {
+      std::ostringstream s;
+      for (int k : x.spc) {
+        if (x.nu[k] == 0) continue;
+        const int a = col[k];
+        s << addW(a, 0, x.nu[k], "dqT");
+        for (int l : x.spc) {
+          if (!has_dq(l)) continue;
+          if (col[l] > 0)
+            s << addW(a, col[l], l == k ? (double)x.nu[k] : x.nu[k] * (sp(k, 0) * sp(l, 1)), "dq" + S(l));
+          else  // an inert species: no column, but its share of s_k
+            s << "      sN[" << k << "] += " << lit(x.nu[k]) << " * (dq" << l << " * C[" << l << "]);\n";
+        }
+        if (x.type != 0) {
+          s << "      " << add1(sM_set, "sM", k, x.nu[k], "dqM");
+          for (int l = 0; l < N; ++l) {
+            const double e = m->blob_host[m->dims.off_eff + N * x.eff + l];
+            if (e == 1.0) continue;
+            if (col[l] > 0)
+              s << addW(a, col[l], x.nu[k] * (e - 1.0) * (l == k ? 1.0 : sp(k, 0) * sp(l, 1)), "dqM");
+            else
+              s << "      sN[" << k << "] += " << lit(x.nu[k] * (e - 1.0)) << " * (dqM * C[" << l << "]);\n";
+          }
+        }
+      }
+      return s.str();
+    };
+    auto dqs = [&](const char* scale) {
+      std::ostringstream s;
+      for (int l : x.spc) {
+        if (!has_dq(l)) continue;
+        const bool inr = std::find(x.r.begin(), x.r.end(), l) != x.r.end();
+        const bool inp = x.rev && std::find(x.p.begin(), x.p.end(), l) != x.p.end();
+        std::string e = inr && inp ? "fd" + S(l) + " - bd" + S(l) : inr ? "fd" + S(l) : inp ? "-bd" + S(l) : "0.0";
+        s << "      const double dq" << l << " = " << (*scale ? std::string(scale) + " * (" + e + ")" : e) << ";\n"
+          << "      (void)dq" << l << ";\n";
+      }
+      return s.str();
+    };
+    std::ostringstream upd;
+    if (x.type != 2) {
+      o << "    const double kf = exp2_fixed(x);\n";
+      if (x.rev) o << "    const double kr = exp2_fixed(x + xc);\n";
+      for (int wj = 1; wj >= 0; --wj) {
+        if (wj) o << "    if (WITH_J) {\n";
+        else o << "    } else {\n";
+        // each branch starts from the same accumulators
+        const auto w0 = w_set, sM0 = sM_set;
+        const auto W0 = W_set;
+        o << product_code("f", "kf", x.r, wj);
+        if (x.rev) o << product_code("b", "kr", x.p, wj);
+        const std::string q0 = x.rev ? "fp - bp" : "fp";
+        if (x.type == 1) o << "      const double dqM = " << q0 << ";\n      (void)dqM;\n      const double q = Mc * dqM;\n";
+        else o << "      const double q = " << q0 << ";\n";
+        for (int k : x.spc)
+          if (x.nu[k] != 0) o << "      " << add1(w_set, "w", k, x.nu[k], "q");
+        if (wj) {
+          o << dl.str();
+          if (x.rev) o << "      const double dKc = " << dKc << ";\n";
+          if (!x.rev) o << "      const double dqT = q * dk;\n";
+          else if (x.type == 1) o << "      const double dqT = q * dk + (Mc * bp) * dKc;\n";
+          else o << "      const double dqT = q * dk + bp * dKc;\n";
+          o << dqs(x.type == 1 ? "Mc" : "") << rows();
+          w_set = w0;  // the other branch makes the same first updates of w
+        }
+        (void)W0;
+        (void)sM0;
+      }
+      o << "    }\n  }\n";
+      continue;
+    }
+    // Troe falloff: the expressions of rate_compute, the rate constants from the
+    // fixed-point exponents
+    const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
+    o << "    int64_t xd = " << fixed_const(tr[0]) << ";  // k0 / kinf\n"
+      << fixed_term("xd", tr[1] - x.b, false, "L", 60) << fixed_term("xd", -(tr[2] - x.E), true, "I", 69)
+      << "    const double kinf = exp2_fixed(x), Pr = exp2_fixed(xd) * Mc;\n"
+      << "    if (Pr > 0.0) {\n"
+      << "      double e3, e1;\n      exp_rate2(-T * " << lit(tr[4]) << ", -T * " << lit(tr[5]) << ", e3, e1);\n"
+      << "      const double e2 = exp_rate(" << lit(-tr[6]) << " * invT);\n"
+      << "      const double invKc = " << (x.rev ? "exp2_fixed(xc)" : "0.0") << ";\n"
+      << "      const double Fc = " << lit(1.0 - tr[3]) << " * e3 + " << lit(tr[3]) << " * e1 + e2;\n"
+      << "      const double Lc = log10_rate(Fc), cc = -0.4 - 0.67 * Lc, nn = 0.75 - 1.27 * Lc;\n"
+      << "      const double xl = log10_rate(Pr) + cc, den = nn - 0.14 * xl, den2 = den * den;\n"
+      << "      const double q1 = den2 * rcp_any(den2 + xl * xl);\n"
+      << "      const double F = exp_rate(LN10 * (Lc * q1)), onePr = rcp_any(1.0 + Pr);\n"
+      << "      const double kf = kinf * Pr * onePr * F, kr = kf * invKc;\n";
+    for (int wj = 1; wj >= 0; --wj) {
+      const auto w0 = w_set;
+      o << (wj ? "      if (WITH_J) {\n" : "      } else {\n") << product_code("f", "kf", x.r, wj);
+      if (x.rev) o << product_code("b", "kr", x.p, wj);
+      o << "      const double q = " << (x.rev ? "fp - bp" : "fp") << ";\n";
+      for (int k : x.spc)
+        if (x.nu[k] != 0) o << "      " << add1(w_set, "w", k, x.nu[k], "q");
+      if (wj) {
+        std::string Pf, Pb;
+        for (int k : x.r) Pf += (Pf.empty() ? "C[" : " * C[") + S(k) + "]";
+        for (int k : x.p) Pb += (Pb.empty() ? "C[" : " * C[") + S(k) + "]";
+        o << "      const double k0 = exp2_fixed(x + xd), rden = rcp_any(den), f1 = xl * rden;\n"
+          << "      const double df1_dL = nn * rden * rden;\n"
+          << "      const double df1_dLc = (-0.67 * den - xl * (-1.27 + 0.67 * 0.14)) * (rden * rden);\n"
+          << "      const double g2 = 2.0 * Lc * f1 * q1 * q1;\n"
+          << "      const double gpr = onePr - g2 * df1_dL, dlogF_dLc = q1 - g2 * df1_dLc;\n"
+          << "      const double dFc = " << lit(-(1.0 - tr[3]) * tr[4]) << " * e3 + " << lit(-tr[3] * tr[5])
+          << " * e1 + " << lit(tr[6]) << " * invT2 * e2;\n"
+          << "      const double dki = " << lit(x.b) << " * invT + " << lit(x.E) << " * invT2;\n"
+          << "      const double dk0 = " << lit(tr[1]) << " * invT + " << lit(tr[2]) << " * invT2;\n"
+          << "      const double dk = dki + gpr * (dk0 - dki) + dlogF_dLc * dFc * rcp_any(Fc);\n"
+          << "      const double dKc = " << dKc << ";\n"
+          << "      const double dqT = q * dk" << (x.rev ? " + bp * dKc" : "") << ";\n      (void)dKc;\n"
+          << "      const double dqM = k0 * F * gpr * onePr * (" << Pf << (x.rev ? " - " + Pb + " * invKc" : std::string())
+          << ");\n"
+          << dqs("") << rows();
+        w_set = w0;
+      }
+    }
+    o << "      }\n    }\n  }\n";
+  }
+  // heat release and f
+  o << "  double Hw = 0.0;\n";
+  for (int a = 1; a < NA; ++a) o << "  Hw += hRT[" << act[a] - 1 << "] * w[" << act[a] - 1 << "];\n";
+  for (int k = 0; k < N; ++k) {
+    if (col[k] > 0) o << "  f[" << 1 + k << "] = " << lit(sp(k, 0)) << " * (w[" << k << "] * invrho);\n";
+    else o << "  f[" << 1 + k << "] = 0.0;\n";
+  }
+  o << "  const double RT = RU * T;\n  f[0] = -(Hw * RT) * (invrho * invcp);\n";
+  // -J: row k holds -S'_kl = -(W_k / W_l) dw_k/dC_l; with s_k = sum_l S_kl C_l and
+  // a_k = W_k (Wbar / rho) (w_k - s_k) + W_k sM_k: d f_k/dY_l = S'_kl + a_k / W_l
+  // (gen_eval); the temperature row sums the finished rows
+  o << "  if (WITH_J) {\n    const double wb = Wbar * invrho;\n    double dcp = 0.0, cpf = 0.0;\n";
+  for (int a = 0; a < NA; ++a) o << "    double tr" << a << " = 0.0;\n";
+  for (int a = 1; a < NA; ++a) {
+    const int k = act[a] - 1;
+    o << "    {  // row of species " << k << "\n";
+    for (int b = 0; b < NA; ++b) o << "      const double v" << b << " = " << W(a, b) << ";\n";
+    o << "      double s = 0.0;\n";
+    for (int b = 1; b < NA; ++b) o << "      s -= v" << b << " * (rho * y[" << act[b] << "]);\n";
+    o << "      s = s * " << lit(sp(k, 1)) << ";\n";
+    if (any_collider) o << "      s += sM[" << k << "] * ctot;\n";
+    if (any_inert) o << "      s += sN[" << k << "];\n";
+    o << "      const double ws = w[" << k << "] - s, hw = hRT[" << k << "] * " << lit(sp(k, 1)) << ";\n"
+      << "      const double ak = " << lit(sp(k, 0)) << " * (wb * ws" << (any_collider ? " + sM[" + S(k) + "]" : std::string())
+      << ");\n"
+      << "      const double n0 = " << lit(sp(k, 0)) << " * invrho * (v0 - ws * invT);\n      " << W(a, 0)
+      << " = n0;\n      tr0 += hw * n0;\n";
+    for (int b = 1; b < NA; ++b)
+      o << "      const double n" << b << " = v" << b << " - ak * " << lit(sp(act[b] - 1, 1)) << ";\n      " << W(a, b)
+        << " = n" << b << ";\n      tr" << b << " += hw * n" << b << ";\n";
+    o << "    }\n";
+  }
+  for (int k = 0; k < N; ++k) {
+    const std::vector<double> d = {sp(k, 3), 2.0 * sp(k, 4), 3.0 * sp(k, 5), 4.0 * sp(k, 6)};
+    std::vector<double> dw(d);
+    for (double& v : dw) v *= sp(k, 1);
+    o << "    dcp += y[" << 1 + k << "] * (" << horner(dw, "T") << ");\n";
+    if (col[k] > 0) o << "    cpf += cpW[" << k << "] * f[" << 1 + k << "];\n";
+  }
+  o << "    const double rc = RU * invcp;\n    " << W(0, 0) << " = rc * (cpf + f[0] * dcp - T * tr0);\n";
+  for (int b = 1; b < NA; ++b)
+    o << "    " << W(0, b) << " = rc * (f[0] * cpW[" << act[b] - 1 << "] - T * tr" << b << ");\n";
+  o << "  }\n  return true;\n}\n\n";
+}
+
 }  // namespace
 
+// state entries (0: T, 1 + k: Y_k) of the generated kernel's linear systems: the
+// temperature and the species that some reaction changes
+static std::vector<int> active_entries(const df_mech* m) {
+  std::vector<int> act = {0};
+  const std::vector<Rx> rx = reactions_of(m);
+  for (int k = 0; k < m->dims.N; ++k)
+    if (std::any_of(rx.begin(), rx.end(), [k](const Rx& x) { return x.nu[k] != 0; })) act.push_back(1 + k);
+  return act;
+}
+
 std::string jit_thread_source(const df_mech* m) {
+  const int N = m->dims.N, n = N + 1;
+  const std::vector<Rx> rx = reactions_of(m);
+  const std::vector<int> act = active_entries(m);
+  const int NA = (int)act.size();
+  const double T_low = fixed_T_low(m, rx);
   std::ostringstream o;
-  o << "// generated for a " << m->dims.N << "-species / " << m->dims.M << "-reaction mechanism\n"
+  o << "// generated for a " << N << "-species / " << m->dims.M << "-reaction mechanism\n"
     << "#include \"integrate_thread.cuh\"\n\nnamespace df {\n\n";
   emit_eval(o, m);
+  if (T_low > 0.0) emit_fixed(o, m, rx, act, T_low);
+  std::string list;
+  for (int a : act) list += (list.empty() ? "" : ", ") + std::to_string(a);
   o << "struct GenEval {\n"
-    << "  static constexpr bool kSpeciesVectors = false;\n"
-    << "  template <int NS, bool WITH_J, bool CONSTV, int ST>\n"
-    << "  __device__ __forceinline__ static double run(const MechView& mv, double pc, const double (&y)[NS + 1],\n"
-    << "                                               double (&f)[NS + 1], SVT<double, ST> scratch, SVT<double, ST>,\n"
-    << "                                               SVT<double, ST>, SVT<double, ST>, SVT<double, ST>,\n"
-    << "                                               SVT<double, ST> Jv) {\n"
-    << "    static_assert(!CONSTV, \"generated evaluation: constant pressure\");\n"
-    << "    return gen_eval<WITH_J, ST>(mv, pc, y, f, Jv, scratch);\n  }\n};\n\n}  // namespace df\n";
+    << "  static constexpr bool kGenerated = true;\n"
+    << "  static constexpr int kN = " << N << ", kNA = " << NA << ";\n"
+    << "  // state entry (0: T, 1 + k: Y_k) of row a of the linear systems\n"
+    << "  __device__ static constexpr int act(int a) {\n    constexpr int t[] = {" << list << "};\n    return t[a];\n  }\n"
+    << "  // any state, one copy for all kernels of the module: the FP64 evaluation,\n"
+    << "  // its full Jacobian compacted and negated\n"
+    << "  template <bool WITH_J>\n"
+    << "  __device__ __noinline__ static void general(const MechView& mv, double pc, const double* y, double* f, double* W) {\n"
+    << "    double yl[" << n << "], fl[" << n << "], J[WITH_J ? " << n * n << " : 1], sM[" << N << "];\n"
+    << "    for (int i = 0; i < " << n << "; ++i) yl[i] = y[i];\n"
+    << "    gen_eval<WITH_J, 1>(mv, pc, yl, fl, SVT<double, 1>{J, 1}, SVT<double, 1>{sM, 1});\n"
+    << "    for (int i = 0; i < " << n << "; ++i) f[i] = fl[i];\n"
+    << "    if (WITH_J)\n#pragma unroll 1\n      for (int a = 0; a < " << NA << "; ++a)\n"
+    << "#pragma unroll 1\n        for (int b = 0; b < " << NA << "; ++b) W[a * " << NA << " + b] = -J[act(a) * " << n
+    << " + act(b)];\n  }\n"
+    << "  // f and, with WITH_J, -J over act() (row-major)\n"
+    << "  template <bool WITH_J, int ST>\n"
+    << "  __device__ __forceinline__ static void run(const MechView& mv, double pc, const double (&y)[" << n
+    << "], double (&f)[" << n << "], SVT<double, ST> W) {\n";
+  if (T_low > 0.0) o << "    if (gen_fixed<WITH_J, ST>(mv, pc, y, f, W)) return;\n";
+  o << "    double yl[" << n << "], fl[" << n << "], Wl[WITH_J ? " << NA * NA << " : 1];\n"
+    << "#pragma unroll\n    for (int i = 0; i < " << n << "; ++i) yl[i] = y[i];\n"
+    << "    general<WITH_J>(mv, pc, yl, fl, Wl);\n"
+    << "#pragma unroll\n    for (int i = 0; i < " << n << "; ++i) f[i] = fl[i];\n"
+    << "    if (WITH_J)\n#pragma unroll 1\n      for (int i = 0; i < " << NA * NA << "; ++i) W[i] = Wl[i];\n"
+    << "  }\n};\n\n}  // namespace df\n";
   return o.str();
 }
 
@@ -430,22 +981,27 @@ std::string header_dir() {
   return "";
 }
 
-// one compiled module per (device, generated source)
+// one compiled module per (device, kernel variant, generated source), built when
+// the variant is first launched: a program that uses one block size compiles one
+// kernel
 struct Module {
   bool ok = false;
   std::string why;
   CUmodule mod = nullptr;
-  std::map<int, CUfunction> fn;  // threads per block -> kernel
-  CUfunction fn_ign = nullptr;    // 32 threads, refining the ignition time (IntegArgs.t_ign)
+  CUfunction fn = nullptr;
   size_t compile_ms = 0;
   bool from_cache = false;
+  int per_thread = 0;  // doubles of shared memory per thread: W and one vector
 };
 
 std::mutex g_mu;
-std::map<std::pair<int, std::string>, Module> g_modules;
+std::map<std::pair<int, std::string>, Module> g_modules;  // key: device * kVariants + variant, source
 
-constexpr int kThreads[] = {32, 64};
-constexpr int kIgnThreads = 32;  // the block size of the kernel that refines the ignition time
+// the kernel variants: 32 and 64 threads per block, and 32 threads refining the
+// ignition time (IntegArgs.t_ign)
+constexpr int kVariants = 3, kIgnVariant = 2;
+constexpr int kVariantThreads[kVariants] = {32, 64, 32};
+static_assert(kVariants <= JIT_VARIANTS, "df_mech keeps one module per variant");
 
 // ---------------------------------------------------------------------------
 // on-disk cache of compiled modules: <dir>/<key>.cubin and <key>.names (the
@@ -513,7 +1069,7 @@ uint64_t headers_hash(const std::string& inc) {
   std::call_once(once, [&] {
     uint64_t acc = 1469598103934665603ull;
     const char* files[] = {"integrate_thread.cuh", "rosenbrock.cuh", "chem_thread.cuh", "dev_common.cuh",
-                           "exp2fix.cuh", "exp2fix_table.inc", "fastlog.cuh", "fastlog_table.inc", "dual.cuh"};
+                           "exp2fix.cuh", "exp2fix_table.inc", "log2fix.cuh", "log2fix_table.inc", "dual.cuh"};
     for (const char* fn : files) {
       std::string d;
       read_file(inc + "/" + fn, &d);
@@ -524,7 +1080,7 @@ uint64_t headers_hash(const std::string& inc) {
   return h;
 }
 
-// resolve the kernels and the table of a loaded cubin, upload the tables
+// resolve the kernel and the table of a loaded cubin, upload the tables
 bool finish_module(Module& r, const Driver& drv, const std::vector<char>& cubin,
                    const std::vector<std::string>& lowered) {
   if (drv.load(&r.mod, cubin.data()) != CUDA_SUCCESS) {
@@ -532,25 +1088,11 @@ bool finish_module(Module& r, const Driver& drv, const std::vector<char>& cubin,
     r.mod = nullptr;
     return false;
   }
-  for (size_t i = 0; i < sizeof(kThreads) / sizeof(kThreads[0]); ++i) {
-    CUfunction f = nullptr;
-    if (i >= lowered.size() || lowered[i].empty() || drv.get_function(&f, r.mod, lowered[i].c_str()) != CUDA_SUCCESS) {
-      r.why = "generated kernel not found in the module";
-      drv.unload(r.mod);
-      r.mod = nullptr;
-      return false;
-    }
-    r.fn[kThreads[i]] = f;
-  }
-  {
-    const size_t i = sizeof(kThreads) / sizeof(kThreads[0]);
-    if (i >= lowered.size() || lowered[i].empty() ||
-        drv.get_function(&r.fn_ign, r.mod, lowered[i].c_str()) != CUDA_SUCCESS) {
-      r.why = "generated kernel (ignition time) not found in the module";
-      drv.unload(r.mod);
-      r.mod = nullptr;
-      return false;
-    }
+  if (lowered.size() != 2 || lowered[0].empty() || drv.get_function(&r.fn, r.mod, lowered[0].c_str()) != CUDA_SUCCESS) {
+    r.why = "generated kernel not found in the module";
+    drv.unload(r.mod);
+    r.mod = nullptr;
+    return false;
   }
   CUdeviceptr tab = 0;
   size_t tab_bytes = 0;
@@ -580,9 +1122,9 @@ bool finish_module(Module& r, const Driver& drv, const std::vector<char>& cubin,
 
 // Version of the cached entries (the cubin and its lowered-name list, and what
 // finish_module expects of them); raised whenever either changes.
-constexpr int kCacheFormat = 3;
+constexpr int kCacheFormat = 4;
 
-Module build_module(int dev, const df_mech* m, const std::string& src) {
+Module build_module(int dev, const df_mech* m, const std::string& src, int variant) {
   Module r;
   const Driver& drv = driver();
   if (!drv.ok) {
@@ -602,10 +1144,8 @@ Module build_module(int dev, const df_mech* m, const std::string& src) {
   }
   const Nvrtc& nv = nvrtc();
   const std::string arch = "--gpu-architecture=sm_" + std::to_string(major * 10 + minor) + "a";
-  std::vector<std::string> names;
-  for (int t : kThreads) names.push_back(jit_kernel_name(m->dims.N, t));
-  names.push_back(jit_kernel_name(m->dims.N, kIgnThreads, true));
-  names.push_back("&df::c_tab");
+  const std::vector<std::string> names = {jit_kernel_name(m->dims.N, kVariantThreads[variant], variant == kIgnVariant),
+                                          "&df::c_tab"};
   const std::string incopt = "-I" + inc;
   const char* opts[] = {arch.c_str(), "-std=c++17", incopt.c_str(), "-default-device", "-lineinfo",
                         "-diag-suppress=177"};
@@ -613,7 +1153,8 @@ Module build_module(int dev, const df_mech* m, const std::string& src) {
   // architecture, the NVRTC version, the compile options (the include path
   // left out: a moved tree keeps its entries) and the entry format
   const std::string dir = cache_dir();
-  std::string keysrc = src + arch + std::to_string(nv.version) + "|format " + std::to_string(kCacheFormat);
+  std::string keysrc =
+      src + names[0] + arch + std::to_string(nv.version) + "|format " + std::to_string(kCacheFormat);
   for (const char* o : opts)
     if (o != incopt.c_str()) keysrc += std::string("|") + o;
   char key[32] = {0};
@@ -685,32 +1226,30 @@ int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, cuda
   *launched = false;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return DF_OK;
-  Module* md = static_cast<Module*>(m->jit_module[dev]);
+  // the variant that refines the ignition time has one block size
+  int variant = a.t_ign ? kIgnVariant : 0;
+  while (variant < kIgnVariant && kVariantThreads[variant] != threads) ++variant;
+  if (!a.t_ign && variant == kIgnVariant) return DF_OK;  // no generated kernel for this block size
+  threads = kVariantThreads[variant];
+  Module* md = static_cast<Module*>(m->jit_module[dev][variant]);
   if (!md) {  // first launch on this device: generate, and compile unless cached
     const std::string src = jit_thread_source(m);
     std::lock_guard<std::mutex> lock(g_mu);
-    auto key = std::make_pair(dev, src);
+    auto key = std::make_pair(dev * kVariants + variant, src);
     auto it = g_modules.find(key);
-    if (it == g_modules.end()) it = g_modules.emplace(key, build_module(dev, m, src)).first;
+    if (it == g_modules.end()) it = g_modules.emplace(key, build_module(dev, m, src, variant)).first;
     md = &it->second;
-    m->jit_module[dev] = md;
+    const int na = (int)active_entries(m).size();
+    md->per_thread = na * (na + 1);
+    m->jit_module[dev][variant] = md;
     m->jit_note = !md->ok          ? md->why
                   : md->from_cache ? std::string("generated kernel loaded from the on-disk cache")
                                    : "generated kernel compiled in " + std::to_string(md->compile_ms) + " ms";
   }
   if (!md->ok) return DF_OK;
-  CUfunction fk = nullptr;
-  if (a.t_ign) {  // the variant that refines the ignition time, in its block size
-    fk = md->fn_ign;
-    threads = kIgnThreads;
-  } else {
-    auto f = md->fn.find(threads);
-    if (f == md->fn.end()) return DF_OK;  // no generated kernel for this block size
-    fk = f->second;
-  }
+  const CUfunction fk = md->fn;
   const Driver& drv = driver();
-  const int N = m->dims.N;
-  const int per_thread = (N + 1) * (N + 1) + 6 * (N + 1);  // J and the stage vectors
+  const int per_thread = md->per_thread;
   IntegArgs args = a;
   // the mechanism if staging it leaves as many blocks on an SM as reading it
   // through L1, the per-thread workspace

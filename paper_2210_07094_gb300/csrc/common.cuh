@@ -14,6 +14,8 @@
 #include "dev_common.cuh"
 
 
+constexpr int JIT_VARIANTS = 3;  // kernels generated for a mechanism (codegen.cu)
+
 // the opaque handle
 struct df_mech {
   df::MechDims dims;
@@ -41,9 +43,10 @@ struct df_mech {
   // launch used it, and its state (compile time, or why it is unavailable)
   int jit_used = 0;
   std::string jit_note;
-  // the module compiled for this mechanism on each device (owned by the
-  // process-wide cache in codegen.cu; null until the first launch)
-  void* jit_module[64] = {nullptr};
+  // the modules compiled for this mechanism on each device, one per kernel
+  // variant (owned by the process-wide cache in codegen.cu; null until the
+  // variant's first launch)
+  void* jit_module[64][JIT_VARIANTS] = {};
 };
 
 namespace df {

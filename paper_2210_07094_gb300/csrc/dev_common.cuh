@@ -61,6 +61,8 @@ constexpr int RX_REC = 5;
 // Troe record (TR_REC doubles): lnA0 - lnA, beta0, Ea0/R, alpha, 1/T***, 1/T*, T**, pad
 constexpr int TR_REC = 8;
 // efficiency record: N doubles per third-body / falloff reaction
+// then, past the total (never staged into shared memory): ln A_j log2(e) 2^53 as
+// 64-bit integers, and 1 if every one of them lies in the fixed-point range
 
 struct RxMeta {
   uint8_t reac[3];
@@ -78,6 +80,8 @@ static_assert(sizeof(RxSlots) == 8, "slot layout");
 struct MechDims {
   int N, M, n_eff, n_troe;
   int off_sp, off_rx, off_tr, off_eff, total;  // offsets in doubles
+  __host__ __device__ int off_fix() const { return total; }
+  __host__ __device__ int allocated() const { return total + M + 1; }
 };
 
 inline MechDims mech_dims(int N, int M, int n_eff, int n_troe) {
@@ -119,6 +123,25 @@ __device__ __forceinline__ double rcp_nr(double a) {
   const double r1 = r0 * fma(-a, r0, 2.0);
   return r1 * fma(-a, r1, 2.0);
 }
+
+// |a| in [2^-95, 2^97): its FP32 image and that of its reciprocal are normal
+__device__ __forceinline__ bool rcp_in_range(double a) {
+  return ((uint32_t)__double2hiint(a) & 0x7fffffffu) - 0x3a000000u < 0x46000000u - 0x3a000000u;
+}
+
+// 1/a for an a in that range, three FP64 operations: the seed's argument and the
+// seed change format through integer operations (a conversion instruction
+// occupies the FP64 pipe), the seed's relative error 2^-20 enters cubed
+__device__ __forceinline__ double rcp_fast(double a) {
+  const uint32_t hi = (uint32_t)__double2hiint(a), sign = hi & 0x80000000u;
+  uint32_t r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=r"(r) : "r"(((hi << 3) - 0xc0000000u) | sign));
+  const double r0 = __hiloint2double((int)((((r & 0x7fffffffu) >> 3) + 0x38000000u) | sign), (int)(r << 29));
+  const double e = fma(-a, r0, 1.0);
+  return fma(r0, fma(e, e, e), r0);
+}
+
+__device__ __forceinline__ double rcp_any(double a) { return rcp_in_range(a) ? rcp_fast(a) : 1.0 / a; }
 
 #endif
 

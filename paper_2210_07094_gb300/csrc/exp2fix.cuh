@@ -23,7 +23,7 @@ namespace df {
 
 #include "exp2fix_table.inc"
 
-__device__ __forceinline__ uint64_t wmad(uint32_t a, uint32_t b, uint64_t c) { return (uint64_t)a * b + c; }
+__host__ __device__ __forceinline__ uint64_t wmad(uint32_t a, uint32_t b, uint64_t c) { return (uint64_t)a * b + c; }
 
 // the high 64 bits of a 64 x 64 bit product to within 3 units (the product of
 // the low words and the carries out of the cross products' low words dropped)
@@ -51,8 +51,10 @@ __device__ __forceinline__ double exp2_fixed(int64_t X) {
 // x log2(e) as floor(x log2(e) 2^53), |x| < 512: the 53-bit mantissa (at bit
 // 62) times log2(e)/2, shifted by the exponent; a negative x takes the
 // complement, so both signs are floors
-__device__ __forceinline__ int64_t exp_arg_fixed(double x) {
-  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+__host__ __device__ __forceinline__ int64_t exp_arg_fixed(double x) {
+  uint64_t bits;
+  memcpy(&bits, &x, 8);
+  const uint32_t hi = (uint32_t)(bits >> 32), lo = (uint32_t)bits;
   constexpr uint32_t ch = (uint32_t)(EXP2FIX_LOG2E_HALF >> 32), cl = (uint32_t)EXP2FIX_LOG2E_HALF;
   const uint32_t mh = 0x40000000u | ((hi << 10) & 0x3fffffffu) | (lo >> 22), ml = lo << 10;
   const uint64_t p = wmad(mh, ch, wmad(ml, ch, (uint64_t)mh * cl) >> 32);
@@ -61,8 +63,25 @@ __device__ __forceinline__ int64_t exp_arg_fixed(double x) {
   return (int64_t)(p >> s) ^ (int64_t)((int32_t)hi >> 31);
 }
 
+// floor(x 2^S) of a positive double whose exponent lets it fit (x 2^S < 2^63)
+template <int S>
+__device__ __forceinline__ uint64_t pos_fixed(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint64_t m = ((uint64_t)(0x40000000u | ((hi << 10) & 0x3fffffffu) | (lo >> 22)) << 32) | (lo << 10);
+  return m >> (1085 - S - (int)(hi >> 20));
+}
+
+// a b 2^-64 to within 3 units
+__device__ __forceinline__ uint64_t mul_fixed(uint64_t a, uint64_t b) {
+  return mulhi64_3((uint32_t)(a >> 32), (uint32_t)a, (uint32_t)(b >> 32), (uint32_t)b);
+}
+
 // |x| >= 512, inf and NaN (an integer test of the high word)
 __device__ __forceinline__ bool exp_is_big(double x) { return (__double2hiint(x) & 0x7fffffff) >= 0x40800000; }
+
+// the ln A the fixed-point rate arguments are built for: they stay within +- 1000
+// octaves with what the generator allows the temperature terms
+__host__ __device__ inline bool lnA_fits_fixed(double lnA) { return lnA > -277.0 && lnA < 277.0; }
 
 __device__ __forceinline__ double exp_rate(double x) {
   return exp_is_big(x) ? exp(x) : exp2_fixed(exp_arg_fixed(x));

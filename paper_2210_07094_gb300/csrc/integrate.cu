@@ -687,9 +687,20 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
   }
 }
 
-__global__ void k_set_lnA(double* blob, int off_rx, int M, const double* lnA) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < M) blob[off_rx + RX_REC * j] = lnA[j];
+// ln A into the reaction records and, as fixed-point logarithms, behind the blob;
+// one block, which also says whether all of them fit
+__global__ void k_set_lnA(double* blob, MechDims d, const double* lnA) {
+  long long* fix = reinterpret_cast<long long*>(blob + d.off_fix());
+  int fits = 1;
+  for (int j = threadIdx.x; j < d.M; j += blockDim.x) {
+    const double a = lnA[j];
+    blob[d.off_rx + RX_REC * j] = a;
+    const bool ok = lnA_fits_fixed(a);
+    fix[j] = ok ? exp_arg_fixed(a) : 0;
+    fits = fits && ok;
+  }
+  fits = __syncthreads_and(fits);
+  if (threadIdx.x == 0) fix[d.M] = fits;
 }
 
 int launch_set_lnA(df_mech* m, const double* lnA, cudaStream_t st) {
@@ -698,11 +709,11 @@ int launch_set_lnA(df_mech* m, const double* lnA, cudaStream_t st) {
   if (lnA == nullptr) {
     // restore the file's values: copy the host records back
     for (int j = 0; j < M; ++j) m->blob_host[m->dims.off_rx + RX_REC * j] = m->lnA_file[j];
-    return cuda_check(cudaMemcpyAsync(m->blob_dev, m->blob_host.data(), sizeof(double) * m->dims.total,
+    return cuda_check(cudaMemcpyAsync(m->blob_dev, m->blob_host.data(), sizeof(double) * m->dims.allocated(),
                                       cudaMemcpyHostToDevice, st),
                       "restore lnA");
   }
-  k_set_lnA<<<(M + 127) / 128, 128, 0, st>>>(m->blob_dev, m->dims.off_rx, M, lnA);
+  k_set_lnA<<<1, 128, 0, st>>>(m->blob_dev, m->dims, lnA);
   return cuda_check(cudaGetLastError(), "set lnA kernel");
 }
 

@@ -45,11 +45,11 @@ struct IntegArgs {
 constexpr unsigned FULL = 0xffffffffu;
 
 // per-thread shared-memory doubles of the thread path: the species vectors C,
-// wdot, g/RT, h/RT, cp/R (when the evaluation policy keeps them there), the
-// matrix J / W and the six stage vectors
-template <int NS, class EVAL = BlobEval>
+// wdot, g/RT, h/RT, cp/R, the matrix J / W and the six stage vectors (a generated
+// evaluation needs W and one vector only, see ros_attempt_gen)
+template <int NS>
 __host__ __device__ constexpr int thread_ws_doubles() {
-  return (EVAL::kSpeciesVectors ? 5 * NS : 0) + (NS + 1) * (NS + 1) + 6 * (NS + 1);
+  return 5 * NS + (NS + 1) * (NS + 1) + 6 * (NS + 1);
 }
 
 __host__ __device__ inline int blob_smem_doubles(const MechDims& d) { return (d.total + 1) & ~1; }
@@ -73,20 +73,10 @@ __global__ void __launch_bounds__(128, 1) k_integrate_thread(IntegArgs a) {
     boff = blob_smem_doubles(a.d);
   }
   __syncthreads();
-  const MechView mv = make_view(blob, a.d);
+  MechView mv = make_view(blob, a.d);
+  mv.fix = reinterpret_cast<const long long*>(a.blob + a.d.off_fix());
   double* ws = smem + boff + tid;
   typedef SVT<double, BT> V;
-  constexpr int nv = EVAL::kSpeciesVectors ? NS : 0;
-  // without species vectors in shared memory (the generated evaluation) the
-  // first view is the evaluation's scratch while J is built: the stage vectors'
-  // storage, idle then
-  V C{ws + (nv > 0 ? 0 : (n * n) * stride), stride};
-  V wdot{ws + nv * stride, stride};
-  V gRT{ws + 2 * nv * stride, stride};
-  V hRT{ws + 3 * nv * stride, stride};
-  V cpR{ws + 4 * nv * stride, stride};
-  V Jv{ws + 5 * nv * stride, stride};
-  V Kv{ws + (5 * nv + n * n) * stride, stride};
   const RosTab& tb = c_tab[a.method];
   const int lane = tid & 31;
   const unsigned long long nwork = a.nwork_dev ? *a.nwork_dev : (unsigned long long)a.nwork;
@@ -174,9 +164,19 @@ __global__ void __launch_bounds__(128, 1) k_integrate_thread(IntegArgs a) {
     double en;
     double fT;
     const double t0 = t;
-    const bool ok = ros_attempt<NS, CONSTV, BT, EVAL>(mv, tb, pc, y, h, a.rtol, a.atolY, a.atolT, C, wdot, gRT, hRT,
-                                                cpR, Jv, Kv, stride, ys, en, nullptr, nacc == 0 && nrej == 0, &last,
-                                                &fT);
+    bool ok;
+    if constexpr (EVAL::kGenerated) {
+      static_assert(NS == EVAL::kN && !CONSTV, "generated evaluation: its own mechanism, constant pressure");
+      ok = ros_attempt_gen<BT, EVAL>(mv, tb, pc, y, h, a.rtol, a.atolY, a.atolT, V{ws, stride},
+                                     V{ws + EVAL::kNA * EVAL::kNA * stride, stride}, ys, en, nacc == 0 && nrej == 0,
+                                     last, fT);
+    } else {
+      V C{ws, stride}, wdot{ws + NS * stride, stride}, gRT{ws + 2 * NS * stride, stride},
+          hRT{ws + 3 * NS * stride, stride}, cpR{ws + 4 * NS * stride, stride}, Jv{ws + 5 * NS * stride, stride},
+          Kv{ws + (5 * NS + n * n) * stride, stride};
+      ok = ros_attempt<NS, CONSTV, BT>(mv, tb, pc, y, h, a.rtol, a.atolY, a.atolT, C, wdot, gRT, hRT, cpR, Jv, Kv,
+                                       stride, ys, en, nullptr, nacc == 0 && nrej == 0, &last, &fT);
+    }
     const int nacc0 = nacc;
     step_control(tb, ok, en, last, a.dt, y, ys, t, h, nacc, nrej, last_rej, done, ss);
     if (nacc > nacc0) {  // dT/dt at the start of an accepted substep

@@ -16,6 +16,7 @@
 #include <sstream>
 
 #include "common.cuh"
+#include "exp2fix.cuh"
 
 namespace df {
 namespace {
@@ -273,12 +274,21 @@ int parse_mechanism(const char* path, df_mech* m) {
   }
   MechDims d = mech_dims(N, M, n_eff, n_troe);
   m->dims = d;
-  m->blob_host.assign(d.total, 0.0);
+  m->blob_host.assign(d.allocated(), 0.0);
   std::copy(spec.begin(), spec.end(), m->blob_host.begin() + d.off_sp);
   std::copy(rec.begin(), rec.end(), m->blob_host.begin() + d.off_rx);
   std::copy(troe.begin(), troe.end(), m->blob_host.begin() + d.off_tr);
   std::copy(eff.begin(), eff.end(), m->blob_host.begin() + d.off_eff);
   m->lnA_file = lnA;
+  for (int j = 0; j <= M; ++j) {
+    int64_t v = 1;
+    if (j < M) {
+      v = lnA_fits_fixed(lnA[j]) ? exp_arg_fixed(lnA[j]) : 0;
+    } else {
+      for (double a : lnA) v = v && lnA_fits_fixed(a);
+    }
+    memcpy(&m->blob_host[d.off_fix() + j], &v, 8);
+  }
   // species -> (reaction, net stoichiometric coefficient nu''_kj - nu'_kj) lists
   std::vector<std::vector<std::pair<int, int>>> lists(N);
   for (int j = 0; j < M; ++j) {

@@ -5,7 +5,7 @@
 #include "../../include/df_probe.h"
 #include "exp2fix.cuh"
 #include "fastexp.cuh"
-#include "fastlog.cuh"
+#include "log2fix.cuh"
 
 namespace df {
 
@@ -53,7 +53,7 @@ __global__ void k_exp_rate_probe(const double* x, double* y, long long n) {
 
 __global__ void k_log_probe(const double* x, double* y, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = log_tab(x[i]);
+  if (i < n) y[i] = log_rate(x[i]);
 }
 
 }  // namespace df

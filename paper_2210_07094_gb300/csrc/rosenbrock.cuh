@@ -27,6 +27,9 @@ struct RosTab {
   // and err = K_{s-1}.  Both tables are (mark_stiffly_accurate); the kernels
   // rely on it and the host uploads no other table.
   int stiff_acc;
+  // the last stage's state is the previous stage's plus the previous stage
+  // (a_{s-1,j} = a_{s-2,j} for j < s - 2, a_{s-1,s-2} = 1): so in both tables
+  int tail;
 };
 
 #ifndef __CUDACC_RTC__  // host-side table builders
@@ -35,6 +38,9 @@ static void mark_stiffly_accurate(RosTab& t) {
   bool sa = l > 0 && t.m[l] == 1.0 && t.newf[l] != 0;
   for (int j = 0; j < l; ++j) sa = sa && t.m[j] == t.a[l][j] && t.e[j] == 0.0;
   t.stiff_acc = sa && t.e[l] == 1.0 ? 1 : 0;
+  bool tl = l > 1 && t.a[l][l - 1] == 1.0 && t.newf[l - 1] != 0 && t.newf[l] != 0;
+  for (int j = 0; j < l - 1; ++j) tl = tl && t.a[l][j] == t.a[l - 1][j];
+  t.tail = tl ? 1 : 0;
 }
 
 static RosTab make_rodas4() {
@@ -123,21 +129,14 @@ __device__ __forceinline__ double first_step_limit(const double (&y)[n], const d
 
 // pc: the reactor's fixed state parameter, pressure [dyn/cm^2] (CONSTV false)
 // or density [g/cm^3] (CONSTV true; see eval_thread)
-// Evaluation of f (and J) for ros_attempt: the mechanism-independent kernels
-// read the mechanism from its blob (eval_thread); a kernel generated for one
-// mechanism supplies its own policy with the same interface.
+// The kernels' evaluation policy: the mechanism-independent kernels read the
+// mechanism from its blob (eval_thread); a kernel generated for one mechanism
+// brings its own (see ros_attempt_gen).
 struct BlobEval {
-  static constexpr bool kSpeciesVectors = true;  // uses the per-thread C, wdot, g, h, cp vectors
-  template <int NS, bool WITH_J, bool CONSTV, int ST>
-  __device__ __forceinline__ static double run(const MechView& mv, double pc, const double (&y)[NS + 1],
-                                               double (&f)[NS + 1], SVT<double, ST> C, SVT<double, ST> wdot,
-                                               SVT<double, ST> gRT, SVT<double, ST> hRT, SVT<double, ST> cpR,
-                                               SVT<double, ST> Jv) {
-    return eval_thread<NS, WITH_J, double, CONSTV, ST>(mv, pc, y, f, C, wdot, gRT, hRT, cpR, Jv);
-  }
+  static constexpr bool kGenerated = false;
 };
 
-template <int NS, bool CONSTV = false, int ST = 0, class EVAL = BlobEval>
+template <int NS, bool CONSTV = false, int ST = 0>
 __device__ __forceinline__ bool ros_attempt(const MechView& mv, const RosTab& tb, double pc, const double (&y)[NS + 1],
                                             double& h, double rtol, double atolY, double atolT, SVT<double, ST> C,
                                             SVT<double, ST> wdot, SVT<double, ST> gRT, SVT<double, ST> hRT,
@@ -146,7 +145,7 @@ __device__ __forceinline__ bool ros_attempt(const MechView& mv, const RosTab& tb
                                             bool first = false, bool* last = nullptr, double* fT = nullptr) {
   constexpr int n = NS + 1;
   double fs[n];
-  EVAL::template run<NS, true, CONSTV, ST>(mv, pc, y, fs, C, wdot, gRT, hRT, cpR, Jv);
+  eval_thread<NS, true, double, CONSTV, ST>(mv, pc, y, fs, C, wdot, gRT, hRT, cpR, Jv);
   if (fT) *fT = fs[0];
   if (first) {
     const double hl = first_step_limit<n>(y, fs);
@@ -173,7 +172,7 @@ __device__ __forceinline__ bool ros_attempt(const MechView& mv, const RosTab& tb
         for (int j = 0; j < s; ++j) acc += tb.a[s][j] * Kv[j * n + i];
         ynew[i] = acc;
       }
-      EVAL::template run<NS, false, CONSTV, ST>(mv, pc, ynew, fs, C, wdot, gRT, hRT, cpR, Jv);
+      eval_thread<NS, false, double, CONSTV, ST>(mv, pc, ynew, fs, C, wdot, gRT, hRT, cpR, Jv);
     }
     // stage right-hand side, solved in place in the K slot of this stage
     SVT<double, ST> Ks{&Kv[s * n], stride};
@@ -200,6 +199,147 @@ __device__ __forceinline__ bool ros_attempt(const MechView& mv, const RosTab& tb
     const double sc = (i == 0 ? atolT : atolY) + rtol * fmax(fabs(y[i]), fabs(yn));
     const double r = e * rcp_nr(sc);
     e2 += r * r;
+  }
+  en = sqrt(e2 * (1.0 / n));
+  return ok && fin && isfinite(en);
+}
+
+// The attempt with a generated evaluation (EVAL, see codegen.cu).  NA is the
+// order of the linear systems: the temperature and the species that some
+// reaction changes.  An inert species has a zero row in J, so its stage vectors
+// are zero and its column never matters: on the H2/air mechanism the systems are
+// 9 x 9 instead of 10 x 10 (N2), 27% fewer operations in the factorisation.
+// EVAL writes -J (compact, row-major) where W = I/(h gamma) - J is wanted.
+//
+// Shared memory holds only W and one vector, NA (NA + 1) doubles per thread: the
+// stage vectors of the finished stages, read once per later stage in long
+// independent runs, go to local memory (about 1% of the attempt's time), and the
+// substitutions run in registers.  On the 9-species mechanism that is 90
+// doubles instead of 160, eight warps per SM instead of five, two for every
+// FP64 pipe: one warp's integer work and shared-memory waits hide behind the
+// other's FP64 work.  With the fixed-point rate exponents of gen_fixed, 2^20
+// cells of the bimodal 9-species field went from 41.6 to 24.4 ms, 96 cells (one
+// warp's latency) from 432 to 257 us.
+template <int ST, class EVAL>
+__device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab& tb, double pc,
+                                                const double (&y)[EVAL::kN + 1], double& h, double rtol, double atolY,
+                                                double atolT, SVT<double, ST> W, SVT<double, ST> X,
+                                                double (&ynew)[EVAL::kN + 1], double& en, bool first, bool& last,
+                                                double& fT) {
+  constexpr int n = EVAL::kN + 1, NA = EVAL::kNA;
+  double fs[n];
+  double K[5][NA];  // finished stages (local memory: indexed by the stage loop)
+  EVAL::template run<true, ST>(mv, pc, y, fs, W);
+  fT = fs[0];
+  if (first) {
+    const double hl = first_step_limit<n>(y, fs);
+    if (hl < h) {
+      h = hl;
+      last = false;
+    }
+  }
+  const double hgi = rcp_nr(h * tb.gamma);
+#pragma unroll
+  for (int i = 0; i < NA; ++i) W[i * NA + i] += hgi;
+  int piv[NA];
+  const bool ok = lu_factor<NA, ST>(W, piv);
+  const double ih = rcp_nr(h);
+  double e2 = 0.0;
+  bool fin = true;
+#pragma unroll
+  for (int i = 0; i < n; ++i) ynew[i] = y[i];
+#pragma unroll 1
+  for (int s = 0; s < tb.s; ++s) {
+    const bool tail = tb.tail && s == tb.s - 1;
+    double r[NA];
+    if (s == 0) {
+#pragma unroll
+      for (int a = 0; a < NA; ++a) X[a] = fs[EVAL::act(a)];
+    } else {
+      // the stage's state and the sum of c_sj K_j in one pass over the stages
+      const bool newf = tb.newf[s] != 0;
+      double g[NA];
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        g[a] = y[EVAL::act(a)];
+        r[a] = 0.0;
+      }
+      if (tail) {
+#pragma unroll 1
+        for (int j = 0; j < s; ++j) {
+          const double c = tb.c[s][j];
+#pragma unroll
+          for (int a = 0; a < NA; ++a) r[a] += c * K[j][a];
+        }
+#pragma unroll
+        for (int a = 0; a < NA; ++a) ynew[EVAL::act(a)] += K[s - 1][a];
+      } else {
+#pragma unroll 1
+        for (int j = 0; j < s; ++j) {
+          const double c = tb.c[s][j], aj = tb.a[s][j];
+#pragma unroll
+          for (int a = 0; a < NA; ++a) {
+            const double k = K[j][a];
+            r[a] += c * k;
+            g[a] += aj * k;
+          }
+        }
+        if (newf) {
+#pragma unroll
+          for (int a = 0; a < NA; ++a) ynew[EVAL::act(a)] = g[a];
+        }
+      }
+      if (newf) {
+#pragma unroll
+        for (int a = 0; a < NA; ++a) X[a] = r[a];  // waits in shared memory for the evaluation
+        EVAL::template run<false, ST>(mv, pc, ynew, fs, W);
+#pragma unroll
+        for (int a = 0; a < NA; ++a) X[a] = fma(ih, X[a], fs[EVAL::act(a)]);
+      } else {
+#pragma unroll
+        for (int a = 0; a < NA; ++a) X[a] = fma(ih, r[a], fs[EVAL::act(a)]);
+      }
+    }
+    // row permutation in shared memory, the substitutions in registers
+#pragma unroll 1
+    for (int k = 0; k < NA; ++k) {
+      const int p = piv[k];
+      if (p != k) {
+        const double t = X[k];
+        X[k] = X[p];
+        X[p] = t;
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < NA; ++a) r[a] = X[a];
+#pragma unroll
+    for (int k = 0; k < NA; ++k) {
+#pragma unroll
+      for (int i = k + 1; i < NA; ++i) r[i] -= W[i * NA + k] * r[k];
+    }
+#pragma unroll
+    for (int k = NA - 1; k >= 0; --k) {
+      r[k] *= W[k * NA + k];
+#pragma unroll
+      for (int i = 0; i < k; ++i) r[i] -= W[i * NA + k] * r[k];
+    }
+    if (s < tb.s - 1) {
+#pragma unroll
+      for (int a = 0; a < NA; ++a) K[s][a] = r[a];
+    } else {
+      // stiffly accurate tables: the last stage is the error estimate, and
+      // y_new = Y_{s-1} + K_{s-1} (see ros_attempt)
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        const int i = EVAL::act(a);
+        const double yn = ynew[i] + r[a];
+        fin = fin && (__double2hiint(yn) & 0x7ff00000) != 0x7ff00000;
+        ynew[i] = yn;
+        const double sc = (i == 0 ? atolT : atolY) + rtol * fmax(fabs(y[i]), fabs(yn));
+        const double q = r[a] * rcp_nr(sc);
+        e2 += q * q;
+      }
+    }
   }
   en = sqrt(e2 * (1.0 / n));
   return ok && fin && isfinite(en);
