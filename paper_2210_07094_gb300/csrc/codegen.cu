@@ -328,11 +328,11 @@ std::string fixed_term(const std::string& dst, double c, bool log2e, const char*
   return "    " + dst + (c < 0.0 ? " -= " : " += ") + "(int64_t)" + e + ";\n";
 }
 
-// c log2(e) in units of 2^-53
-std::string fixed_const(double c) {
+// c, or c log2(e), in units of 2^-53
+std::string fixed_const(double c, bool log2e) {
   uint64_t l;
   int sh;
-  fixed_literal(c, true, 53, &l, &sh);
+  fixed_literal(c, log2e, 53, &l, &sh);
   return std::string(c < 0.0 ? "-" : "") + "(int64_t)(" + hex64(l) + (sh ? " << " + std::to_string(sh) : "") + ")";
 }
 
@@ -372,6 +372,113 @@ std::vector<Rx> reactions_of(const df_mech* m) {
   return out;
 }
 
+// The unknowns of the generated kernel's linear systems.  A species that no
+// reaction changes is inert.  Of the others the mole changes live in the column
+// space of the stoichiometric matrix: with as many fewer dimensions as elements
+// are conserved, dn_e = sum_r b_er dn_r expresses some species (elim) by the rest
+// (keep), exactly, for the production rates, every stage vector of a Rosenbrock
+// step and the step itself.  The systems then cover the kept species and the
+// temperature.  Eliminated are molecules of non-positive formation enthalpy (the
+// species that carry the mass, so that a sum's rounding is small beside them)
+// with the most reactions (whose production rates need not be summed).
+struct Systems {
+  std::vector<int> act;    // reacting species, ascending
+  std::vector<int> keep;   // species of the systems' rows, ascending
+  std::vector<int> elim;   // eliminated species, ascending
+  std::vector<std::vector<double>> b;  // [elim][keep]
+  int na() const { return (int)keep.size() + 1; }
+  // doubles of shared memory per thread: the matrix and a vector, or the kept
+  // species' rows over all reacting species while the Jacobian is summed
+  int per_thread() const {
+    return std::max(na() * (na() + 1), (int)(keep.size() * (act.size() + 1)));
+  }
+};
+
+struct Ratio {
+  long long p = 0, q = 1;
+};
+bool ratio_sub_mul(Ratio* a, Ratio f, Ratio x) {  // a -= f x; false on overflow
+  long long p, q, u, v, w;
+  if (__builtin_mul_overflow(f.p, x.p, &p) || __builtin_mul_overflow(f.q, x.q, &q) ||
+      __builtin_mul_overflow(a->p, q, &u) || __builtin_mul_overflow(p, a->q, &v) || __builtin_sub_overflow(u, v, &w) ||
+      __builtin_mul_overflow(a->q, q, &q))
+    return false;
+  const long long g = std::max(1ll, std::__gcd(w < 0 ? -w : w, q < 0 ? -q : q));
+  a->p = w / g;
+  a->q = q / g;
+  return true;
+}
+
+Systems systems_of(const df_mech* m, const std::vector<Rx>& rx) {
+  const int N = m->dims.N, M = (int)rx.size();
+  Systems s;
+  std::vector<int> entries(N, 0);
+  for (int k = 0; k < N; ++k) {
+    for (const Rx& x : rx) entries[k] += x.nu[k] != 0;
+    if (entries[k]) s.act.push_back(k);
+  }
+  auto stable = [&](int k) {  // h(298 K)
+    const double* a = &m->blob_host[m->dims.off_sp + SP_REC * k + 2];
+    const double T = 298.0;
+    return a[0] * T + T * T * (a[1] / 2 + T * (a[2] / 3 + T * (a[3] / 4 + T * a[4] / 5))) + a[5] <= 1500.0;
+  };
+  std::vector<int> order = s.act;  // the last ones that depend on the earlier ones are eliminated
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+    return std::make_pair(stable(a), entries[a]) < std::make_pair(stable(b), entries[b]);
+  });
+  // row echelon form of the kept species' rows, each with its combination of them
+  struct Row {
+    std::vector<Ratio> v;   // M entries
+    std::vector<Ratio> c;   // by position in `kept`
+    int pivot;
+  };
+  std::vector<Row> basis;
+  std::vector<int> kept;
+  std::vector<std::pair<int, std::vector<Ratio>>> dep;
+  bool ok = true;
+  for (int k : order) {
+    Row r;
+    r.v.resize(M);
+    for (int j = 0; j < M; ++j) r.v[j].p = rx[j].nu[k];
+    r.c.assign(order.size(), Ratio());
+    for (const Row& e : basis) {
+      if (r.v[e.pivot].p == 0) continue;
+      Ratio f{r.v[e.pivot].p * e.v[e.pivot].q, r.v[e.pivot].q * e.v[e.pivot].p};
+      if (f.q < 0) f = Ratio{-f.p, -f.q};
+      for (int j = 0; j < M && ok; ++j) ok = ratio_sub_mul(&r.v[j], f, e.v[j]);
+      for (size_t i = 0; i < r.c.size() && ok; ++i) ok = ratio_sub_mul(&r.c[i], f, e.c[i]);
+    }
+    if (!ok) break;
+    r.pivot = -1;
+    for (int j = 0; j < M && r.pivot < 0; ++j)
+      if (r.v[j].p != 0) r.pivot = j;
+    if (r.pivot < 0) {
+      dep.emplace_back(k, r.c);  // nu_k + sum_i c_i nu_kept[i] = 0
+    } else {
+      r.c[kept.size()].p += 1;
+      kept.push_back(k);
+      basis.push_back(r);
+    }
+  }
+  if (!ok) {  // no elimination
+    s.keep = s.act;
+    return s;
+  }
+  s.keep = kept;
+  std::sort(s.keep.begin(), s.keep.end());
+  std::sort(dep.begin(), dep.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
+  for (const auto& d : dep) {
+    s.elim.push_back(d.first);
+    std::vector<double> b;
+    for (int k : s.keep) {
+      const Ratio c = d.second[std::find(kept.begin(), kept.end(), k) - kept.begin()];
+      b.push_back(-(double)c.p / (double)c.q + 0.0);
+    }
+    s.b.push_back(b);
+  }
+  return s;
+}
+
 // the temperatures the fixed-point evaluation covers: from the lowest one at
 // which every exponent, with any ln A of lnA_fits_fixed, stays within 1000 octaves
 // (sampled every 2% and with 5% to spare); 0 if there is none
@@ -382,9 +489,12 @@ double fixed_T_low(const df_mech* m, const std::vector<Rx>& rx) {
     double worst = 0.0;
     for (double T = lo; T < kFixTHi * 1.02; T *= 1.02) {
       std::vector<double> g(m->dims.N);
-      for (int k = 0; k < m->dims.N; ++k)
+      for (int k = 0; k < m->dims.N; ++k) {
+        worst = std::max(worst, std::fabs(sp(k, 2) + T * (sp(k, SP_H) + T * (sp(k, SP_H + 1) + T * (sp(k, SP_H + 2) +
+                                          T * sp(k, SP_H + 3)))) + sp(k, 7) / T));
         g[k] = L2E * ((sp(k, 2) - sp(k, 8)) - sp(k, 2) * std::log(T) -
                       T * (sp(k, 3) / 2 + T * (sp(k, 4) / 6 + T * (sp(k, 5) / 12 + T * sp(k, 6) / 20))) + sp(k, 7) / T);
+      }
       for (const Rx& x : rx) {
         const double kf = 400.0 + L2E * std::fabs(x.b * std::log(T) - x.E / T);
         double sg = -x.dnu * L2E * (LOG_PSTD_RU - std::log(T));
@@ -448,9 +558,78 @@ std::string product_code(const std::string& name, const std::string& K, std::vec
   return o.str();
 }
 
-// The evaluation the generated kernel runs: f and -J, the latter compact over
-// the temperature and the species some reaction changes (the inert ones have
-// zero rows).  The exponents of the rate constants -- ln A + b ln T - E/T, the
+// The same as unpacked numbers from the rate constant `K`: `name`p, and with
+// derivatives the doubles `name`d<l>; `name`s is the sign word of the product
+std::string fx_product_code(const std::string& name, const std::string& K, std::vector<int> e, bool deriv) {
+  std::ostringstream o;
+  auto X = [](int k) { return "x" + std::to_string(k); };
+  auto hi = [](int k) { return "(uint32_t)__double2hiint(C[" + std::to_string(k) + "])"; };
+  auto sgn = [&](std::vector<int> v) {
+    std::string s;
+    for (int k : v) s += (s.empty() ? "" : " ^ ") + hi(k);
+    return s.empty() ? std::string("0u") : s;
+  };
+  auto mul = [](const std::string& a, const std::string& b) { return "fx_mul(" + a + ", " + b + ")"; };
+  if (e.size() == 3 && e[0] != e[1]) {  // equal species first
+    if (e[0] == e[2]) std::swap(e[1], e[2]);
+    else if (e[1] == e[2]) std::swap(e[0], e[2]);
+  }
+  o << "    const uint32_t " << name << "s = " << sgn(e) << ";\n";
+  if (!deriv) {
+    std::string p = K;
+    for (int k : e) p = mul(p, X(k));
+    o << "    const Fx " << name << "p = " << p << ";\n";
+    return o.str();
+  }
+  auto fx = [&](const char* v, const std::string& x) { o << "    const Fx " << name << v << " = " << x << ";\n"; };
+  // d/dC_l = mult v, v an unpacked number with the sign of the other species
+  auto d = [&](int l, int mult, const std::string& v, std::vector<int> others) {
+    const std::string p = "fx_pack(" + v + (mult == 2 ? ".m, " + v + ".e + 1" : std::string()) + ", " + sgn(others) + ")";
+    o << "    const double " << name << "d" << l << " = " << (mult == 3 ? "3.0 * " : "") << p << ";\n";
+  };
+  if (e.size() == 1) {
+    fx("t", K);
+    d(e[0], 1, name + "t", {});
+    fx("p", mul(name + "t", X(e[0])));
+  } else if (e.size() == 2 && e[0] == e[1]) {
+    fx("t", mul(K, X(e[0])));
+    d(e[0], 2, name + "t", {e[0]});
+    fx("p", mul(name + "t", X(e[0])));
+  } else if (e.size() == 2) {
+    fx("t", mul(K, X(e[0])));
+    fx("u", mul(K, X(e[1])));
+    d(e[1], 1, name + "t", {e[0]});
+    d(e[0], 1, name + "u", {e[1]});
+    fx("p", mul(name + "t", X(e[1])));
+  } else if (e[0] == e[1] && e[1] == e[2]) {
+    fx("t", mul(mul(K, X(e[0])), X(e[0])));
+    d(e[0], 3, name + "t", {e[0], e[0]});
+    fx("p", mul(name + "t", X(e[0])));
+  } else if (e[0] == e[1]) {
+    fx("t", mul(K, X(e[0])));
+    fx("u", mul(name + "t", X(e[0])));
+    fx("v", mul(name + "t", X(e[2])));
+    d(e[2], 1, name + "u", {e[0], e[0]});
+    d(e[0], 2, name + "v", {e[0], e[2]});
+    fx("p", mul(name + "u", X(e[2])));
+  } else {
+    fx("t", mul(K, X(e[0])));
+    fx("u", mul(name + "t", X(e[1])));
+    fx("v", mul(name + "t", X(e[2])));
+    fx("y", mul(mul(K, X(e[1])), X(e[2])));
+    d(e[2], 1, name + "u", {e[0], e[1]});
+    d(e[1], 1, name + "v", {e[0], e[2]});
+    d(e[0], 1, name + "y", {e[1], e[2]});
+    fx("p", mul(name + "u", X(e[2])));
+  }
+  return o.str();
+}
+
+// Where two products meet in a sum the text says which one is fused, so that the
+// module's kernels, compiled apart, round alike.
+//
+// The evaluation the generated kernel runs: f and -J, the latter over the kept
+// species and the temperature (Systems).  The exponents of the rate constants -- ln A + b ln T - E/T, the
 // sums of g_k/RT and the pressure term, all times log2(e) -- are 64-bit
 // fixed-point sums in units of 2^-53 octave: an addition is two integer
 // instructions where an FP64 one occupies the pipe for 64 cycles, a product
@@ -458,14 +637,20 @@ std::string product_code(const std::string& name, const std::string& K, std::vec
 // accurate than the rounded FP64 sums it replaces.  Only what multiplies
 // concentrations stays in FP64.  Returns false (nothing written) for states
 // outside the range the fixed-point words cover; the caller then takes gen_eval.
-void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& rx, const std::vector<int>& act,
-                double T_low) {
-  const int N = m->dims.N, NA = (int)act.size();
+// Without J only the kept species' entries of f and f[0] are written.
+void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& rx, const Systems& sys, double T_low) {
+  const int N = m->dims.N, NA = sys.na(), NR = NA - 1, wid = (int)sys.act.size() + 1;
   auto sp = [&](int k, int i) { return m->blob_host[m->dims.off_sp + SP_REC * k + i]; };
-  std::vector<int> col(N, -1);  // species -> compact index
-  for (int a = 1; a < NA; ++a) col[act[a] - 1] = a;
+  std::vector<int> col(N, -1), row(N, -1);  // reacting species -> column while J is summed; kept species -> row
+  for (size_t a = 0; a < sys.act.size(); ++a) col[sys.act[a]] = (int)a + 1;
+  for (int a = 0; a < NR; ++a) row[sys.keep[a]] = a;
+  // d Y_elim[e] / d Y_keep[a]
+  auto beta = [&](size_t e, int a) { return sys.b[e][a] * (sp(sys.elim[e], 0) * sp(sys.keep[a], 1)); };
   auto S = [](int k) { return std::to_string(k); };
-  auto W = [&](int a, int b) { return "W[" + std::to_string(a * NA + b) + "]"; };
+  // the sums: a row per kept species, d/dT and the reacting species (column 0 and
+  // col); then, in place row by row, the matrix, the temperature last
+  auto W = [&](int a, int b) { return "W[" + std::to_string(a * wid + b) + "]"; };
+  auto Wn = [&](int a, int b) { return "W[" + std::to_string(a * NA + b) + "]"; };
   bool any_collider = false, any_inert = false;  // any_inert: a rate depends on an inert species alone
   std::vector<bool> used(N, false);  // species whose g/RT some reaction needs
   for (const Rx& x : rx) {
@@ -500,45 +685,60 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     << "  const uint64_t t2 = mul_fixed(t1, t1);\n";
   bool t3 = false, t4 = false;
   for (int k = 0; k < N; ++k) {
-    t3 = t3 || (used[k] && sp(k, 5) != 0.0);
-    t4 = t4 || (used[k] && sp(k, 6) != 0.0);
+    t3 = t3 || ((used[k] || col[k] > 0) && sp(k, 5) != 0.0);
+    t4 = t4 || ((used[k] || col[k] > 0) && sp(k, 6) != 0.0);
   }
   if (t3) o << "  const uint64_t t3 = mul_fixed(t2, t1);\n";
   if (t4) o << "  const uint64_t t4 = mul_fixed(t2, t2);\n";
-  o << "  const int64_t lp = " << fixed_const(LOG_PSTD_RU) << " - (int64_t)(L >> 7);  // log2(p_std / (R T))\n"
+  o << "  const int64_t lp = " << fixed_const(LOG_PSTD_RU, true) << " - (int64_t)(L >> 7);  // log2(p_std / (R T))\n"
     << "  int64_t G[NS];  // g_k/RT log2(e)\n";
   for (int k = 0; k < N; ++k) {
     if (!used[k]) continue;
     const std::string g = "G[" + S(k) + "]";
-    o << "  {\n    " << g << " = " << fixed_const(sp(k, 2) - sp(k, 8)) << ";\n"
+    o << "  {\n    " << g << " = " << fixed_const(sp(k, 2) - sp(k, 8), true) << ";\n"
       << fixed_term(g, -sp(k, 2), false, "L", 60) << fixed_term(g, -0.5 * sp(k, 3), true, "t1", 50)
       << fixed_term(g, -sp(k, 4) / 6.0, true, "t2", 36) << fixed_term(g, -sp(k, 5) / 12.0, true, "t3", 22)
       << fixed_term(g, -sp(k, 6) / 20.0, true, "t4", 8) << fixed_term(g, sp(k, 7), true, "I", 69) << "  }\n";
   }
   for (int k = 0; k < N; ++k) o << "  C[" << k << "] *= rho;\n";
   if (any_collider) {
-    o << "  double ctot = C[0];\n";
-    for (int k = 1; k < N; ++k) o << "  ctot += C[" << k << "];\n";
+    o << "  const double ctot = rho * sumYW;\n";
   }
-  // species enthalpies h/RT of the reacting species; with J also times 1/T
-  o << "  double hRT[NS], hT[NS], w[NS], sM[NS], sN[NS];\n  const double invT2 = invT * invT;\n"
-    << "  (void)hT; (void)sM; (void)sN; (void)invT2;\n";
-  for (int a = 1; a < NA; ++a) {
-    const int k = act[a] - 1;
-    std::vector<double> hs = {sp(k, 2), sp(k, SP_H), sp(k, SP_H + 1), sp(k, SP_H + 2), sp(k, SP_H + 3)};
-    o << "  hRT[" << k << "] = " << horner(hs, "T") << " + " << lit(sp(k, 7)) << " * invT;\n"
-      << "  if (WITH_J) hT[" << k << "] = hRT[" << k << "] * invT;\n";
+  for (int k = 0; k < N; ++k) o << "  const Fx x" << k << " = fx_factor(C[" << k << "]);\n  (void)x" << k << ";\n";
+  // h/RT of the kept species with the eliminated ones' shares (the heat release
+  // and the temperature row need no others); with J also of every reacting
+  // species, in fixed point, for d ln K_c/dT
+  o << "  double hk[NS], w[NS], sM[NS], sN[NS];\n  int64_t H[NS];\n  const double invT2 = invT * invT;\n"
+    << "  (void)H; (void)sM; (void)sN; (void)invT2;\n";
+  auto enthalpy = [&](const std::string& dst, const std::vector<double>& c) {
+    return "    " + dst + " = " + fixed_const(c[0], false) + ";\n" + fixed_term(dst, c[1], false, "t1", 50) +
+           fixed_term(dst, c[2], false, "t2", 36) + fixed_term(dst, c[3], false, "t3", 22) +
+           fixed_term(dst, c[4], false, "t4", 8) + fixed_term(dst, c[5], false, "I", 69);
+  };
+  auto hcoef = [&](int k) {
+    return std::vector<double>{sp(k, 2), sp(k, SP_H), sp(k, SP_H + 1), sp(k, SP_H + 2), sp(k, SP_H + 3), sp(k, 7)};
+  };
+  for (int a = 0; a < NR; ++a) {
+    std::vector<double> c = hcoef(sys.keep[a]);
+    for (size_t e = 0; e < sys.elim.size(); ++e) {
+      const std::vector<double> ce = hcoef(sys.elim[e]);
+      for (int i = 0; i < 6; ++i) c[i] += sys.b[e][a] * ce[i];
+    }
+    o << "  {\n    int64_t h;\n" << enthalpy("h", c) << "    hk[" << sys.keep[a] << "] = fixed_to_double(h);\n  }\n";
   }
+  o << "  if (WITH_J) {\n";
+  for (int k : sys.act) o << enthalpy("H[" + S(k) + "]", hcoef(k));
+  o << "  }\n";
   // accumulators start at zero where their first contribution is conditional
   // (falloff reactions without a low-pressure rate contribute nothing)
-  std::vector<bool> w_set(N, false), sM_set(N, false), W_set(NA * NA, false);
+  std::vector<bool> w_set(N, false), sM_set(N, false), W_set(NR * wid, false);
   {
-    std::vector<bool> wz(N, true), Wz(NA * NA, true), sMz(N, true);
-    std::vector<bool> seen_w(N, false), seen_W(NA * NA, false), seen_M(N, false);
+    std::vector<bool> wz(N, true), Wz(NR * wid, true), sMz(N, true);
+    std::vector<bool> seen_w(N, false), seen_W(NR * wid, false), seen_M(N, false);
     for (const Rx& x : rx) {
       for (int k : x.spc) {
-        if (x.nu[k] == 0) continue;
-        const int a = col[k];
+        const int a = row[k];
+        if (x.nu[k] == 0 || a < 0) continue;
         if (!seen_w[k]) wz[k] = x.type == 2;
         seen_w[k] = true;
         if (x.type != 0) {
@@ -549,20 +749,19 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
         for (int l : x.spc)
           if (col[l] > 0 && (x.rev || std::find(x.r.begin(), x.r.end(), l) != x.r.end())) cols.push_back(col[l]);
         for (int c : cols) {
-          if (!seen_W[a * NA + c]) Wz[a * NA + c] = x.type == 2;
-          seen_W[a * NA + c] = true;
+          if (!seen_W[a * wid + c]) Wz[a * wid + c] = x.type == 2;
+          seen_W[a * wid + c] = true;
         }
         if (x.type != 0)
           for (int l = 0; l < N; ++l)
             if (m->blob_host[m->dims.off_eff + N * x.eff + l] != 1.0 && col[l] > 0) {
               const int c = col[l];
-              if (!seen_W[a * NA + c]) Wz[a * NA + c] = true;
-              seen_W[a * NA + c] = true;
+              if (!seen_W[a * wid + c]) Wz[a * wid + c] = true;
+              seen_W[a * wid + c] = true;
             }
       }
     }
-    for (int a = 1; a < NA; ++a) {
-      const int k = act[a] - 1;
+    for (int k : sys.keep) {
       if (wz[k]) {
         o << "  w[" << k << "] = 0.0;\n";
         w_set[k] = true;
@@ -574,19 +773,19 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
       if (any_inert) o << "  if (WITH_J) sN[" << k << "] = 0.0;\n";
     }
     o << "  if (WITH_J) {\n";
-    for (int a = 1; a < NA; ++a)
-      for (int b = 0; b < NA; ++b)
-        if (Wz[a * NA + b]) {
+    for (int a = 0; a < NR; ++a)
+      for (int b = 0; b < wid; ++b)
+        if (Wz[a * wid + b]) {
           o << "    " << W(a, b) << " = 0.0;\n";
-          W_set[a * NA + b] = true;
+          W_set[a * wid + b] = true;
         }
     o << "  }\n";
   }
   // the rows take -d w_k/d(...) , species columns pre-scaled by W_k / W_l
   auto addW = [&](int a, int b, double c, const std::string& v) {
     std::ostringstream s;
-    const bool set = W_set[a * NA + b];
-    W_set[a * NA + b] = true;
+    const bool set = W_set[a * wid + b];
+    W_set[a * wid + b] = true;
     s << "      " << W(a, b);
     if (c == 1.0) s << (set ? " -= " : " = -") << v << ";\n";
     else if (c == -1.0) s << (set ? " += " : " = ") << v << ";\n";
@@ -623,11 +822,11 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     }
     // d ln k / dT and d ln K_c / dT
     std::ostringstream dl;
-    dl << "      const double dk = " << lit(x.b) << " * invT + " << lit(x.E) << " * invT2;\n";
-    std::string dKc = "0.0";
+    dl << "      const double dk = fma(" << lit(x.E) << ", invT2, " << lit(x.b) << " * invT);\n";
+    std::string dKc = "fixed_to_double(" + S(-x.dnu) + "LL * (1LL << 53)";
     for (int k : x.spc)
-      for (int i = 0; i < std::abs(x.nu[k]); ++i) dKc += (x.nu[k] > 0 ? " + hT[" : " - hT[") + S(k) + "]";
-    for (int i = 0; i < std::abs(x.dnu); ++i) dKc += x.dnu > 0 ? " - invT" : " + invT";
+      for (int i = 0; i < std::abs(x.nu[k]); ++i) dKc += (x.nu[k] > 0 ? " + H[" : " - H[") + S(k) + "]";
+    dKc += ") * invT";
     auto has_dq = [&](int l) {
       return std::find(x.r.begin(), x.r.end(), l) != x.r.end() ||
              (x.rev && std::find(x.p.begin(), x.p.end(), l) != x.p.end());
@@ -636,8 +835,8 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     auto rows = [&]() {
       std::ostringstream s;
       for (int k : x.spc) {
-        if (x.nu[k] == 0) continue;
-        const int a = col[k];
+        const int a = row[k];
+        if (x.nu[k] == 0 || a < 0) continue;
         s << addW(a, 0, x.nu[k], "dqT");
         for (int l : x.spc) {
           if (!has_dq(l)) continue;
@@ -674,32 +873,28 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     };
     std::ostringstream upd;
     if (x.type != 2) {
-      o << "    const double kf = exp2_fixed(x);\n";
-      if (x.rev) o << "    const double kr = exp2_fixed(x + xc);\n";
+      o << "    const Fx kf = fx_exp2(x);\n";
+      if (x.rev) o << "    const Fx kr = fx_exp2(x + xc);\n";
       for (int wj = 1; wj >= 0; --wj) {
         if (wj) o << "    if (WITH_J) {\n";
         else o << "    } else {\n";
-        // each branch starts from the same accumulators
-        const auto w0 = w_set, sM0 = sM_set;
-        const auto W0 = W_set;
-        o << product_code("f", "kf", x.r, wj);
-        if (x.rev) o << product_code("b", "kr", x.p, wj);
-        const std::string q0 = x.rev ? "fp - bp" : "fp";
+        const auto w0 = w_set;  // both branches start from the same accumulators
+        o << fx_product_code("f", "kf", x.r, wj);
+        if (x.rev) o << fx_product_code("b", "kr", x.p, wj);
+        const std::string q0 = x.rev ? "fx_diff(fp, fs, bp, bs)" : "fx_pack(fp, fs)";
         if (x.type == 1) o << "      const double dqM = " << q0 << ";\n      (void)dqM;\n      const double q = Mc * dqM;\n";
         else o << "      const double q = " << q0 << ";\n";
         for (int k : x.spc)
-          if (x.nu[k] != 0) o << "      " << add1(w_set, "w", k, x.nu[k], "q");
+          if (x.nu[k] != 0 && row[k] >= 0) o << "      " << add1(w_set, "w", k, x.nu[k], "q");
         if (wj) {
           o << dl.str();
-          if (x.rev) o << "      const double dKc = " << dKc << ";\n";
+          if (x.rev) o << "      const double dKc = " << dKc << ", pb = fx_pack(bp, bs);\n";
           if (!x.rev) o << "      const double dqT = q * dk;\n";
-          else if (x.type == 1) o << "      const double dqT = q * dk + (Mc * bp) * dKc;\n";
-          else o << "      const double dqT = q * dk + bp * dKc;\n";
+          else if (x.type == 1) o << "      const double dqT = fma(q, dk, (Mc * pb) * dKc);\n";
+          else o << "      const double dqT = fma(q, dk, pb * dKc);\n";
           o << dqs(x.type == 1 ? "Mc" : "") << rows();
           w_set = w0;  // the other branch makes the same first updates of w
         }
-        (void)W0;
-        (void)sM0;
       }
       o << "    }\n  }\n";
       continue;
@@ -707,44 +902,44 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     // Troe falloff: the expressions of rate_compute, the rate constants from the
     // fixed-point exponents
     const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
-    o << "    int64_t xd = " << fixed_const(tr[0]) << ";  // k0 / kinf\n"
+    o << "    int64_t xd = " << fixed_const(tr[0], true) << ";  // k0 / kinf\n"
       << fixed_term("xd", tr[1] - x.b, false, "L", 60) << fixed_term("xd", -(tr[2] - x.E), true, "I", 69)
       << "    const double kinf = exp2_fixed(x), Pr = exp2_fixed(xd) * Mc;\n"
       << "    if (Pr > 0.0) {\n"
       << "      double e3, e1;\n      exp_rate2(-T * " << lit(tr[4]) << ", -T * " << lit(tr[5]) << ", e3, e1);\n"
       << "      const double e2 = exp_rate(" << lit(-tr[6]) << " * invT);\n"
       << "      const double invKc = " << (x.rev ? "exp2_fixed(xc)" : "0.0") << ";\n"
-      << "      const double Fc = " << lit(1.0 - tr[3]) << " * e3 + " << lit(tr[3]) << " * e1 + e2;\n"
+      << "      const double Fc = fma(" << lit(1.0 - tr[3]) << ", e3, fma(" << lit(tr[3]) << ", e1, e2));\n"
       << "      const double Lc = log10_rate(Fc), cc = -0.4 - 0.67 * Lc, nn = 0.75 - 1.27 * Lc;\n"
       << "      const double xl = log10_rate(Pr) + cc, den = nn - 0.14 * xl, den2 = den * den;\n"
-      << "      const double q1 = den2 * rcp_any(den2 + xl * xl);\n"
+      << "      const double q1 = den2 * rcp_any(fma(xl, xl, den2));\n"
       << "      const double F = exp_rate(LN10 * (Lc * q1)), onePr = rcp_any(1.0 + Pr);\n"
       << "      const double kf = kinf * Pr * onePr * F, kr = kf * invKc;\n";
     for (int wj = 1; wj >= 0; --wj) {
       const auto w0 = w_set;
       o << (wj ? "      if (WITH_J) {\n" : "      } else {\n") << product_code("f", "kf", x.r, wj);
       if (x.rev) o << product_code("b", "kr", x.p, wj);
-      o << "      const double q = " << (x.rev ? "fp - bp" : "fp") << ";\n";
+      o << "      const double q = " << (x.rev ? "__dsub_rn(fp, bp)" : "fp") << ";\n";
       for (int k : x.spc)
-        if (x.nu[k] != 0) o << "      " << add1(w_set, "w", k, x.nu[k], "q");
+        if (x.nu[k] != 0 && row[k] >= 0) o << "      " << add1(w_set, "w", k, x.nu[k], "q");
       if (wj) {
         std::string Pf, Pb;
         for (int k : x.r) Pf += (Pf.empty() ? "C[" : " * C[") + S(k) + "]";
         for (int k : x.p) Pb += (Pb.empty() ? "C[" : " * C[") + S(k) + "]";
         o << "      const double k0 = exp2_fixed(x + xd), rden = rcp_any(den), f1 = xl * rden;\n"
           << "      const double df1_dL = nn * rden * rden;\n"
-          << "      const double df1_dLc = (-0.67 * den - xl * (-1.27 + 0.67 * 0.14)) * (rden * rden);\n"
+          << "      const double df1_dLc = fma(-0.67, den, -(xl * (-1.27 + 0.67 * 0.14))) * (rden * rden);\n"
           << "      const double g2 = 2.0 * Lc * f1 * q1 * q1;\n"
-          << "      const double gpr = onePr - g2 * df1_dL, dlogF_dLc = q1 - g2 * df1_dLc;\n"
-          << "      const double dFc = " << lit(-(1.0 - tr[3]) * tr[4]) << " * e3 + " << lit(-tr[3] * tr[5])
-          << " * e1 + " << lit(tr[6]) << " * invT2 * e2;\n"
-          << "      const double dki = " << lit(x.b) << " * invT + " << lit(x.E) << " * invT2;\n"
-          << "      const double dk0 = " << lit(tr[1]) << " * invT + " << lit(tr[2]) << " * invT2;\n"
-          << "      const double dk = dki + gpr * (dk0 - dki) + dlogF_dLc * dFc * rcp_any(Fc);\n"
+          << "      const double gpr = fma(-g2, df1_dL, onePr), dlogF_dLc = fma(-g2, df1_dLc, q1);\n"
+          << "      const double dFc = fma(" << lit(-(1.0 - tr[3]) * tr[4]) << ", e3, fma(" << lit(-tr[3] * tr[5])
+          << ", e1, " << lit(tr[6]) << " * invT2 * e2));\n"
+          << "      const double dki = fma(" << lit(x.E) << ", invT2, " << lit(x.b) << " * invT);\n"
+          << "      const double dk0 = fma(" << lit(tr[2]) << ", invT2, " << lit(tr[1]) << " * invT);\n"
+          << "      const double dk = fma(dlogF_dLc * dFc, rcp_any(Fc), fma(gpr, dk0 - dki, dki));\n"
           << "      const double dKc = " << dKc << ";\n"
-          << "      const double dqT = q * dk" << (x.rev ? " + bp * dKc" : "") << ";\n      (void)dKc;\n"
-          << "      const double dqM = k0 * F * gpr * onePr * (" << Pf << (x.rev ? " - " + Pb + " * invKc" : std::string())
-          << ");\n"
+          << "      const double dqT = " << (x.rev ? "fma(q, dk, bp * dKc)" : "q * dk") << ";\n      (void)dKc;\n"
+          << "      const double dqM = k0 * F * gpr * onePr * "
+          << (x.rev ? "fma(-(" + Pb + "), invKc, " + Pf + ")" : "(" + Pf + ")") << ";\n"
           << dqs("") << rows();
         w_set = w0;
       }
@@ -753,35 +948,49 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
   }
   // heat release and f
   o << "  double Hw = 0.0;\n";
-  for (int a = 1; a < NA; ++a) o << "  Hw += hRT[" << act[a] - 1 << "] * w[" << act[a] - 1 << "];\n";
-  for (int k = 0; k < N; ++k) {
-    if (col[k] > 0) o << "  f[" << 1 + k << "] = " << lit(sp(k, 0)) << " * (w[" << k << "] * invrho);\n";
-    else o << "  f[" << 1 + k << "] = 0.0;\n";
+  for (int k : sys.keep) o << "  Hw += hk[" << k << "] * w[" << k << "];\n";
+  for (int k : sys.keep) o << "  f[" << 1 + k << "] = " << lit(sp(k, 0)) << " * (w[" << k << "] * invrho);\n";
+  o << "  const double RT = RU * T;\n  f[0] = -(Hw * RT) * (invrho * invcp);\n  if (WITH_J) {\n";
+  for (size_t e = 0; e < sys.elim.size(); ++e) {
+    o << "    f[" << 1 + sys.elim[e] << "] = 0.0";
+    for (int a = 0; a < NR; ++a)
+      if (sys.b[e][a] != 0.0) o << " + " << lit(beta(e, a)) << " * f[" << 1 + sys.keep[a] << "]";
+    o << ";\n";
   }
-  o << "  const double RT = RU * T;\n  f[0] = -(Hw * RT) * (invrho * invcp);\n";
+  for (int k = 0; k < N; ++k)
+    if (col[k] < 0) o << "    f[" << 1 + k << "] = 0.0;\n";
   // -J: row k holds -S'_kl = -(W_k / W_l) dw_k/dC_l; with s_k = sum_l S_kl C_l and
   // a_k = W_k (Wbar / rho) (w_k - s_k) + W_k sM_k: d f_k/dY_l = S'_kl + a_k / W_l
-  // (gen_eval); the temperature row sums the finished rows
-  o << "  if (WITH_J) {\n    const double wb = Wbar * invrho;\n    double dcp = 0.0, cpf = 0.0;\n";
-  for (int a = 0; a < NA; ++a) o << "    double tr" << a << " = 0.0;\n";
-  for (int a = 1; a < NA; ++a) {
-    const int k = act[a] - 1;
-    o << "    {  // row of species " << k << "\n";
-    for (int b = 0; b < NA; ++b) o << "      const double v" << b << " = " << W(a, b) << ";\n";
+  // (gen_eval); a kept species' column takes beta times the eliminated ones'; the
+  // temperature row sums the finished rows
+  o << "    const double wb = Wbar * invrho;\n    double dcp = 0.0, cpf = 0.0;\n";
+  for (int b = 0; b < NA; ++b) o << "    double tr" << b << " = 0.0;\n";
+  for (int a = 0; a < NR; ++a) {
+    const int k = sys.keep[a];
+    o << "    {  // row of species " << k << "\n      const double v0 = " << W(a, 0) << ";\n";
+    for (int l : sys.act) o << "      const double v" << 1 + l << " = " << W(a, col[l]) << ";\n";
     o << "      double s = 0.0;\n";
-    for (int b = 1; b < NA; ++b) o << "      s -= v" << b << " * (rho * y[" << act[b] << "]);\n";
+    for (int l : sys.act) o << "      s -= v" << 1 + l << " * (rho * y[" << 1 + l << "]);\n";
     o << "      s = s * " << lit(sp(k, 1)) << ";\n";
-    if (any_collider) o << "      s += sM[" << k << "] * ctot;\n";
+    if (any_collider) o << "      s = fma(sM[" << k << "], ctot, s);\n";
     if (any_inert) o << "      s += sN[" << k << "];\n";
-    o << "      const double ws = w[" << k << "] - s, hw = hRT[" << k << "] * " << lit(sp(k, 1)) << ";\n"
+    o << "      const double ws = w[" << k << "] - s, hw = hk[" << k << "] * " << lit(sp(k, 1)) << ";\n"
       << "      const double ak = " << lit(sp(k, 0)) << " * (wb * ws" << (any_collider ? " + sM[" + S(k) + "]" : std::string())
-      << ");\n"
-      << "      const double n0 = " << lit(sp(k, 0)) << " * invrho * (v0 - ws * invT);\n      " << W(a, 0)
-      << " = n0;\n      tr0 += hw * n0;\n";
-    for (int b = 1; b < NA; ++b)
-      o << "      const double n" << b << " = v" << b << " - ak * " << lit(sp(act[b] - 1, 1)) << ";\n      " << W(a, b)
-        << " = n" << b << ";\n      tr" << b << " += hw * n" << b << ";\n";
-    o << "    }\n";
+      << ");\n";
+    for (int b = 0; b < NR; ++b) {
+      const int l = sys.keep[b];
+      double iw = sp(l, 1);
+      o << "      const double n" << b << " = v" << 1 + l;
+      for (size_t e = 0; e < sys.elim.size(); ++e)
+        if (sys.b[e][b] != 0.0) {
+          o << " + " << lit(beta(e, b)) << " * v" << 1 + sys.elim[e];
+          iw += beta(e, b) * sp(sys.elim[e], 1);
+        }
+      o << " - ak * " << lit(iw) << ";\n      " << Wn(a, b) << " = n" << b << ";\n      tr" << b << " += hw * n" << b
+        << ";\n";
+    }
+    o << "      const double nT = " << lit(sp(k, 0)) << " * invrho * (v0 - ws * invT);\n      " << Wn(a, NR)
+      << " = nT;\n      tr" << NR << " += hw * nT;\n    }\n";
   }
   for (int k = 0; k < N; ++k) {
     const std::vector<double> d = {sp(k, 3), 2.0 * sp(k, 4), 3.0 * sp(k, 5), 4.0 * sp(k, 6)};
@@ -790,54 +999,66 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     o << "    dcp += y[" << 1 + k << "] * (" << horner(dw, "T") << ");\n";
     if (col[k] > 0) o << "    cpf += cpW[" << k << "] * f[" << 1 + k << "];\n";
   }
-  o << "    const double rc = RU * invcp;\n    " << W(0, 0) << " = rc * (cpf + f[0] * dcp - T * tr0);\n";
-  for (int b = 1; b < NA; ++b)
-    o << "    " << W(0, b) << " = rc * (f[0] * cpW[" << act[b] - 1 << "] - T * tr" << b << ");\n";
-  o << "  }\n  return true;\n}\n\n";
+  o << "    const double rc = RU * invcp;\n";
+  for (int b = 0; b < NR; ++b) {
+    o << "    " << Wn(NR, b) << " = rc * fma(f[0], cpW[" << sys.keep[b] << "]";
+    for (size_t e = 0; e < sys.elim.size(); ++e)
+      if (sys.b[e][b] != 0.0) o << " + " << lit(beta(e, b)) << " * cpW[" << sys.elim[e] << "]";
+    o << ", -(T * tr" << b << "));\n";
+  }
+  o << "    " << Wn(NR, NR) << " = rc * fma(-T, tr" << NR << ", fma(f[0], dcp, cpf));\n  }\n  return true;\n}\n\n";
 }
 
 }  // namespace
 
-// state entries (0: T, 1 + k: Y_k) of the generated kernel's linear systems: the
-// temperature and the species that some reaction changes
-static std::vector<int> active_entries(const df_mech* m) {
-  std::vector<int> act = {0};
-  const std::vector<Rx> rx = reactions_of(m);
-  for (int k = 0; k < m->dims.N; ++k)
-    if (std::any_of(rx.begin(), rx.end(), [k](const Rx& x) { return x.nu[k] != 0; })) act.push_back(1 + k);
-  return act;
-}
-
 std::string jit_thread_source(const df_mech* m) {
   const int N = m->dims.N, n = N + 1;
   const std::vector<Rx> rx = reactions_of(m);
-  const std::vector<int> act = active_entries(m);
-  const int NA = (int)act.size();
+  const Systems sys = systems_of(m, rx);
+  const int NA = sys.na(), NE = (int)sys.elim.size();
   const double T_low = fixed_T_low(m, rx);
   std::ostringstream o;
   o << "// generated for a " << N << "-species / " << m->dims.M << "-reaction mechanism\n"
     << "#include \"integrate_thread.cuh\"\n\nnamespace df {\n\n";
   emit_eval(o, m);
-  if (T_low > 0.0) emit_fixed(o, m, rx, act, T_low);
-  std::string list;
-  for (int a : act) list += (list.empty() ? "" : ", ") + std::to_string(a);
+  if (T_low > 0.0) emit_fixed(o, m, rx, sys, T_low);
+  std::string act, elim, beta;
+  for (int k : sys.keep) act += std::to_string(1 + k) + ", ";
+  for (int k : sys.elim) elim += std::to_string(1 + k) + ", ";
+  for (int e = 0; e < NE; ++e) {
+    beta += "{";
+    for (int a = 0; a < NA; ++a) {
+      const double b = a < NA - 1 ? sys.b[e][a] * (m->blob_host[m->dims.off_sp + SP_REC * sys.elim[e]] *
+                                                   m->blob_host[m->dims.off_sp + SP_REC * sys.keep[a] + 1])
+                                  : 0.0;
+      beta += lit(b) + ", ";
+    }
+    beta += "}, ";
+  }
   o << "struct GenEval {\n"
     << "  static constexpr bool kGenerated = true;\n"
-    << "  static constexpr int kN = " << N << ", kNA = " << NA << ";\n"
+    << "  static constexpr int kN = " << N << ", kNA = " << NA << ", kNE = " << NE << ";\n"
+    << "  static constexpr int kWords = " << sys.per_thread() << ";  // shared doubles per thread\n"
     << "  // state entry (0: T, 1 + k: Y_k) of row a of the linear systems\n"
-    << "  __device__ static constexpr int act(int a) {\n    constexpr int t[] = {" << list << "};\n    return t[a];\n  }\n"
-    << "  // any state, one copy for all kernels of the module: the FP64 evaluation,\n"
-    << "  // its full Jacobian compacted and negated\n"
+    << "  __device__ static constexpr int act(int a) {\n    constexpr int t[] = {" << act << "0};\n    return t[a];\n  }\n"
+    << "  // state entry of eliminated species e, and d Y_e / d Y of row a\n"
+    << "  __device__ static constexpr int elim(int e) {\n    constexpr int t[] = {" << elim << "0};\n    return t[e];\n  }\n"
+    << "  __device__ static constexpr double beta(int e, int a) {\n    constexpr double t[][" << NA << "] = {" << beta
+    << "{0.0}};\n    return t[e][a];\n  }\n"
+    << "  // any state, one copy for all evaluations: the FP64 evaluation, its full\n"
+    << "  // Jacobian reduced to the systems' and negated\n"
     << "  template <bool WITH_J>\n"
     << "  __device__ __noinline__ static void general(const MechView& mv, double pc, const double* y, double* f, double* W) {\n"
     << "    double yl[" << n << "], fl[" << n << "], J[WITH_J ? " << n * n << " : 1], sM[" << N << "];\n"
     << "    for (int i = 0; i < " << n << "; ++i) yl[i] = y[i];\n"
     << "    gen_eval<WITH_J, 1>(mv, pc, yl, fl, SVT<double, 1>{J, 1}, SVT<double, 1>{sM, 1});\n"
     << "    for (int i = 0; i < " << n << "; ++i) f[i] = fl[i];\n"
-    << "    if (WITH_J)\n#pragma unroll 1\n      for (int a = 0; a < " << NA << "; ++a)\n"
-    << "#pragma unroll 1\n        for (int b = 0; b < " << NA << "; ++b) W[a * " << NA << " + b] = -J[act(a) * " << n
-    << " + act(b)];\n  }\n"
-    << "  // f and, with WITH_J, -J over act() (row-major)\n"
+    << "    if (WITH_J) {\n#pragma unroll 1\n      for (int a = 0; a < kNA; ++a) {\n"
+    << "#pragma unroll 1\n        for (int b = 0; b < kNA; ++b) {\n"
+    << "          double v = J[act(a) * " << n << " + act(b)];\n"
+    << "          for (int e = 0; e < kNE; ++e) v += beta(e, b) * J[act(a) * " << n << " + elim(e)];\n"
+    << "          W[a * kNA + b] = -v;\n        }\n      }\n    }\n  }\n"
+    << "  // f (without J only the entries act()) and, with WITH_J, -J over act() (row-major)\n"
     << "  template <bool WITH_J, int ST>\n"
     << "  __device__ __forceinline__ static void run(const MechView& mv, double pc, const double (&y)[" << n
     << "], double (&f)[" << n << "], SVT<double, ST> W) {\n";
@@ -1239,8 +1460,7 @@ int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, cuda
     auto it = g_modules.find(key);
     if (it == g_modules.end()) it = g_modules.emplace(key, build_module(dev, m, src, variant)).first;
     md = &it->second;
-    const int na = (int)active_entries(m).size();
-    md->per_thread = na * (na + 1);
+    md->per_thread = systems_of(m, reactions_of(m)).per_thread();
     m->jit_module[dev][variant] = md;
     m->jit_note = !md->ok          ? md->why
                   : md->from_cache ? std::string("generated kernel loaded from the on-disk cache")

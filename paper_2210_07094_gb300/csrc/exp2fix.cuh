@@ -31,9 +31,9 @@ __device__ __forceinline__ uint64_t mulhi64_3(uint32_t ah, uint32_t al, uint32_t
   return wmad(ah, bh, (uint64_t)__umulhi(ah, bl)) + __umulhi(al, bh);
 }
 
-// 2^((X + 1/2) 2^-53): X is the floor of a value, its mean the half unit above.
-// |X| < 1022 2^53 (normal results).
-__device__ __forceinline__ double exp2_fixed(int64_t X) {
+// 2^((X + 1/2) 2^-53) = r 2^(e - 63) with r in [2^63, 2^64): X is the floor of a
+// value, its mean the half unit above
+__device__ __forceinline__ uint64_t exp2_parts(int64_t X, int& e) {
   const uint32_t xh = (uint32_t)((uint64_t)X >> 32), xl = (uint32_t)X;
   const uint64_t t = __ldg(reinterpret_cast<const unsigned long long*>(g_exp2fix_tab) + ((xh >> 13) & 255u));
   const uint32_t gh = (xh << 19) | (xl >> 13), gl = (xl << 19) | (1u << 18);
@@ -42,10 +42,80 @@ __device__ __forceinline__ double exp2_fixed(int64_t X) {
   const uint64_t h1 = EXP2FIX_A1 + (mulhi64_3(gh, gl, (uint32_t)(h2 >> 32), (uint32_t)h2) >> 10);  // 2^72
   const uint64_t p = mulhi64_3(gh, gl, (uint32_t)(h1 >> 32), (uint32_t)h1);                       // 2^72
   const uint64_t q = mulhi64_3((uint32_t)(t >> 32), (uint32_t)t, (uint32_t)(p >> 32), (uint32_t)p);
-  const uint64_t r = t + (q >> 8);  // in [2^63, 2^64)
-  // the leading 53 bits, rounded; the leading one adds 1 to the exponent field
-  const uint64_t e = (uint64_t)((uint32_t)(((int32_t)xh >> 21) + 1022) << 20) << 32;
-  return __longlong_as_double((long long)(e + (r >> 11) + ((r >> 10) & 1u)));
+  e = (int32_t)xh >> 21;
+  return t + (q >> 8);
+}
+
+// the same as a double, |X| < 1022 2^53 (normal results): the leading 53 bits,
+// rounded; the leading one adds 1 to the exponent field
+__device__ __forceinline__ double exp2_fixed(int64_t X) {
+  int e;
+  const uint64_t r = exp2_parts(X, e);
+  const uint64_t f = (uint64_t)((uint32_t)(e + 1022) << 20) << 32;
+  return __longlong_as_double((long long)(f + (r >> 11) + ((r >> 10) & 1u)));
+}
+
+// Rates as unpacked floating-point numbers m 2^e: a product of a rate constant
+// with up to three concentrations is a chain of integer multiplications, seven
+// instructions each where an FP64 multiplication occupies its pipe for 64 cycles.
+// The constant enters with 64 bits, each concentration with 53 at bit 62, and a
+// product drops at most two leading bits, so 57 remain after three: no rounding
+// until the number is packed.  The sign is the top bit of the concentrations'
+// exclusive or, carried beside.
+struct Fx {
+  uint64_t m;
+  int e;
+};
+
+__device__ __forceinline__ Fx fx_exp2(int64_t X) {
+  Fx a;
+  a.m = exp2_parts(X, a.e);
+  a.e -= 63;
+  return a;
+}
+
+// a finite double for fx_mul (e: the exponent's share of the product); zeros and
+// subnormals become numbers that pack to zero
+__device__ __forceinline__ Fx fx_factor(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x), e = (hi >> 20) & 0x7ffu;
+  Fx a;
+  a.m = ((uint64_t)(0x40000000u | ((hi << 10) & 0x3fffffffu) | (lo >> 22)) << 32) | (lo << 10);
+  a.e = e ? (int)e - 1021 : -100000;
+  return a;
+}
+
+__device__ __forceinline__ Fx fx_mul(Fx a, Fx c) {
+  Fx p;
+  p.m = mulhi64_3((uint32_t)(a.m >> 32), (uint32_t)a.m, (uint32_t)(c.m >> 32), (uint32_t)c.m);
+  p.e = a.e + c.e;
+  return p;
+}
+
+// sign m 2^e as a double (truncated), 0 below the normal range, infinity above it
+__device__ __forceinline__ double fx_pack(uint64_t m, int e, uint32_t sign) {
+  const int lz = __clzll((long long)m);
+  const uint64_t r = m << (lz & 63);
+  const uint32_t f = (uint32_t)(e - lz + 1085);  // exponent field - 1
+  uint64_t b = ((uint64_t)(f << 20) << 32) + (r >> 11);
+  if (f >= 2046u || m == 0) b = (int)f < 0 || m == 0 ? 0 : 0x7ff0000000000000ull;
+  return __longlong_as_double((long long)(b | ((uint64_t)(sign & 0x80000000u) << 32)));
+}
+__device__ __forceinline__ double fx_pack(Fx a, uint32_t sign) { return fx_pack(a.m, a.e, sign); }
+
+// a - b, signs apart; both m below 2^63
+__device__ __forceinline__ double fx_diff(Fx a, uint32_t sa, Fx b, uint32_t sb) {
+  const int d = a.e - b.e;
+  const uint64_t am = a.m >> min(max(-d, 0) + 1, 63), bm = b.m >> min(max(d, 0) + 1, 63);
+  const int64_t opp = (int64_t)((int32_t)(sa ^ sb) >> 31);  // all ones: the magnitudes add
+  const int64_t v = (int64_t)am - (((int64_t)bm ^ opp) - opp);
+  const int64_t neg = v >> 63;
+  return fx_pack((uint64_t)((v ^ neg) - neg), max(a.e, b.e) + 1, sa ^ (uint32_t)(neg >> 32));
+}
+
+// v 2^-53 as a double
+__device__ __forceinline__ double fixed_to_double(int64_t v) {
+  const int64_t neg = v >> 63;
+  return fx_pack((uint64_t)((v ^ neg) - neg), -53, (uint32_t)(neg >> 32));
 }
 
 // x log2(e) as floor(x log2(e) 2^53), |x| < 512: the 53-bit mantissa (at bit

@@ -205,21 +205,22 @@ __device__ __forceinline__ bool ros_attempt(const MechView& mv, const RosTab& tb
 }
 
 // The attempt with a generated evaluation (EVAL, see codegen.cu).  NA is the
-// order of the linear systems: the temperature and the species that some
-// reaction changes.  An inert species has a zero row in J, so its stage vectors
-// are zero and its column never matters: on the H2/air mechanism the systems are
-// 9 x 9 instead of 10 x 10 (N2), 27% fewer operations in the factorisation.
+// order of the linear systems: the temperature and the species that neither are
+// inert nor follow from the others by the conservation of the elements, which
+// holds exactly for every stage vector (Systems in codegen.cu).  On the H2/air
+// mechanism they are 7 x 7 (N2 inert, H and O conserved) instead of 10 x 10: a
+// third of the operations in the factorisation, half in the solves.
 // EVAL writes -J (compact, row-major) where W = I/(h gamma) - J is wanted.
 //
-// Shared memory holds only W and one vector, NA (NA + 1) doubles per thread: the
-// stage vectors of the finished stages, read once per later stage in long
-// independent runs, go to local memory (about 1% of the attempt's time), and the
-// substitutions run in registers.  On the 9-species mechanism that is 90
-// doubles instead of 160, eight warps per SM instead of five, two for every
-// FP64 pipe: one warp's integer work and shared-memory waits hide behind the
-// other's FP64 work.  With the fixed-point rate exponents of gen_fixed, 2^20
-// cells of the bimodal 9-species field went from 41.6 to 24.4 ms, 96 cells (one
-// warp's latency) from 432 to 257 us.
+// Shared memory holds only W and one vector per thread: the stage vectors of the
+// finished stages, read once per later stage in long independent runs, go to
+// local memory (about 1% of the attempt's time), and the substitutions run in
+// registers.  That leaves room for eight warps per SM, two for every FP64 pipe (the
+// registers allow no more: with 168 instead of 255 per thread a third warp per
+// pipe made 2^20 cells 22.1 instead of 19.3 ms).
+// 2^20 cells of the bimodal 9-species field: 41.6 ms with the 10 x 10 systems at
+// five warps per SM, 24.4 with 9 x 9 at eight, 21.0 with the rate products on the
+// integer pipes, 19.3 with 7 x 7.
 template <int ST, class EVAL>
 __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab& tb, double pc,
                                                 const double (&y)[EVAL::kN + 1], double& h, double rtol, double atolY,
@@ -248,6 +249,14 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
   bool fin = true;
 #pragma unroll
   for (int i = 0; i < n; ++i) ynew[i] = y[i];
+  // the eliminated species' share of an increment d of the others
+  auto elim_of = [](int e, const double(&d)[NA]) {
+    double v = 0.0;
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+      if (EVAL::beta(e, a) != 0.0) v += EVAL::beta(e, a) * d[a];
+    return v;
+  };
 #pragma unroll 1
   for (int s = 0; s < tb.s; ++s) {
     const bool tail = tb.tail && s == tb.s - 1;
@@ -260,10 +269,7 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
       const bool newf = tb.newf[s] != 0;
       double g[NA];
 #pragma unroll
-      for (int a = 0; a < NA; ++a) {
-        g[a] = y[EVAL::act(a)];
-        r[a] = 0.0;
-      }
+      for (int a = 0; a < NA; ++a) g[a] = r[a] = 0.0;
       if (tail) {
 #pragma unroll 1
         for (int j = 0; j < s; ++j) {
@@ -272,7 +278,12 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
           for (int a = 0; a < NA; ++a) r[a] += c * K[j][a];
         }
 #pragma unroll
-        for (int a = 0; a < NA; ++a) ynew[EVAL::act(a)] += K[s - 1][a];
+        for (int a = 0; a < NA; ++a) {
+          g[a] = K[s - 1][a];
+          ynew[EVAL::act(a)] += g[a];
+        }
+#pragma unroll
+        for (int e = 0; e < EVAL::kNE; ++e) ynew[EVAL::elim(e)] += elim_of(e, g);
       } else {
 #pragma unroll 1
         for (int j = 0; j < s; ++j) {
@@ -286,7 +297,9 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
         }
         if (newf) {
 #pragma unroll
-          for (int a = 0; a < NA; ++a) ynew[EVAL::act(a)] = g[a];
+          for (int a = 0; a < NA; ++a) ynew[EVAL::act(a)] = y[EVAL::act(a)] + g[a];
+#pragma unroll
+          for (int e = 0; e < EVAL::kNE; ++e) ynew[EVAL::elim(e)] = y[EVAL::elim(e)] + elim_of(e, g);
         }
       }
       if (newf) {
@@ -330,13 +343,14 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
       // stiffly accurate tables: the last stage is the error estimate, and
       // y_new = Y_{s-1} + K_{s-1} (see ros_attempt)
 #pragma unroll
-      for (int a = 0; a < NA; ++a) {
-        const int i = EVAL::act(a);
-        const double yn = ynew[i] + r[a];
+      for (int a = 0; a < NA + EVAL::kNE; ++a) {
+        const int i = a < NA ? EVAL::act(a) : EVAL::elim(a - NA);
+        const double ei = a < NA ? r[a < NA ? a : 0] : elim_of(a - NA, r);
+        const double yn = ynew[i] + ei;
         fin = fin && (__double2hiint(yn) & 0x7ff00000) != 0x7ff00000;
         ynew[i] = yn;
         const double sc = (i == 0 ? atolT : atolY) + rtol * fmax(fabs(y[i]), fabs(yn));
-        const double q = r[a] * rcp_nr(sc);
+        const double q = ei * rcp_nr(sc);
         e2 += q * q;
       }
     }

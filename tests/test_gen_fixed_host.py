@@ -39,6 +39,9 @@ struct D3 { int x, y, z; };
 static D3 threadIdx, blockIdx, blockDim, gridDim;
 static inline uint32_t __umulhi(uint32_t a, uint32_t b) { return (uint32_t)(((uint64_t)a * b) >> 32); }
 static inline int __clz(unsigned x) { return x ? __builtin_clz(x) : 32; }
+static inline int __clzll(long long x) { return x ? __builtin_clzll(x) : 64; }
+template <class T> T min(T a, T b) { return a < b ? a : b; }
+template <class T> T max(T a, T b) { return a > b ? a : b; }
 static inline uint64_t bits_of(double x) { uint64_t u; memcpy(&u, &x, 8); return u; }
 static inline double of_bits(uint64_t u) { double x; memcpy(&x, &u, 8); return x; }
 static inline int __double2hiint(double x) { return (int)(bits_of(x) >> 32); }
@@ -55,6 +58,7 @@ static inline int __popc(unsigned) { return 0; }
 template <class T> T __shfl_sync(unsigned, T v, int) { return v; }
 template <class T> T __shfl_down_sync(unsigned, T v, int) { return v; }
 static inline void __syncthreads() {}
+static inline double __dsub_rn(double a, double b) { return a - b; }
 """
 
 DRIVER = r"""
@@ -99,40 +103,62 @@ int main() {
     for (int i = 0; i < n; ++i) {
       const double tol = 100 * fabs(f2[i] - fe[i]) + 1e-11 * (i ? nf : fabs(fe[0])) + 1e-280;
       wf = fmax(wf, fabs(f[i] - fe[i]) / tol);
-      wp = fmax(wp, fabs(f[i] - fp_[i]) / tol);
+      for (int a = 0; a < NA; ++a)  // without J only the systems' entries
+        if (GenEval::act(a) == i) wp = fmax(wp, fabs(f[i] - fp_[i]) / tol);
     }
+    // the columns over the kept species: beta times the eliminated ones' added
+    auto red = [&](const double* A, int ra, int b) {
+      double v = A[ra + GenEval::act(b)];
+      for (int e = 0; e < GenEval::kNE; ++e) v += GenEval::beta(e, b) * A[ra + GenEval::elim(e)];
+      return v;
+    };
     for (int a = 0; a < NA; ++a) {
       double nr = 1e-300;
       const int ra = GenEval::act(a) * n;
-      for (int b = 0; b < NA; ++b) nr = fmax(nr, fabs(J[ra + GenEval::act(b)]));
-      if (a == 0) {  // the temperature row sums h_k times the species rows: its terms
+      for (int j = 0; j < n; ++j) nr = fmax(nr, fabs(J[ra + j]));
+      if (ra == 0) {  // the temperature row sums h_k times the species rows: its terms
         const double T = y[0];
         double cp = 0;
         for (int k = 0; k < N; ++k) {
           const double* c = mv.sp + SP_REC * k + 2;
           cp += y[1 + k] * mv.sp[SP_REC * k + 1] * (c[0] + T * (c[1] + T * (c[2] + T * (c[3] + T * c[4]))));
         }
-        for (int b = 0; b < NA; ++b) {
+        for (int j = 0; j < n; ++j) {
           double s = 0;
           for (int k = 0; k < N; ++k) {
             const double* c = mv.sp + SP_REC * k + 2;
             const double h = c[0] + T * (c[1] / 2 + T * (c[2] / 3 + T * (c[3] / 4 + T * c[4] / 5))) + c[5] / T;
-            s += fabs(T * h * mv.sp[SP_REC * k + 1] * J[(1 + k) * n + GenEval::act(b)]);
+            s += fabs(T * h * mv.sp[SP_REC * k + 1] * J[(1 + k) * n + j]);
           }
           nr = fmax(nr, s / fabs(cp));
         }
       }
       for (int b = 0; b < NA; ++b) {
-        const int id = ra + GenEval::act(b);
-        const double e = fabs(W[a * NA + b] + J[id]) / (100 * fabs(J2[id] - J[id]) + 1e-11 * nr);
+        const double j = red(J, ra, b), e = fabs(W[a * NA + b] + j) / (100 * fabs(red(J2, ra, b) - j) + 1e-11 * nr);
         if (!(e <= wj)) wj = e;
       }
     }
-    for (int i = 0; i < n; ++i) {  // rows outside act() are zero
-      bool act = false;
-      for (int a = 0; a < NA; ++a) act = act || GenEval::act(a) == i;
-      for (int j = 0; j < n && !act; ++j)
-        if (J[i * n + j] != 0.0 || fe[i] != 0.0 || f[i] != 0.0) return 5;
+    auto row_max = [&](int i) {
+      double v = 0;
+      for (int j = 0; j < n; ++j) v = fmax(v, fabs(J[i * n + j]));
+      return v;
+    };
+    for (int i = 0; i < n; ++i) {  // the other rows are zero or follow from the systems'
+      int e = 0, act = 0;
+      for (int a = 0; a < NA; ++a) act += GenEval::act(a) == i;
+      while (e < GenEval::kNE && GenEval::elim(e) != i) ++e;
+      if (act + (e < GenEval::kNE) > 1) return 5;
+      for (int j = -1; j < n && !act; ++j) {
+        double v = j < 0 ? fe[i] : J[i * n + j], terms = j < 0 ? nf : row_max(i);
+        for (int a = 0; a < NA && e < GenEval::kNE; ++a) {
+          const int ra = GenEval::act(a);
+          const double t = GenEval::beta(e, a) * (j < 0 ? fe[ra] : J[ra * n + j]);
+          v -= t;
+          terms += fabs(GenEval::beta(e, a)) * (j < 0 ? nf : row_max(ra));
+        }
+        if (!(fabs(v) <= 1e-11 * terms)) return 6;
+        if (e == GenEval::kNE && f[i] != 0.0) return 7;
+      }
     }
   }
   printf("inside %d f %g J %g plain %g\n", inside, wf, wj, wp);
