@@ -392,6 +392,11 @@ struct Systems {
   int per_thread() const {
     return std::max(na() * (na() + 1), (int)(keep.size() * (act.size() + 1)));
   }
+  // further words, for the exponents of a group of reactions.  More words make
+  // longer runs of independent work, but what shared memory does not take is L1 for
+  // the threads' local memory (states, stage vectors): 2^20 cells of the 9-species
+  // field take 16.6, 15.9, 16.1, 16.9, 18.6 ms with 12, 20, 28, 36, 52 words.
+  static constexpr int exponents() { return 20; }
 };
 
 struct Ratio {
@@ -496,12 +501,16 @@ double fixed_T_low(const df_mech* m, const std::vector<Rx>& rx) {
                       T * (sp(k, 3) / 2 + T * (sp(k, 4) / 6 + T * (sp(k, 5) / 12 + T * sp(k, 6) / 20))) + sp(k, 7) / T);
       }
       for (const Rx& x : rx) {
+        worst = std::max(worst, std::fabs(x.b) + std::fabs(x.E) / T);
         const double kf = 400.0 + L2E * std::fabs(x.b * std::log(T) - x.E / T);
         double sg = -x.dnu * L2E * (LOG_PSTD_RU - std::log(T));
         for (int k : x.spc) sg += x.nu[k] * g[k];
         worst = std::max({worst, kf, kf + std::fabs(sg)});
         if (x.type == 2) {
           const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
+          // the centring must be a positive number for its logarithm
+          const double Fc = (1.0 - tr[3]) * std::exp(-T * tr[4]) + tr[3] * std::exp(-T * tr[5]) + std::exp(-tr[6] / T);
+          if (!(Fc > 1e-60 && Fc < 1e60)) worst = INFINITY;
           const double d = L2E * std::fabs(tr[0] + (tr[1] - x.b) * std::log(T) - (tr[2] - x.E) / T);
           worst = std::max({worst, d, kf + d, std::fabs(sg)});
         }
@@ -512,54 +521,9 @@ double fixed_T_low(const df_mech* m, const std::vector<Rx>& rx) {
   return 0.0;
 }
 
-// "K C[a] C[b] ..." and, with derivatives, d(K prod C)/dC_l of each distinct
-// species: statements that define `name`p and `name`d<l>
-std::string product_code(const std::string& name, const std::string& K, std::vector<int> e, bool deriv) {
-  std::ostringstream o;
-  auto C = [](int k) { return "C[" + std::to_string(k) + "]"; };
-  auto d = [&](int k) { return name + "d" + std::to_string(k); };
-  if (!deriv) {
-    o << "    const double " << name << "p = " << K;
-    for (int k : e) o << " * " << C(k);
-    o << ";\n";
-    return o.str();
-  }
-  // equal species first
-  if (e.size() == 3 && e[0] != e[1]) {
-    if (e[0] == e[2]) std::swap(e[1], e[2]);
-    else if (e[1] == e[2]) std::swap(e[0], e[2]);
-  }
-  const std::string t = "    const double ";
-  if (e.size() == 1) {
-    o << t << d(e[0]) << " = " << K << ";\n" << t << name << "p = " << K << " * " << C(e[0]) << ";\n";
-  } else if (e.size() == 2) {
-    if (e[0] == e[1]) {
-      o << t << name << "t = " << K << " * " << C(e[0]) << ";\n"
-        << t << d(e[0]) << " = 2.0 * " << name << "t;\n" << t << name << "p = " << name << "t * " << C(e[0]) << ";\n";
-    } else {
-      o << t << d(e[0]) << " = " << K << " * " << C(e[1]) << ";\n" << t << d(e[1]) << " = " << K << " * " << C(e[0])
-        << ";\n" << t << name << "p = " << d(e[1]) << " * " << C(e[1]) << ";\n";
-    }
-  } else if (e[0] == e[1] && e[1] == e[2]) {
-    o << t << name << "t = " << K << " * " << C(e[0]) << " * " << C(e[0]) << ";\n"
-      << t << d(e[0]) << " = 3.0 * " << name << "t;\n" << t << name << "p = " << name << "t * " << C(e[0]) << ";\n";
-  } else if (e[0] == e[1]) {
-    o << t << name << "t = " << K << " * " << C(e[0]) << ";\n"
-      << t << d(e[2]) << " = " << name << "t * " << C(e[0]) << ";\n"
-      << t << d(e[0]) << " = 2.0 * (" << name << "t * " << C(e[2]) << ");\n"
-      << t << name << "p = " << d(e[2]) << " * " << C(e[2]) << ";\n";
-  } else {
-    o << t << name << "t = " << K << " * " << C(e[0]) << ";\n"
-      << t << d(e[2]) << " = " << name << "t * " << C(e[1]) << ";\n"
-      << t << d(e[1]) << " = " << name << "t * " << C(e[2]) << ";\n"
-      << t << d(e[0]) << " = " << K << " * (" << C(e[1]) << " * " << C(e[2]) << ");\n"
-      << t << name << "p = " << d(e[2]) << " * " << C(e[2]) << ";\n";
-  }
-  return o.str();
-}
-
-// The same as unpacked numbers from the rate constant `K`: `name`p, and with
-// derivatives the doubles `name`d<l>; `name`s is the sign word of the product
+// The product of the rate constant `K` and the concentrations C[e], unpacked: `name`p,
+// and with derivatives by each distinct species the doubles `name`d<l>; `name`s is
+// the sign word of the product
 std::string fx_product_code(const std::string& name, const std::string& K, std::vector<int> e, bool deriv) {
   std::ostringstream o;
   auto X = [](int k) { return "x" + std::to_string(k); };
@@ -664,7 +628,7 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
   }
   o << "template <bool WITH_J, int ST>\n"
     << "__device__ __forceinline__ bool gen_fixed(const MechView& mv, const double pc, const double (&y)[" << N + 1
-    << "], double (&f)[" << N + 1 << "], SVT<double, ST> W) {\n"
+    << "], double (&f)[" << N + 1 << "], SVT<double, ST> W, SVT<double, ST> E) {\n"
     << "  constexpr int NS = " << N << ";\n"
     << "  const double T = y[0];\n"
     << "  if (!mv.fix[" << m->dims.M << "] || !(T >= " << lit(T_low) << " && T < " << lit(kFixTHi) << ")) return false;\n"
@@ -705,11 +669,8 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     o << "  const double ctot = rho * sumYW;\n";
   }
   for (int k = 0; k < N; ++k) o << "  const Fx x" << k << " = fx_factor(C[" << k << "]);\n  (void)x" << k << ";\n";
-  // h/RT of the kept species with the eliminated ones' shares (the heat release
-  // and the temperature row need no others); with J also of every reacting
-  // species, in fixed point, for d ln K_c/dT
-  o << "  double hk[NS], w[NS], sM[NS], sN[NS];\n  int64_t H[NS];\n  const double invT2 = invT * invT;\n"
-    << "  (void)H; (void)sM; (void)sN; (void)invT2;\n";
+  // h/RT: with J of every reacting species, in fixed point, for d ln K_c/dT
+  o << "  double w[NS], sM[NS], sN[NS];\n  int64_t H[NS];\n  (void)H; (void)sM; (void)sN;\n";
   auto enthalpy = [&](const std::string& dst, const std::vector<double>& c) {
     return "    " + dst + " = " + fixed_const(c[0], false) + ";\n" + fixed_term(dst, c[1], false, "t1", 50) +
            fixed_term(dst, c[2], false, "t2", 36) + fixed_term(dst, c[3], false, "t3", 22) +
@@ -718,14 +679,6 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
   auto hcoef = [&](int k) {
     return std::vector<double>{sp(k, 2), sp(k, SP_H), sp(k, SP_H + 1), sp(k, SP_H + 2), sp(k, SP_H + 3), sp(k, 7)};
   };
-  for (int a = 0; a < NR; ++a) {
-    std::vector<double> c = hcoef(sys.keep[a]);
-    for (size_t e = 0; e < sys.elim.size(); ++e) {
-      const std::vector<double> ce = hcoef(sys.elim[e]);
-      for (int i = 0; i < 6; ++i) c[i] += sys.b[e][a] * ce[i];
-    }
-    o << "  {\n    int64_t h;\n" << enthalpy("h", c) << "    hk[" << sys.keep[a] << "] = fixed_to_double(h);\n  }\n";
-  }
   o << "  if (WITH_J) {\n";
   for (int k : sys.act) o << enthalpy("H[" + S(k) + "]", hcoef(k));
   o << "  }\n";
@@ -802,17 +755,51 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     else s << (st ? " += " : " = ") << c << ".0 * " << v << ";\n";
     return s.str();
   };
-  for (size_t j = 0; j < rx.size(); ++j) {
-    const Rx& x = rx[j];
-    o << "  {  // rate " << j << "\n    int64_t x = mv.fix[" << j << "];\n"
-      << fixed_term("x", x.b, false, "L", 60) << fixed_term("x", -x.E, true, "I", 69);
-    if (x.rev) {
+  // the exponents of the reactions [j, j1) and then all their powers of two: of an
+  // elementary or third-body reaction k_f and (reversible) k_r, of a falloff
+  // reaction k_inf, k_0 / k_inf and (reversible) 1 / K_c
+  const int cap = Systems::exponents();
+  std::vector<int> slot(rx.size());
+  auto exponents = [&](size_t j0) {
+    size_t j1 = j0;
+    int n = 0;
+    for (; j1 < rx.size(); ++j1) {
+      const int words = 1 + (rx[j1].type == 2 ? 1 : 0) + (rx[j1].rev ? 1 : 0);
+      if (n + words > cap) break;
+      slot[j1] = n;
+      n += words;
+    }
+    auto E = [&](int i) { return "    E[" + std::to_string(i) + "] = __longlong_as_double("; };
+    for (size_t j = j0; j < j1; ++j) {
+      const Rx& x = rx[j];
+      o << "  {\n    int64_t x = mv.fix[" << j << "];\n"
+        << fixed_term("x", x.b, false, "L", 60) << fixed_term("x", -x.E, true, "I", 69) << E(slot[j]) << "x);\n";
       std::string sg;
       for (int k : x.spc)
         for (int i = 0; i < std::abs(x.nu[k]); ++i) sg += (x.nu[k] > 0 ? " + G[" : " - G[") + S(k) + "]";
       for (int i = 0; i < std::abs(x.dnu); ++i) sg += x.dnu > 0 ? " - lp" : " + lp";
-      o << "    const int64_t xc = 0" << sg << ";\n";
+      if (x.type == 2) {
+        const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
+        o << "    int64_t xd = " << fixed_const(tr[0], true) << ";\n"
+          << fixed_term("xd", tr[1] - x.b, false, "L", 60) << fixed_term("xd", -(tr[2] - x.E), true, "I", 69)
+          << E(slot[j] + 1) << "xd);\n";
+        if (x.rev) o << E(slot[j] + 2) << "(int64_t)0" << sg << ");\n";
+      } else if (x.rev) {
+        o << E(slot[j] + 1) << "x" << sg << ");\n";
+      }
+      o << "  }\n";
     }
+    const int padded = (n + 3) / 4 * 4;
+    for (int i = n; i < padded; ++i) o << E(i).substr(2) << "0);\n";
+    o << "  fx_exp2_all<" << padded << ">(E);\n";
+    return j1;
+  };
+  size_t group_end = 0;
+  for (size_t j = 0; j < rx.size(); ++j) {
+    const Rx& x = rx[j];
+    if (j == group_end) group_end = exponents(j);
+    auto K = [&](int i) { return "fx_word(E[" + std::to_string(i) + "])"; };
+    o << "  {  // rate " << j << "\n";
     if (x.type != 0) {
       o << "    double Mc = ctot;\n";
       for (int l = 0; l < N; ++l) {
@@ -822,11 +809,13 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     }
     // d ln k / dT and d ln K_c / dT
     std::ostringstream dl;
-    dl << "      const double dk = fma(" << lit(x.E) << ", invT2, " << lit(x.b) << " * invT);\n";
+    // (times T: the column d/dT takes the factor 1/T when the row is finished)
+    dl << "      int64_t bE = " << fixed_const(x.b, false) << ";\n"
+       << fixed_term("bE", x.E, false, "I", 69) << "      const double dk = fixed_to_double(bE);\n";
     std::string dKc = "fixed_to_double(" + S(-x.dnu) + "LL * (1LL << 53)";
     for (int k : x.spc)
       for (int i = 0; i < std::abs(x.nu[k]); ++i) dKc += (x.nu[k] > 0 ? " + H[" : " - H[") + S(k) + "]";
-    dKc += ") * invT";
+    dKc += ")";
     auto has_dq = [&](int l) {
       return std::find(x.r.begin(), x.r.end(), l) != x.r.end() ||
              (x.rev && std::find(x.p.begin(), x.p.end(), l) != x.p.end());
@@ -873,8 +862,8 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     };
     std::ostringstream upd;
     if (x.type != 2) {
-      o << "    const Fx kf = fx_exp2(x);\n";
-      if (x.rev) o << "    const Fx kr = fx_exp2(x + xc);\n";
+      o << "    const Fx kf = " << K(slot[j]) << ";\n";
+      if (x.rev) o << "    const Fx kr = " << K(slot[j] + 1) << ";\n";
       for (int wj = 1; wj >= 0; --wj) {
         if (wj) o << "    if (WITH_J) {\n";
         else o << "    } else {\n";
@@ -899,52 +888,72 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
       o << "    }\n  }\n";
       continue;
     }
-    // Troe falloff: the expressions of rate_compute, the rate constants from the
-    // fixed-point exponents
+    // Troe falloff: the expressions of rate_compute with logarithms to base 2, in
+    // fixed point up to the quotient; k = k_inf Pr/(1 + Pr) F as an unpacked number
     const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
-    o << "    int64_t xd = " << fixed_const(tr[0], true) << ";  // k0 / kinf\n"
-      << fixed_term("xd", tr[1] - x.b, false, "L", 60) << fixed_term("xd", -(tr[2] - x.E), true, "I", 69)
-      << "    const double kinf = exp2_fixed(x), Pr = exp2_fixed(xd) * Mc;\n"
-      << "    if (Pr > 0.0) {\n"
+    uint64_t c67, c127, c14;
+    int none;
+    fixed_literal(0.67, false, 64, &c67, &none);
+    fixed_literal(1.27, false, 63, &c127, &none);
+    fixed_literal(0.14, false, 64, &c14, &none);
+    const double L10 = 3.32192809488736234787;  // log2(10)
+    auto q52 = [](double v) { return std::to_string((long long)std::llround(std::ldexp(v, 52))) + "LL"; };
+    o << "    const Fx kinf = " << K(slot[j]) << ";\n"
+      << "    const double Pr = fx_pack(" << K(slot[j] + 1) << ", 0u) * Mc;\n"
+      << "    if (Pr >= 0x1p-1022) {\n"
       << "      double e3, e1;\n      exp_rate2(-T * " << lit(tr[4]) << ", -T * " << lit(tr[5]) << ", e3, e1);\n"
       << "      const double e2 = exp_rate(" << lit(-tr[6]) << " * invT);\n"
-      << "      const double invKc = " << (x.rev ? "exp2_fixed(xc)" : "0.0") << ";\n"
       << "      const double Fc = fma(" << lit(1.0 - tr[3]) << ", e3, fma(" << lit(tr[3]) << ", e1, e2));\n"
-      << "      const double Lc = log10_rate(Fc), cc = -0.4 - 0.67 * Lc, nn = 0.75 - 1.27 * Lc;\n"
-      << "      const double xl = log10_rate(Pr) + cc, den = nn - 0.14 * xl, den2 = den * den;\n"
-      << "      const double q1 = den2 * rcp_any(fma(xl, xl, den2));\n"
-      << "      const double F = exp_rate(LN10 * (Lc * q1)), onePr = rcp_any(1.0 + Pr);\n"
-      << "      const double kf = kinf * Pr * onePr * F, kr = kf * invKc;\n";
+      << "      const int64_t lc = log2_q52(Fc), lx = log2_q52(Pr) - " << q52(0.4 * L10) << " - mul_fixed_signed(lc, "
+      << hex64(c67) << ");\n"
+      << "      const int64_t ln = " << q52(0.75 * L10) << " - 2 * mul_fixed_signed(lc, " << hex64(c127) << ");\n"
+      << "      const double xl = q52_to_double(lx), den = q52_to_double(ln - mul_fixed_signed(lx, " << hex64(c14) << "));\n"
+      << "      const double Lc = q52_to_double(lc), den2 = den * den;\n"
+      << "      const double q1 = den2 * rcp_any(fma(xl, xl, den2)), onePr = rcp_any(1.0 + Pr);\n"
+      << "      const Fx kf = fx_mul(fx_mul(kinf, fx_factor(Pr * onePr)), fx_exp2_factor(Lc * q1));\n";
+    if (x.rev) {
+      o << "      Fx kr = " << K(slot[j] + 2) << ";\n      kr.e += 64;\n      kr = fx_mul(kf, kr);\n";
+    }
     for (int wj = 1; wj >= 0; --wj) {
       const auto w0 = w_set;
-      o << (wj ? "      if (WITH_J) {\n" : "      } else {\n") << product_code("f", "kf", x.r, wj);
-      if (x.rev) o << product_code("b", "kr", x.p, wj);
-      o << "      const double q = " << (x.rev ? "__dsub_rn(fp, bp)" : "fp") << ";\n";
+      o << (wj ? "      if (WITH_J) {\n" : "      } else {\n") << fx_product_code("f", "kf", x.r, wj);
+      if (x.rev) o << fx_product_code("b", "kr", x.p, wj);
+      o << "      const double q = " << (x.rev ? "fx_diff(fp, fs, bp, bs)" : "fx_pack(fp, fs)") << ";\n";
       for (int k : x.spc)
         if (x.nu[k] != 0 && row[k] >= 0) o << "      " << add1(w_set, "w", k, x.nu[k], "q");
       if (wj) {
-        std::string Pf, Pb;
-        for (int k : x.r) Pf += (Pf.empty() ? "C[" : " * C[") + S(k) + "]";
-        for (int k : x.p) Pb += (Pb.empty() ? "C[" : " * C[") + S(k) + "]";
-        o << "      const double k0 = exp2_fixed(x + xd), rden = rcp_any(den), f1 = xl * rden;\n"
+        o << "      const double nn = q52_to_double(ln), rden = rcp_any(den), f1 = xl * rden;\n"
           << "      const double df1_dL = nn * rden * rden;\n"
           << "      const double df1_dLc = fma(-0.67, den, -(xl * (-1.27 + 0.67 * 0.14))) * (rden * rden);\n"
           << "      const double g2 = 2.0 * Lc * f1 * q1 * q1;\n"
           << "      const double gpr = fma(-g2, df1_dL, onePr), dlogF_dLc = fma(-g2, df1_dLc, q1);\n"
-          << "      const double dFc = fma(" << lit(-(1.0 - tr[3]) * tr[4]) << ", e3, fma(" << lit(-tr[3] * tr[5])
-          << ", e1, " << lit(tr[6]) << " * invT2 * e2));\n"
-          << "      const double dki = fma(" << lit(x.E) << ", invT2, " << lit(x.b) << " * invT);\n"
-          << "      const double dk0 = fma(" << lit(tr[2]) << ", invT2, " << lit(tr[1]) << " * invT);\n"
-          << "      const double dk = fma(dlogF_dLc * dFc, rcp_any(Fc), fma(gpr, dk0 - dki, dki));\n"
-          << "      const double dKc = " << dKc << ";\n"
-          << "      const double dqT = " << (x.rev ? "fma(q, dk, bp * dKc)" : "q * dk") << ";\n      (void)dKc;\n"
-          << "      const double dqM = k0 * F * gpr * onePr * "
-          << (x.rev ? "fma(-(" + Pb + "), invKc, " + Pf + ")" : "(" + Pf + ")") << ";\n"
-          << dqs("") << rows();
+          << "      const double dFc = fma(T, fma(" << lit(-(1.0 - tr[3]) * tr[4]) << ", e3, " << lit(-tr[3] * tr[5])
+          << " * e1), " << lit(tr[6]) << " * (invT * e2));\n"
+          << "      const double dki = fma(" << lit(x.E) << ", invT, " << lit(x.b) << ");\n"
+          << "      const double dk0 = fma(" << lit(tr[2]) << ", invT, " << lit(tr[1]) << ");\n"
+          << "      const double dk = fma(dlogF_dLc * dFc, rcp_any(Fc), fma(gpr, dk0 - dki, dki));\n";
+        if (x.rev)
+          o << "      const double dKc = " << dKc << ", pb = fx_pack(bp, bs);\n"
+            << "      const double dqT = fma(q, dk, pb * dKc);\n";
+        else
+          o << "      const double dqT = q * dk;\n";
+        // dk/d[M] = k gpr / [M]
+        o << "      const double dqM = q * (gpr * rcp_any(Mc));\n" << dqs("") << rows();
         w_set = w0;
       }
     }
     o << "      }\n    }\n  }\n";
+  }
+  // h/RT of the kept species with the eliminated ones' shares (the heat release
+  // and the temperature row need no others)
+  o << "  double hk[NS];\n";
+  for (int a = 0; a < NR; ++a) {
+    std::vector<double> c = hcoef(sys.keep[a]);
+    for (size_t e = 0; e < sys.elim.size(); ++e) {
+      const std::vector<double> ce = hcoef(sys.elim[e]);
+      for (int i = 0; i < 6; ++i) c[i] += sys.b[e][a] * ce[i];
+    }
+    o << "  {\n    int64_t h;\n" << enthalpy("h", c) << "    hk[" << sys.keep[a] << "] = fixed_to_double(h);\n  }\n";
   }
   // heat release and f
   o << "  double Hw = 0.0;\n";
@@ -989,7 +998,7 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
       o << " - ak * " << lit(iw) << ";\n      " << Wn(a, b) << " = n" << b << ";\n      tr" << b << " += hw * n" << b
         << ";\n";
     }
-    o << "      const double nT = " << lit(sp(k, 0)) << " * invrho * (v0 - ws * invT);\n      " << Wn(a, NR)
+    o << "      const double nT = " << lit(sp(k, 0)) << " * ((v0 - ws) * (invrho * invT));\n      " << Wn(a, NR)
       << " = nT;\n      tr" << NR << " += hw * nT;\n    }\n";
   }
   for (int k = 0; k < N; ++k) {
@@ -1038,7 +1047,7 @@ std::string jit_thread_source(const df_mech* m) {
   o << "struct GenEval {\n"
     << "  static constexpr bool kGenerated = true;\n"
     << "  static constexpr int kN = " << N << ", kNA = " << NA << ", kNE = " << NE << ";\n"
-    << "  static constexpr int kWords = " << sys.per_thread() << ";  // shared doubles per thread\n"
+    << "  static constexpr int kWords = " << sys.per_thread() << ";  // shared doubles per thread before the exponents'\n"
     << "  // state entry (0: T, 1 + k: Y_k) of row a of the linear systems\n"
     << "  __device__ static constexpr int act(int a) {\n    constexpr int t[] = {" << act << "0};\n    return t[a];\n  }\n"
     << "  // state entry of eliminated species e, and d Y_e / d Y of row a\n"
@@ -1061,8 +1070,8 @@ std::string jit_thread_source(const df_mech* m) {
     << "  // f (without J only the entries act()) and, with WITH_J, -J over act() (row-major)\n"
     << "  template <bool WITH_J, int ST>\n"
     << "  __device__ __forceinline__ static void run(const MechView& mv, double pc, const double (&y)[" << n
-    << "], double (&f)[" << n << "], SVT<double, ST> W) {\n";
-  if (T_low > 0.0) o << "    if (gen_fixed<WITH_J, ST>(mv, pc, y, f, W)) return;\n";
+    << "], double (&f)[" << n << "], SVT<double, ST> W, SVT<double, ST> E) {\n";
+  if (T_low > 0.0) o << "    if (gen_fixed<WITH_J, ST>(mv, pc, y, f, W, E)) return;\n";
   o << "    double yl[" << n << "], fl[" << n << "], Wl[WITH_J ? " << NA * NA << " : 1];\n"
     << "#pragma unroll\n    for (int i = 0; i < " << n << "; ++i) yl[i] = y[i];\n"
     << "    general<WITH_J>(mv, pc, yl, fl, Wl);\n"
@@ -1212,7 +1221,7 @@ struct Module {
   CUfunction fn = nullptr;
   size_t compile_ms = 0;
   bool from_cache = false;
-  int per_thread = 0;  // doubles of shared memory per thread: W and one vector
+  int per_thread = 0;  // doubles of shared memory per thread: the systems and the exponents
 };
 
 std::mutex g_mu;
@@ -1460,7 +1469,10 @@ int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, cuda
     auto it = g_modules.find(key);
     if (it == g_modules.end()) it = g_modules.emplace(key, build_module(dev, m, src, variant)).first;
     md = &it->second;
-    md->per_thread = systems_of(m, reactions_of(m)).per_thread();
+    {
+      const Systems sys = systems_of(m, reactions_of(m));
+      md->per_thread = sys.per_thread() + Systems::exponents();
+    }
     m->jit_module[dev][variant] = md;
     m->jit_note = !md->ok          ? md->why
                   : md->from_cache ? std::string("generated kernel loaded from the on-disk cache")

@@ -67,13 +67,6 @@ struct Fx {
   int e;
 };
 
-__device__ __forceinline__ Fx fx_exp2(int64_t X) {
-  Fx a;
-  a.m = exp2_parts(X, a.e);
-  a.e -= 63;
-  return a;
-}
-
 // a finite double for fx_mul (e: the exponent's share of the product); zeros and
 // subnormals become numbers that pack to zero
 __device__ __forceinline__ Fx fx_factor(double x) {
@@ -110,6 +103,59 @@ __device__ __forceinline__ double fx_diff(Fx a, uint32_t sa, Fx b, uint32_t sb) 
   const int64_t v = (int64_t)am - (((int64_t)bm ^ opp) - opp);
   const int64_t neg = v >> 63;
   return fx_pack((uint64_t)((v ^ neg) - neg), max(a.e, b.e) + 1, sa ^ (uint32_t)(neg >> 32));
+}
+
+// 2^((X + 1/2) 2^-53) of n exponents in a vector of 64-bit words, in place, |X| <
+// 1022 2^53: the leading 53 bits and the exponent (e + 1024) in the low 11.  Four
+// at a time, independent chains in one loop body: a warp alone on its
+// sub-partition waits out the latency of each dependent integer instruction
+// otherwise, and the code is there once.
+template <int N, class V>
+__device__ __forceinline__ void fx_exp2_all(V S) {
+#pragma unroll 1
+  for (int i = 0; i < N; i += 4) {
+    uint64_t m[4];
+    int e[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) m[k] = exp2_parts(__double_as_longlong(S[i + k]), e[k]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      S[i + k] = __longlong_as_double((long long)((m[k] & ~0x7ffull) | (uint32_t)((e[k] + 1024) & 0x7ff)));
+  }
+}
+
+// one of them; the bits the exponent took count as half a unit
+__device__ __forceinline__ Fx fx_word(double w) {
+  const uint64_t u = (uint64_t)__double_as_longlong(w);
+  Fx a;
+  a.m = (u & ~0x7ffull) | 0x400u;
+  a.e = (int)((uint32_t)u & 0x7ffu) - (1024 + 63);
+  return a;
+}
+
+// 2^v as a factor for fx_mul, |v| < 1000
+__device__ __forceinline__ Fx fx_exp2_factor(double v) {
+  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v), e = (hi >> 20) & 0x7ffu;
+  const uint64_t m = ((uint64_t)(0x40000000u | ((hi << 10) & 0x3fffffffu) | (lo >> 22)) << 32) | (lo << 10);
+  const uint32_t s = e < 969u ? 63u : 1032u - e;  // floor(|v| 2^53), then the complement
+  Fx a;
+  a.m = exp2_parts((int64_t)(m >> s) ^ (int64_t)((int32_t)hi >> 31), a.e);
+  a.e += 1;
+  return a;
+}
+
+// v 2^-52 as a double
+__device__ __forceinline__ double q52_to_double(int64_t v) {
+  const int64_t neg = v >> 63;
+  return fx_pack((uint64_t)((v ^ neg) - neg), -52, (uint32_t)(neg >> 32));
+}
+
+// v c 2^-64 to within 3 units
+__device__ __forceinline__ int64_t mul_fixed_signed(int64_t v, uint64_t c) {
+  const int64_t neg = v >> 63;
+  const uint64_t a = (uint64_t)((v ^ neg) - neg);
+  const uint64_t p = mulhi64_3((uint32_t)(a >> 32), (uint32_t)a, (uint32_t)(c >> 32), (uint32_t)c);
+  return ((int64_t)p ^ neg) - neg;
 }
 
 // v 2^-53 as a double

@@ -52,6 +52,16 @@ __host__ __device__ constexpr int thread_ws_doubles() {
   return 5 * NS + (NS + 1) * (NS + 1) + 6 * (NS + 1);
 }
 
+// a cell's state: registers, or (the generated kernels) local memory
+template <bool GENERATED>
+struct StateOf {
+  typedef double type;
+};
+template <>
+struct StateOf<true> {
+  typedef volatile double type;
+};
+
 __host__ __device__ inline int blob_smem_doubles(const MechDims& d) { return (d.total + 1) & ~1; }
 
 // BT > 0: the kernel is launched with exactly BT threads per block, the
@@ -84,7 +94,7 @@ __global__ void __launch_bounds__(128, 1) k_integrate_thread(IntegArgs a) {
   int64_t cell = -1;
   bool exhausted = false, done = false, last_rej = false;
   int status = 0, nacc = 0, nrej = 0, istep = 0;
-  double y[n];
+  typename StateOf<EVAL::kGenerated>::type y[n];
   double t = 0.0, h = 0.0, fbest = -INFINITY, tbest = 0.0;
   PeakTrack pk;
   if (IGN) pk.reset();
@@ -119,12 +129,14 @@ __global__ void __launch_bounds__(128, 1) k_integrate_thread(IntegArgs a) {
         const unsigned long long idx = base + __popc(m & ((1u << lane) - 1u));
         if (idx < nwork) {
           cell = a.order ? (int64_t)a.order[idx] : (int64_t)idx;
-          y[0] = a.T[cell];
-          bool ok = isfinite(y[0]) && y[0] > 0.0;
+          const double T = a.T[cell];
+          bool ok = isfinite(T) && T > 0.0;
+          y[0] = T;
 #pragma unroll
           for (int k = 0; k < NS; ++k) {
-            y[1 + k] = a.Y[(int64_t)k * a.ncells + cell];
-            ok = ok && isfinite(y[1 + k]);
+            const double v = a.Y[(int64_t)k * a.ncells + cell];
+            y[1 + k] = v;
+            ok = ok && isfinite(v);
           }
           const double pc = a.p[cell];
           ok = ok && isfinite(pc) && pc > 0.0;
@@ -160,7 +172,7 @@ __global__ void __launch_bounds__(128, 1) k_integrate_thread(IntegArgs a) {
       h = a.dt - t;
       last = true;
     }
-    double ys[n];
+    typename StateOf<EVAL::kGenerated>::type ys[n];
     double en;
     double fT;
     const double t0 = t;
@@ -168,8 +180,8 @@ __global__ void __launch_bounds__(128, 1) k_integrate_thread(IntegArgs a) {
     if constexpr (EVAL::kGenerated) {
       static_assert(NS == EVAL::kN && !CONSTV, "generated evaluation: its own mechanism, constant pressure");
       ok = ros_attempt_gen<BT, EVAL>(mv, tb, pc, y, h, a.rtol, a.atolY, a.atolT, V{ws, stride},
-                                     V{ws + EVAL::kNA * EVAL::kNA * stride, stride}, ys, en, nacc == 0 && nrej == 0,
-                                     last, fT);
+                                     V{ws + EVAL::kNA * EVAL::kNA * stride, stride},
+                                     V{ws + EVAL::kWords * stride, stride}, ys, en, nacc == 0 && nrej == 0, last, fT);
     } else {
       V C{ws, stride}, wdot{ws + NS * stride, stride}, gRT{ws + 2 * NS * stride, stride},
           hRT{ws + 3 * NS * stride, stride}, cpR{ws + 4 * NS * stride, stride}, Jv{ws + 5 * NS * stride, stride},

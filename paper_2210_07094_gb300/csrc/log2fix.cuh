@@ -37,6 +37,13 @@ __device__ __forceinline__ uint64_t log2_fixed(double x) {
   return ((uint64_t)((hi >> 20) - 1023u) << 60) + log2_mantissa_fixed(hi, (uint32_t)__double2loint(x));
 }
 
+// log2(x) 2^52 of a normal positive double
+__device__ __forceinline__ int64_t log2_q52(double x) {
+  const int hi = __double2hiint(x);
+  return ((int64_t)((hi >> 20) - 1023) << 52) +
+         (int64_t)((log2_mantissa_fixed((uint32_t)hi, (uint32_t)__double2loint(x)) + 128u) >> 8);
+}
+
 // ln(x) log_b(e) for any x; hi + lo = ln 2 log_b(e) with hi rounded to 42 bits, so
 // that a multiple of it by the exponent is exact.  Zero, negative, subnormal,
 // infinite and NaN arguments go to the library's log.  Four FP64 operations.

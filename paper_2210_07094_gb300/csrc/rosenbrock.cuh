@@ -121,9 +121,9 @@ constexpr double FIRST_STEP_THETA = 0.5;
 
 template <int n>
 __device__ __forceinline__ double first_step_limit(const double (&y)[n], const double (&f)[n]) {
-  double r = fabs(f[0]) * rcp_nr(fabs(y[0]));
+  double r = fabs(f[0]) * rcp_any(fabs(y[0]));
 #pragma unroll
-  for (int i = 1; i < n; ++i) r = fmax(r, fabs(f[i]) * rcp_nr(fmax(fabs(y[i]), 1e-6)));
+  for (int i = 1; i < n; ++i) r = fmax(r, fabs(f[i]) * rcp_any(fmax(fabs(y[i]), 1e-6)));
   return r > 0.0 ? FIRST_STEP_THETA / r : INFINITY;
 }
 
@@ -215,25 +215,31 @@ __device__ __forceinline__ bool ros_attempt(const MechView& mv, const RosTab& tb
 // Shared memory holds only W and one vector per thread: the stage vectors of the
 // finished stages, read once per later stage in long independent runs, go to
 // local memory (about 1% of the attempt's time), and the substitutions run in
-// registers.  That leaves room for eight warps per SM, two for every FP64 pipe (the
+// registers.  So do (volatile) the state and the stage state, which the evaluation
+// takes as its own copies: 40 registers that it would otherwise not have.  That leaves room for eight warps per SM, two for every FP64 pipe (the
 // registers allow no more: with 168 instead of 255 per thread a third warp per
 // pipe made 2^20 cells 22.1 instead of 19.3 ms).
 // 2^20 cells of the bimodal 9-species field: 41.6 ms with the 10 x 10 systems at
 // five warps per SM, 24.4 with 9 x 9 at eight, 21.0 with the rate products on the
-// integer pipes, 19.3 with 7 x 7.
+// integer pipes, 19.3 with 7 x 7, 15.9 with the exponents in groups and the states
+// in local memory.
 template <int ST, class EVAL>
 __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab& tb, double pc,
-                                                const double (&y)[EVAL::kN + 1], double& h, double rtol, double atolY,
-                                                double atolT, SVT<double, ST> W, SVT<double, ST> X,
-                                                double (&ynew)[EVAL::kN + 1], double& en, bool first, bool& last,
-                                                double& fT) {
+                                                const volatile double (&y)[EVAL::kN + 1], double& h, double rtol,
+                                                double atolY, double atolT, SVT<double, ST> W, SVT<double, ST> X,
+                                                SVT<double, ST> E, volatile double (&ynew)[EVAL::kN + 1], double& en,
+                                                bool first, bool& last, double& fT) {
   constexpr int n = EVAL::kN + 1, NA = EVAL::kNA;
-  double fs[n];
+  double fs[n], ys[n];
   double K[5][NA];  // finished stages (local memory: indexed by the stage loop)
-  EVAL::template run<true, ST>(mv, pc, y, fs, W);
+#pragma unroll
+  for (int i = 0; i < n; ++i) ys[i] = y[i];
+  EVAL::template run<true, ST>(mv, pc, ys, fs, W, E);
   fT = fs[0];
   if (first) {
-    const double hl = first_step_limit<n>(y, fs);
+#pragma unroll
+    for (int i = 0; i < n; ++i) ys[i] = y[i];
+    const double hl = first_step_limit<n>(ys, fs);
     if (hl < h) {
       h = hl;
       last = false;
@@ -247,8 +253,6 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
   const double ih = rcp_nr(h);
   double e2 = 0.0;
   bool fin = true;
-#pragma unroll
-  for (int i = 0; i < n; ++i) ynew[i] = y[i];
   // the eliminated species' share of an increment d of the others
   auto elim_of = [](int e, const double(&d)[NA]) {
     double v = 0.0;
@@ -278,12 +282,14 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
           for (int a = 0; a < NA; ++a) r[a] += c * K[j][a];
         }
 #pragma unroll
+        for (int i = 0; i < n; ++i) ys[i] = ynew[i];
+#pragma unroll
         for (int a = 0; a < NA; ++a) {
           g[a] = K[s - 1][a];
-          ynew[EVAL::act(a)] += g[a];
+          ys[EVAL::act(a)] += g[a];
         }
 #pragma unroll
-        for (int e = 0; e < EVAL::kNE; ++e) ynew[EVAL::elim(e)] += elim_of(e, g);
+        for (int e = 0; e < EVAL::kNE; ++e) ys[EVAL::elim(e)] += elim_of(e, g);
       } else {
 #pragma unroll 1
         for (int j = 0; j < s; ++j) {
@@ -297,15 +303,19 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
         }
         if (newf) {
 #pragma unroll
-          for (int a = 0; a < NA; ++a) ynew[EVAL::act(a)] = y[EVAL::act(a)] + g[a];
+          for (int i = 0; i < n; ++i) ys[i] = y[i];
 #pragma unroll
-          for (int e = 0; e < EVAL::kNE; ++e) ynew[EVAL::elim(e)] = y[EVAL::elim(e)] + elim_of(e, g);
+          for (int a = 0; a < NA; ++a) ys[EVAL::act(a)] += g[a];
+#pragma unroll
+          for (int e = 0; e < EVAL::kNE; ++e) ys[EVAL::elim(e)] += elim_of(e, g);
         }
       }
       if (newf) {
 #pragma unroll
         for (int a = 0; a < NA; ++a) X[a] = r[a];  // waits in shared memory for the evaluation
-        EVAL::template run<false, ST>(mv, pc, ynew, fs, W);
+#pragma unroll
+        for (int i = 0; i < n; ++i) ynew[i] = ys[i];
+        EVAL::template run<false, ST>(mv, pc, ys, fs, W, E);
 #pragma unroll
         for (int a = 0; a < NA; ++a) X[a] = fma(ih, X[a], fs[EVAL::act(a)]);
       } else {
@@ -349,9 +359,17 @@ __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab
         const double yn = ynew[i] + ei;
         fin = fin && (__double2hiint(yn) & 0x7ff00000) != 0x7ff00000;
         ynew[i] = yn;
-        const double sc = (i == 0 ? atolT : atolY) + rtol * fmax(fabs(y[i]), fabs(yn));
-        const double q = ei * rcp_nr(sc);
+        const double yi = y[i];
+        const double sc = (i == 0 ? atolT : atolY) + rtol * fmax(fabs(yi), fabs(yn));
+        const double q = ei * rcp_any(sc);
         e2 += q * q;
+      }
+#pragma unroll
+      for (int i = 0; i < n; ++i) {  // the inert species
+        bool moves = false;
+#pragma unroll
+        for (int a = 0; a < NA + EVAL::kNE; ++a) moves = moves || i == (a < NA ? EVAL::act(a) : EVAL::elim(a - NA));
+        if (!moves) ynew[i] = y[i];
       }
     }
   }
@@ -415,9 +433,9 @@ struct StepState {
   double hacc, erracc;
 };
 
-template <int n>
+template <int n, class Y>  // Y: double or volatile double
 __device__ __forceinline__ void step_control(const RosTab& tb, bool ok, double en, bool last, double dt,
-                                             double (&y)[n], const double (&ynew)[n], double& t, double& h,
+                                             Y (&y)[n], const Y (&ynew)[n], double& t, double& h,
                                              int& nacc, int& nrej, bool& last_rej, bool& done, StepState& ss) {
   // the accept test in FP64, the step-size factors in FP32 (a heuristic's
   // factors need no more; FP32 powf runs on the wide pipes, FP64 pow on the

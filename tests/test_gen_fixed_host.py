@@ -79,15 +79,16 @@ int main() {
   int inside = 0;
   double wf = 0, wj = 0, wp = 0;
   for (int t = 0; t < 2000; ++t) {
-    double y[n], y2[n], f[n], fe[n], f2[n], fp_[n], W[NA * NA], W0[NA * NA], J[n * n], J2[n * n], sM[n], s = 0;
+    double y[n], y2[n], f[n], fe[n], f2[n], fp_[n], W[GenEval::kWords], W0[GenEval::kWords], ex[128], J[n * n], J2[n * n], sM[n], s = 0;
     y[0] = t % 50 == 0 ? 30.0 + 12000.0 * U() : 240.0 + 3000.0 * U();
     for (int k = 0; k < N; ++k) s += y[1 + k] = pow(10.0, -9.0 * U()) * (U() < 0.05 ? -1e-6 : 1.0);
     for (int k = 0; k < N; ++k) y[1 + k] /= s;
     const double pc = 1.01325e6 * pow(10.0, 2.0 * U() - 0.5);
+    SVT<double, 1> E{ex, 1};
     for (double& v : W) v = NAN;
     for (double& v : W0) v = NAN;
-    const bool in = gen_fixed<true, 1>(mv, pc, y, f, SVT<double, 1>{W, 1});
-    if (in != gen_fixed<false, 1>(mv, pc, y, fp_, SVT<double, 1>{W0, 1})) return 3;
+    const bool in = gen_fixed<true, 1>(mv, pc, y, f, SVT<double, 1>{W, 1}, E);
+    if (in != gen_fixed<false, 1>(mv, pc, y, fp_, SVT<double, 1>{W0, 1}, E)) return 3;
     if (!in) {
       for (double v : W) if (v == v) return 4;  // nothing may be written
       continue;
