@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
     boff = (a.d.total + 1) & ~1;
   }
   __syncthreads();
-  const MechView mv = make_view(blob, a.d);
+  const MechView mv = make_view(blob, a.d, a.blob);
   const int M = a.d.M;
   double* base = smem + boff;
   // Dual vectors (value part at even offsets)

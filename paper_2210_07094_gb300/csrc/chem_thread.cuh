@@ -48,18 +48,28 @@ struct MechView {
   const double* rx;
   const double* tr;
   const double* eff;
-  const long long* fix;  // ln A as fixed-point logarithms (generated evaluation only)
+  const long long* fix;  // the fixed-point words (FixLayout), always in global memory
   int M;
+  int fg, fr, ff;        // offsets of their species, reaction and falloff records
+  double T_low;          // the fixed-point arguments cover T_low <= T < FIX_T_HIGH; infinity: none
 };
 
-__device__ __forceinline__ MechView make_view(const double* blob, const MechDims& d) {
+// blob: the mechanism as the kernel reads it (shared or global memory); global: in
+// global memory, with the words behind it
+__device__ __forceinline__ MechView make_view(const double* blob, const MechDims& d, const double* global) {
   MechView v;
   v.sp = blob + d.off_sp;
   v.rx = blob + d.off_rx;
   v.tr = blob + d.off_tr;
   v.eff = blob + d.off_eff;
-  v.fix = nullptr;
   v.M = d.M;
+  const FixLayout F(d.N, d.M, d.n_troe);
+  v.fix = reinterpret_cast<const long long*>(global + d.off_fix());
+  v.fg = F.g;
+  v.fr = F.rate;
+  v.ff = F.falloff;
+  v.T_low = __longlong_as_double(v.fix[F.T_low]);
+  if (!(v.T_low > 0.0) || !v.fix[F.flag]) v.T_low = INFINITY;
   return v;
 }
 
@@ -280,6 +290,182 @@ __device__ __forceinline__ void rate_one(const MechView& mv, const double* r, in
   rate_compute<NS, WITH_J>(mv, g, T, lnT, invT, lnP0RT, o);
 }
 
+// ---------------------------------------------------------------------------
+// The fixed-point form of the rates for a mechanism read from its blob (the
+// generated kernels have it as literals, gen_fixed in codegen.cu): the exponents
+// are 64-bit sums in units of 2^-53 octave, the products of rate constants and
+// concentrations unpacked numbers (Fx), so that a reaction's net rate takes the
+// FP64 pipe, 64 cycles per warp instruction, only for its collider.
+// ---------------------------------------------------------------------------
+struct FixState {
+  uint64_t L, I, t1, t2, t3, t4;  // log2 T 2^60, 1/T 2^69, T 2^50, T^2 2^36, T^3 2^22, T^4 2^8
+  int64_t lp;                     // log2(p_std / (R T)) 2^53
+};
+
+__device__ __forceinline__ bool fixed_covers(const MechView& mv, double T) { return T >= mv.T_low && T < FIX_T_HIGH; }
+
+__device__ __forceinline__ FixState fix_state(double T, double invT) {
+  FixState s;
+  s.L = log2_fixed(T);
+  s.I = pos_fixed<69>(invT);
+  s.t1 = pos_fixed<50>(T);
+  s.t2 = mul_fixed(s.t1, s.t1);
+  s.t3 = mul_fixed(s.t2, s.t1);
+  s.t4 = mul_fixed(s.t2, s.t2);
+  // ln(p_std / R) log2(e) 2^53, from its parts (a literal of the sum)
+  s.lp = -(int64_t)0xcb7954cba85db7ll - (int64_t)(s.L >> 7);
+  return s;
+}
+
+// c times a fixed-point monomial, c signed
+__device__ __forceinline__ int64_t fix_term(long long c, uint64_t mono) { return mul_fixed_signed(c, mono); }
+
+// g_k/RT log2(e) 2^53 from the species' record
+__device__ __forceinline__ int64_t fix_gibbs(const long long* c, const FixState& s) {
+  int64_t v = fix_term(__ldg(c + 2), s.t1) + fix_term(__ldg(c + 3), s.t2) + fix_term(__ldg(c + 6), s.I);
+  const long long c3 = __ldg(c + 4), c4 = __ldg(c + 5);
+  if (c3 | c4) v += fix_term(c3, s.t3) + fix_term(c4, s.t4);
+  return __ldg(c) + fix_term(__ldg(c + 1), s.L) + 4 * v;
+}
+
+__device__ __forceinline__ uint32_t hi_word(double x) { return (uint32_t)__double2hiint(x); }
+
+// 2^X as a number, and a number as a factor of fx_mul
+__device__ __forceinline__ Fx fx_exp2(int64_t X) {
+  Fx a;
+  a.m = exp2_parts(X, a.e);
+  a.e -= 63;
+  return a;
+}
+__device__ __forceinline__ Fx fx_as_factor(Fx a) {
+  a.e += 64;
+  return a;
+}
+
+// The exponents of reaction j: of k_f (k_inf of a falloff reaction) and of k_r (1 / K_c
+// of a falloff reaction; 0 for an irreversible one).  G holds the species' g/RT
+// log2(e) 2^53 as 64-bit integers in the doubles' storage.
+template <class Vec>
+__device__ __forceinline__ void rate_exponents(const MechView& mv, int j, const double* r, const FixState& fs,
+                                               const Vec& G, int64_t& x, int64_t& xr) {
+  const RxMeta mt = load_meta(r);
+  const int nr = mt.nrnp & 15, np = mt.nrnp >> 4;
+  const long long* rr = mv.fix + mv.fr + 2 * j;
+  x = __ldg(mv.fix + j) + fix_term(__ldg(rr), fs.L) + 4 * fix_term(__ldg(rr + 1), fs.I);
+  auto g = [&](int k) { return (int64_t)__double_as_longlong(G[k]); };
+  int64_t xc = g(mt.prod[0]) - g(mt.reac[0]) - (np - nr) * fs.lp;
+  if (np > 1) xc += g(mt.prod[1]);
+  if (np > 2) xc += g(mt.prod[2]);
+  if (nr > 1) xc -= g(mt.reac[1]);
+  if (nr > 2) xc -= g(mt.reac[2]);
+  xr = (mt.flags & 4) == 0 ? 0 : (mt.flags & 3) == 2 ? xc : add_exponents(x, xc);
+}
+
+// rate_gather and rate_compute in fixed point: the same results but for rounding.
+// se: sparse efficiencies (the warp path), else the dense row.  (The powers of two
+// of eight reactions at a time, as in the generated kernels, were slower here: the
+// loops wait for the reactions' records; 16411 source terms 76 instead of 64 us.)
+template <int NS, bool WITH_J, class Vec>
+__device__ __forceinline__ void rate_fixed(const MechView& mv, int j, const double* r, int Nrt, double T, double invT,
+                                           const FixState& fs, const Vec& C, const Vec& G, const Vec& hRT, RateOut& o,
+                                           const SparseEff* se = nullptr) {
+  const int N = NS > 0 ? NS : Nrt;
+  int64_t x, xr;
+  rate_exponents(mv, j, r, fs, G, x, xr);
+  Fx kf = fx_exp2(x), kr = fx_exp2(xr);
+  const RxMeta mt = load_meta(r);
+  const RxSlots sl = load_slots(r);
+  o.active = true;
+  o.mt = mt;
+  o.sl = sl;
+  const int nr = mt.nrnp & 15, np = mt.nrnp >> 4, type = mt.flags & 3;
+  const bool rev = (mt.flags & 4) != 0;
+  o.cr[0] = C[mt.reac[0]];
+  o.cr[1] = nr > 1 ? C[mt.reac[1]] : 1.0;
+  o.cr[2] = nr > 2 ? C[mt.reac[2]] : 1.0;
+  o.cp[0] = C[mt.prod[0]];
+  o.cp[1] = np > 1 ? C[mt.prod[1]] : 1.0;
+  o.cp[2] = np > 2 ? C[mt.prod[2]] : 1.0;
+  double sh = 0.0;
+  if (WITH_J) {
+    sh = hRT[mt.prod[0]] - hRT[mt.reac[0]];
+    if (np > 1) sh += hRT[mt.prod[1]];
+    if (np > 2) sh += hRT[mt.prod[2]];
+    if (nr > 1) sh -= hRT[mt.reac[1]];
+    if (nr > 2) sh -= hRT[mt.reac[2]];
+  }
+  double Mc = 1.0;
+  if (type != 0) {
+    if (se) {
+      Mc = se->ctot;
+      for (int t = se->off[sl.eff]; t < se->off[sl.eff + 1]; ++t) {
+        const int* e = se->ent + 3 * t;
+        Mc += __hiloint2double(e[2], e[1]) * C[e[0]];
+      }
+    } else {
+      const double* ef = mv.eff + N * sl.eff;
+      Mc = 0.0;
+#pragma unroll
+      for (int l = 0; l < N; ++l) Mc += ef[l] * C[l];
+    }
+  }
+  const double beta = r[1], EaR = r[2];
+  double dlnk = 0.0, gpr = 0.0;
+  if (WITH_J) dlnk = fma(EaR, invT, beta) * invT;
+  if (type == 2) {
+    // Troe falloff, logarithms to base 2 (see rate_compute); kr holds 1 / K_c here
+    const double* tr = mv.tr + TR_REC * sl.troe;
+    const long long* rt = mv.fix + mv.ff + 3 * sl.troe;
+    const int64_t xd = __ldg(rt) + fix_term(__ldg(rt + 1), fs.L) + 4 * fix_term(__ldg(rt + 2), fs.I);
+    const double Pr = fx_pack(fx_exp2(xd), 0u) * Mc;
+    if (!(Pr >= 0x1p-1022)) {  // no low-pressure rate or no collider: k = 0
+      o.active = false;
+      return;
+    }
+    double e3, e1;
+    exp_rate2(-T * tr[4], -T * tr[5], e3, e1);
+    const double e2 = exp_rate(-tr[6] * invT);
+    const double Fc = fma(1.0 - tr[3], e3, fma(tr[3], e1, e2));
+    const int64_t lc = log2_q52(Fc);
+    // 0.67 2^64, 1.27 2^63, 0.14 2^64
+    constexpr uint64_t C067 = 12359318529385400320ull, C127 = 11713682486805565440ull, C014 = 2582544170319337472ull;
+    constexpr int64_t Q04 = 5984253652114523ll, Q075 = 11220475597714730ll;  // 0.4 and 0.75 log2(10) 2^52
+    const int64_t lx = log2_q52(Pr) - Q04 - mul_fixed_signed(lc, C067), ln = Q075 - 2 * mul_fixed_signed(lc, C127);
+    const double xl = q52_to_double(lx), den = q52_to_double(ln - mul_fixed_signed(lx, C014)), Lc = q52_to_double(lc);
+    const double den2 = den * den, q1 = den2 * rcp_any(fma(xl, xl, den2)), onePr = rcp_any(1.0 + Pr);
+    kf = fx_mul(fx_mul(kf, fx_factor(Pr * onePr)), fx_exp2_factor(Lc * q1));
+    kr = fx_mul(kf, fx_as_factor(kr));
+    if (WITH_J) {
+      const double nn = q52_to_double(ln), rden = rcp_any(den), f1 = xl * rden;
+      const double df1_dLc = fma(-0.67, den, -(xl * (-1.27 + 0.67 * 0.14))) * (rden * rden);
+      const double g2 = 2.0 * Lc * f1 * q1 * q1;
+      gpr = fma(-g2, nn * rden * rden, onePr);  // d ln k / d ln Pr
+      const double dFc = fma(-(1.0 - tr[3]) * tr[4], e3, fma(-tr[3] * tr[5], e1, tr[6] * invT * invT * e2));
+      const double dlnk0 = fma(tr[2], invT, tr[1]) * invT;
+      dlnk = fma(fma(-g2, df1_dLc, q1) * dFc, rcp_any(Fc), fma(gpr, dlnk0 - dlnk, dlnk));
+    }
+  }
+  const uint32_t sf = hi_word(o.cr[0]) ^ hi_word(o.cr[1]) ^ hi_word(o.cr[2]);
+  const uint32_t sb = hi_word(o.cp[0]) ^ hi_word(o.cp[1]) ^ hi_word(o.cp[2]);
+  const Fx pf = fx_mul(fx_mul(fx_mul(kf, fx_factor(o.cr[0])), fx_factor(o.cr[1])), fx_factor(o.cr[2]));
+  Fx pb = fx_mul(fx_mul(fx_mul(kr, fx_factor(o.cp[0])), fx_factor(o.cp[1])), fx_factor(o.cp[2]));
+  if (!rev) {
+    pb.m = 0;
+    pb.e = -100000;  // must not set the scale of the difference
+  }
+  const double q0 = fx_diff(pf, sf, pb, sb);
+  o.q = type == 1 ? Mc * q0 : q0;
+  if (WITH_J) {
+    const double kfd = fx_pack(kf, 0u), krd = rev ? fx_pack(kr, 0u) : 0.0, pbd = fx_pack(pb, sb);
+    o.fk = type == 1 ? Mc * kfd : kfd;
+    o.rk = type == 1 ? Mc * krd : krd;
+    // dk/d[M] = k gpr / [M] for falloff
+    o.dqdM = type == 1 ? q0 : type == 2 ? q0 * (gpr * rcp_any(Mc)) : 0.0;
+    const double dlnKc = (sh - (double)(np - nr)) * invT;
+    o.dqdT = fma(o.q, dlnk, (type == 1 ? Mc * pbd : pbd) * dlnKc);
+  }
+}
+
 // Optional accumulation of d/d ln A_j of a weighted sum of the right-hand side
 // (the discrete adjoint's parameter gradient), inside eval_vjp.  Mode 1: the
 // weights are eval_vjp's cotangent r of dy/dt, i.e. th[j] += r . d f / d ln A_j
@@ -325,22 +511,36 @@ __device__ __forceinline__ S eval_thread(const MechView& mv, const double pc, co
   constexpr int n = NS + 1;
   constexpr double EV = CONSTV ? 1.0 : 0.0;  // U/(RT) = H/(RT) - 1, cv/R = cp/R - 1
   const S T = y[0];
-  const S lnT = fast_log(T);
   const S invT = 1.0 / T;
   S sumYW(0.0), cpm(0.0);
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     const double* a = mv.sp + SP_REC * k + 2;
-    const double* ah = mv.sp + SP_REC * k + SP_H;  // a2/2 .. a5/5
-    const double* as = mv.sp + SP_REC * k + SP_S;  // a3/2 .. a5/4
     const S cpk = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4])));
     cpR[k] = cpk;
-    const S hk = a[0] + T * (ah[0] + T * (ah[1] + T * (ah[2] + T * ah[3]))) + a[5] * invT;
-    const S sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
-    hRT[k] = hk;
-    gRT[k] = hk - sk;
     sumYW += y[1 + k] * mv.sp[SP_REC * k + 1];
     cpm += y[1 + k] * (cpk - EV) * mv.sp[SP_REC * k + 1];
+  }
+  // fixed-point rates where the temperature is covered and the concentrations
+  // are finite
+  const bool fixed = fixed_covers(mv, T) && rcp_in_range(sumYW) && rcp_in_range(pc);
+  FixState fst;
+  S lnT(0.0);
+  if (fixed) fst = fix_state(T, invT);
+  else lnT = fast_log(T);
+#pragma unroll 1
+  for (int k = 0; k < NS; ++k) {
+    const double* a = mv.sp + SP_REC * k + 2;
+    const double* ah = mv.sp + SP_REC * k + SP_H;  // a2/2 .. a5/5
+    const S hk = a[0] + T * (ah[0] + T * (ah[1] + T * (ah[2] + T * ah[3]))) + a[5] * invT;
+    hRT[k] = hk;
+    if (fixed) {
+      gRT[k] = __longlong_as_double(fix_gibbs(mv.fix + mv.fg + 7 * k, fst));
+    } else {
+      const double* as = mv.sp + SP_REC * k + SP_S;  // a3/2 .. a5/4
+      const S sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
+      gRT[k] = hk - sk;
+    }
   }
   cpm = cpm * RU;  // cp, or cv at constant volume
   const S rho = CONSTV ? S(pc) : pc * invT / (RU * sumYW);
@@ -358,7 +558,9 @@ __device__ __forceinline__ S eval_thread(const MechView& mv, const double pc, co
   const S lnP0RT = LOG_PSTD_RU - lnT;
   for (int j = 0; j < mv.M; ++j) {
     RateOutT<S> ro;
-    rate_one<NS, WITH_J>(mv, mv.rx + RX_REC * j, NS, T, lnT, invT, lnP0RT, C, gRT, hRT, ro);
+    if (fixed) rate_fixed<NS, WITH_J>(mv, j, mv.rx + RX_REC * j, NS, T, invT, fst, C, gRT, hRT, ro);
+    else
+      rate_one<NS, WITH_J>(mv, mv.rx + RX_REC * j, NS, T, lnT, invT, lnP0RT, C, gRT, hRT, ro);
     if (!ro.active) continue;
     const RxMeta mt = ro.mt;
     const int nr = mt.nrnp & 15, np = mt.nrnp >> 4;

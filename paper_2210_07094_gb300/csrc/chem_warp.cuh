@@ -93,22 +93,32 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
   PV C{ws + L.C}, gRT{ws + L.gRT}, hRT{ws + L.hRT};
   double* wdot = ws + L.wdot;  // the g/RT slots, once the rates have read them
   const double T = y[0];
-  const double lnT = log_rate(T);
-  const double invT = rcp_nr(T);
-  // thermo and sum Y/W
+  const double invT = rcp_any(T);
+  // thermo and sum Y/W; the rates in fixed point (rate_fixed; the g/RT slots then
+  // hold 64-bit integers) where the temperature is covered and the concentrations
+  // are finite
   double sYW = 0.0;
+  for (int k = lane; k < N; k += 32) sYW += y[1 + k] * mv.sp[SP_REC * k + 1];
+  const double sumYW = warp_sum(sYW);
+  const bool fixed = fixed_covers(mv, T) && rcp_in_range(sumYW) && rcp_in_range(pc);
+  FixState fst;
+  double lnT = 0.0;
+  if (fixed) fst = fix_state(T, invT);
+  else lnT = log_rate(T);
   for (int k = lane; k < N; k += 32) {
     const double* a = mv.sp + SP_REC * k + 2;
     const double* ah = mv.sp + SP_REC * k + SP_H;  // a2/2 .. a5/5
-    const double* as = mv.sp + SP_REC * k + SP_S;  // a3/2 .. a5/4
     const double hk = a[0] + T * (ah[0] + T * (ah[1] + T * (ah[2] + T * ah[3]))) + a[5] * invT;
-    const double sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
     hRT[k] = hk;
-    gRT[k] = hk - sk;
-    sYW += y[1 + k] * mv.sp[SP_REC * k + 1];
+    if (fixed) {
+      gRT[k] = __longlong_as_double(fix_gibbs(mv.fix + mv.fg + 7 * k, fst));
+    } else {
+      const double* as = mv.sp + SP_REC * k + SP_S;  // a3/2 .. a5/4
+      const double sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
+      gRT[k] = hk - sk;
+    }
   }
-  const double sumYW = warp_sum(sYW);
-  const double Wbar = rcp_nr(sumYW);
+  const double Wbar = rcp_any(sumYW);
   const double rho = CONSTV ? pc : pc * invT * Wbar * (1.0 / RU);
   double cs = 0.0;
   for (int k = lane; k < N; k += 32) {
@@ -125,7 +135,8 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
   // reactions: one lane per reaction
   for (int j = lane; j < mv.M; j += 32) {
     RateOut ro;
-    rate_one<0, WITH_J>(mv, mv.rx + RX_REC * j, N, T, lnT, invT, lnP0RT, C, gRT, hRT, ro, &se);
+    if (fixed) rate_fixed<0, WITH_J>(mv, j, mv.rx + RX_REC * j, N, T, invT, fst, C, gRT, hRT, ro, &se);
+    else rate_one<0, WITH_J>(mv, mv.rx + RX_REC * j, N, T, lnT, invT, lnP0RT, C, gRT, hRT, ro, &se);
     if (ro.active) {
       ws[L.q + j] = ro.q;
       if (WITH_J) {
@@ -183,8 +194,8 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
   __syncwarp();
   const double cpm = RU * warp_sum(cpp);
   const double Hw = RU * T * warp_sum(hwp);
-  const double invrho = rcp_nr(rho);
-  const double invcp = rcp_nr(cpm);
+  const double invrho = rcp_any(rho);
+  const double invcp = rcp_any(cpm);
   for (int k = lane; k < N; k += 32) f[1 + k] = mv.sp[SP_REC * k] * wdot[k] * invrho;
   const double fT = -Hw * invrho * invcp;
   if (lane == 0) f[0] = fT;
@@ -210,16 +221,24 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
         const double* r = mv.rx + RX_REC * j;
         const RxMeta mt = load_meta(r);
         const int nr = mt.nrnp & 15, np = mt.nrnp >> 4;
-        const double fk = ws[L.fk + j], rk = ws[L.rk + j];
         row[0] += nu * ws[L.dT + j];
-        const double c0 = C[mt.reac[0]], c1 = nr > 1 ? C[mt.reac[1]] : 1.0, c2 = nr > 2 ? C[mt.reac[2]] : 1.0;
-        row[1 + mt.reac[0]] += nu * fk * c1 * c2;
-        if (nr > 1) row[1 + mt.reac[1]] += nu * fk * c0 * c2;
-        if (nr > 2) row[1 + mt.reac[2]] += nu * fk * c0 * c1;
-        const double d0 = C[mt.prod[0]], d1 = np > 1 ? C[mt.prod[1]] : 1.0, d2 = np > 2 ? C[mt.prod[2]] : 1.0;
-        row[1 + mt.prod[0]] -= nu * rk * d1 * d2;
-        if (np > 1) row[1 + mt.prod[1]] -= nu * rk * d0 * d2;
-        if (np > 2) row[1 + mt.prod[2]] -= nu * rk * d0 * d1;
+        // nu fk c c' and -nu rk c c' as unpacked products (Fx): one FP64 addition
+        // per entry instead of three multiplications and an addition
+        auto side = [&](double k, const uint8_t* sp, int cnt, uint32_t sign) {
+          const double c0 = C[sp[0]], c1 = cnt > 1 ? C[sp[1]] : 1.0, c2 = cnt > 2 ? C[sp[2]] : 1.0;
+          const uint32_t s = sign ^ hi_word(k) ^ hi_word(nu);
+          Fx v = fx_factor(k);
+          v.m <<= 1;
+          v.e += -64 - 1;  // fx_factor's share back to the number's own exponent
+          v = fx_mul(v, fx_factor(nu));
+          const Fx f0 = fx_factor(c0), f1 = fx_factor(c1), f2 = fx_factor(c2);
+          const Fx v2 = fx_mul(v, f2);
+          row[1 + sp[0]] += fx_pack(fx_mul(v2, f1), s ^ hi_word(c1) ^ hi_word(c2));
+          if (cnt > 1) row[1 + sp[1]] += fx_pack(fx_mul(v2, f0), s ^ hi_word(c0) ^ hi_word(c2));
+          if (cnt > 2) row[1 + sp[2]] += fx_pack(fx_mul(fx_mul(v, f0), f1), s ^ hi_word(c0) ^ hi_word(c1));
+        };
+        side(ws[L.fk + j], mt.reac, nr, 0u);
+        side(ws[L.rk + j], mt.prod, np, 0x80000000u);
         if ((mt.flags & 3) != 0) {
           const int sl = load_slots(r).eff;
           const double cM = nu * ws[L.dM + sl];
@@ -313,7 +332,7 @@ __device__ bool warp_lu(double* A, int* piv, int n) {
       }
     }
     __syncwarp();
-    const double inv = rcp_nr(A[k * n + k]);
+    const double inv = rcp_any(A[k * n + k]);
     __syncwarp();
     for (int i = k + 1 + lane; i < n; i += 32) A[i * n + k] *= inv;
     for (int i = lane; i < k; i += 32) A[i * n + k] *= inv;  // U'_ik = U_ik / U_kk (row i < k is final)

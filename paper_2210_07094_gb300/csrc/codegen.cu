@@ -41,6 +41,7 @@
 
 #include "common.cuh"
 #include "integrate_thread.cuh"
+#include "reactions.cuh"
 
 namespace df {
 
@@ -49,17 +50,6 @@ namespace {
 // ---------------------------------------------------------------------------
 // source generation
 // ---------------------------------------------------------------------------
-RxMeta meta_of(const df_mech* m, int j) {
-  RxMeta mt;
-  memcpy(&mt, &m->blob_host[m->dims.off_rx + RX_REC * j + 3], 8);
-  return mt;
-}
-RxSlots slots_of(const df_mech* m, int j) {
-  RxSlots sl;
-  memcpy(&sl, &m->blob_host[m->dims.off_rx + RX_REC * j + 4], 8);
-  return sl;
-}
-
 // exact decimal-free spelling of a double (C++17 hexadecimal literal)
 std::string lit(double v) {
   char b[64];
@@ -287,30 +277,6 @@ void emit_eval(std::ostringstream& o, const df_mech* m) {
 // the fixed-point evaluation
 // ---------------------------------------------------------------------------
 
-// |c| 2^s, or |c| log2(e) 2^s, as a 64-bit integer and the left shift its use
-// still needs (0 unless the value is too large for 64 bits).  Integer
-// arithmetic only: the same digits on every host.
-void fixed_literal(double c, bool log2e, int s, uint64_t* lit, int* shift) {
-  *lit = 0;
-  *shift = 0;
-  if (c == 0.0) return;
-  int e;
-  const uint64_t m = (uint64_t)std::ldexp(std::frexp(std::fabs(c), &e), 53);  // |c| = m 2^(e - 53)
-  const unsigned __int128 p = log2e ? (unsigned __int128)m * EXP2FIX_LOG2E_HALF : (unsigned __int128)m << 63;
-  int bits = 64;
-  while (bits < 128 && (p >> bits) != 0) ++bits;
-  const int r0 = 116 - e - s;  // |c| (log2 e) 2^s = p 2^-r0
-  int r = std::max(r0, bits - 64);
-  if (r > 126) return;
-  unsigned __int128 v = (p + ((unsigned __int128)1 << (r - 1))) >> r;
-  if ((v >> 64) != 0) {
-    ++r;
-    v = (p + ((unsigned __int128)1 << (r - 1))) >> r;
-  }
-  *lit = (uint64_t)v;
-  *shift = r - r0;
-}
-
 std::string hex64(uint64_t v) {
   char b[32];
   snprintf(b, sizeof b, "0x%llxull", (unsigned long long)v);
@@ -334,42 +300,6 @@ std::string fixed_const(double c, bool log2e) {
   int sh;
   fixed_literal(c, log2e, 53, &l, &sh);
   return std::string(c < 0.0 ? "-" : "") + "(int64_t)(" + hex64(l) + (sh ? " << " + std::to_string(sh) : "") + ")";
-}
-
-constexpr double kFixTHi = 8000.0;
-
-struct Rx {
-  std::vector<int> r, p;  // species entries
-  std::vector<int> nu;    // net coefficients, by species
-  std::vector<int> spc;   // species of the reaction
-  int type = 0, eff = -1, troe = -1, dnu = 0;
-  bool rev = false;
-  double b = 0, E = 0;
-};
-
-std::vector<Rx> reactions_of(const df_mech* m) {
-  std::vector<Rx> out(m->dims.M);
-  for (int j = 0; j < m->dims.M; ++j) {
-    Rx& x = out[j];
-    const RxMeta mt = meta_of(m, j);
-    const RxSlots sl = slots_of(m, j);
-    for (int i = 0; i < (mt.nrnp & 15); ++i) x.r.push_back(mt.reac[i]);
-    for (int i = 0; i < (mt.nrnp >> 4); ++i) x.p.push_back(mt.prod[i]);
-    x.nu.assign(m->dims.N, 0);
-    for (int k : x.r) x.nu[k] -= 1;
-    for (int k : x.p) x.nu[k] += 1;
-    for (const auto* side : {&x.r, &x.p})
-      for (int k : *side)
-        if (std::find(x.spc.begin(), x.spc.end(), k) == x.spc.end()) x.spc.push_back(k);
-    x.type = mt.flags & 3;
-    x.rev = (mt.flags & 4) != 0;
-    x.eff = sl.eff;
-    x.troe = sl.troe;
-    x.dnu = (int)x.p.size() - (int)x.r.size();
-    x.b = m->blob_host[m->dims.off_rx + RX_REC * j + 1];
-    x.E = m->blob_host[m->dims.off_rx + RX_REC * j + 2];
-  }
-  return out;
 }
 
 // The unknowns of the generated kernel's linear systems.  A species that no
@@ -484,43 +414,6 @@ Systems systems_of(const df_mech* m, const std::vector<Rx>& rx) {
   return s;
 }
 
-// the temperatures the fixed-point evaluation covers: from the lowest one at
-// which every exponent, with any ln A of lnA_fits_fixed, stays within 1000 octaves
-// (sampled every 2% and with 5% to spare); 0 if there is none
-double fixed_T_low(const df_mech* m, const std::vector<Rx>& rx) {
-  const double L2E = 1.4426950408889634;
-  auto sp = [&](int k, int i) { return m->blob_host[m->dims.off_sp + SP_REC * k + i]; };
-  for (double lo : {100.0, 150.0, 200.0, 250.0, 300.0, 400.0}) {
-    double worst = 0.0;
-    for (double T = lo; T < kFixTHi * 1.02; T *= 1.02) {
-      std::vector<double> g(m->dims.N);
-      for (int k = 0; k < m->dims.N; ++k) {
-        worst = std::max(worst, std::fabs(sp(k, 2) + T * (sp(k, SP_H) + T * (sp(k, SP_H + 1) + T * (sp(k, SP_H + 2) +
-                                          T * sp(k, SP_H + 3)))) + sp(k, 7) / T));
-        g[k] = L2E * ((sp(k, 2) - sp(k, 8)) - sp(k, 2) * std::log(T) -
-                      T * (sp(k, 3) / 2 + T * (sp(k, 4) / 6 + T * (sp(k, 5) / 12 + T * sp(k, 6) / 20))) + sp(k, 7) / T);
-      }
-      for (const Rx& x : rx) {
-        worst = std::max(worst, std::fabs(x.b) + std::fabs(x.E) / T);
-        const double kf = 400.0 + L2E * std::fabs(x.b * std::log(T) - x.E / T);
-        double sg = -x.dnu * L2E * (LOG_PSTD_RU - std::log(T));
-        for (int k : x.spc) sg += x.nu[k] * g[k];
-        worst = std::max({worst, kf, kf + std::fabs(sg)});
-        if (x.type == 2) {
-          const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
-          // the centring must be a positive number for its logarithm
-          const double Fc = (1.0 - tr[3]) * std::exp(-T * tr[4]) + tr[3] * std::exp(-T * tr[5]) + std::exp(-tr[6] / T);
-          if (!(Fc > 1e-60 && Fc < 1e60)) worst = INFINITY;
-          const double d = L2E * std::fabs(tr[0] + (tr[1] - x.b) * std::log(T) - (tr[2] - x.E) / T);
-          worst = std::max({worst, d, kf + d, std::fabs(sg)});
-        }
-      }
-    }
-    if (worst * 1.05 <= 1000.0) return lo;  // false for NaN and infinity
-  }
-  return 0.0;
-}
-
 // The product of the rate constant `K` and the concentrations C[e], unpacked: `name`p,
 // and with derivatives by each distinct species the doubles `name`d<l>; `name`s is
 // the sign word of the product
@@ -602,7 +495,8 @@ std::string fx_product_code(const std::string& name, const std::string& K, std::
 // concentrations stays in FP64.  Returns false (nothing written) for states
 // outside the range the fixed-point words cover; the caller then takes gen_eval.
 // Without J only the kept species' entries of f and f[0] are written.
-void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& rx, const Systems& sys, double T_low) {
+void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& rx, const Systems& sys, double T_low,
+                bool saturates) {
   const int N = m->dims.N, NA = sys.na(), NR = NA - 1, wid = (int)sys.act.size() + 1;
   auto sp = [&](int k, int i) { return m->blob_host[m->dims.off_sp + SP_REC * k + i]; };
   std::vector<int> col(N, -1), row(N, -1);  // reacting species -> column while J is summed; kept species -> row
@@ -631,7 +525,7 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     << "], double (&f)[" << N + 1 << "], SVT<double, ST> W, SVT<double, ST> E) {\n"
     << "  constexpr int NS = " << N << ";\n"
     << "  const double T = y[0];\n"
-    << "  if (!mv.fix[" << m->dims.M << "] || !(T >= " << lit(T_low) << " && T < " << lit(kFixTHi) << ")) return false;\n"
+    << "  if (!mv.fix[" << m->dims.M << "] || !(T >= " << lit(T_low) << " && T < " << lit(FIX_T_HIGH) << ")) return false;\n"
     << "  double C[NS], cpW[NS];  // cpW: cp_k / (R W_k)\n"
     << "  double sumYW = 0.0, cpm = 0.0;\n";
   for (int k = 0; k < N; ++k) {
@@ -785,7 +679,7 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
           << E(slot[j] + 1) << "xd);\n";
         if (x.rev) o << E(slot[j] + 2) << "(int64_t)0" << sg << ");\n";
       } else if (x.rev) {
-        o << E(slot[j] + 1) << "x" << sg << ");\n";
+        o << E(slot[j] + 1) << (saturates ? "add_exponents(x, (int64_t)0" + sg + ")" : "x" + sg) << ");\n";
       }
       o << "  }\n";
     }
@@ -1025,12 +919,15 @@ std::string jit_thread_source(const df_mech* m) {
   const std::vector<Rx> rx = reactions_of(m);
   const Systems sys = systems_of(m, rx);
   const int NA = sys.na(), NE = (int)sys.elim.size();
-  const double T_low = fixed_T_low(m, rx);
+  // down to 300 K without the test for saturation where the mechanism allows it
+  double T_low = fixed_T_low(m, rx, false);
+  const bool saturates = !(T_low > 0.0 && T_low <= 300.0);
+  if (saturates) T_low = fixed_T_low(m, rx, true);
   std::ostringstream o;
   o << "// generated for a " << N << "-species / " << m->dims.M << "-reaction mechanism\n"
     << "#include \"integrate_thread.cuh\"\n\nnamespace df {\n\n";
   emit_eval(o, m);
-  if (T_low > 0.0) emit_fixed(o, m, rx, sys, T_low);
+  if (T_low > 0.0) emit_fixed(o, m, rx, sys, T_low, saturates);
   std::string act, elim, beta;
   for (int k : sys.keep) act += std::to_string(1 + k) + ", ";
   for (int k : sys.elim) elim += std::to_string(1 + k) + ", ";

@@ -61,8 +61,8 @@ constexpr int RX_REC = 5;
 // Troe record (TR_REC doubles): lnA0 - lnA, beta0, Ea0/R, alpha, 1/T***, 1/T*, T**, pad
 constexpr int TR_REC = 8;
 // efficiency record: N doubles per third-body / falloff reaction
-// then, past the total (never staged into shared memory): ln A_j log2(e) 2^53 as
-// 64-bit integers, and 1 if every one of them lies in the fixed-point range
+// then, past the total (never staged into shared memory), the 64-bit words of the
+// fixed-point rate arguments (FixLayout)
 
 struct RxMeta {
   uint8_t reac[3];
@@ -81,8 +81,25 @@ struct MechDims {
   int N, M, n_eff, n_troe;
   int off_sp, off_rx, off_tr, off_eff, total;  // offsets in doubles
   __host__ __device__ int off_fix() const { return total; }
-  __host__ __device__ int allocated() const { return total + M + 1; }
+  __host__ __device__ int allocated() const;
 };
+
+// The words behind the blob, all values times log2(e) unless noted:
+//   lnA     M      ln A_j 2^53
+//   flag    1      1 if every ln A fits (lnA_fits_fixed)
+//   T_low   1      the lowest temperature the fixed-point arguments cover, as a
+//                  double; 0: the mechanism does not fit, nothing below is set
+//   g       7 N    g_k/RT: the constant 2^53, then the signed coefficients of log2 T
+//                  (plain a1, 2^57), T (2^65), T^2 (2^79), T^3 (2^93), T^4 (2^107)
+//                  and 1/T (2^46)
+//   rate    2 M    b (no log2(e), 2^57) and -E/R (2^46)
+//   falloff 3 n_troe  ln A0 - ln A (2^53), b0 - b (2^57), -(E0 - E)/R (2^46)
+struct FixLayout {
+  int flag, T_low, g, rate, falloff, words;
+  __host__ __device__ FixLayout(int N, int M, int n_troe)
+      : flag(M), T_low(M + 1), g(M + 2), rate(g + 7 * N), falloff(rate + 2 * M), words(falloff + 3 * n_troe) {}
+};
+__host__ __device__ inline int MechDims::allocated() const { return total + FixLayout(N, M, n_troe).words; }
 
 inline MechDims mech_dims(int N, int M, int n_eff, int n_troe) {
   MechDims d;

@@ -195,9 +195,18 @@ __device__ __forceinline__ uint64_t mul_fixed(uint64_t a, uint64_t b) {
 // |x| >= 512, inf and NaN (an integer test of the high word)
 __device__ __forceinline__ bool exp_is_big(double x) { return (__double2hiint(x) & 0x7fffffff) >= 0x40800000; }
 
-// the ln A the fixed-point rate arguments are built for: they stay within +- 1000
-// octaves with what the generator allows the temperature terms
-__host__ __device__ inline bool lnA_fits_fixed(double lnA) { return lnA > -277.0 && lnA < 277.0; }
+// the fixed-point arguments cover temperatures below this (and from FixLayout.T_low)
+constexpr double FIX_T_HIGH = 8000.0;
+
+// the ln A the fixed-point rate arguments are built for (150 octaves): the sums stay
+// within what 64 bits hold with what fixed_T_low allows the temperature terms
+__host__ __device__ inline bool lnA_fits_fixed(double lnA) { return lnA > -104.0 && lnA < 104.0; }
+
+// x + xc, both within 1022 2^53 and their sum below 1000 2^53, but not below
+// -1000 2^53 (a constant of 2^-1000)
+__device__ __forceinline__ int64_t add_exponents(int64_t x, int64_t xc) {
+  return (x >> 1) + (xc >> 1) < -(500ll << 53) ? -(1000ll << 53) : x + xc;
+}
 
 __device__ __forceinline__ double exp_rate(double x) {
   return exp_is_big(x) ? exp(x) : exp2_fixed(exp_arg_fixed(x));

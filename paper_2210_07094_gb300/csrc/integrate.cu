@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(128) k_eval_thread(EvalArgs a) {
     boff = blob_smem_doubles(a.d);
   }
   __syncthreads();
-  const MechView mv = make_view(blob, a.d);
+  const MechView mv = make_view(blob, a.d, a.blob);
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + tid;
   if (c >= a.ncells) return;
   double* ws = smem + boff + tid;
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(256, 1) k_integrate_warp(IntegArgs a, const in
     boff = blob_smem_doubles(a.d);
   }
   __syncthreads();
-  const MechView mv = make_view(blob, a.d);
+  const MechView mv = make_view(blob, a.d, a.blob);
   const int N = a.d.N, n = N + 1;
   double* ws = smem + boff + (size_t)warp * L.total;
   double* y = ws + L.y;
@@ -270,7 +270,7 @@ template <bool WITH_J>
 __global__ void __launch_bounds__(256) k_eval_warp(EvalArgs a, const int* csr, WarpWS L) {
   extern __shared__ double smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const MechView mv = make_view(a.blob, a.d);
+  const MechView mv = make_view(a.blob, a.d, a.blob);
   const int N = a.d.N, n = N + 1;
   const int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   if (c >= a.ncells) return;
@@ -561,8 +561,17 @@ int integrate_warp_dispatch(df_mech* m, const IntegArgs& a0, cudaStream_t st, in
 
 }  // namespace
 
+// One cell per warp for an evaluation of few cells of a mechanism with reactions
+// for the lanes: a cell per thread takes one thread's time through all reactions
+// whatever the number of cells (source term of the 9-species mechanism 62 us up to
+// 16000 cells), a cell per warp takes 39 us up to 500 cells, 52 at 2000, 75 at 4000.
+static bool few_cells(const df_mech* m, int64_t ncells) {
+  return m->dims.M >= 16 && ncells <= (int64_t)16 * m->num_sms;
+}
+
 int launch_rhs(const df_mech* m, int64_t ncells, const double* T, const double* p,
                const double* Y, double* dydt, double* qdot, cudaStream_t st) {
+  if (few_cells(m, ncells)) return eval_warp_dispatch(m, ncells, T, p, Y, dydt, qdot, nullptr, st);
   switch (m->dims.N) {
 #define X(NS) \
   case NS:    \
@@ -576,6 +585,7 @@ int launch_rhs(const df_mech* m, int64_t ncells, const double* T, const double* 
 
 int launch_jacobian(const df_mech* m, int64_t ncells, const double* T, const double* p,
                     const double* Y, double* J, cudaStream_t st) {
+  if (few_cells(m, ncells)) return eval_warp_dispatch(m, ncells, T, p, Y, nullptr, nullptr, J, st);
   switch (m->dims.N) {
 #define X(NS) \
   case NS:    \

@@ -83,8 +83,7 @@ __global__ void __launch_bounds__(128, 1) k_integrate_thread(IntegArgs a) {
     boff = blob_smem_doubles(a.d);
   }
   __syncthreads();
-  MechView mv = make_view(blob, a.d);
-  mv.fix = reinterpret_cast<const long long*>(a.blob + a.d.off_fix());
+  const MechView mv = make_view(blob, a.d, a.blob);
   double* ws = smem + boff + tid;
   typedef SVT<double, BT> V;
   const RosTab& tb = c_tab[a.method];

@@ -16,7 +16,7 @@
 #include <sstream>
 
 #include "common.cuh"
-#include "exp2fix.cuh"
+#include "reactions.cuh"
 
 namespace df {
 namespace {
@@ -143,6 +143,54 @@ bool num_of(const JVal* v, double* out) {
 }
 
 }  // namespace
+
+// the fixed-point words behind the blob (FixLayout)
+static void write_fixed(df_mech* m) {
+  const MechDims& d = m->dims;
+  const FixLayout F(d.N, d.M, d.n_troe);
+  std::vector<int64_t> w(F.words, 0);
+  bool fits = true;
+  for (int j = 0; j < d.M; ++j) {
+    const bool ok = lnA_fits_fixed(m->lnA_file[j]);
+    w[j] = ok ? exp_arg_fixed(m->lnA_file[j]) : 0;
+    fits = fits && ok;
+  }
+  w[F.flag] = fits;
+  const std::vector<Rx> rx = reactions_of(m);
+  double T_low = fixed_T_low(m, rx, true);
+  auto put = [&](int at, double c, bool log2e, int s) {  // c 2^s, signed; T_low = 0 if it takes more than 63 bits
+    uint64_t l;
+    int shift;
+    fixed_literal(c, log2e, s, &l, &shift);
+    if (shift || (l >> 63) != 0) T_low = 0.0;
+    w[at] = c < 0.0 ? -(int64_t)l : (int64_t)l;
+  };
+  for (int k = 0; k < d.N; ++k) {
+    const double* a = &m->blob_host[d.off_sp + SP_REC * k + 2];
+    const int g = F.g + 7 * k;
+    put(g, a[0] - a[6], true, 53);
+    put(g + 1, -a[0], false, 57);
+    put(g + 2, -a[1] / 2.0, true, 65);
+    put(g + 3, -a[2] / 6.0, true, 79);
+    put(g + 4, -a[3] / 12.0, true, 93);
+    put(g + 5, -a[4] / 20.0, true, 107);
+    put(g + 6, a[5], true, 46);
+  }
+  for (int j = 0; j < d.M; ++j) {
+    const Rx& x = rx[j];
+    put(F.rate + 2 * j, x.b, false, 57);
+    put(F.rate + 2 * j + 1, -x.E, true, 46);
+    if (x.type == 2) {
+      const double* tr = &m->blob_host[d.off_tr + TR_REC * x.troe];
+      const int t = F.falloff + 3 * x.troe;
+      if (std::isfinite(tr[0])) put(t, tr[0], true, 53);
+      put(t + 1, tr[1] - x.b, false, 57);
+      put(t + 2, -(tr[2] - x.E), true, 46);
+    }
+  }
+  memcpy(&w[F.T_low], &T_low, 8);
+  memcpy(&m->blob_host[d.off_fix()], w.data(), 8 * w.size());
+}
 
 int parse_mechanism(const char* path, df_mech* m) {
   std::ifstream f(path, std::ios::binary);
@@ -280,15 +328,7 @@ int parse_mechanism(const char* path, df_mech* m) {
   std::copy(troe.begin(), troe.end(), m->blob_host.begin() + d.off_tr);
   std::copy(eff.begin(), eff.end(), m->blob_host.begin() + d.off_eff);
   m->lnA_file = lnA;
-  for (int j = 0; j <= M; ++j) {
-    int64_t v = 1;
-    if (j < M) {
-      v = lnA_fits_fixed(lnA[j]) ? exp_arg_fixed(lnA[j]) : 0;
-    } else {
-      for (double a : lnA) v = v && lnA_fits_fixed(a);
-    }
-    memcpy(&m->blob_host[d.off_fix() + j], &v, 8);
-  }
+  write_fixed(m);
   // species -> (reaction, net stoichiometric coefficient nu''_kj - nu'_kj) lists
   std::vector<std::vector<std::pair<int, int>>> lists(N);
   for (int j = 0; j < M; ++j) {

@@ -1,5 +1,5 @@
-"""The generated fixed-point evaluation (gen_fixed) against the generated FP64 one
-(gen_eval) on the host: the same source text compiled by g++ with the device
+"""The generated fixed-point evaluation (gen_fixed) and the mechanism-independent one
+(eval_thread with rate_fixed) against the generated FP64 one (gen_eval) on the host: the same source text compiled by g++ with the device
 intrinsics it uses written out, so that f and every Jacobian entry are compared
 for all reaction forms without a GPU."""
 import os
@@ -72,12 +72,11 @@ int main() {
   if (fread(&d, sizeof d, 1, fp) != 1) return 2;
   std::vector<double> blob(d.allocated());
   if (fread(blob.data(), 8, blob.size(), fp) != blob.size()) return 2;
-  MechView mv = make_view(blob.data(), d);
-  mv.fix = (const long long*)(blob.data() + d.off_fix());
+  MechView mv = make_view(blob.data(), d, blob.data());
   std::mt19937_64 r(1);
   auto U = [&] { return (r() >> 11) * 0x1p-53; };
   int inside = 0;
-  double wf = 0, wj = 0, wp = 0;
+  double wf = 0, wj = 0, wp = 0, bf = 0, bj = 0;
   for (int t = 0; t < 2000; ++t) {
     double y[n], y2[n], f[n], fe[n], f2[n], fp_[n], W[GenEval::kWords], W0[GenEval::kWords], ex[128], J[n * n], J2[n * n], sM[n], s = 0;
     y[0] = t % 50 == 0 ? 30.0 + 12000.0 * U() : 240.0 + 3000.0 * U();
@@ -101,12 +100,41 @@ int main() {
     gen_eval<true, 1>(mv, pc, y2, f2, SVT<double, 1>{J2, 1}, S);
     double nf = 1e-300;
     for (int i = 1; i < n; ++i) nf = fmax(nf, fabs(fe[i]));
+    // the temperature's rate sums h_k times the species' rates: its terms
+    double f0 = 1e-300, cp0 = 0;
+    for (int k = 0; k < N; ++k) {
+      const double* c = mv.sp + SP_REC * k + 2;
+      const double T = y[0], iW = mv.sp[SP_REC * k + 1];
+      cp0 += y[1 + k] * iW * (c[0] + T * (c[1] + T * (c[2] + T * (c[3] + T * c[4]))));
+      f0 += fabs(T * iW * fe[1 + k] * (c[0] + T * (c[1] / 2 + T * (c[2] / 3 + T * (c[3] / 4 + T * c[4] / 5))) + c[5] / T));
+    }
+    f0 /= fabs(cp0);
     for (int i = 0; i < n; ++i) {
-      const double tol = 100 * fabs(f2[i] - fe[i]) + 1e-11 * (i ? nf : fabs(fe[0])) + 1e-280;
+      const double tol = 100 * fabs(f2[i] - fe[i]) + 1e-11 * (i ? nf : f0) + 1e-280;
       wf = fmax(wf, fabs(f[i] - fe[i]) / tol);
       for (int a = 0; a < NA; ++a)  // without J only the systems' entries
         if (GenEval::act(a) == i) wp = fmax(wp, fabs(f[i] - fp_[i]) / tol);
     }
+    // the mechanism-independent evaluation, which reads the same arguments from the blob
+    // against itself in FP64 (no temperature covered)
+    double fb[n], fs[n], fq[n], v5[5][N], Jb[n * n], Js[n * n], Jq[n * n], cf[n] = {}, cJ[n * n] = {};
+    MechView mvs = mv;
+    mvs.T_low = INFINITY;
+    auto sv = [](double* p) { return SVT<double, 1>{p, 1}; };
+    auto blob_eval = [&](const MechView& v, const double(&z)[n], double(&ff)[n], double* JJ) {
+      eval_thread<N, true, double, false, 1>(v, pc, z, ff, sv(v5[0]), sv(v5[1]), sv(v5[2]), sv(v5[3]), sv(v5[4]), sv(JJ));
+    };
+    blob_eval(mv, y, fb, Jb);
+    blob_eval(mvs, y, fs, Js);
+    for (int q = 0; q < n; ++q) {  // the change with each entry of the state (1 + 4e-16)
+      double z[n];
+      for (int i = 0; i < n; ++i) z[i] = y[i] * (i == q ? 1 + 4e-16 : 1);
+      blob_eval(mvs, z, fq, Jq);
+      for (int i = 0; i < n; ++i) cf[i] = fmax(cf[i], fabs(fq[i] - fs[i]));
+      for (int i = 0; i < n * n; ++i) cJ[i] = fmax(cJ[i], fabs(Jq[i] - Js[i]));
+    }
+    for (int i = 0; i < n; ++i)
+      bf = fmax(bf, fabs(fb[i] - fs[i]) / (100 * cf[i] + 1e-11 * (i ? nf : f0) + 1e-280));
     // the columns over the kept species: beta times the eliminated ones' added
     auto red = [&](const double* A, int ra, int b) {
       double v = A[ra + GenEval::act(b)];
@@ -135,6 +163,9 @@ int main() {
         }
       }
       for (int b = 0; b < NA; ++b) {
+        const int id = ra + GenEval::act(b);
+        const double d = fabs(Jb[id] - Js[id]) / (100 * cJ[id] + 1e-11 * nr);
+        if (!(d <= bj)) bj = d;
         const double j = red(J, ra, b), e = fabs(W[a * NA + b] + j) / (100 * fabs(red(J2, ra, b) - j) + 1e-11 * nr);
         if (!(e <= wj)) wj = e;
       }
@@ -162,8 +193,8 @@ int main() {
       }
     }
   }
-  printf("inside %d f %g J %g plain %g\n", inside, wf, wj, wp);
-  return inside >= 1000 && wf <= 1 && wj <= 1 && wp <= 1 ? 0 : 1;
+  printf("inside %d f %g J %g plain %g blob f %g J %g\n", inside, wf, wj, wp, bf, bj);
+  return inside >= 1000 && wf <= 1 && wj <= 1 && wp <= 1 && bf <= 1 && bj <= 1 && mv.T_low < 500 ? 0 : 1;
 }
 """
 
