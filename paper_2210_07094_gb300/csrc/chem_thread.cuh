@@ -690,21 +690,38 @@ __device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, co
                                          SVT<S> wdot, SVT<S> gRT, SVT<S> hRT, SVT<S> cpR, SVT<S> sig, SVT<S> v,
                                          const ThetaHook* hook = nullptr) {
   const S T = y[0];
-  const S lnT = fast_log(T);
   const S invT = 1.0 / T;
   S sumYW(0.0), cpm(0.0);
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     const double* a = mv.sp + SP_REC * k + 2;
     const S cpk = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4])));
-    const double* ah = mv.sp + SP_REC * k + SP_H;  // a2/2 .. a5/5
-    const double* as = mv.sp + SP_REC * k + SP_S;  // a3/2 .. a5/4
-    const S hk = a[0] + T * (ah[0] + T * (ah[1] + T * (ah[2] + T * ah[3]))) + a[5] * invT;
-    const S sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
-    hRT[k] = hk;
-    gRT[k] = hk - sk;
     sumYW += y[1 + k] * mv.sp[SP_REC * k + 1];
     cpm += y[1 + k] * cpk * mv.sp[SP_REC * k + 1];
+  }
+  // the rates in fixed point (rate_fixed) for the plain evaluation
+  FixState fst;
+  bool fixed = false;
+  if constexpr (sizeof(S) == sizeof(double)) {
+    fixed = fixed_covers(mv, T) && rcp_in_range(sumYW) && rcp_in_range(pc);
+    if (fixed) fst = fix_state(T, invT);
+  }
+  S lnT(0.0);
+  if (!fixed) lnT = fast_log(T);
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const double* a = mv.sp + SP_REC * k + 2;
+    const double* ah = mv.sp + SP_REC * k + SP_H;  // a2/2 .. a5/5
+    const S hk = a[0] + T * (ah[0] + T * (ah[1] + T * (ah[2] + T * ah[3]))) + a[5] * invT;
+    hRT[k] = hk;
+    if (fixed) {
+      if constexpr (sizeof(S) == sizeof(double))
+        gRT[k] = __longlong_as_double(fix_gibbs(mv.fix + mv.fg + 7 * k, fst));
+    } else {
+      const double* as = mv.sp + SP_REC * k + SP_S;  // a3/2 .. a5/4
+      const S sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
+      gRT[k] = hk - sk;
+    }
   }
   cpm = cpm * RU;
   const S rho = pc * invT / (RU * sumYW);
@@ -732,7 +749,12 @@ __device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, co
   const S lnP0RT = LOG_PSTD_RU - lnT;
   for (int j = 0; j < mv.M; ++j) {
     RateOutT<S> ro;
-    rate_one<NS, true>(mv, mv.rx + RX_REC * j, NS, T, lnT, invT, lnP0RT, C, gRT, hRT, ro);
+    if (fixed) {
+      if constexpr (sizeof(S) == sizeof(double))
+        rate_fixed<NS, true>(mv, j, mv.rx + RX_REC * j, NS, T, invT, fst, C, gRT, hRT, ro);
+    } else {
+      rate_one<NS, true>(mv, mv.rx + RX_REC * j, NS, T, lnT, invT, lnP0RT, C, gRT, hRT, ro);
+    }
     if (!ro.active) continue;
     const RxMeta mt = ro.mt;
     const int nr = mt.nrnp & 15, np = mt.nrnp >> 4;
