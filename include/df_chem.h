@@ -197,9 +197,8 @@ int df_chem_integrate(const df_mech* mech, int64_t ncells, double* T, const doub
  *                steps gets DF_CELL_MAXSTEPS and a zero gradient
  *  workspace     device memory owned by the caller: at least the compact size
  *                8 * (ncells*max_steps*(N+2) + ceil(ncells/16)*M) + 256
- *                bytes (the ln A partial sums take ceil(ncells/B)*M doubles,
- *                B the 16 to 32 cells of one block, which the library picks
- *                from the device's shared memory); df_chem_adjoint_workspace_size() returns the size with
+ *                bytes (the ln A partial sums take ceil(ncells/32)*M doubles
+ *                of it); df_chem_adjoint_workspace_size() returns the size with
  *                the stored stages, 8 * ncells*max_steps*(7n + n^2) bytes more
  *                (n = N + 1).  On return its first ncells*max_steps*(N+2)
  *                doubles hold the checkpoints [cell][step][T, Y_1..Y_N, h] of

@@ -59,33 +59,29 @@ struct AdjArgs {
   int32_t* nsub;
   double* ckpt;     // [ncells][cap][n + 1]: y_i then h_i
   double* partial;  // [gridDim.x][M]
-  int stage_blob;
   // optional [cap][7n + n^2][ncells] (cell fastest, so a warp's accesses
   // coalesce): the accepted step's stage vectors K_s (6n), LU factors of W
   // (n^2) and row pivots (n), kept by the forward sweep so that the reverse
   // sweep need not recompute the step; null: the reverse sweep recomputes it
   double* stages;
-  int hook_cp;  // 8 NS: the Dual cpR vector's offset (doubles, units of the block size)
+  int hook_cp;  // 4 NS: the cpR vector's offset (doubles, units of the block size)
 };
 
-// Per-thread shared-memory doubles.  Without KEEP (the reverse sweep
-// recomputes each step): Dual C, wdot, gRT, hRT, cpR, sigma, v (14 NS) + W
-// (n^2) + K, Kbar (12 n) + theta (M).  With KEEP (the forward sweep stores each
-// accepted step's stages and LU factors in the workspace and the reverse sweep
-// reads them there): the dual vectors, then a region of max(n^2, 6n + M) that
-// holds Kbar and theta in the reverse sweep and W in the forward sweep; the
-// forward sweep's K sits in the derivative halves of the dual vectors, unused
-// until the reverse sweep (6n <= 7NS for NS >= 6).  In both, the ln A hook's
-// scratch u, ud shares the Dual cpR vector (eval_vjp writes cpR only after its
-// reaction loop, the one place that reads u), and its weights are the
-// cotangent eval_vjp is given.  Less shared memory per thread, more warps per
-// SM on the narrow FP64 pipe.
-__host__ __device__ constexpr int adj_layout_doubles(int NS, int M, bool keep) {
-  return keep ? 14 * NS + ((NS + 1) * (NS + 1) > 6 * (NS + 1) + M ? (NS + 1) * (NS + 1) : 6 * (NS + 1) + M)
-              : 14 * NS + (NS + 1) * (NS + 1) + 12 * (NS + 1) + M;
-}
+// The sweeps of a launch: both in one kernel, which recomputes each step's stages
+// and factors, or, where the workspace keeps them, one kernel each.
+enum Sweep { BOTH, FORWARD, REVERSE };
 
-__host__ __device__ constexpr bool adj_keep_possible(int NS) { return 6 * (NS + 1) <= 7 * NS; }
+// Per-thread shared-memory doubles: C, wdot, gRT, hRT, cpR, then sigma and v for
+// the reverse sweep; W (n^2) where the step is computed; theta (M) for the reverse
+// sweep.  K and Kbar are in local memory.  The ln A hook's scratch u shares the
+// cpR vector (eval_vjp writes cpR only after its reaction loop, the one place that
+// reads u).  The less shared memory a thread takes, the more warps an SM holds: eight
+// for the reverse sweep of 9 species (255 registers a thread), six for the forward one,
+// two on each of the narrow FP64 pipes, so that one's dependent chains overlap the other's.
+__host__ __device__ constexpr int adj_layout_doubles(int NS, int M, Sweep sw) {
+  const int n = NS + 1;
+  return sw == FORWARD ? 5 * NS + n * n : sw == REVERSE ? 7 * NS + M : 7 * NS + n * n + M;
+}
 
 // read-only view of the stored stages in the workspace: element i at p[i * s],
 // s = ncells (64-bit offsets)
@@ -95,71 +91,26 @@ struct GV {
   __device__ __forceinline__ double operator[](int i) const { return p[(int64_t)i * s]; }
 };
 
-// The sweeps of a launch: both in one kernel, or (with stored stages) one kernel
-// each.  Apart, the forward sweep needs the species vectors, W and K (K in local
-// memory), the reverse sweep the dual vectors alone, with Kbar and theta in local
-// memory: six and seven warps per SM instead of four, one of which every FP64 pipe
-// had to itself.  65536 cells, 25 reactions, gradients of Y and ln A for a loss on T
-// and the heat release, with eval_vjp's rates in fixed point: 12.16 -> 9.57 ms.
-enum Sweep { BOTH, FORWARD, REVERSE };
-constexpr int ADJ_LOCAL_M = 64;  // theta's room in the reverse kernel's local memory
-
-template <int NS, bool KEEP = false, Sweep SW = BOTH>
+template <int NS, Sweep SW>
 __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
-  static_assert(!KEEP || 6 * (NS + 1) <= 7 * NS, "KEEP: the forward K must fit the dual derivative halves");
-  static_assert(SW == BOTH || KEEP, "separate sweeps: stored stages");
   constexpr int n = NS + 1;
   extern __shared__ double smem[];
   const int tid = threadIdx.x, stride = blockDim.x;
-  int boff = 0;
-  const double* blob = a.blob;
-  if (a.stage_blob) {
-    for (int i = tid; i < a.d.total; i += stride) smem[i] = a.blob[i];
-    blob = smem;
-    boff = (a.d.total + 1) & ~1;
-  }
-  __syncthreads();
-  const MechView mv = make_view(blob, a.d, a.blob);
+  const MechView mv = make_view(a.blob, a.d, a.blob);
   const int M = a.d.M;
-  double* base = smem + boff;
-  // Dual vectors (value part at even offsets)
-  Dual* dbase = reinterpret_cast<Dual*>(base) + tid;
-  SVT<Dual> dC{dbase, stride}, dW{dbase + NS * stride, stride}, dG{dbase + 2 * NS * stride, stride},
-      dH{dbase + 3 * NS * stride, stride}, dCp{dbase + 4 * NS * stride, stride},
-      dS{dbase + 5 * NS * stride, stride}, dV{dbase + 6 * NS * stride, stride};
-  // double views of the same storage
-  double* vb = base + 2 * tid;
-  SV C{vb, 2 * stride}, wd{vb + 2 * NS * stride, 2 * stride}, gRT{vb + 4 * NS * stride, 2 * stride},
-      hRT{vb + 6 * NS * stride, 2 * stride}, cpR{vb + 8 * NS * stride, 2 * stride},
-      sg{vb + 10 * NS * stride, 2 * stride}, vs{vb + 12 * NS * stride, 2 * stride};
-  double* rest = base + (14 * NS) * stride + tid;
-  SV Wv{rest, stride};  // the forward sweep's W (both layouts) and the recomputed one
-  SV Kv = KEEP ? SV{vb + 1, 2 * stride} : SV{rest + n * n * stride, stride};
-  const int kstride = SW == FORWARD ? 1 : KEEP ? 2 * stride : stride;  // stride of a stage vector inside Kv
-  double* kb0 = KEEP ? rest : rest + (n * n + 6 * n) * stride;
-  SV Kb{kb0, stride};
-  SV th{kb0 + 6 * n * stride, stride};
-  double kl[SW == BOTH ? 1 : 6 * n], tl[SW == REVERSE ? ADJ_LOCAL_M : 1];
-  if (SW == FORWARD) {  // species vectors, then W
-    C = SV{base + tid, stride};
-    wd = SV{base + tid + NS * stride, stride};
-    gRT = SV{base + tid + 2 * NS * stride, stride};
-    hRT = SV{base + tid + 3 * NS * stride, stride};
-    cpR = SV{base + tid + 4 * NS * stride, stride};
-    Wv = SV{base + tid + 5 * NS * stride, stride};
-    Kv = SV{kl, 1};
-  }
-  if (SW == REVERSE) {
-    Kb = SV{kl, 1};
-    th = SV{tl, 1};
-  }
-  // the ln A hook's scratch: the Dual cpR vector (its value halves for the
-  // double evaluation), at an offset the launch passes in: where the compiler
-  // can see that the scratch and cpR coincide it schedules eval_vjp with
-  // several hundred bytes of register spills
-  SV uu{vb + a.hook_cp * stride, 2 * stride};
-  SVT<Dual> uD{reinterpret_cast<Dual*>(vb + a.hook_cp * stride), stride};
-  const int th_off = 14 * NS + (KEEP ? 6 * n : n * n + 12 * n);  // theta's offset (units of stride)
+  double* base = smem + tid;
+  SV C{base, stride}, wd{base + NS * stride, stride}, gRT{base + 2 * NS * stride, stride},
+      hRT{base + 3 * NS * stride, stride}, cpR{base + 4 * NS * stride, stride}, sg{base + 5 * NS * stride, stride},
+      vs{base + 6 * NS * stride, stride};
+  SV Wv{base + (SW == FORWARD ? 5 : 7) * NS * stride, stride};
+  const int th_off = 7 * NS + (SW == BOTH ? n * n : 0);  // theta's offset (units of stride)
+  SV th{base + th_off * stride, stride};
+  double kf[SW == REVERSE ? 1 : 6 * n], kb[SW == FORWARD ? 1 : 6 * n];
+  SV Kv{kf, 1}, Kb{kb, 1};
+  // the ln A hook's scratch: the cpR vector, at an offset the launch passes in:
+  // where the compiler can see that the scratch and cpR coincide it schedules
+  // eval_vjp with several hundred bytes of register spills
+  SV uu{base + a.hook_cp * stride, stride};
   const RosTab& tb = c_tab_adj;
   if (SW != FORWARD)
     for (int j = 0; j < M; ++j) th[j] = 0.0;
@@ -194,7 +145,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
       for (int i = 0; i < n; ++i) yold[i] = y[i];
       int pv[n];
       const bool sok = ros_attempt<NS>(mv, tb, pc, y, h, a.rtol, a.atolY, a.atolT, C, wd, gRT, hRT, cpR, Wv, Kv,
-                                       kstride, ynew, en, pv, nacc == 0 && nrej == 0, &last);
+                                       1, ynew, en, pv, nacc == 0 && nrej == 0, &last);
       const double hstep = h;  // the step actually taken (the first one may be cut)
       const int before = nacc;
       step_control(tb, sok, en, last, a.dt, y, ynew, t, h, nacc, nrej, last_rej, done, ss);
@@ -245,9 +196,6 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
         }
       }
     }
-    if (KEEP && SW == BOTH) {  // the forward sweep's W overlaid theta, u, ud and Kbar
-      for (int j = 0; j < M; ++j) th[j] = 0.0;
-    }
     double lam[n];
     if (status == DF_CELL_OK) {
       // ---- cotangent at the final state --------------------------------
@@ -260,11 +208,11 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
         // f_T d(rho cp)/dy: one transposed product with e_T (which also adds the
         // ln A terms of Q through the hook) and the closed-form derivative of
         // rho cp = (p/T) A/B, A = sum_k Y_k cp_k/(R W_k), B = sum_k Y_k/W_k
-        ThetaHook hk{2, gq, th, uu, uD};
+        ThetaHook hk{2, gq, th, uu};
         double e0[n], b0[n], fq[n];
 #pragma unroll
         for (int i = 0; i < n; ++i) e0[i] = i == 0 ? 1.0 : 0.0;
-        eval_vjp<NS, double>(mv, pc, y, e0, b0, fq, C, wd, gRT, hRT, cpR, sg, vs, &hk);
+        eval_vjp<NS>(mv, pc, y, e0, b0, fq, C, wd, gRT, hRT, cpR, sg, vs, &hk);
         const double T = y[0];
         double A = 0.0, B = 0.0, dA = 0.0;
 #pragma unroll
@@ -290,27 +238,16 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
         for (int i = 0; i < n; ++i) yi[i] = slot[i];
         double hs = slot[n];
         int piv[n];
-        // this step's stages and LU factors: read in place from the workspace
-        // (KEEP), copied from it, or recomputed
-        typedef typename std::conditional<KEEP, GV, SV>::type StageView;
-        StageView Wr, Kr;
-        if constexpr (KEEP) {
+        // this step's stages and LU factors: read in place from the workspace, or recomputed
+        typename std::conditional<SW == REVERSE, GV, SV>::type Wr, Kr;
+        if constexpr (SW == REVERSE) {
           const double* sp = a.stages + (int64_t)istep * (7 * n + n * n) * a.ncells + cell;
           Kr = GV{sp, a.ncells};
           Wr = GV{sp + (int64_t)6 * n * a.ncells, a.ncells};
 #pragma unroll
           for (int i = 0; i < n; ++i) piv[i] = (int)sp[(int64_t)(6 * n + n * n + i) * a.ncells];
         } else {
-          if (a.stages) {  // the forward sweep kept this step's stages and factors
-            const double* sp = a.stages + (int64_t)istep * (7 * n + n * n) * a.ncells + cell;
-            for (int i = 0; i < 6 * n; ++i) Kv[i] = sp[i * a.ncells];
-            for (int i = 0; i < n * n; ++i) Wv[i] = sp[(6 * n + i) * a.ncells];
-#pragma unroll
-            for (int i = 0; i < n; ++i) piv[i] = (int)sp[(6 * n + n * n + i) * a.ncells];
-          } else {
-            ros_attempt<NS>(mv, tb, pc, yi, hs, a.rtol, a.atolY, a.atolT, C, wd, gRT, hRT, cpR, Wv, Kv, stride, ynew,
-                            en, piv);
-          }
+          ros_attempt<NS>(mv, tb, pc, yi, hs, a.rtol, a.atolY, a.atolT, C, wd, gRT, hRT, cpR, Wv, Kv, 1, ynew, en, piv);
           Kr = Kv;
           Wr = Wv;
         }
@@ -362,33 +299,19 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
             for (int j = 0; j < s; ++j) acc += tb.a[s][j] * Kr[j * n + i];
             ysg[i] = acc;
           }
-          // the first stage is evaluated at the step's start, where the dual
-          // evaluation below is: its value part stands in for this product
-          if (s > 0) {
-            ThetaHook hk{1, 0.0, th, uu, uD};
-            double bj[n];
-            eval_vjp<NS, double>(mv, pc, ysg, r, bj, fs, C, wd, gRT, hRT, cpR, sg, vs, &hk);
+          ThetaHook hk{1, 0.0, th, uu};
+          double bj[n];
+          eval_vjp<NS>(mv, pc, ysg, r, bj, fs, C, wd, gRT, hRT, cpR, sg, vs, &hk);
 #pragma unroll
-            for (int jc = 0; jc < n; ++jc) {
-              yb[jc] += bj[jc];
-              for (int j = 0; j < s; ++j) Kb[j * n + jc] += tb.a[s][j] * bj[jc];
-            }
+          for (int jc = 0; jc < n; ++jc) {
+            yb[jc] += bj[jc];
+            for (int j = 0; j < s; ++j) Kb[j * n + jc] += tb.a[s][j] * bj[jc];
           }
-          // W depends on y through J(y): d/de [J(y + e K_s)^T Rbar] and the ln A analogue
-          {
-            Dual yd[n], fd[n], bd[n];
 #pragma unroll
-            for (int i = 0; i < n; ++i) yd[i] = Dual(yi[i], Kr[s * n + i]);
-            ThetaHook hk{1, 0.0, th, uu, uD, s == 0 ? 1 : 0};
-            eval_vjp<NS, Dual>(mv, pc, yd, r, bd, fd, dC, dW, dG, dH, dCp, dS, dV, &hk);
-            if (s == 0) {
-#pragma unroll
-              for (int jc = 0; jc < n; ++jc) yb[jc] += bd[jc].v;
-            }
-#pragma unroll
-            for (int jc = 0; jc < n; ++jc) yb[jc] += bd[jc].d;
-          }
+          for (int i = 0; i < n; ++i) Kb[s * n + i] = r[i];
         }
+        // W depends on y through J(y), in every stage
+        second_order<NS>(mv, pc, yi, tb.s, Kr, Kb, yb, C, wd, gRT, hRT, cpR, vs, th);
 #pragma unroll
         for (int i = 0; i < n; ++i) lam[i] = yb[i];
       }
@@ -407,15 +330,11 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_thread(AdjArgs a) {
   }
   // fixed-order sum of the per-thread ln A gradients of this block
   if (SW == FORWARD) return;
-  if (SW == REVERSE) {  // through shared memory (the dual vectors are done with; M <= 14 NS)
-    __syncthreads();
-    for (int j = 0; j < M; ++j) base[(size_t)j * stride + tid] = th[j];
-  }
   __syncthreads();
   if (a.partial) {
     for (int j = tid; j < M; j += stride) {
       double acc = 0.0;
-      for (int q = 0; q < stride; ++q) acc += base[(size_t)((SW == REVERSE ? 0 : th_off) + j) * stride + q];
+      for (int q = 0; q < stride; ++q) acc += smem[(size_t)(th_off + j) * stride + q];
       a.partial[(int64_t)blockIdx.x * M + j] = acc;
     }
   }
@@ -440,26 +359,9 @@ static int ensure_adj_table(int dev) {
   return rc;
 }
 
-// Threads (cells) per block: as many, up to one warp, as let four blocks share
-// an SM.  Each of an SM's four sub-partitions has its own FP64 unit, and a
-// thread's workspace is too large for two warps per sub-partition, so a
-// fourth block keeps the fourth unit busy: four blocks of 31 threads do more
-// work than three of 32 (the 9-species layout: 226 doubles per thread).  Both
-// layouts use the count of the one with stored stages, so that their per-block
-// ln A partial sums group the cells alike and the gradients agree bitwise.  The
-// separate sweeps take whole warps.
-static bool adj_apart(const df_mech* m) {  // separate sweeps with stored stages
-  return adj_keep_possible(m->dims.N) && m->dims.M <= ADJ_LOCAL_M && m->dims.M <= 14 * m->dims.N;
-}
-
-static int adj_threads(const df_mech* m) {
-  const int NS = m->dims.N;
-  if (adj_apart(m)) return 32;
-  const long per = adj_layout_doubles(NS, m->dims.M, adj_keep_possible(NS));
-  const long budget = (long)m->smem_per_sm / 4 - (long)m->smem_reserved_per_block;  // bytes per block
-  const long t = budget / (long)sizeof(double) / per;
-  return t >= 16 && t < 32 ? (int)t : 32;
-}
+// Threads (cells) per block, in all layouts: their per-block ln A partial sums
+// group the cells alike, so the gradients agree bitwise.
+constexpr int ADJ_THREADS = 32;
 
 // Workspace: checkpoints [ncells][cap][n + 1], then the per-block ln A
 // partials, then (with_stages) the stored stages [cap][7n + n^2][ncells].
@@ -468,7 +370,7 @@ static int adj_threads(const df_mech* m) {
 static bool adj_compact_doubles(const df_mech* m, int64_t ncells, int cap, size_t* out) {
   if (ncells < 0 || cap < 1) return false;
   const size_t n = (size_t)m->dims.N + 1;
-  const size_t threads = (size_t)adj_threads(m);
+  const size_t threads = ADJ_THREADS;
   const size_t blocks = ((size_t)ncells + threads - 1) / threads;
   size_t ck = 0, part = 0;
   if (__builtin_mul_overflow((size_t)ncells, (size_t)cap, &ck) || __builtin_mul_overflow(ck, n + 1, &ck) ||
@@ -492,69 +394,34 @@ bool adjoint_workspace_bytes(const df_mech* m, int64_t ncells, int cap, bool wit
   return true;
 }
 
-template <int NS, bool KEEP>
-static int adjoint_dispatch_layout(const df_mech* m, AdjArgs a, cudaStream_t st, double* g_lnA) {
-  const int threads = adj_threads(m);
-  const size_t per = (size_t)adj_layout_doubles(NS, m->dims.M, KEEP) * threads;
-  a.hook_cp = 8 * NS;
-  // the mechanism is staged in shared memory unless that leaves fewer blocks
-  // on an SM than reading it through L1
-  const size_t sm_staged = sizeof(double) * (((m->dims.total + 1) & ~1) + per);
-  const size_t sm_plain = sizeof(double) * per;
-  auto blocks_per_sm = [m](size_t b) {
-    return b > m->max_smem_optin ? (size_t)0 : m->smem_per_sm / (b + m->smem_reserved_per_block);
-  };
-  a.stage_blob = blocks_per_sm(sm_staged) >= blocks_per_sm(sm_plain) ? 1 : 0;
-  const size_t sm = a.stage_blob ? sm_staged : sm_plain;
+template <int NS, Sweep SW>
+static int launch_sweep(const df_mech* m, const AdjArgs& a, int64_t blocks, cudaStream_t st) {
+  const size_t sm = sizeof(double) * adj_layout_doubles(NS, m->dims.M, SW) * ADJ_THREADS;
   if (sm > m->max_smem_optin) return set_error(DF_EUNSUPPORTED, "adjoint workspace exceeds shared memory");
-  auto kf = k_adjoint_thread<NS, KEEP>;
-  int rc = cuda_check(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
+  int rc = cuda_check(cudaFuncSetAttribute(k_adjoint_thread<NS, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
                       "set adjoint shared memory");
   if (rc) return rc;
-  const int64_t blocks = (a.ncells + threads - 1) / threads;
-  kf<<<(unsigned)blocks, threads, sm, st>>>(a);
-  rc = cuda_check(cudaGetLastError(), "adjoint kernel launch");
+  k_adjoint_thread<NS, SW><<<(unsigned)blocks, ADJ_THREADS, sm, st>>>(a);
+  return cuda_check(cudaGetLastError(), "adjoint kernel launch");
+}
+
+template <int NS>
+static int adjoint_dispatch(const df_mech* m, AdjArgs a, cudaStream_t st, double* g_lnA) {
+  const int64_t blocks = (a.ncells + ADJ_THREADS - 1) / ADJ_THREADS;
+  a.hook_cp = 4 * NS;
+  int rc;
+  if (a.stages) {
+    rc = launch_sweep<NS, FORWARD>(m, a, blocks, st);
+    if (!rc) rc = launch_sweep<NS, REVERSE>(m, a, blocks, st);
+  } else {
+    rc = launch_sweep<NS, BOTH>(m, a, blocks, st);
+  }
   if (rc) return rc;
   if (g_lnA && m->dims.M > 0) {
     k_adjoint_reduce<<<(m->dims.M + 127) / 128, 128, 0, st>>>(a.partial, blocks, m->dims.M, g_lnA);
     rc = cuda_check(cudaGetLastError(), "adjoint reduction launch");
   }
   return rc;
-}
-
-// the smaller layout when the stages are kept in the workspace and the
-// forward sweep's stage vectors fit the dual derivative halves
-template <int NS>
-static int adjoint_dispatch(const df_mech* m, AdjArgs a, cudaStream_t st, double* g_lnA) {
-  if constexpr (adj_keep_possible(NS)) {
-    if (a.stages && adj_apart(m) && a.cap < (1 << 26)) {
-      const int threads = adj_threads(m);
-      const int64_t blocks = (a.ncells + threads - 1) / threads;
-      a.stage_blob = 0;
-      a.hook_cp = 8 * NS;
-      auto kf = k_adjoint_thread<NS, true, FORWARD>;
-      auto kr = k_adjoint_thread<NS, true, REVERSE>;
-      const int sf = (int)sizeof(double) * (5 * NS + (NS + 1) * (NS + 1)) * threads;
-      const int sr = (int)sizeof(double) * 14 * NS * threads;
-      int rc = cuda_check(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, sf),
-                          "set adjoint shared memory");
-      if (!rc)
-        rc = cuda_check(cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, sr),
-                        "set adjoint shared memory");
-      if (rc) return rc;
-      kf<<<(unsigned)blocks, threads, sf, st>>>(a);
-      kr<<<(unsigned)blocks, threads, sr, st>>>(a);
-      rc = cuda_check(cudaGetLastError(), "adjoint kernel launch");
-      if (rc) return rc;
-      if (g_lnA && m->dims.M > 0) {
-        k_adjoint_reduce<<<(m->dims.M + 127) / 128, 128, 0, st>>>(a.partial, blocks, m->dims.M, g_lnA);
-        rc = cuda_check(cudaGetLastError(), "adjoint reduction launch");
-      }
-      return rc;
-    }
-    if (a.stages) return adjoint_dispatch_layout<NS, true>(m, a, st, g_lnA);
-  }
-  return adjoint_dispatch_layout<NS, false>(m, a, st, g_lnA);
 }
 
 int launch_adjoint(const df_mech* m, int64_t ncells, const double* T0, const double* p, const double* Y0,
@@ -599,7 +466,8 @@ int launch_adjoint(const df_mech* m, int64_t ncells, const double* T0, const dou
   adj_compact_doubles(m, ncells, cap, &compact);  // fits: checked above
   a.ckpt = static_cast<double*>(ws);
   a.partial = static_cast<double*>(ws) + (size_t)ncells * cap * (n + 1);
-  a.stages = keep_stages ? static_cast<double*>(ws) + compact : nullptr;
+  // (the forward kernel packs the step count beside the status)
+  a.stages = keep_stages && cap < (1 << 26) ? static_cast<double*>(ws) + compact : nullptr;
   switch (m->dims.N) {
     case 3:
       return adjoint_dispatch<3>(m, a, st, g_lnA);

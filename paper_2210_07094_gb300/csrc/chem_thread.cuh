@@ -471,29 +471,14 @@ __device__ __forceinline__ void rate_fixed(const MechView& mv, int j, const doub
 // weights are eval_vjp's cotangent r of dy/dt, i.e. th[j] += r . d f / d ln A_j
 // = q_j sum_k nu_kj u_k with u_k = (W_k r_{Y_k} - r_T H_k / cp) / rho.  Mode 2:
 // heat release, th[j] += g * d qdot / d ln A_j with qdot = -0.1 sum_k H_k wdot_k
-// [W/m^3].  With a Dual scalar only the derivative part is accumulated, or,
-// with both set, the value part and then the derivative part (a Dual
-// evaluation that also stands in for the double one at the same point).  The
-// scratch u may be the storage of eval_vjp's cpR vector: eval_vjp reads u only
-// in its reaction loop and writes cpR after it.
+// [W/m^3].  The scratch u may be the storage of eval_vjp's cpR vector: eval_vjp
+// reads u only in its reaction loop and writes cpR after it.
 struct ThetaHook {
   int mode;        // 0: off
   double g;        // mode 2: weight
   SV th;           // per-thread accumulator, M entries
-  SV u;            // per-thread scratch, N entries (double evaluation)
-  SVT<Dual> uD;    // per-thread scratch, N entries (Dual evaluation)
-  int both = 0;    // Dual evaluation: accumulate the value part too
+  SV u;            // per-thread scratch, N entries
 };
-
-__device__ __forceinline__ void th_add(const ThetaHook& h, int j, double x) { h.th[j] += x; }
-__device__ __forceinline__ void th_add(const ThetaHook& h, int j, const Dual& x) {
-  if (h.both) h.th[j] += x.v;
-  h.th[j] += x.d;
-}
-__device__ __forceinline__ void u_store(const ThetaHook& h, int k, double x) { h.u[k] = x; }
-__device__ __forceinline__ void u_store(const ThetaHook& h, int k, const Dual& x) { h.uD[k] = x; }
-__device__ __forceinline__ double u_load(const ThetaHook& h, int k, double) { return h.u[k]; }
-__device__ __forceinline__ Dual u_load(const ThetaHook& h, int k, const Dual&) { return h.uD[k]; }
 
 // Evaluate f = dy/dt for y = (T, Y) and, when WITH_J, the analytic Jacobian
 // J = df/dy (row-major in the strided view Jv, n x n with n = NS + 1).
@@ -683,82 +668,77 @@ __device__ __forceinline__ S eval_thread(const MechView& mv, const double pc, co
 // with e the temperature row's own terms (e_T = -(cpf + f_T dcp/dT) / cp,
 // e_i = -f_T cp_i / cp).  Also returns f = dy/dt (f may alias nothing) and, with
 // a hook, its ln A terms.  sig and v are N-entry scratch vectors; cpR receives
-// cp_k/R after the reaction loop (the hook's u, ud may share its storage).
-template <int NS, class S = double>
-__device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, const S (&y)[NS + 1],
-                                         const double (&r)[NS + 1], S (&b)[NS + 1], S (&f)[NS + 1], SVT<S> C,
-                                         SVT<S> wdot, SVT<S> gRT, SVT<S> hRT, SVT<S> cpR, SVT<S> sig, SVT<S> v,
+// cp_k/R after the reaction loop (the hook's u may share its storage).
+template <int NS>
+__device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, const double (&y)[NS + 1],
+                                         const double (&r)[NS + 1], double (&b)[NS + 1], double (&f)[NS + 1], SV C,
+                                         SV wdot, SV gRT, SV hRT, SV cpR, SV sig, SV v,
                                          const ThetaHook* hook = nullptr) {
-  const S T = y[0];
-  const S invT = 1.0 / T;
-  S sumYW(0.0), cpm(0.0);
+  const double T = y[0];
+  const double invT = 1.0 / T;
+  double sumYW = 0.0, cpm = 0.0;
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     const double* a = mv.sp + SP_REC * k + 2;
-    const S cpk = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4])));
+    const double cpk = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4])));
     sumYW += y[1 + k] * mv.sp[SP_REC * k + 1];
     cpm += y[1 + k] * cpk * mv.sp[SP_REC * k + 1];
   }
-  // the rates in fixed point (rate_fixed) for the plain evaluation
+  // the rates in fixed point (rate_fixed) where it covers the state
   FixState fst;
-  bool fixed = false;
-  if constexpr (sizeof(S) == sizeof(double)) {
-    fixed = fixed_covers(mv, T) && rcp_in_range(sumYW) && rcp_in_range(pc);
-    if (fixed) fst = fix_state(T, invT);
-  }
-  S lnT(0.0);
-  if (!fixed) lnT = fast_log(T);
+  const bool fixed = fixed_covers(mv, T) && rcp_in_range(sumYW) && rcp_in_range(pc);
+  double lnT = 0.0;
+  if (fixed) fst = fix_state(T, invT);
+  else lnT = fast_log(T);
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     const double* a = mv.sp + SP_REC * k + 2;
     const double* ah = mv.sp + SP_REC * k + SP_H;  // a2/2 .. a5/5
-    const S hk = a[0] + T * (ah[0] + T * (ah[1] + T * (ah[2] + T * ah[3]))) + a[5] * invT;
+    const double hk = a[0] + T * (ah[0] + T * (ah[1] + T * (ah[2] + T * ah[3]))) + a[5] * invT;
     hRT[k] = hk;
     if (fixed) {
-      if constexpr (sizeof(S) == sizeof(double))
-        gRT[k] = __longlong_as_double(fix_gibbs(mv.fix + mv.fg + 7 * k, fst));
+      gRT[k] = __longlong_as_double(fix_gibbs(mv.fix + mv.fg + 7 * k, fst));
     } else {
       const double* as = mv.sp + SP_REC * k + SP_S;  // a3/2 .. a5/4
-      const S sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
+      const double sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
       gRT[k] = hk - sk;
     }
   }
   cpm = cpm * RU;
-  const S rho = pc * invT / (RU * sumYW);
-  const S invrho = 1.0 / rho;
-  const S invcp = 1.0 / cpm;
+  const double rho = pc * invT / (RU * sumYW);
+  const double invrho = 1.0 / rho;
+  const double invcp = 1.0 / cpm;
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     C[k] = rho * y[1 + k] * mv.sp[SP_REC * k + 1];
-    wdot[k] = S(0.0);
-    v[k] = S(0.0);
-    const S ck = -(invcp * (RU * T) * hRT[k] * mv.sp[SP_REC * k + 1]);
+    wdot[k] = 0.0;
+    v[k] = 0.0;
+    const double ck = -(invcp * (RU * T) * hRT[k] * mv.sp[SP_REC * k + 1]);
     sig[k] = mv.sp[SP_REC * k] * (r[1 + k] + r[0] * ck);
   }
   if (hook && hook->mode) {
 #pragma unroll
     for (int k = 0; k < NS; ++k) {
-      const S Hk = RU * T * hRT[k];
-      S uk;
+      const double Hk = RU * T * hRT[k];
+      double uk;
       if (hook->mode == 1) uk = (mv.sp[SP_REC * k] * r[1 + k] - r[0] * Hk * invcp) * invrho;
       else uk = -0.1 * hook->g * Hk;
-      u_store(*hook, k, uk);
+      hook->u[k] = uk;
     }
   }
-  S vT(0.0);
-  const S lnP0RT = LOG_PSTD_RU - lnT;
+  double vT = 0.0;
+  const double lnP0RT = LOG_PSTD_RU - lnT;
   for (int j = 0; j < mv.M; ++j) {
-    RateOutT<S> ro;
+    RateOut ro;
     if (fixed) {
-      if constexpr (sizeof(S) == sizeof(double))
-        rate_fixed<NS, true>(mv, j, mv.rx + RX_REC * j, NS, T, invT, fst, C, gRT, hRT, ro);
+      rate_fixed<NS, true>(mv, j, mv.rx + RX_REC * j, NS, T, invT, fst, C, gRT, hRT, ro);
     } else {
       rate_one<NS, true>(mv, mv.rx + RX_REC * j, NS, T, lnT, invT, lnP0RT, C, gRT, hRT, ro);
     }
     if (!ro.active) continue;
     const RxMeta mt = ro.mt;
     const int nr = mt.nrnp & 15, np = mt.nrnp >> 4;
-    const S q = ro.q;
+    const double q = ro.q;
     wdot[mt.reac[0]] -= q;
     if (nr > 1) wdot[mt.reac[1]] -= q;
     if (nr > 2) wdot[mt.reac[2]] -= q;
@@ -766,20 +746,20 @@ __device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, co
     if (np > 1) wdot[mt.prod[1]] += q;
     if (np > 2) wdot[mt.prod[2]] += q;
     if (hook && hook->mode) {
-      S w = u_load(*hook, mt.prod[0], q) - u_load(*hook, mt.reac[0], q);
-      if (np > 1) w += u_load(*hook, mt.prod[1], q);
-      if (np > 2) w += u_load(*hook, mt.prod[2], q);
-      if (nr > 1) w -= u_load(*hook, mt.reac[1], q);
-      if (nr > 2) w -= u_load(*hook, mt.reac[2], q);
-      th_add(*hook, j, q * w);
+      double w = hook->u[mt.prod[0]] - hook->u[mt.reac[0]];
+      if (np > 1) w += hook->u[mt.prod[1]];
+      if (np > 2) w += hook->u[mt.prod[2]];
+      if (nr > 1) w -= hook->u[mt.reac[1]];
+      if (nr > 2) w -= hook->u[mt.reac[2]];
+      hook->th[j] += q * w;
     }
-    S w = sig[mt.prod[0]] - sig[mt.reac[0]];
+    double w = sig[mt.prod[0]] - sig[mt.reac[0]];
     if (np > 1) w += sig[mt.prod[1]];
     if (np > 2) w += sig[mt.prod[2]];
     if (nr > 1) w -= sig[mt.reac[1]];
     if (nr > 2) w -= sig[mt.reac[2]];
     vT += w * ro.dqdT;
-    const S wf = w * ro.fk, wr = w * ro.rk;
+    const double wf = w * ro.fk, wr = w * ro.rk;
     v[mt.reac[0]] += wf * (ro.cr[1] * ro.cr[2]);
     if (nr > 1) v[mt.reac[1]] += wf * (ro.cr[0] * ro.cr[2]);
     if (nr > 2) v[mt.reac[2]] += wf * (ro.cr[0] * ro.cr[1]);
@@ -789,7 +769,7 @@ __device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, co
     const int type = mt.flags & 3;
     if (type != 0) {
       const double* ef = mv.eff + NS * ro.sl.eff;
-      const S wM = w * ro.dqdM;
+      const double wM = w * ro.dqdM;
 #pragma unroll
       for (int l = 0; l < NS; ++l) v[l] += wM * ef[l];
     }
@@ -801,7 +781,7 @@ __device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, co
     const double* a = mv.sp + SP_REC * k + 2;
     cpR[k] = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4])));
   }
-  S Hw(0.0), sw(0.0), svc(0.0);
+  double Hw = 0.0, sw = 0.0, svc = 0.0;
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     Hw += hRT[k] * wdot[k];
@@ -812,7 +792,7 @@ __device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, co
 #pragma unroll
   for (int k = 0; k < NS; ++k) f[1 + k] = mv.sp[SP_REC * k] * wdot[k] * invrho;
   f[0] = -(Hw * invrho * invcp);
-  S dcp(0.0), cpf(0.0);
+  double dcp = 0.0, cpf = 0.0;
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
     const double* a = mv.sp + SP_REC * k + 2;
@@ -822,15 +802,271 @@ __device__ __forceinline__ void eval_vjp(const MechView& mv, const double pc, co
   }
   dcp = dcp * RU;
   cpf = cpf * RU;
-  const S D = sw - svc;
-  const S Wbar = 1.0 / sumYW;
+  const double D = sw - svc;
+  const double Wbar = 1.0 / sumYW;
   b[0] = invrho * (vT + invT * D) - r[0] * (invcp * (cpf + f[0] * dcp));
-  const S DW = Wbar * invrho * D;
-  const S fcp = r[0] * f[0] * invcp * RU;
+  const double DW = Wbar * invrho * D;
+  const double fcp = r[0] * f[0] * invcp * RU;
 #pragma unroll
   for (int i = 0; i < NS; ++i) {
     const double iWi = mv.sp[SP_REC * i + 1];
     b[1 + i] = (v[i] + DW) * iWi - fcp * cpR[i] * iWi;
+  }
+}
+
+// The second-derivative terms of the reverse sweep over one Rosenbrock step:
+//   b += grad_y G,  th_j += dG/d ln A_j,  G(y) = sum_s r_s . J(y) K_s
+// (J = df/dy, r_s the stages' cotangents): d/de [J(y + e K_s)^T r_s] summed over
+// the stages, since both are the second derivatives of f contracted with r_s and
+// K_s.  All stages act on J at the same y, so one pass over the reactions does:
+//   r_s . f = sum_k u_k wdot_k,  u_k = (W_k r_k - r_T H_k / cp) / rho,
+//   G = sum_j [q_T z_T + sum_l q_{C_l} z_l] - sum_k omega_k wdot_k
+//       - (A1 Hc / cp + f_T rho A2 / cp) / rho
+// with z_j = sum_k nu_kj Z_k, Z_k = sum_s u_k (K_T, dC_1 .. dC_N), dC the change of
+// the concentrations along K (dC_l = rho K_l / W_l + C_l theta, theta = -(K_T/T +
+// S_K/S), S = sum Y_l/W_l), omega_k = sum_s u_k theta, A1 = sum_s r_T K_T,
+// A2 = sum_s r_T dcp, Hc = sum_k wdot_k Cp_k.  Per reaction: q and its first
+// derivatives as Duals along z_j, whose derivative halves are the gradient of
+// q_T z_T + sum q_C z_C.  A Dual evaluation per stage (six per step, each with
+// every exponential and every species sum in Duals) took two thirds of the sweep:
+// gradients of 65536 cells, 25 reactions, with the integration 9.57 -> 6.44 ms.
+// K: element i of stage s at K[s n + i]; R likewise.  v, wdot, ...: scratch of NS.
+template <int NS, class KView>
+__device__ __forceinline__ void second_order(const MechView& mv, const double pc, const double (&y)[NS + 1], int ns,
+                                             const KView& K, const SV& R, double (&b)[NS + 1], SV C, SV wdot, SV gRT,
+                                             SV hRT, SV cpR, SV v, SV th) {
+  constexpr int n = NS + 1, ZC = n + 1;  // a row of Z: z_T, z_1 .. z_N, omega
+  const double T = y[0], invT = 1.0 / T, lnT = fast_log(T), lnP0RT = LOG_PSTD_RU - lnT;
+  double S = 0.0, cp = 0.0, dcp = 0.0;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const double* a = mv.sp + SP_REC * k + 2;
+    const double* ah = mv.sp + SP_REC * k + SP_H;
+    const double* as = mv.sp + SP_REC * k + SP_S;
+    const double iW = mv.sp[SP_REC * k + 1];
+    const double cpk = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4])));
+    const double hk = a[0] + T * (ah[0] + T * (ah[1] + T * (ah[2] + T * ah[3]))) + a[5] * invT;
+    const double sk = a[0] * lnT + T * (a[1] + T * (as[0] + T * (as[1] + T * as[2]))) + a[6];
+    cpR[k] = cpk;
+    hRT[k] = hk;
+    gRT[k] = hk - sk;
+    S += y[1 + k] * iW;
+    cp += y[1 + k] * cpk * iW;
+    dcp += y[1 + k] * (a[1] + T * (2.0 * a[2] + T * (3.0 * a[3] + T * 4.0 * a[4]))) * iW;
+  }
+  cp *= RU;
+  dcp *= RU;
+  const double invS = 1.0 / S, rho = pc * invT / (RU * S), vol = 1.0 / rho, icp = 1.0 / cp, RT = RU * T;
+  double Z[NS * ZC], t[NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    C[k] = rho * y[1 + k] * mv.sp[SP_REC * k + 1];
+    wdot[k] = 0.0;
+    v[k] = 0.0;
+    t[k] = 0.0;
+  }
+#pragma unroll 1
+  for (int i = 0; i < NS * ZC; ++i) Z[i] = 0.0;
+  double A1 = 0.0, A2 = 0.0, A3 = 0.0;
+#pragma unroll 1
+  for (int s = 0; s < ns; ++s) {
+    const double KT = K[s * n], rT = R[s * n];
+    double X[NS], SK = 0.0, dc = 0.0;
+#pragma unroll
+    for (int l = 0; l < NS; ++l) {
+      X[l] = K[s * n + 1 + l] * mv.sp[SP_REC * l + 1];
+      SK += X[l];
+      dc += X[l] * cpR[l];
+    }
+    const double theta = -(KT * invT + SK * invS);
+    A1 += rT * KT;
+    A2 += rT * (RU * dc + KT * dcp);
+    A3 += rT * theta;
+#pragma unroll
+    for (int l = 0; l < NS; ++l) {
+      X[l] = rho * X[l] + C[l] * theta;
+      t[l] += rT * X[l];
+    }
+    const double rH = rT * RT * icp;
+#pragma unroll 1
+    for (int k = 0; k < NS; ++k) {
+      const double u = vol * (mv.sp[SP_REC * k] * R[s * n + 1 + k] - rH * hRT[k]);
+      double* z = Z + k * ZC;
+      z[0] += u * KT;
+#pragma unroll
+      for (int l = 0; l < NS; ++l) z[1 + l] += u * X[l];
+      z[n] += u * theta;
+    }
+  }
+  // weights of q_j's own derivatives from the terms with wdot: sum nu (cA cpR + cB hRT) - omega_j
+  const double cA = -vol * icp * A1 * RU, cB = vol * icp * icp * A2 * RT;
+  double G1T = 0.0, kw = 0.0, kT = 0.0, Q1 = 0.0, Q2 = 0.0, gT = 0.0;
+#pragma unroll 1
+  for (int j = 0; j < mv.M; ++j) {
+    const double* rx = mv.rx + RX_REC * j;
+    RxIn<double> g;
+    rate_gather<NS, true>(mv, rx, NS, C, gRT, hRT, g);
+    if (g.lnA == -INFINITY) continue;
+    const RxMeta mt = g.mt;
+    const int nr = mt.nrnp & 15, np = mt.nrnp >> 4, type = mt.flags & 3, dnu = np - nr;
+    auto col = [&](int m) {
+      double z = Z[mt.prod[0] * ZC + m] - Z[mt.reac[0] * ZC + m];
+      if (np > 1) z += Z[mt.prod[1] * ZC + m];
+      if (np > 2) z += Z[mt.prod[2] * ZC + m];
+      if (nr > 1) z -= Z[mt.reac[1] * ZC + m];
+      if (nr > 2) z -= Z[mt.reac[2] * ZC + m];
+      return z;
+    };
+    double scp = cpR[mt.prod[0]] - cpR[mt.reac[0]];
+    if (np > 1) scp += cpR[mt.prod[1]];
+    if (np > 2) scp += cpR[mt.prod[2]];
+    if (nr > 1) scp -= cpR[mt.reac[1]];
+    if (nr > 2) scp -= cpR[mt.reac[2]];
+    const double zT = col(0), om = col(n), gw = cA * scp + cB * g.sh;
+    Dual Mc(1.0), cr[3], cpd[3];
+    double Mt = 0.0;
+    const double* ef = nullptr;
+    if (type != 0) {
+      ef = mv.eff + NS * load_slots(rx).eff;
+      Mc = Dual(g.Mc);
+#pragma unroll 1
+      for (int l = 0; l < NS; ++l) {
+        Mc.d += ef[l] * col(1 + l);
+        Mt += ef[l] * t[l];
+      }
+    }
+    cr[0] = Dual(g.cr[0], col(1 + mt.reac[0]));
+    cpd[0] = Dual(g.cp[0], col(1 + mt.prod[0]));
+    cr[1] = cr[2] = cpd[1] = cpd[2] = Dual(1.0);
+    if (nr > 1) cr[1] = Dual(g.cr[1], col(1 + mt.reac[1]));
+    if (nr > 2) cr[2] = Dual(g.cr[2], col(1 + mt.reac[2]));
+    if (np > 1) cpd[1] = Dual(g.cp[1], col(1 + mt.prod[1]));
+    if (np > 2) cpd[2] = Dual(g.cp[2], col(1 + mt.prod[2]));
+    Dual fk, rk, qT, qM(0.0), q;
+    double dl = 0.0, dlr = 0.0, ddl = 0.0, ddlr = 0.0;
+    if (type == 2) {
+      RxIn<Dual> gd;
+      gd.lnA = g.lnA;
+      gd.beta = g.beta;
+      gd.EaR = g.EaR;
+      gd.mt = mt;
+      gd.sl = g.sl;
+      for (int i = 0; i < 3; ++i) {
+        gd.cr[i] = cr[i];
+        gd.cp[i] = cpd[i];
+      }
+      gd.sg = Dual(g.sg, -g.sh * invT * zT);
+      gd.sh = Dual(g.sh, (scp - g.sh) * invT * zT);
+      gd.Mc = Mc;
+      RateOutT<Dual> ro;
+      rate_compute<NS, true>(mv, gd, Dual(T, zT), Dual(lnT, zT * invT), Dual(invT, -zT * invT * invT),
+                             Dual(lnP0RT, -zT * invT), ro);
+      if (!ro.active) continue;
+      fk = ro.fk;
+      rk = ro.rk;
+      qT = ro.dqdT;
+      qM = ro.dqdM;
+    } else {
+      const double lnkf = g.lnA + g.beta * lnT - g.EaR * invT;
+      double kf, kr;
+      exp_pair(lnkf, lnkf + (dnu == 0 ? g.sg : g.sg - (double)dnu * lnP0RT), kf, kr);
+      if ((mt.flags & 4) == 0) kr = 0.0;
+      // d ln k / dT of both directions and their derivatives
+      const double e = g.EaR * invT, i2 = invT * invT;
+      dl = (g.beta + e) * invT;
+      ddl = -(g.beta + 2.0 * e) * i2;
+      dlr = dl - (g.sh - (double)dnu) * invT;
+      ddlr = ddl - (scp - 2.0 * g.sh + (double)dnu) * i2;
+      fk = Dual(kf, kf * (dl * zT));
+      rk = Dual(kr, kr * (dlr * zT));
+    }
+    // the derivatives by the concentrations, and both directions' rates
+    Dual xr[3], xp[3];
+    auto side = [](int m, const Dual& k, const Dual (&c)[3], Dual (&x)[3]) {
+      if (m == 1) {
+        x[0] = k;
+      } else if (m == 2) {
+        x[0] = k * c[1];
+        x[1] = k * c[0];
+      } else {
+        x[0] = k * (c[1] * c[2]);
+        x[1] = k * (c[0] * c[2]);
+        x[2] = k * (c[0] * c[1]);
+      }
+      return x[0] * c[0];
+    };
+    Dual F = side(nr, fk, cr, xr), B = side(np, rk, cpd, xp);
+    if (type == 1) {
+      qM = F - B;
+      F *= Mc;
+      B *= Mc;
+      for (int i = 0; i < 3; ++i) {
+        if (i < nr) xr[i] *= Mc;
+        if (i < np) xp[i] *= Mc;
+      }
+    }
+    q = F - B;
+    if (type != 2) qT = Dual(dl * F.v - dlr * B.v, dl * F.d - dlr * B.d + zT * (ddl * F.v - ddlr * B.v));
+    double e = A1 * qT.v + Mt * qM.v, d = (double)nr * F.v - (double)np * B.v + qM.v * Mc.v;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if (i < nr) {
+        v[mt.reac[i]] += xr[i].d + gw * xr[i].v;
+        wdot[mt.reac[i]] -= q.v;
+        e += t[mt.reac[i]] * xr[i].v;
+      }
+      if (i < np) {
+        v[mt.prod[i]] -= xp[i].d + gw * xp[i].v;
+        wdot[mt.prod[i]] += q.v;
+        e -= t[mt.prod[i]] * xp[i].v;
+      }
+    }
+    if (type != 0) {
+      const double m = qM.d + gw * qM.v;
+#pragma unroll
+      for (int l = 0; l < NS; ++l) v[l] += m * ef[l];
+    }
+    gT += qT.d + qT.v * (gw - om);
+    th[j] += q.d + q.v * (gw - om);
+    G1T += qT.v * zT;
+    kw += om * d;
+    kT += zT * d;
+    Q1 += g.sh * e;
+    Q2 += scp * e;
+  }
+  Q1 *= RT;
+  Q2 *= RU;
+  double Hw = 0.0, Hc = 0.0, Hcc = 0.0, Ww = 0.0, WZ = 0.0, D = 0.0, dA2 = 0.0;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const double* a = mv.sp + SP_REC * k + 2;
+    const double iW = mv.sp[SP_REC * k + 1], w = wdot[k];
+    const double c1 = a[1] + T * (2.0 * a[2] + T * (3.0 * a[3] + T * 4.0 * a[4]));
+    const double c2 = 2.0 * a[2] + T * (6.0 * a[3] + T * 12.0 * a[4]);
+    Hw += hRT[k] * w;
+    Hc += cpR[k] * w;
+    Hcc += c1 * w;
+    Ww += Z[k * ZC + n] * w;
+    WZ += Z[k * ZC] * w;
+    D += v[k] * C[k];
+    dA2 += (t[k] - C[k] * A3) * vol * c1 + A1 * y[1 + k] * c2 * iW;
+  }
+  Hw *= RT;
+  Hc *= RU;
+  Hcc *= RU;
+  dA2 *= RU;
+  const double vi = vol * icp, vii = vi * icp;
+  const double Gb = -vi * A1 * Hc, Gc = vii * A2 * Hw;
+  const double Pv = G1T + kw - Ww + Gb + Gc - D;  // times d ln vol
+  const double Pc = vii * (Q1 - A3 * Hw) - icp * (Gb + 2.0 * Gc);
+  const double th1 = invT * (kT - WZ);
+  b[0] += Pv * invT + Pc * dcp + invT * th1 + gT + vi * (A3 * Hc - Q2 - A1 * Hcc) + vii * (A2 * Hc + Hw * dA2);
+  const double Py = (Pv - (kw - Ww) - th1) * invS, H1 = vii * Hw * A1;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const double* a = mv.sp + SP_REC * k + 2;
+    const double c1 = a[1] + T * (2.0 * a[2] + T * (3.0 * a[3] + T * 4.0 * a[4]));
+    b[1 + k] += mv.sp[SP_REC * k + 1] * (Py + rho * v[k] + RU * (Pc * cpR[k] + H1 * c1));
   }
 }
 
