@@ -22,18 +22,24 @@ struct PV {
   __device__ __forceinline__ double& operator[](int i) const { return p[i]; }
 };
 
-// per-warp workspace layout (offsets in doubles)
+// per-warp workspace layout (offsets in doubles); qJ: the rates of progress of an
+// evaluation with J
 struct WarpWS {
-  int y, ys, f, wdot, C, gRT, hRT, q, fk, rk, dT, dM, J, K, piv, total;
+  int y, ys, f, wdot, C, gRT, hRT, q, qJ, fk, rk, dT, dM, J, K, piv, total;
 };
 
-// Seven cells of the 50-species mechanism fit an SM where six did with one
-// slot per quantity: the production rates share the g/RT slots (the rates
+// The fewer doubles a cell takes, the more cells an SM holds (one warp each, two on
+// every FP64 pipe with eight).  The production rates share the g/RT slots (the rates
 // read g/RT before the per-species sums write the production rates, and the
-// temperature row reuses the slots after the last read of the production
-// rates); d q / d[M] has one slot per third-body reaction; d q / dT lives in
-// the stage vectors while the Jacobian is built (no stage vector is live
-// then) where they have room; cp/R is recomputed where it is needed.
+// temperature row reuses the slots after the last read of the production rates);
+// d q / d[M] has one slot per third-body reaction; cp/R is recomputed where it is
+// needed.  While the Jacobian is evaluated no factors and no stage vectors are live:
+// q and d q / dT, read by the species sums before the first entry of J is written,
+// lie in J's own storage, and the rate factors of the two directions in the slots of
+// the stage vectors and of the plain evaluations' q, where those have room.  50
+// species, 300 reactions: 3515 doubles, eight cells per SM; with slots of their own
+// for the rates 4115 and seven.  8192 cells, with warp_solve in
+// registers: 141.7 -> 126.4 ms.
 __host__ __device__ inline WarpWS warp_ws_layout(int N, int M, int n_eff) {
   const int n = N + 1;
   WarpWS w;
@@ -45,8 +51,6 @@ __host__ __device__ inline WarpWS warp_ws_layout(int N, int M, int n_eff) {
   w.wdot = w.gRT;
   w.hRT = o; o += N;
   w.q = o; o += M;
-  w.fk = o; o += M;
-  w.rk = o; o += M;
   w.dM = o; o += n_eff > 0 ? n_eff : 1;
   w.J = o; o += n * n;
   w.K = o; o += 6 * n;
@@ -54,11 +58,19 @@ __host__ __device__ inline WarpWS warp_ws_layout(int N, int M, int n_eff) {
   // before that stage vector is written, and the candidate state overwrites
   // it element by element after each lane has read its own elements
   w.ys = w.K + 5 * n;
-  if (M <= 6 * n) {
-    w.dT = w.K;
+  w.qJ = w.q;
+  if (2 * M <= n * n) {
+    w.qJ = w.J;
+    w.dT = w.J + M;
+    w.fk = w.q;
   } else {
-    w.dT = o;
-    o += M;
+    w.dT = o; o += M;
+    w.fk = o; o += M;
+  }
+  if (M <= 6 * n) {
+    w.rk = w.K;
+  } else {
+    w.rk = o; o += M;
   }
   w.piv = o; o += (n + 1) / 2;  // ints, two per double slot
   w.total = (o + 1) & ~1;
@@ -128,17 +140,18 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
   }
   // third-body [M] = sum_l C_l + the sparse corrections (eps_l - 1) C_l; the
   // table follows the species lists and the lane assignment in csr
-  const int* effs = csr + N + 1 + 2 * csr[N] + 64;
+  const int* effs = csr + 2 * N + 1 + 2 * csr[N] + 64;
   const SparseEff se{effs + 1, effs + 2 + effs[0], warp_sum(cs)};
   __syncwarp();
   const double lnP0RT = LOG_PSTD_RU - lnT;
   // reactions: one lane per reaction
+  const int qo = WITH_J ? L.qJ : L.q;
   for (int j = lane; j < mv.M; j += 32) {
     RateOut ro;
     if (fixed) rate_fixed<0, WITH_J>(mv, j, mv.rx + RX_REC * j, N, T, invT, fst, C, gRT, hRT, ro, &se);
     else rate_one<0, WITH_J>(mv, mv.rx + RX_REC * j, N, T, lnT, invT, lnP0RT, C, gRT, hRT, ro, &se);
     if (ro.active) {
-      ws[L.q + j] = ro.q;
+      ws[qo + j] = ro.q;
       if (WITH_J) {
         ws[L.fk + j] = ro.fk;
         ws[L.rk + j] = ro.rk;
@@ -146,7 +159,7 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
         if ((ro.mt.flags & 3) != 0) ws[L.dM + ro.sl.eff] = ro.dqdM;
       }
     } else {
-      ws[L.q + j] = 0.0;
+      ws[qo + j] = 0.0;
       if (WITH_J) {
         ws[L.fk + j] = 0.0;
         ws[L.rk + j] = 0.0;
@@ -166,20 +179,33 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
   const int ba = ka >= 0 ? csr[ka] : 0, la = ka >= 0 ? csr[ka + 1] - ba : 0;
   const int bb = kb >= 0 ? csr[kb] : 0, lb = kb >= 0 ? csr[kb + 1] - bb : 0;
   double cpp = 0.0, hwp = 0.0;
+  double ja = 0.0, jb = 0.0;  // with J: the rows' sums of d q / dT
   {
     // one running sum, one multiply-add per entry: the first list's sum is
     // set aside where the second list starts
-    double acc = 0.0, wa = 0.0, wb = 0.0;
+    double acc = 0.0, wa = 0.0, wb = 0.0, jac = 0.0;
     for (int t = 0; t < la + lb; ++t) {
       if (t == la) {
         wa = acc;
         acc = 0.0;
+        if (WITH_J) {
+          ja = jac;
+          jac = 0.0;
+        }
       }
       const int e = t < la ? ba + t : bb + (t - la);
-      acc = fma(small_int_to_double(csr[N + 2 + 2 * e]), ws[L.q + csr[N + 1 + 2 * e]], acc);
+      const int j = csr[N + 1 + 2 * e];
+      const double nu = small_int_to_double(csr[N + 2 + 2 * e]);
+      acc = fma(nu, ws[qo + j], acc);
+      if (WITH_J) jac = fma(nu, ws[L.dT + j], jac);
     }
-    if (lb > 0) wb = acc;
-    else wa = acc;
+    if (lb > 0) {
+      wb = acc;
+      jb = jac;
+    } else {
+      wa = acc;
+      ja = jac;
+    }
     if (ka >= 0) {
       wdot[ka] = wa;
       cpp += y[1 + ka] * (cp_species(mv, ka, T) - EV) * mv.sp[SP_REC * ka + 1];
@@ -203,14 +229,11 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
     double* J = ws + L.J;
     // concentration-space rows of this lane's species: one loop over the
     // concatenation of their reaction lists (as for the production rates)
+    // (the sums above read the last of q and d q / dT before the first entry is written)
     if (ka >= 0)
-      for (int c = 0; c < n; ++c) J[(1 + ka) * n + c] = 0.0;
+      for (int c = 0; c < n; ++c) J[(1 + ka) * n + c] = c == 0 ? ja : 0.0;
     if (kb >= 0)
-      for (int c = 0; c < n; ++c) J[(1 + kb) * n + c] = 0.0;
-    // collider columns d q_j / d[M] eps_l: the unit part summed per row (sMa,
-    // sMb; added to every species column in the conversion below), the
-    // corrections eps_l - 1 entered where the efficiency is not 1
-    double sMa = 0.0, sMb = 0.0;
+      for (int c = 0; c < n; ++c) J[(1 + kb) * n + c] = c == 0 ? jb : 0.0;
     for (int t = 0; t < la + lb; ++t) {
       const bool first = t < la;
       const int e = first ? ba + t : bb + (t - la);
@@ -221,7 +244,6 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
         const double* r = mv.rx + RX_REC * j;
         const RxMeta mt = load_meta(r);
         const int nr = mt.nrnp & 15, np = mt.nrnp >> 4;
-        row[0] += nu * ws[L.dT + j];
         // nu fk c c' and -nu rk c c' as unpacked products (Fx): one FP64 addition
         // per entry instead of three multiplications and an addition
         auto side = [&](double k, const uint8_t* sp, int cnt, uint32_t sign) {
@@ -239,16 +261,29 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
         };
         side(ws[L.fk + j], mt.reac, nr, 0u);
         side(ws[L.rk + j], mt.prod, np, 0x80000000u);
-        if ((mt.flags & 3) != 0) {
-          const int sl = load_slots(r).eff;
-          const double cM = nu * ws[L.dM + sl];
-          if (first) sMa += cM;
-          else sMb += cM;
-          for (int u = se.off[sl]; u < se.off[sl + 1]; ++u) {
-            const int* q = se.ent + 3 * u;
-            row[1 + q[0]] += cM * __hiloint2double(q[2], q[1]);
-          }
-        }
+      }
+    }
+    // collider columns d q_j / d[M] eps_l: the unit part summed per row (sMa,
+    // sMb; added to every species column in the conversion below), the
+    // corrections eps_l - 1 entered where the efficiency is not 1.  A loop of its
+    // own over the third-body entries, which lead each list: inside the loop above
+    // nearly every round had some lane with one (30 of 300 reactions), and the
+    // other lanes waited for its corrections.  187k -> 150k cycles per Jacobian;
+    // 126.4 -> 120.1 ms.
+    double sMa = 0.0, sMb = 0.0;
+    const int* ntb = csr + N + 1 + 2 * csr[N] + 64;  // third-body entries of each list
+    const int ta = ka >= 0 ? ntb[ka] : 0, tb = kb >= 0 ? ntb[kb] : 0;
+    for (int t = 0; t < ta + tb; ++t) {
+      const bool first = t < ta;
+      const int e = first ? ba + t : bb + (t - ta);
+      double* row = J + (1 + (first ? ka : kb)) * n;
+      const int sl = load_slots(mv.rx + RX_REC * csr[N + 1 + 2 * e]).eff;
+      const double cM = small_int_to_double(csr[N + 2 + 2 * e]) * ws[L.dM + sl];
+      if (first) sMa += cM;
+      else sMb += cM;
+      for (int u = se.off[sl]; u < se.off[sl + 1]; ++u) {
+        const int* q = se.ent + 3 * u;
+        row[1 + q[0]] += cM * __hiloint2double(q[2], q[1]);
       }
     }
     // -> (T, Y) space, row by row
@@ -299,16 +334,18 @@ __device__ double warp_eval(const MechView& mv, const int* csr, int N, double pc
 }
 
 // LU with partial pivoting of the n x n row-major matrix A (shared memory),
-// whole rows swapped, reciprocal pivots on the diagonal, and the columns of U
+// whole rows swapped (perm[i]: the row of A that became row i), reciprocal pivots on the diagonal, and the columns of U
 // above the diagonal divided by their pivot (U'_ik = U_ik / U_kk, for the
 // back substitution of warp_solve).  Returns false if a pivot is zero or not
 // finite.  The pivot search compares the magnitudes' bit patterns as 64-bit
 // integers (non-negative doubles order like their patterns), so it runs on
 // the integer pipe instead of the narrow FP64 one; a NaN sorts above every
 // finite value, is picked, and fails the finiteness test.
-__device__ bool warp_lu(double* A, int* piv, int n) {
+__device__ bool warp_lu(double* A, int* perm, int n) {
   const int lane = threadIdx.x & 31;
   bool ok = true;
+  for (int i = lane; i < n; i += 32) perm[i] = i;
+  __syncwarp();
   for (int k = 0; k < n; ++k) {
     long long best = -1;
     int bi = k;
@@ -323,7 +360,11 @@ __device__ bool warp_lu(double* A, int* piv, int n) {
       if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
     }
     ok = ok && (best > 0) && (best < 0x7FF0000000000000LL);
-    if (lane == 0) piv[k] = bi;
+    if (lane == 0) {
+      const int r = perm[k];
+      perm[k] = perm[bi];
+      perm[bi] = r;
+    }
     if (bi != k) {
       for (int j = lane; j < n; j += 32) {
         const double t = A[k * n + j];
@@ -362,35 +403,65 @@ __device__ bool warp_lu(double* A, int* piv, int n) {
   return ok;
 }
 
-// x <- A^{-1} x with the factors of warp_lu (x in shared memory)
-__device__ void warp_solve(const double* A, const int* piv, double* x, int n) {
+// x <- A^{-1} x with the factors of warp_lu (x in shared memory, n <= 96).  Lane l
+// holds x_l, x_{l+32}, x_{l+64} in registers and each step's x_k is broadcast by a
+// shuffle: the chain of a step is the shuffle and one multiply-add, with the
+// loads of A ahead of it.  Through shared memory (load, multiply-add, store and
+// two barriers per step) a solve of order 51 took 34k cycles with seven
+// cells per SM, this 28.5k with eight (two warps per FP64 pipe, which sets the rest).
+__device__ void warp_solve(const double* A, const int* perm, double* x, int n) {
   const int lane = threadIdx.x & 31;
-  if (lane == 0) {
-    for (int k = 0; k < n; ++k) {
-      const int p = piv[k];
-      if (p != k) {
-        const double t = x[k];
-        x[k] = x[p];
-        x[p] = t;
-      }
-    }
+  const int r0 = lane, r1 = lane + 32, r2 = lane + 64;
+  double x0 = r0 < n ? x[perm[r0]] : 0.0, x1 = r1 < n ? x[perm[r1]] : 0.0, x2 = r2 < n ? x[perm[r2]] : 0.0;
+  const double *a0 = A + min(r0, n - 1) * n, *a1 = A + min(r1, n - 1) * n, *a2 = A + min(r2, n - 1) * n;
+  const int n0 = min(n, 32), n1 = min(n, 64);
+  // L, column by column; rows past n keep harmless values (never read or stored)
+#pragma unroll 4
+  for (int k = 0; k < n0; ++k) {
+    const double xk = __shfl_sync(WFULL, x0, k);
+    const double u0 = x0 - a0[k] * xk;
+    if (lane > k) x0 = u0;
+    if (n > 32) x1 -= a1[k] * xk;
+    if (n > 64) x2 -= a2[k] * xk;
   }
-  __syncwarp();
-  for (int k = 0; k < n; ++k) {
-    const double xk = x[k];
-    __syncwarp();
-    for (int i = k + 1 + lane; i < n; i += 32) x[i] -= A[i * n + k] * xk;
-    __syncwarp();
+#pragma unroll 4
+  for (int k = 32; k < n1; ++k) {
+    const double xk = __shfl_sync(WFULL, x1, k - 32);
+    const double u1 = x1 - a1[k] * xk;
+    if (r1 > k) x1 = u1;
+    if (n > 64) x2 -= a2[k] * xk;
+  }
+  for (int k = 64; k < n; ++k) {
+    const double xk = __shfl_sync(WFULL, x2, k - 64);
+    const double u2 = x2 - a2[k] * xk;
+    if (r2 > k) x2 = u2;
   }
   // back substitution on b~ (x_k = b~_k / U_kk): b~_i -= U'_ik b~_k for i < k,
   // with U' = U scaled by its column pivots, then one scaling pass
-  for (int k = n - 1; k > 0; --k) {
-    const double bk = x[k];
-    __syncwarp();
-    for (int i = lane; i < k; i += 32) x[i] -= A[i * n + k] * bk;
-    __syncwarp();
+  for (int k = n - 1; k >= 64; --k) {
+    const double xk = __shfl_sync(WFULL, x2, k - 64);
+    const double u2 = x2 - a2[k] * xk;
+    if (r2 < k) x2 = u2;
+    x0 -= a0[k] * xk;
+    x1 -= a1[k] * xk;
   }
-  for (int i = lane; i < n; i += 32) x[i] *= A[i * n + i];
+#pragma unroll 4
+  for (int k = n1 - 1; k >= 32; --k) {
+    const double xk = __shfl_sync(WFULL, x1, k - 32);
+    const double u1 = x1 - a1[k] * xk;
+    if (r1 < k) x1 = u1;
+    x0 -= a0[k] * xk;
+  }
+#pragma unroll 4
+  for (int k = n0 - 1; k > 0; --k) {
+    const double xk = __shfl_sync(WFULL, x0, k);
+    const double u0 = x0 - a0[k] * xk;
+    if (lane < k) x0 = u0;
+  }
+  __syncwarp();  // every lane has read x
+  if (r0 < n) x[r0] = x0 * a0[r0];
+  if (r1 < n) x[r1] = x1 * a1[r1];
+  if (r2 < n) x[r2] = x2 * a2[r2];
   __syncwarp();
 }
 

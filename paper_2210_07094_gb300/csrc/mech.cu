@@ -340,6 +340,14 @@ int parse_mechanism(const char* path, df_mech* m) {
     for (int k = 0; k < N; ++k)
       if (nu[k] != 0) lists[k].emplace_back(j, nu[k]);
   }
+  // the third-body entries lead each list (the Jacobian rows' collider columns loop over them alone)
+  std::vector<int> ntb(N);
+  for (int k = 0; k < N; ++k)
+    ntb[k] = (int)(std::stable_partition(lists[k].begin(), lists[k].end(), [&](const std::pair<int, int>& e) {
+                     RxMeta meta;
+                     memcpy(&meta, &rec[RX_REC * e.first + 3], 8);
+                     return (meta.flags & 3) != 0;
+                   }) - lists[k].begin());
   m->csr_host.assign(N + 1, 0);
   for (int k = 0; k < N; ++k) m->csr_host[k + 1] = m->csr_host[k] + (int)lists[k].size();
   for (int k = 0; k < N; ++k)
@@ -350,17 +358,11 @@ int parse_mechanism(const char* path, df_mech* m) {
   // Lane assignment of the warp path's species loops (production rates and
   // Jacobian rows): at most two species per lane, balanced by the cost of
   // their reaction lists (longest first, each to the least-loaded lane that
-  // still has a free slot).  A third-body entry adds a full row of
-  // efficiencies to the Jacobian row.  Table: 32 x (k0, k1), -1 = none.
+  // still has a free slot; a third-body entry counts twice, for its collider
+  // columns).  Table: 32 x (k0, k1), -1 = none, then the N third-body counts.
   std::vector<std::pair<long, int>> cost(N);
   for (int k = 0; k < N; ++k) {
-    long c = 0;
-    for (auto& e : lists[k]) {
-      RxMeta meta;
-      memcpy(&meta, &rec[RX_REC * e.first + 3], 8);
-      c += 13 + (((meta.flags & 3) != 0) ? N : 0);
-    }
-    cost[k] = {c, k};
+    cost[k] = {(long)lists[k].size() + ntb[k], k};
   }
   std::stable_sort(cost.begin(), cost.end(),
                    [](const std::pair<long, int>& a, const std::pair<long, int>& b) { return a.first > b.first; });
@@ -377,6 +379,7 @@ int parse_mechanism(const char* path, df_mech* m) {
     load[best] += ck.first;
   }
   m->csr_host.insert(m->csr_host.end(), asg.begin(), asg.end());
+  m->csr_host.insert(m->csr_host.end(), ntb.begin(), ntb.end());
   // Sparse third-body efficiencies for the warp path: [n_eff], offsets
   // [n_eff + 1] (in triples), then per slot the (species, low word, high word)
   // triples of eps_l - 1 for every species whose efficiency is not 1.
