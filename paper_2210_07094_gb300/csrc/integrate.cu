@@ -537,7 +537,10 @@ int integrate_warp_dispatch(df_mech* m, const IntegArgs& a0, cudaStream_t st, in
   const WarpWS L = warp_ws_layout(m->dims.N, m->dims.M, m->dims.n_eff);
   int warps, stage;
   size_t sm;
-  const int max_warps = threads > 0 ? threads / 32 : 8;
+  // fewer cells than eight per SM: over all the SMs (64 cells of 50 species in blocks of
+  // eight warps left 144 of 152 SMs idle: 27 -> 17.6 ms; a cell's arithmetic is its own)
+  const int64_t per_sm = (a0.nwork + m->num_sms - 1) / m->num_sms;
+  const int max_warps = threads > 0 ? threads / 32 : (int)std::max<int64_t>(1, std::min<int64_t>(8, per_sm));
   int rc = warp_shape(m, L, true, max_warps, &warps, &stage, &sm);
   if (rc) return rc;
   IntegArgs a = a0;
