@@ -80,6 +80,8 @@ struct df_dnn {
   cudaGraphExec_t train_exec = nullptr;
   int64_t train_n = -1;
   cudaStream_t cap_stream = nullptr;  // private stream the step is captured on
+  cudaStream_t cap_side = nullptr;    // and the one its weight gradients fork to
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool no_graph = false;              // capture unavailable here: enqueue the kernels directly
   // inference scratch (chunk rows)
   int64_t chunk = 0;
@@ -477,17 +479,65 @@ __global__ void k_set_train_scalars(float* sc, float lr, float c1, float c2) {
 // Adam (Kingma & Ba 2015, Algorithm 1) in FP32 on the master weights; the
 // coefficients beta and 1 - beta are rounded to FP32 from their FP64 values
 // (1 - (float)0.999 would be 5e-5 off 0.001)
-__global__ void k_adam(float* P, float* m1, float* m2, const float* g, int64_t n, const float* sc, float b1,
-                       float omb1, float b2, float omb2, float eps) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float lr = sc[0], c1 = sc[1], c2 = sc[2];
-  const float gi = g[i];
-  const float a = b1 * m1[i] + omb1 * gi;
-  const float b = b2 * m2[i] + omb2 * (gi * gi);
-  m1[i] = a;
-  m2[i] = b;
-  P[i] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+struct AdamArgs {
+  float *P, *m1, *m2;
+  const float* g;
+  const float* sc;
+  float b1, omb1, b2, omb2, eps;
+  DnnLayout L;
+  __nv_bfloat16 *wb[4], *wtb[4];
+  int first[6];  // first block of each layer's weights, of the biases, and the grid's size
+};
+
+__device__ __forceinline__ float adam_one(const AdamArgs& a, int64_t i, float lr, float c1, float c2) {
+  const float gi = a.g[i];
+  const float m = a.b1 * a.m1[i] + a.omb1 * gi;
+  const float v = a.b2 * a.m2[i] + a.omb2 * (gi * gi);
+  a.m1[i] = m;
+  a.m2[i] = v;
+  const float p = a.P[i] - lr * (m / c1) / (sqrtf(v / c2) + a.eps);
+  a.P[i] = p;
+  return p;
+}
+
+// Adam and the bf16 copies (see k_dnn_cast) in one launch: a block per 32 x 32 tile of
+// the four weight matrices, then 256 biases per block.  Bound by the launch and by
+// the 46 MB it moves (L2 resident between steps); the update and four casts apart
+// re-read the weights and took five launches, 31 us of a training step's nodes.
+__global__ void k_adam(AdamArgs a) {
+  __shared__ __nv_bfloat16 tile[32][33];
+  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
+  const float lr = a.sc[0], c1 = a.sc[1], c2 = a.sc[2];
+  const int b = blockIdx.x;
+  if (b >= a.first[4]) {
+    int64_t i = (int64_t)(b - a.first[4]) * 256 + ty * 32 + tx;
+    for (int l = 0; l < 4; ++l) {
+      if (i < a.L.out(l)) {
+        adam_one(a, a.L.off[2 * l + 1] + i, lr, c1, c2);
+        return;
+      }
+      i -= a.L.out(l);
+    }
+    return;
+  }
+  int l = 0;
+  while (b >= a.first[l + 1]) ++l;
+  const int out = a.L.out(l), in = a.L.in(l), nx = (in + 31) / 32;
+  const int c0 = (b - a.first[l]) % nx * 32, r0 = (b - a.first[l]) / nx * 32;
+  for (int j = ty; j < 32; j += 8) {
+    const int r = r0 + j, c = c0 + tx;
+    if (r < out && c < in) {
+      const int64_t e = (int64_t)r * in + c;
+      const __nv_bfloat16 w = __float2bfloat16_rn(adam_one(a, a.L.off[2 * l] + e, lr, c1, c2));
+      a.wb[l][e] = w;
+      tile[j][tx] = w;
+    }
+  }
+  __syncthreads();
+  for (int j = ty; j < 32; j += 8) {
+    const int c = c0 + j, r = r0 + tx;
+    if (r < out && c < in) a.wtb[l][(int64_t)c * out + r] = tile[tx][j];
+  }
 }
 
 struct PostArgs {
@@ -978,6 +1028,9 @@ void df_dnn_free(df_dnn* d) {
                   d->rawb, d->fb_flag, d->bT, d->bp, d->bY, d->bYn, d->train_sc, d->splitk_ws};
   if (d->train_exec) cudaGraphExecDestroy(d->train_exec);
   if (d->cap_stream) cudaStreamDestroy(d->cap_stream);
+  if (d->cap_side) cudaStreamDestroy(d->cap_side);
+  if (d->ev_fork) cudaEventDestroy(d->ev_fork);
+  if (d->ev_join) cudaEventDestroy(d->ev_join);
   if (d->side) cudaStreamDestroy(d->side);
   if (d->ev_ranged) cudaEventDestroy(d->ev_ranged);
   if (d->ev_fallback) cudaEventDestroy(d->ev_fallback);
@@ -1047,7 +1100,21 @@ int df_dnn_fit_norm(df_dnn* d, int64_t n, const double* T, const double* p, cons
 
 // The kernels of one forward and backward pass on the staged batch (bT, bp,
 // bY, bYn): the loss partials and the gradients (d->grads), no update.
-static int dnn_grad_enqueue(df_dnn* d, int64_t n, int64_t n_norm, cudaStream_t st) {
+// side (a stream of the same capture, or null): the weight and bias gradients and the
+// loss sum go there, beside the chain of the dZ products that st holds, and join st at
+// the end.  One after the other they were a third of the step: SMs that a product's last
+// wave leaves idle, and the small reductions' launches, then hide behind the chain.  4096 pairs:
+// 266 -> 224 us a step (with k_adam below in one launch).  The
+// split-K workspace stays with one stream at a time: st's only user of it (the output
+// layer) is ahead of the fork.
+static int dnn_grad_enqueue(df_dnn* d, int64_t n, int64_t n_norm, cudaStream_t st, cudaStream_t side = nullptr) {
+  int frc = DF_OK;
+  const cudaStream_t ws = side ? side : st;
+  auto fork = [&]() {  // ws continues from here on st
+    if (!side || frc) return;
+    frc = cuda_check(cudaEventRecord(d->ev_fork, st), "fork the gradients");
+    if (!frc) frc = cuda_check(cudaStreamWaitEvent(side, d->ev_fork, 0), "fork the gradients");
+  };
   const DnnLayout& L = d->L;
   const int64_t B = d->B;
   const int64_t M = (n + 7) / 8 * 8;  // rows used by the GEMMs (K of the weight gradients)
@@ -1087,27 +1154,34 @@ static int dnn_grad_enqueue(df_dnn* d, int64_t n, int64_t n_norm, cudaStream_t s
   if (rc) return rc;
   const int nbl = (int)((M + LOSS_ROWS - 1) / LOSS_ROWS);
   k_dnn_loss<<<nbl, LOSS_ROWS, 0, st>>>(d->U, d->tgt, n, n_norm, M, N, d->dU, d->dUT, B, d->loss_part);
-  k_sum_partials<<<1, 32, 0, st>>>(d->loss_part, nbl, d->loss_part + nbl);
+  fork();
+  k_sum_partials<<<1, 32, 0, ws>>>(d->loss_part, nbl, d->loss_part + nbl);
   // backward: layer 4
   rc = gemm(d, d->dUT, (int)B, d->HT[2], (int)B, DNN_OUT, L.w[2], (int)M, EPI_F32, nullptr, G + L.off[6], L.w[2],
-            nullptr, 0, nullptr, 0, nullptr, 0, st);
-  k_dnn_rowsum<<<DNN_OUT, 256, 0, st>>>(d->dUT, B, DNN_OUT, M, G + L.off[7]);
+            nullptr, 0, nullptr, 0, nullptr, 0, ws);
+  k_dnn_rowsum<<<DNN_OUT, 256, 0, ws>>>(d->dUT, B, DNN_OUT, M, G + L.off[7]);
   // dZ3 = (dU W4) * gelu'(Z3)
   if (!rc)
     rc = gemm(d, d->dU, 0, d->wtb[3], 0, (int)M, L.w[2], DNN_OUT, EPI_BWD_DZ, nullptr, nullptr, 0, d->dZ[2], L.w[2],
               d->dZT[2], (int)B, d->Z[2], L.w[2], st);
   for (int l = 2; l >= 0 && !rc; --l) {
+    fork();
     // weight gradient of layer l: dZ_l^T . H_{l-1}  (H_{-1} = X)
     const __nv_bfloat16* hinT = l > 0 ? d->HT[l - 1] : d->XT;
     const int in_w = L.in(l);
     rc = gemm(d, d->dZT[l], (int)B, hinT, (int)B, L.w[l], in_w, (int)M, EPI_F32, nullptr, G + L.off[2 * l], in_w,
-              nullptr, 0, nullptr, 0, nullptr, 0, st);
-    k_dnn_rowsum<<<L.w[l], 256, 0, st>>>(d->dZT[l], B, L.w[l], M, G + L.off[2 * l + 1]);
+              nullptr, 0, nullptr, 0, nullptr, 0, ws);
+    k_dnn_rowsum<<<L.w[l], 256, 0, l > 0 ? ws : st>>>(d->dZT[l], B, L.w[l], M, G + L.off[2 * l + 1]);
     if (!rc && l > 0)
       rc = gemm(d, d->dZ[l], 0, d->wtb[l], 0, (int)M, L.w[l - 1], L.w[l], EPI_BWD_DZ, nullptr, nullptr, 0,
                 d->dZ[l - 1], L.w[l - 1], d->dZT[l - 1], (int)B, d->Z[l - 1], L.w[l - 1], st);
   }
-  return cuda_check(cudaGetLastError(), "gradient kernels");
+  if (side) {  // also after an error: a capture is only ended once its streams have joined
+    const int jrc = cuda_check(cudaEventRecord(d->ev_join, side), "join the gradients");
+    if (!frc) frc = jrc ? jrc : cuda_check(cudaStreamWaitEvent(st, d->ev_join, 0), "join the gradients");
+  }
+  if (!rc) rc = frc;
+  return rc ? rc : cuda_check(cudaGetLastError(), "gradient kernels");
 }
 
 // Adam (bias-corrected, scalars of this step in train_sc) on the master
@@ -1116,16 +1190,25 @@ static int dnn_adam_enqueue(df_dnn* d, cudaStream_t st) {
   const DnnLayout& L = d->L;
   const float b1 = (float)d->o.beta1, b2 = (float)d->o.beta2;
   const float omb1 = (float)(1.0 - d->o.beta1), omb2 = (float)(1.0 - d->o.beta2);
-  k_adam<<<(unsigned)((L.total + 255) / 256), 256, 0, st>>>(d->params, d->m1, d->m2, d->grads, L.total,
-                                                             d->train_sc, b1, omb1, b2, omb2, (float)d->o.adam_eps);
+  AdamArgs a{d->params, d->m1, d->m2, d->grads, d->train_sc, b1, omb1, b2, omb2, (float)d->o.adam_eps, L, {}, {}, {}};
+  int blocks = 0, biases = 0;
+  for (int l = 0; l < 4; ++l) {
+    a.wb[l] = d->wb[l];
+    a.wtb[l] = d->wtb[l];
+    a.first[l] = blocks;
+    blocks += ((L.in(l) + 31) / 32) * ((L.out(l) + 31) / 32);
+    biases += L.out(l);
+  }
+  a.first[4] = blocks;
+  a.first[5] = blocks + (biases + 255) / 256;
+  k_adam<<<(unsigned)a.first[5], dim3(32, 8), 0, st>>>(a);
   int rc = cuda_check(cudaGetLastError(), "Adam kernel");
-  if (!rc) rc = dnn_cast_all(d, st);
   return rc;
 }
 
 // The kernels of one training step on the staged batch.
-static int dnn_train_enqueue(df_dnn* d, int64_t n, cudaStream_t st) {
-  int rc = dnn_grad_enqueue(d, n, n, st);
+static int dnn_train_enqueue(df_dnn* d, int64_t n, cudaStream_t st, cudaStream_t side = nullptr) {
+  int rc = dnn_grad_enqueue(d, n, n, st, side);
   if (!rc) rc = dnn_adam_enqueue(d, st);
   return rc;
 }
@@ -1191,13 +1274,17 @@ int df_dnn_train_step(df_dnn* d, int64_t n, const double* T, const double* p, co
     d->train_n = -1;
     if (!d->cap_stream)
       rc = cuda_check(cudaStreamCreateWithFlags(&d->cap_stream, cudaStreamNonBlocking), "capture stream");
+    if (!rc && !d->cap_side)
+      rc = cuda_check(cudaStreamCreateWithFlags(&d->cap_side, cudaStreamNonBlocking), "capture stream");
+    if (!rc && !d->ev_fork) rc = cuda_check(cudaEventCreateWithFlags(&d->ev_fork, cudaEventDisableTiming), "event");
+    if (!rc && !d->ev_join) rc = cuda_check(cudaEventCreateWithFlags(&d->ev_join, cudaEventDisableTiming), "event");
     if (rc) return rc;
     if (cudaStreamBeginCapture(d->cap_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
       cudaGetLastError();
       d->no_graph = true;  // capture unavailable: run the kernels as they are from now on
       return train_step_loss(d, n, n, dnn_train_enqueue(d, n, st), loss_out, st);
     }
-    const int erc = dnn_train_enqueue(d, n, d->cap_stream);
+    const int erc = dnn_train_enqueue(d, n, d->cap_stream, d->cap_side);
     cudaGraph_t g = nullptr;
     rc = cuda_check(cudaStreamEndCapture(d->cap_stream, &g), "end capture");
     if (erc) {
