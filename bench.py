@@ -33,26 +33,27 @@ METRIC = "cell-steps/s (9-species chemistry substep, FP64 integrator)"
 UNIT = "cell-steps/s"
 # FP64 operations per Rosenbrock substep attempt (accepted or rejected) of the
 # 9-species / 25-reaction mechanism on the thread-per-cell path: ncu's executed
-# DP thread-instruction counters (2*DFMA + DADD + DMUL = 3.6363e+10) of one timed
-# launch on the 2^20-cell field (the kernel generated for the mechanism, in the
-# autotuned 32-thread shape) divided by the 2199716 attempts that launch
-# counted.
-FLOP_PER_SUBSTEP = 16531
-# dram__bytes_read.sum + dram__bytes_write.sum of that launch (same kernel build)
-TRAFFIC_PER_LAUNCH = 231775232 + 235842048
+# DP thread-instruction counters (2*DFMA + DADD + DMUL = 2.5085e+09) of one
+# launch on 2^18 cells of the field (the kernel generated for the mechanism, in
+# 32-thread blocks) divided by the 550051 attempts that launch counted.  The
+# rates' products and exponentials run in 64-bit fixed point on the integer
+# pipes and are not in this count.
+FLOP_PER_SUBSTEP = 4560
+# dram__bytes_read.sum + dram__bytes_write.sum of the 2^20-cell launch (same kernel build)
+TRAFFIC_PER_LAUNCH = 524287232 + 530153472
 # hash of the device sources that kernel is built from, when the two counters
 # above were taken; a different hash at run time marks them stale in the line
 COUNTERS_SOURCES = ("integrate_thread.cuh", "rosenbrock.cuh", "chem_thread.cuh", "dev_common.cuh", "exp2fix.cuh",
                     "exp2fix_table.inc", "log2fix.cuh", "log2fix_table.inc", "codegen.cu")
-COUNTERS_SOURCE_HASH = "1f85abfcfe201580"
+COUNTERS_SOURCE_HASH = "3569d8b71e4f40b1"
 # the same for the 50-species one-warp-per-cell path: FP64 operations per
 # substep from ncu's DP thread-instruction counters of one launch on 8192 cells
 # of the 50-species field (2*DFMA + DADD + DMUL over its substeps), and the
 # hash of the sources of that kernel when they were taken
-FLOP_PER_SUBSTEP_50 = 352115
+FLOP_PER_SUBSTEP_50 = 248787
 COUNTERS50_SOURCES = ("integrate.cu", "chem_warp.cuh", "chem_thread.cuh", "dev_common.cuh", "exp2fix.cuh",
                       "exp2fix_table.inc", "log2fix.cuh", "log2fix_table.inc")
-COUNTERS50_SOURCE_HASH = "b9f7ab353c77172e"
+COUNTERS50_SOURCE_HASH = "1b194d4e1fcdd5a0"
 
 
 def counters_source_hash(names=COUNTERS_SOURCES) -> str:
@@ -402,7 +403,7 @@ def profile_case(args):
     DFMA chains per thread (FP64 dependent latency against throughput).
     adjoint: one df_chem_adjoint call on the adjoint workload (65536 cells of
     the 9-species field, cotangents of sum T(dt) + sum qdot(dt), stored
-    stages): one launch of the adjoint kernel.
+    stages): one launch each of the forward and the reverse sweep.
     h2: two thread-per-cell integrator launches (warm-up, measured) on 2^18
     cells of the bimodal 9-species field, in the launch shape the autotuner
     picks for the full field (32-thread blocks, as many per SM as fit, hottest
@@ -710,9 +711,9 @@ def main():
                 "frac": achieved / (fp64_peak / 1e3),
                 "counters_current": fresh,
                 "traffic": TRAFFIC_PER_LAUNCH if (ncells == NCELLS and fresh) else None,
-                "traffic_note": "ncu DRAM bytes of one 2^20-cell launch; 2.6x the 180 MB of cell state read "
-                                "and written, from 8-byte accesses in hottest-first cell order (32-byte sectors); "
-                                "0.1% of HBM bandwidth over the launch",
+                "traffic_note": "ncu DRAM bytes of one 2^20-cell launch; 5.9x the 180 MB of cell state read "
+                                "and written: 8-byte accesses in hottest-first cell order (32-byte sectors) and "
+                                "local memory (stage vectors) evicted from L2; 1% of HBM bandwidth over the launch",
                 "peak_source": "measured FP64 DFMA throughput (df_probe_fp64_peak), this GPU, this run",
                 "flop_per_substep": FLOP_PER_SUBSTEP}
     line = {

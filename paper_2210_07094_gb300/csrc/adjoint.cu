@@ -9,8 +9,9 @@
 // paper has no adjoint; this is the sensitivity / calibration extension of the
 // chemistry substep of Sec. 2.3.
 //
-// Per accepted step, in reverse: recompute the stages K_s and the LU of
-// W = I/(h gamma) - J(y) from the checkpoint (y_i, h_i), then with
+// Per accepted step, in reverse: read the stages K_s and the LU of
+// W = I/(h gamma) - J(y) that the forward sweep stored (or recompute them from the
+// checkpoint (y_i, h_i)), then with
 // Kbar_s = m_s lambda (+ later-stage terms):
 //   Rbar_s = W^{-T} Kbar_s
 //   Kbar_j += (c_sj / h) Rbar_s                           (j < s)
@@ -18,9 +19,9 @@
 //   thbar  += (df/dlnA)(Y_s)^T Rbar_s
 //   lambda += d/de [J(y + e K_s)^T Rbar_s]               (W depends on y)
 //   thbar  += d/de [(df/dlnA)(y + e K_s)^T Rbar_s]
-// The directional derivatives come from forward-mode dual numbers through the
-// same rate and Jacobian code as the integrator (exact, no differencing).
-// qdot's gradient at the final state: n dual evaluations of the right-hand side.
+// The products J^T r come from eval_vjp (reverse mode, no Jacobian formed), the last
+// two lines, summed over the stages, from second_order in one pass (exact, no
+// differencing).  qdot's gradient at the final state: one product J^T e_T and closed forms.
 //
 // Cells are assigned statically (cell = global thread index) and the per-cell
 // ln A gradients are summed over threads in a fixed order, then over blocks by a

@@ -1,8 +1,8 @@
 // First-order forward-mode dual numbers a + b eps (eps^2 = 0) for the device
-// chemistry code.  Pushing a state y + eps K through the Jacobian code gives
-// J(y) and its directional derivative dJ(y)[K] exactly (no differencing); the
-// discrete adjoint uses that for the second-derivative terms of the
-// Rosenbrock step.
+// chemistry code.  A reaction's rate and its derivatives evaluated along a direction of
+// (T, C) give the gradient of their directional derivative exactly (no differencing);
+// the discrete adjoint uses that for the second-derivative terms of the
+// Rosenbrock step (second_order).
 #pragma once
 #include "exp2fix.cuh"
 

@@ -686,7 +686,7 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
                                             m->jit_note + ")");
     return integrate_warp_dispatch(m, a, st, 0, false);
   }
-  // default block: 32 threads (5 warps per SM for the generated kernel; the
+  // default block: 32 threads (8 warps per SM for the generated kernel; the
   // mechanism-independent kernel runs as fast at 32 as at 64)
   const int threads = bt > 0 ? bt : 32;
   switch (m->dims.N) {
