@@ -53,7 +53,7 @@ COUNTERS_SOURCE_HASH = "3569d8b71e4f40b1"
 FLOP_PER_SUBSTEP_50 = 248787
 COUNTERS50_SOURCES = ("integrate.cu", "chem_warp.cuh", "chem_thread.cuh", "dev_common.cuh", "exp2fix.cuh",
                       "exp2fix_table.inc", "log2fix.cuh", "log2fix_table.inc")
-COUNTERS50_SOURCE_HASH = "1b194d4e1fcdd5a0"
+COUNTERS50_SOURCE_HASH = "8df78d8d13b94023"
 
 
 def counters_source_hash(names=COUNTERS_SOURCES) -> str:

@@ -74,7 +74,9 @@ typedef struct df_integ_opts {
                              value, see block_threads); >0: at most this many */
   int32_t order_by_T;     /* 1 (default): hand out cells hottest first (a device
                              counting sort; longest work first, lanes refilled
-                             together get cells of similar stiffness)          */
+                             together get cells of similar stiffness; left out
+                             where every cell starts at once, one warp per
+                             FP64 pipe: the results are the same)              */
   int32_t path;           /* 0: auto -- the path df_chem_autotune chose, else
                              thread per cell where a thread kernel exists (the
                              built species counts 3 and 9; with jit = 0 at

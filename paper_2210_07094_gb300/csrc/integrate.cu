@@ -639,12 +639,7 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
   a.nsub = nsub;
   a.nsteps = nsteps;
   a.t_ign = t_ign;
-  if (!order && o.order_by_T && nwork == ncells && ncells > 1) {
-    int32_t* ord = nullptr;
-    rc = build_order(m, T, ncells, st, &ord);
-    if (rc) return rc;
-    order = ord;
-  } else if (order && nwork_dev && o.order_by_T && nwork > 1) {
+  if (order && nwork_dev && o.order_by_T && nwork > 1) {
     // a cell list counted on the device (the surrogate's fallback cells):
     // hottest first as well, so its stiffest cells do not start last
     int32_t* ord = nullptr;
@@ -671,6 +666,17 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
   if (tuned && m->tuned_path == (warp_path ? 2 : 1)) {
     bt = m->tuned_threads;
     bps = m->tuned_bps;
+  }
+  // Hottest first, unless every cell starts at once on a warp that has an FP64 pipe (four
+  // per SM) to itself: the longest cell then sets the time in any order, and the order's
+  // four launches were a tenth of a call of 96 cells (223 -> 202 us; the sizes
+  // up to the line, bimodal or not, take the same time or a little less).
+  const int64_t alone = bps > 0 ? 0 : (warp_path ? 4 : 128) * (int64_t)m->num_sms;
+  if (!a.order && o.order_by_T && nwork == ncells && ncells > std::max<int64_t>(1, alone)) {
+    int32_t* ord = nullptr;
+    rc = build_order(m, T, ncells, st, &ord);
+    if (rc) return rc;
+    a.order = ord;
   }
   if (warp_path) {
     m->jit_used = 0;
