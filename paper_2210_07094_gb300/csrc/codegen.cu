@@ -283,23 +283,35 @@ std::string hex64(uint64_t v) {
   return b;
 }
 
-// "+= c * mono" in units of 2^-53, mono a fixed-point variable of the given scale
-std::string fixed_term(const std::string& dst, double c, bool log2e, const char* mono, int scale) {
+// "+= c * mono" in units of 2^-bits, mono a fixed-point variable of the given scale
+std::string fixed_term(const std::string& dst, double c, bool log2e, const char* mono, int scale, int bits = 53) {
   uint64_t l;
   int sh;
-  fixed_literal(c, log2e, 117 - scale, &l, &sh);
+  fixed_literal(c, log2e, bits + 64 - scale, &l, &sh);
   if (l == 0) return "";
   std::string e = std::string("mul_fixed(") + mono + ", " + hex64(l) + ")";
   if (sh) e = "(" + e + " << " + std::to_string(sh) + ")";
   return "    " + dst + (c < 0.0 ? " -= " : " += ") + "(int64_t)" + e + ";\n";
 }
 
-// c, or c log2(e), in units of 2^-53
-std::string fixed_const(double c, bool log2e) {
+// c, or c log2(e), in units of 2^-bits
+std::string fixed_const(double c, bool log2e, int bits = 53) {
   uint64_t l;
   int sh;
-  fixed_literal(c, log2e, 53, &l, &sh);
+  fixed_literal(c, log2e, bits, &l, &sh);
   return std::string(c < 0.0 ? "-" : "") + "(int64_t)(" + hex64(l) + (sh ? " << " + std::to_string(sh) : "") + ")";
+}
+
+// The fraction bits, at most 53, with which c0 + T (c1 + T (c2 + T (c3 + T c4))) + c5/T
+// stays within 63 bits at the temperatures from T_low (sampled as in fixed_T_low; a
+// term may wrap, the sum of 64-bit words is the same)
+int enthalpy_bits(const std::vector<double>& c, double T_low) {
+  double worst = 0.0;
+  for (double T = T_low; T < FIX_T_HIGH * 1.02; T *= 1.02)
+    worst = std::max(worst, std::fabs(c[0] + T * (c[1] + T * (c[2] + T * (c[3] + T * c[4]))) + c[5] / T));
+  int bits = 53;
+  while (bits > 0 && worst * 1.05 * std::ldexp(1.0, bits) >= 0x1p63) --bits;
+  return bits;
 }
 
 // The unknowns of the generated kernel's linear systems.  A species that no
@@ -565,16 +577,16 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
   for (int k = 0; k < N; ++k) o << "  const Fx x" << k << " = fx_factor(C[" << k << "]);\n  (void)x" << k << ";\n";
   // h/RT: with J of every reacting species, in fixed point, for d ln K_c/dT
   o << "  double w[NS], sM[NS], sN[NS];\n  int64_t H[NS];\n  (void)H; (void)sM; (void)sN;\n";
-  auto enthalpy = [&](const std::string& dst, const std::vector<double>& c) {
-    return "    " + dst + " = " + fixed_const(c[0], false) + ";\n" + fixed_term(dst, c[1], false, "t1", 50) +
-           fixed_term(dst, c[2], false, "t2", 36) + fixed_term(dst, c[3], false, "t3", 22) +
-           fixed_term(dst, c[4], false, "t4", 8) + fixed_term(dst, c[5], false, "I", 69);
+  auto enthalpy = [&](const std::string& dst, const std::vector<double>& c, int bits) {
+    return "    " + dst + " = " + fixed_const(c[0], false, bits) + ";\n" + fixed_term(dst, c[1], false, "t1", 50, bits) +
+           fixed_term(dst, c[2], false, "t2", 36, bits) + fixed_term(dst, c[3], false, "t3", 22, bits) +
+           fixed_term(dst, c[4], false, "t4", 8, bits) + fixed_term(dst, c[5], false, "I", 69, bits);
   };
   auto hcoef = [&](int k) {
     return std::vector<double>{sp(k, 2), sp(k, SP_H), sp(k, SP_H + 1), sp(k, SP_H + 2), sp(k, SP_H + 3), sp(k, 7)};
   };
   o << "  if (WITH_J) {\n";
-  for (int k : sys.act) o << enthalpy("H[" + S(k) + "]", hcoef(k));
+  for (int k : sys.act) o << enthalpy("H[" + S(k) + "]", hcoef(k), 53);
   o << "  }\n";
   // accumulators start at zero where their first contribution is conditional
   // (falloff reactions without a low-pressure rate contribute nothing)
@@ -839,7 +851,8 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     o << "      }\n    }\n  }\n";
   }
   // h/RT of the kept species with the eliminated ones' shares (the heat release
-  // and the temperature row need no others)
+  // and the temperature row need no others).  A fuel's is its heat of combustion, so
+  // beyond 1024 a sum has fewer fraction bits than 53 (still more digits than a double)
   o << "  double hk[NS];\n";
   for (int a = 0; a < NR; ++a) {
     std::vector<double> c = hcoef(sys.keep[a]);
@@ -847,7 +860,9 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
       const std::vector<double> ce = hcoef(sys.elim[e]);
       for (int i = 0; i < 6; ++i) c[i] += sys.b[e][a] * ce[i];
     }
-    o << "  {\n    int64_t h;\n" << enthalpy("h", c) << "    hk[" << sys.keep[a] << "] = fixed_to_double(h);\n  }\n";
+    const int bits = enthalpy_bits(c, T_low);
+    o << "  {\n    int64_t h;\n" << enthalpy("h", c, bits) << "    hk[" << sys.keep[a] << "] = fixed_to_double(h"
+      << (bits != 53 ? ", " + S(bits) : std::string()) << ");\n  }\n";
   }
   // heat release and f
   o << "  double Hw = 0.0;\n";

@@ -158,10 +158,10 @@ __device__ __forceinline__ int64_t mul_fixed_signed(int64_t v, uint64_t c) {
   return ((int64_t)p ^ neg) - neg;
 }
 
-// v 2^-53 as a double
-__device__ __forceinline__ double fixed_to_double(int64_t v) {
+// v 2^-bits as a double
+__device__ __forceinline__ double fixed_to_double(int64_t v, int bits = 53) {
   const int64_t neg = v >> 63;
-  return fx_pack((uint64_t)((v ^ neg) - neg), -53, (uint32_t)(neg >> 32));
+  return fx_pack((uint64_t)((v ^ neg) - neg), -bits, (uint32_t)(neg >> 32));
 }
 
 // x log2(e) as floor(x log2(e) 2^53), |x| < 512: the 53-bit mantissa (at bit

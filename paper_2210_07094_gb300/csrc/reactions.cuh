@@ -91,19 +91,23 @@ inline double fixed_T_low(const df_mech* m, const std::vector<Rx>& rx, bool satu
   for (double lo : {100.0, 150.0, 200.0, 250.0, 300.0, 400.0}) {
     double worst = 0.0, least = 0.0;
     for (double T = lo; T < FIX_T_HIGH * 1.02; T *= 1.02) {
-      std::vector<double> g(m->dims.N);
+      std::vector<double> g(m->dims.N), h(m->dims.N);
       for (int k = 0; k < m->dims.N; ++k) {
-        worst = std::max(worst, std::fabs(sp(k, 2) + T * (sp(k, SP_H) + T * (sp(k, SP_H + 1) + T * (sp(k, SP_H + 2) +
-                                          T * sp(k, SP_H + 3)))) + sp(k, 7) / T));
+        h[k] = sp(k, 2) + T * (sp(k, SP_H) + T * (sp(k, SP_H + 1) + T * (sp(k, SP_H + 2) + T * sp(k, SP_H + 3)))) +
+               sp(k, 7) / T;
+        worst = std::max(worst, std::fabs(h[k]));
         g[k] = L2E * ((sp(k, 2) - sp(k, 8)) - sp(k, 2) * std::log(T) -
                       T * (sp(k, 3) / 2 + T * (sp(k, 4) / 6 + T * (sp(k, 5) / 12 + T * sp(k, 6) / 20))) + sp(k, 7) / T);
       }
       for (const Rx& x : rx) {
         worst = std::max(worst, std::fabs(x.b) + std::fabs(x.E) / T);
         const double kf = 150.0 + L2E * std::fabs(x.b * std::log(T) - x.E / T);
-        double sg = -x.dnu * L2E * (LOG_PSTD_RU - std::log(T));
-        for (int k : x.spc) sg += x.nu[k] * g[k];
-        worst = std::max({worst, kf + std::max(sg, 0.0), std::fabs(sg)});
+        double sg = -x.dnu * L2E * (LOG_PSTD_RU - std::log(T)), sh = -x.dnu;
+        for (int k : x.spc) {
+          sg += x.nu[k] * g[k];
+          sh += x.nu[k] * h[k];
+        }
+        worst = std::max({worst, kf + std::max(sg, 0.0), std::fabs(sg), std::fabs(sh)});
         least = std::max(least, kf - sg);
         if (x.type == 2) {
           const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
