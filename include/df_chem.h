@@ -97,7 +97,12 @@ typedef struct df_integ_opts {
                              code, compiled with NVRTC on first use and cached;
                              32- and 64-thread blocks; the same operations as
                              the mechanism-independent kernel, cells equal to
-                             rounding), falling back to
+                             rounding), each of three variants (32 threads, 64
+                             threads, ignition time: t_ign given) on its own
+                             first use, which takes the seconds of a compilation
+                             and may lie in a stream capture (a program that
+                             cannot wait there makes a call of each variant it
+                             uses beforehand), falling back to
                              that kernel when runtime compilation is
                              unavailable (df_chem_jit_info says why); compiled
                              modules are kept in an on-disk cache

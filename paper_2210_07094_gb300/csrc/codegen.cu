@@ -1134,6 +1134,11 @@ struct Module {
   size_t compile_ms = 0;
   bool from_cache = false;
   int per_thread = 0;  // doubles of shared memory per thread: the systems and the exponents
+  // compiled, but not loaded or its table not uploaded (a lack of memory, say): the
+  // next launches try these again, so many times
+  std::vector<char> cubin;
+  std::vector<std::string> lowered;
+  int retries = 0;
 };
 
 std::mutex g_mu;
@@ -1222,6 +1227,27 @@ uint64_t headers_hash(const std::string& inc) {
   return h;
 }
 
+// The tables to a module's constants.  The variant's first launch may lie inside a
+// stream capture of the caller, where the legacy stream may not be used: a stream of
+// its own that does not wait for it, and this thread in the capture mode that allows
+// calls beside the captured ones.
+bool upload_tables(CUdeviceptr dst, const RosTab (&t)[2]) {
+  cudaStream_t s = nullptr;
+  bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
+  ok = ok && cudaMemcpyAsync((void*)dst, t, sizeof(t), cudaMemcpyHostToDevice, s) == cudaSuccess;
+  ok = ok && cudaStreamSynchronize(s) == cudaSuccess;
+  if (s) cudaStreamDestroy(s);
+  return ok;
+}
+
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  bool ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+  ~RelaxedCapture() {
+    if (ok) cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+};
+
 // resolve the kernel and the table of a loaded cubin, upload the tables
 bool finish_module(Module& r, const Driver& drv, const std::vector<char>& cubin,
                    const std::vector<std::string>& lowered) {
@@ -1252,7 +1278,8 @@ bool finish_module(Module& r, const Driver& drv, const std::vector<char>& cubin,
     r.mod = nullptr;
     return false;
   }
-  if (cudaMemcpy((void*)tab, t, sizeof(t), cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (!upload_tables(tab, t)) {
+    cudaGetLastError();
     r.why = "upload of the Rosenbrock tables failed";
     drv.unload(r.mod);
     r.mod = nullptr;
@@ -1352,12 +1379,16 @@ Module build_module(int dev, const df_mech* m, const std::string& src, int varia
     lowered.push_back(l ? std::string(l) : std::string());
   }
   nv.destroy(&prog);
-  if (!finish_module(r, drv, cubin, lowered)) return r;
   if (!base.empty()) {  // best effort: a failed write only costs the next process a compile
     std::string nm;
     for (auto& l : lowered) nm += l + "\n";
     if (write_file_atomic(base + ".cubin", std::string(cubin.begin(), cubin.end())))
       write_file_atomic(base + ".names", nm);
+  }
+  if (!finish_module(r, drv, cubin, lowered)) {
+    r.cubin = cubin;
+    r.lowered = lowered;
+    r.retries = 3;
   }
   return r;
 }
@@ -1377,15 +1408,22 @@ int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, cuda
   if (!md) {  // first launch on this device: generate, and compile unless cached
     const std::string src = jit_thread_source(m);
     std::lock_guard<std::mutex> lock(g_mu);
+    const RelaxedCapture relaxed;
     auto key = std::make_pair(dev * kVariants + variant, src);
     auto it = g_modules.find(key);
-    if (it == g_modules.end()) it = g_modules.emplace(key, build_module(dev, m, src, variant)).first;
-    md = &it->second;
-    {
+    if (it == g_modules.end()) {
+      it = g_modules.emplace(key, build_module(dev, m, src, variant)).first;
       const Systems sys = systems_of(m, reactions_of(m));
-      md->per_thread = sys.per_thread() + Systems::exponents();
+      it->second.per_thread = sys.per_thread() + Systems::exponents();
+    } else if (it->second.retries > 0) {
+      Module& r = it->second;
+      r.retries = finish_module(r, driver(), r.cubin, r.lowered) ? 0 : r.retries - 1;
     }
-    m->jit_module[dev][variant] = md;
+    md = &it->second;
+    if (md->retries == 0) {
+      md->cubin = {};
+      m->jit_module[dev][variant] = md;
+    }
     m->jit_note = !md->ok          ? md->why
                   : md->from_cache ? std::string("generated kernel loaded from the on-disk cache")
                                    : "generated kernel compiled in " + std::to_string(md->compile_ms) + " ms";
