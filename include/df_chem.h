@@ -144,7 +144,8 @@ int df_mech_set_lnA(df_mech* mech, const double* lnA, df_stream_t stream);
 
 /* ---------------------------------------------------------------------------
  * Right-hand side and Jacobian (diagnostic entry points; same device code as
- * the integrator).
+ * the integrator).  A cell's result does not depend on how many cells share its
+ * call.
  * ------------------------------------------------------------------------- */
 
 /* dydt[(i) * ncells + c], i = 0 for dT/dt [K/s], i = 1 + k for dY_k/dt [1/s]

@@ -636,7 +636,8 @@ __device__ __forceinline__ S eval_thread(const MechView& mv, const double pc, co
       cpf += (cpR[k] - EV) * iW * f[1 + k];
     }
     dcp = dcp * RU;
-    cpf = cpf * RU;
+    // (where two products meet in a sum the text says which one is fused: eval_lanes.cuh
+    // rounds alike)
 #pragma unroll 1
     for (int jc = 0; jc < n; ++jc) {
       S acc(0.0);
@@ -644,11 +645,11 @@ __device__ __forceinline__ S eval_thread(const MechView& mv, const double pc, co
       for (int k = 0; k < NS; ++k) acc += (hRT[k] - EV) * mv.sp[SP_REC * k + 1] * Jv[(1 + k) * n + jc];
       acc = acc * (RU * T);
       if (jc == 0) {
-        Jv[0] = -(invcp * (acc + cpf)) - f[0] * dcp * invcp;
+        Jv[0] = fma(-invcp, fma(cpf, RU, acc), -(f[0] * dcp * invcp));
       } else {
         const double iWj = mv.sp[SP_REC * (jc - 1) + 1];
         const S cpj = RU * (cpR[jc - 1] - EV) * iWj;
-        Jv[jc] = -(invcp * acc) - f[0] * cpj * invcp;
+        Jv[jc] = fma(-(f[0] * cpj), invcp, -(invcp * acc));
       }
     }
   }

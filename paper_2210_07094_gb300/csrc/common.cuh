@@ -24,6 +24,7 @@ struct df_mech {
   std::vector<int> csr_host;      // species -> (reaction, net nu) lists: [N+1] ptr, pairs
   double* blob_dev = nullptr;     // device copy (lnA may be overridden)
   int* csr_dev = nullptr;
+  int occ_off = 0;                // where the species' occurrences (eval_lanes.cuh) start in it
   int device = 0;
   // persistent-queue and statistics scratch (device): [0] work counter,
   // [1] accepted, [2] rejected, [3] error flag

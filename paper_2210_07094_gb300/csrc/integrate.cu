@@ -18,6 +18,7 @@
 
 #include "common.cuh"
 #include "chem_warp.cuh"
+#include "eval_lanes.cuh"
 #include "integrate_thread.cuh"
 
 namespace df {
@@ -285,6 +286,25 @@ __global__ void __launch_bounds__(256) k_eval_warp(EvalArgs a, const int* csr, W
     for (int e = lane; e < n * n; e += 32) a.J[c * n * n + e] = ws[L.J + e];
 }
 
+template <int NS, bool WITH_J>
+__global__ void __launch_bounds__(128) k_eval_lanes(EvalArgs a, const int* occ, LanesWS L) {
+  constexpr int n = NS + 1;
+  extern __shared__ double smem[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const MechView mv = make_view(a.blob, a.d, a.blob);
+  const int64_t c = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+  if (c >= a.ncells) return;
+  double* ws = smem + (size_t)warp * L.total;
+  if (lane < n) ws[L.y + lane] = lane == 0 ? a.T[c] : a.Y[(int64_t)(lane - 1) * a.ncells + c];
+  __syncwarp();
+  const double q = eval_lanes<NS, WITH_J>(mv, occ, 10.0 * a.p[c], ws, L);
+  __syncwarp();
+  if (a.dydt && lane < n) a.dydt[(int64_t)lane * a.ncells + c] = ws[L.f + lane];
+  if (a.qdot && lane == 0) a.qdot[c] = 0.1 * q;  // erg/(cm^3 s) -> W/m^3
+  if (WITH_J)
+    for (int e = lane; e < n * n; e += 32) a.J[c * n * n + e] = ws[L.J + e];
+}
+
 // ----------------------------------------------------------------------------
 // work order by temperature (hottest first): a counting sort over 1 K bins.
 // Hot cells take the most substeps, so handing them out first shortens the
@@ -401,10 +421,39 @@ size_t thread_smem_bytes(const MechDims& d, int threads, bool stage) {
   return sizeof(double) * ((stage ? blob_smem_doubles(d) : 0) + (size_t)thread_ws_doubles<NS>() * threads);
 }
 
+// A cell per warp (k_eval_lanes, the same bits) where the cells are few: a cell per thread
+// takes one thread's way through all reactions whatever the number of cells.  Cell per thread /
+// cell per warp in us, 152 SMs:
+//                       1 cell     4 per SM   16 per SM  32 per SM
+//   N 9 M 25 source     43 / 14    43 / 14    43 / 25    43 / 51
+//            Jacobian  154 / 29   154 / 29   154 / 67   154 / 131
+//   N 9 M  6 source     23 / 12    23 / 12    23 / 21    23 / 41
+//            Jacobian   68 / 21    72 / 21    72 / 49    72 / 92
+//   N 9 M 70 source     88 / 19    87 / 19    88 / 38    88 / 71
+//            Jacobian  330 / 53   334 / 53   334 / 119  334 / 232
+//   N 3 M  1 source      8 / 8      8 / 8      8 / 12     9 / 23
+//            Jacobian   16 / 10    16 / 12    16 / 25    16 / 43
+static bool few_cells(const df_mech* m, int64_t ncells) {
+  return ncells <= (int64_t)(m->dims.M >= 6 ? 16 : 4) * m->num_sms;
+}
+
 template <int NS>
 int eval_dispatch(const df_mech* m, int64_t ncells, const double* T, const double* p,
                   const double* Y, double* dydt, double* qdot, double* J, cudaStream_t st) {
   EvalArgs a{m->blob_dev, m->dims, ncells, T, p, Y, dydt, qdot, J, 1};
+  if (few_cells(m, ncells)) {
+    // one warp per block while there are SMs for them
+    const LanesWS L = lanes_ws_layout(NS, m->dims.M, m->dims.n_eff, J != nullptr);
+    const size_t per_warp = sizeof(double) * (size_t)L.total;
+    int warps = (int)std::min<int64_t>(4, (ncells + m->num_sms - 1) / m->num_sms);
+    warps = (int)std::min<size_t>(warps, m->max_smem_optin / per_warp);
+    if (warps > 0) {
+      auto kf = J ? k_eval_lanes<NS, true> : k_eval_lanes<NS, false>;
+      cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per_warp * warps));
+      kf<<<(unsigned)((ncells + warps - 1) / warps), 32 * warps, per_warp * warps, st>>>(a, m->csr_dev + m->occ_off, L);
+      return cuda_check(cudaGetLastError(), "chemistry evaluation kernel");
+    }
+  }
   const int threads = 64;
   size_t sm = thread_smem_bytes<NS>(m->dims, threads, true);
   if (sm > m->max_smem_optin) {
@@ -564,17 +613,8 @@ int integrate_warp_dispatch(df_mech* m, const IntegArgs& a0, cudaStream_t st, in
 
 }  // namespace
 
-// One cell per warp for an evaluation of few cells of a mechanism with reactions
-// for the lanes: a cell per thread takes one thread's time through all reactions
-// whatever the number of cells (source term of the 9-species mechanism 62 us up to
-// 16000 cells), a cell per warp takes 39 us up to 500 cells, 52 at 2000, 75 at 4000.
-static bool few_cells(const df_mech* m, int64_t ncells) {
-  return m->dims.M >= 16 && ncells <= (int64_t)16 * m->num_sms;
-}
-
 int launch_rhs(const df_mech* m, int64_t ncells, const double* T, const double* p,
                const double* Y, double* dydt, double* qdot, cudaStream_t st) {
-  if (few_cells(m, ncells)) return eval_warp_dispatch(m, ncells, T, p, Y, dydt, qdot, nullptr, st);
   switch (m->dims.N) {
 #define X(NS) \
   case NS:    \
@@ -588,7 +628,6 @@ int launch_rhs(const df_mech* m, int64_t ncells, const double* T, const double* 
 
 int launch_jacobian(const df_mech* m, int64_t ncells, const double* T, const double* p,
                     const double* Y, double* J, cudaStream_t st) {
-  if (few_cells(m, ncells)) return eval_warp_dispatch(m, ncells, T, p, Y, nullptr, nullptr, J, st);
   switch (m->dims.N) {
 #define X(NS) \
   case NS:    \

@@ -402,6 +402,21 @@ int parse_mechanism(const char* path, df_mech* m) {
     }
   }
   m->csr_host[off0 + n_eff] = ntrip;
+  // the species' occurrences among the reactions' entries: [N + 1] offsets, then 8 j + a
+  m->occ_off = (int)m->csr_host.size();
+  std::vector<std::vector<int>> occ(N);
+  for (int j = 0; j < M; ++j) {
+    RxMeta meta;
+    memcpy(&meta, &rec[RX_REC * j + 3], 8);
+    for (int i = 0; i < (meta.nrnp & 15); ++i) occ[meta.reac[i]].push_back(8 * j + i);
+    for (int i = 0; i < (meta.nrnp >> 4); ++i) occ[meta.prod[i]].push_back(8 * j + 3 + i);
+  }
+  int at = N + 1;
+  for (int k = 0; k <= N; ++k) {
+    m->csr_host.push_back(at);
+    if (k < N) at += (int)occ[k].size();
+  }
+  for (int k = 0; k < N; ++k) m->csr_host.insert(m->csr_host.end(), occ[k].begin(), occ[k].end());
   return DF_OK;
 }
 
