@@ -1395,7 +1395,8 @@ Module build_module(int dev, const df_mech* m, const std::string& src, int varia
 
 }  // namespace
 
-int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, cudaStream_t st, bool* launched) {
+int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, bool order, cudaStream_t st,
+                      bool* launched) {
   *launched = false;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return DF_OK;
@@ -1452,7 +1453,8 @@ int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, cuda
   int64_t blocks = (int64_t)m->num_sms * per_sm;
   const int64_t need = (args.nwork + threads - 1) / threads;
   if (blocks > need) blocks = std::max<int64_t>(1, need);
-  int rc = cuda_check(cudaMemsetAsync(m->counters, 0, 4 * sizeof(unsigned long long), st), "reset work counter");
+  int rc = order_unless_alone(m, args, order, per_sm, threads / 32, 32, st);
+  if (!rc) rc = cuda_check(cudaMemsetAsync(m->counters, 0, 4 * sizeof(unsigned long long), st), "reset work counter");
   if (rc) return rc;
   void* params[] = {&args};
   if (drv.launch(fk, (unsigned)blocks, 1, 1, (unsigned)threads, 1, 1, (unsigned)sm, (CUstream)st, params,

@@ -85,8 +85,13 @@ struct IntegArgs;
 std::string jit_thread_source(const df_mech* m);
 // launch the kernel generated for m with `threads` per block if it can (NVRTC
 // available, the module compiled, a generated kernel for that block size);
-// *launched says whether it did.  Errors only for a failed launch.
-int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, cudaStream_t st, bool* launched);
+// *launched says whether it did; order: as in order_unless_alone.  Errors only for
+// a failed launch.
+int jit_thread_launch(df_mech* m, int threads, int bps, const IntegArgs& a, bool order, cudaStream_t st, bool* launched);
+// with order, give the launch (blocks of `warps` warps with cells_per_warp cells each,
+// per_sm of them resident on an SM) its work order, hottest cell first, unless every
+// cell starts at once on a warp of its own FP64 pipe (integrate.cu)
+int order_unless_alone(df_mech* m, IntegArgs& a, bool order, int per_sm, int warps, int cells_per_warp, cudaStream_t st);
 
 // adjoint (adjoint.cu)
 // with_stages: also room for the stored stages and LU factors of every

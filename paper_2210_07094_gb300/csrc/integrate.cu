@@ -411,6 +411,20 @@ static int build_order(df_mech* m, const double* T, int64_t ncells, cudaStream_t
   return cuda_check(cudaGetLastError(), "order kernels");
 }
 
+// Hottest first, unless every cell starts at once on a warp that has an FP64 pipe (four
+// per SM) to itself: the longest cell then sets the time in any order, and the order's
+// four launches were a tenth of a call of 96 cells (223 -> 202 us; the sizes up to the
+// line, bimodal or not, take the same time or a little less).
+int order_unless_alone(df_mech* m, IntegArgs& a, bool order, int per_sm, int warps, int cells_per_warp,
+                       cudaStream_t st) {
+  const int64_t blocks = (int64_t)m->num_sms * std::min(per_sm, 4 / warps);
+  if (!order || a.ncells <= std::max<int64_t>(1, blocks * warps * cells_per_warp)) return DF_OK;
+  int32_t* ord = nullptr;
+  const int rc = build_order(m, a.T, a.ncells, st, &ord);
+  a.order = ord;
+  return rc;
+}
+
 // ----------------------------------------------------------------------------
 // host launchers
 // ----------------------------------------------------------------------------
@@ -474,12 +488,12 @@ int eval_dispatch(const df_mech* m, int64_t ncells, const double* T, const doubl
 }
 
 template <int NS>
-int integrate_dispatch(df_mech* m, const IntegArgs& a0, cudaStream_t st, int threads, int bps, bool constv,
+int integrate_dispatch(df_mech* m, const IntegArgs& a0, bool order, cudaStream_t st, int threads, int bps, bool constv,
                        bool jit) {
   m->jit_used = 0;
   if (jit && !constv) {  // the kernel generated for this mechanism, if it can run
     bool launched = false;
-    const int rc = jit_thread_launch(m, threads, bps, a0, st, &launched);
+    const int rc = jit_thread_launch(m, threads, bps, a0, order, st, &launched);
     if (rc || launched) return rc;
   }
   IntegArgs a = a0;
@@ -511,7 +525,8 @@ int integrate_dispatch(df_mech* m, const IntegArgs& a0, cudaStream_t st, int thr
   int64_t blocks = (int64_t)m->num_sms * per_sm;
   const int64_t need = (a.nwork + threads - 1) / threads;
   if (blocks > need) blocks = std::max<int64_t>(1, need);
-  rc = cuda_check(cudaMemsetAsync(m->counters, 0, 4 * sizeof(unsigned long long), st), "reset work counter");
+  rc = order_unless_alone(m, a, order, per_sm, threads / 32, 32, st);
+  if (!rc) rc = cuda_check(cudaMemsetAsync(m->counters, 0, 4 * sizeof(unsigned long long), st), "reset work counter");
   if (rc) return rc;
   kf<<<(unsigned)blocks, threads, sm, st>>>(a);
   return cuda_check(cudaGetLastError(), "integrator kernel launch");
@@ -582,7 +597,7 @@ int eval_warp_dispatch(const df_mech* m, int64_t ncells, const double* T, const 
   return cuda_check(cudaGetLastError(), "warp evaluation kernel");
 }
 
-int integrate_warp_dispatch(df_mech* m, const IntegArgs& a0, cudaStream_t st, int threads, bool constv) {
+int integrate_warp_dispatch(df_mech* m, const IntegArgs& a0, bool order, cudaStream_t st, int threads, bool constv) {
   const WarpWS L = warp_ws_layout(m->dims.N, m->dims.M, m->dims.n_eff);
   int warps, stage;
   size_t sm;
@@ -605,7 +620,8 @@ int integrate_warp_dispatch(df_mech* m, const IntegArgs& a0, cudaStream_t st, in
   int64_t blocks = (int64_t)m->num_sms * occ;
   const int64_t need = (a.nwork + warps - 1) / warps;
   if (blocks > need) blocks = std::max<int64_t>(1, need);
-  rc = cuda_check(cudaMemsetAsync(m->counters, 0, 4 * sizeof(unsigned long long), st), "reset work counter");
+  rc = order_unless_alone(m, a, order, occ, warps, 1, st);
+  if (!rc) rc = cuda_check(cudaMemsetAsync(m->counters, 0, 4 * sizeof(unsigned long long), st), "reset work counter");
   if (rc) return rc;
   kf<<<(unsigned)blocks, 32 * warps, sm, st>>>(a, m->csr_dev, L);
   return cuda_check(cudaGetLastError(), "warp integrator kernel launch");
@@ -706,30 +722,20 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
     bt = m->tuned_threads;
     bps = m->tuned_bps;
   }
-  // Hottest first, unless every cell starts at once on a warp that has an FP64 pipe (four
-  // per SM) to itself: the longest cell then sets the time in any order, and the order's
-  // four launches were a tenth of a call of 96 cells (223 -> 202 us; the sizes
-  // up to the line, bimodal or not, take the same time or a little less).
-  const int64_t alone = bps > 0 ? 0 : (warp_path ? 4 : 128) * (int64_t)m->num_sms;
-  if (!a.order && o.order_by_T && nwork == ncells && ncells > std::max<int64_t>(1, alone)) {
-    int32_t* ord = nullptr;
-    rc = build_order(m, T, ncells, st, &ord);
-    if (rc) return rc;
-    a.order = ord;
-  }
+  const bool by_T = !a.order && o.order_by_T && nwork == ncells;
   if (warp_path) {
     m->jit_used = 0;
-    return integrate_warp_dispatch(m, a, st, bt, o.reactor == 1);
+    return integrate_warp_dispatch(m, a, by_T, st, bt, o.reactor == 1);
   }
   if (!thread_ok) {  // the generated kernel only (32- or 64-thread blocks)
     bool launched = false;
     m->jit_used = 0;
-    const int rc = jit_thread_launch(m, bt == 64 ? 64 : 32, bps, a, st, &launched);
+    const int rc = jit_thread_launch(m, bt == 64 ? 64 : 32, bps, a, by_T, st, &launched);
     if (rc || launched) return rc;
     if (o.path == 1)
       return set_error(DF_EUNSUPPORTED, "thread-per-cell path: the generated kernel is unavailable (" +
                                             m->jit_note + ")");
-    return integrate_warp_dispatch(m, a, st, 0, false);
+    return integrate_warp_dispatch(m, a, by_T, st, 0, false);
   }
   // default block: 32 threads (8 warps per SM for the generated kernel; the
   // mechanism-independent kernel runs as fast at 32 as at 64)
@@ -737,7 +743,7 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
   switch (m->dims.N) {
 #define X(NS) \
   case NS:    \
-    return integrate_dispatch<NS>(m, a, st, threads, bps, o.reactor == 1, o.jit == 0);
+    return integrate_dispatch<NS>(m, a, by_T, st, threads, bps, o.reactor == 1, o.jit == 0);
     DF_THREAD_NS_LIST(X)
 #undef X
     default:
