@@ -69,7 +69,10 @@ __device__ __forceinline__ MechView make_view(const double* blob, const MechDims
   v.fr = F.rate;
   v.ff = F.falloff;
   v.T_low = __longlong_as_double(v.fix[F.T_low]);
-  if (!(v.T_low > 0.0) || !v.fix[F.flag]) v.T_low = INFINITY;
+  // with a reaction without a rate in FP64: a test for one in rate_fixed made every
+  // mechanism 1 to 5% slower (constant volume 20011 cells 4.77 -> 4.84 ms, 8192 cells of 50 species
+  // 119.9 -> 122.1, 16411 source terms 64 -> 68 us) and such a one 13% faster
+  if (!(v.T_low > 0.0) || v.fix[F.flag] != 1) v.T_low = INFINITY;
   return v;
 }
 

@@ -52,6 +52,7 @@ namespace {
 // ---------------------------------------------------------------------------
 // exact decimal-free spelling of a double (C++17 hexadecimal literal)
 std::string lit(double v) {
+  if (v == -INFINITY) return "(-INFINITY)";  // ln A0 - ln A of a falloff reaction without a rate
   char b[64];
   snprintf(b, sizeof b, "%a", v);
   return std::string("(") + b + ")";
@@ -532,12 +533,24 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     for (int l = 0; l < N; ++l)
       if (x.type != 0 && col[l] < 0 && m->blob_host[m->dims.off_eff + N * x.eff + l] != 1.0) any_inert = true;
   }
+  // the constants of reactions without a rate: words that pack to zero in every product
+  // (a call, which costs nothing where it is not made: 2^20 cells 15.5 ms, inlined 16.2)
+  o << "template <int ST>\n"
+    << "__device__ __noinline__ void gen_no_rate(const MechView& mv, int j0, int j1, SVT<double, ST> E) {\n"
+    << "  int at = 0;\n"
+    << "#pragma unroll 1\n  for (int j = j0; j < j1; ++j) {\n"
+    << "    const RxMeta mt = load_meta(mv.rx + RX_REC * j);\n"
+    << "    const int words = 1 + ((mt.flags & 3) == 2 ? 1 : 0) + ((mt.flags & 4) != 0 ? 1 : 0);\n"
+    << "    if (mv.fix[j] == FIX_OFF)\n"
+    << "      for (int i = 0; i < words; ++i) E[at + i] = 0.0;\n"
+    << "    at += words;\n  }\n}\n\n";
   o << "template <bool WITH_J, int ST>\n"
     << "__device__ __forceinline__ bool gen_fixed(const MechView& mv, const double pc, const double (&y)[" << N + 1
     << "], double (&f)[" << N + 1 << "], SVT<double, ST> W, SVT<double, ST> E) {\n"
     << "  constexpr int NS = " << N << ";\n"
     << "  const double T = y[0];\n"
-    << "  if (!mv.fix[" << m->dims.M << "] || !(T >= " << lit(T_low) << " && T < " << lit(FIX_T_HIGH) << ")) return false;\n"
+    << "  const long long flag = mv.fix[" << m->dims.M << "];\n"
+    << "  if (!flag || !(T >= " << lit(T_low) << " && T < " << lit(FIX_T_HIGH) << ")) return false;\n"
     << "  double C[NS], cpW[NS];  // cpW: cp_k / (R W_k)\n"
     << "  double sumYW = 0.0, cpm = 0.0;\n";
   for (int k = 0; k < N; ++k) {
@@ -686,7 +699,7 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
       for (int i = 0; i < std::abs(x.dnu); ++i) sg += x.dnu > 0 ? " - lp" : " + lp";
       if (x.type == 2) {
         const double* tr = &m->blob_host[m->dims.off_tr + TR_REC * x.troe];
-        o << "    int64_t xd = " << fixed_const(tr[0], true) << ";\n"
+        o << "    int64_t xd = " << fixed_const(tr[0] == -INFINITY ? 0.0 : tr[0], true) << ";\n"
           << fixed_term("xd", tr[1] - x.b, false, "L", 60) << fixed_term("xd", -(tr[2] - x.E), true, "I", 69)
           << E(slot[j] + 1) << "xd);\n";
         if (x.rev) o << E(slot[j] + 2) << "(int64_t)0" << sg << ");\n";
@@ -697,7 +710,8 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
     }
     const int padded = (n + 3) / 4 * 4;
     for (int i = n; i < padded; ++i) o << E(i).substr(2) << "0);\n";
-    o << "  fx_exp2_all<" << padded << ">(E);\n";
+    o << "  fx_exp2_all<" << padded << ">(E);\n"
+      << "  if (flag == 2) gen_no_rate(mv, " << j0 << ", " << j1 << ", E);\n";
     return j1;
   };
   size_t group_end = 0;

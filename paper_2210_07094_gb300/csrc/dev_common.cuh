@@ -85,8 +85,8 @@ struct MechDims {
 };
 
 // The words behind the blob, all values times log2(e) unless noted:
-//   lnA     M      ln A_j 2^53
-//   flag    1      1 if every ln A fits (lnA_fits_fixed)
+//   lnA     M      ln A_j 2^53, or FIX_OFF for a reaction without a rate
+//   flag    1      0 if some ln A does not fit (fixed_lnA), 2 if one is FIX_OFF, else 1
 //   T_low   1      the lowest temperature the fixed-point arguments cover, as a
 //                  double; 0: the mechanism does not fit, nothing below is set
 //   g       7 N    g_k/RT: the constant 2^53, then the signed coefficients of log2 T

@@ -202,6 +202,15 @@ constexpr double FIX_T_HIGH = 8000.0;
 // within what 64 bits hold with what fixed_T_low allows the temperature terms
 __host__ __device__ inline bool lnA_fits_fixed(double lnA) { return lnA > -104.0 && lnA < 104.0; }
 
+// The word of a reaction's ln A, false if it does not fit.  A reaction without a rate
+// (A = 0, or a falloff reaction whose ln A0 - ln A, d0, is -inf) has one of its own.
+constexpr int64_t FIX_OFF = (int64_t)(1ull << 63);
+__host__ __device__ inline bool fixed_lnA(double lnA, double d0, int64_t* word) {
+  const bool off = lnA == -INFINITY || d0 == -INFINITY, ok = off || lnA_fits_fixed(lnA);
+  *word = off ? FIX_OFF : ok ? exp_arg_fixed(lnA) : 0;
+  return ok;
+}
+
 // x + xc, both within 1022 2^53 and their sum below 1000 2^53, but not below
 // -1000 2^53 (a constant of 2^-1000)
 __device__ __forceinline__ int64_t add_exponents(int64_t x, int64_t xc) {

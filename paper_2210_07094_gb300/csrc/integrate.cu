@@ -752,19 +752,23 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
 }
 
 // ln A into the reaction records and, as fixed-point logarithms, behind the blob;
-// one block, which also says whether all of them fit
+// one block, which also sets the flag (FixLayout)
 __global__ void k_set_lnA(double* blob, MechDims d, const double* lnA) {
   long long* fix = reinterpret_cast<long long*>(blob + d.off_fix());
-  int fits = 1;
+  int fits = 1, off = 0;
   for (int j = threadIdx.x; j < d.M; j += blockDim.x) {
+    double* r = blob + d.off_rx + RX_REC * j;
     const double a = lnA[j];
-    blob[d.off_rx + RX_REC * j] = a;
-    const bool ok = lnA_fits_fixed(a);
-    fix[j] = ok ? exp_arg_fixed(a) : 0;
-    fits = fits && ok;
+    r[0] = a;
+    const double d0 = (load_meta(r).flags & 3) == 2 ? blob[d.off_tr + TR_REC * load_slots(r).troe] : 0.0;
+    int64_t word;
+    fits = fixed_lnA(a, d0, &word) && fits;
+    off = off || word == FIX_OFF;
+    fix[j] = word;
   }
   fits = __syncthreads_and(fits);
-  if (threadIdx.x == 0) fix[d.M] = fits;
+  off = __syncthreads_or(off);
+  if (threadIdx.x == 0) fix[d.M] = !fits ? 0 : off ? 2 : 1;
 }
 
 int launch_set_lnA(df_mech* m, const double* lnA, cudaStream_t st) {

@@ -149,14 +149,14 @@ static void write_fixed(df_mech* m) {
   const MechDims& d = m->dims;
   const FixLayout F(d.N, d.M, d.n_troe);
   std::vector<int64_t> w(F.words, 0);
-  bool fits = true;
-  for (int j = 0; j < d.M; ++j) {
-    const bool ok = lnA_fits_fixed(m->lnA_file[j]);
-    w[j] = ok ? exp_arg_fixed(m->lnA_file[j]) : 0;
-    fits = fits && ok;
-  }
-  w[F.flag] = fits;
   const std::vector<Rx> rx = reactions_of(m);
+  bool fits = true, off = false;
+  for (int j = 0; j < d.M; ++j) {
+    const double d0 = rx[j].type == 2 ? m->blob_host[d.off_tr + TR_REC * rx[j].troe] : 0.0;
+    fits = fixed_lnA(m->lnA_file[j], d0, &w[j]) && fits;
+    off = off || w[j] == FIX_OFF;
+  }
+  w[F.flag] = !fits ? 0 : off ? 2 : 1;
   double T_low = fixed_T_low(m, rx, true);
   auto put = [&](int at, double c, bool log2e, int s) {  // c 2^s, signed; T_low = 0 if it takes more than 63 bits
     uint64_t l;

@@ -115,7 +115,7 @@ inline double fixed_T_low(const df_mech* m, const std::vector<Rx>& rx, bool satu
           const double Fc = (1.0 - tr[3]) * std::exp(-T * tr[4]) + tr[3] * std::exp(-T * tr[5]) + std::exp(-tr[6] / T);
           if (!(Fc > 1e-60 && Fc < 1e60)) worst = INFINITY;
           const double d = L2E * std::fabs(tr[0] + (tr[1] - x.b) * std::log(T) - (tr[2] - x.E) / T);
-          worst = std::max({worst, d, kf + d, std::fabs(sg)});
+          if (tr[0] != -INFINITY) worst = std::max({worst, d, kf + d, std::fabs(sg)});  // else it has no rate
         }
       }
     }
