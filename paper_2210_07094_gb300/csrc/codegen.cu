@@ -560,6 +560,7 @@ void emit_fixed(std::ostringstream& o, const df_mech* m, const std::vector<Rx>& 
       << "  cpW[" << k << "] = " << horner(aw, "T") << ";\n  cpm += y[" << 1 + k << "] * cpW[" << k << "];\n";
   }
   o << "  if (!rcp_in_range(sumYW) || !rcp_in_range(cpm) || !rcp_in_range(pc)) return false;\n"
+    // (cpm RU, 2^26 times cpm, is within what rcp_fast takes: below 2^124)
     << "  const double invT = rcp_fast(T), Wbar = rcp_fast(sumYW), invcp = rcp_fast(cpm * RU);\n"
     << "  const double rho = pc * invT * (Wbar * " << lit(1.0 / RU) << ");\n"
     << "  const double invrho = rcp_any(rho);\n"
