@@ -38,8 +38,9 @@ int df_probe_exp(const double* x, double* y, long long n, int table_bits, void* 
  * 0, or DF_EINVAL for a negative n or a missing buffer. */
 int df_probe_exp_rate(const double* x, double* y, long long n, void* stream);
 
-/* y[i] = ln(x[i]) by the library's own table-driven logarithm (the one the
- * rate kernels use for ln T and the Troe falloff), so that its accuracy can be
+/* y[i] = ln(x[i]) by the library's own logarithm (the one the rate kernels use for
+ * ln T and the Troe falloff: a table and a polynomial in 64-bit fixed point, the
+ * exponent's share and the result in FP64), so that its accuracy can be
  * checked against CUDA's log.  x, y: device memory; asynchronous on `stream`.
  * DF_EINVAL for n < 0 or null arrays with n > 0. */
 int df_probe_log(const double* x, double* y, long long n, void* stream);

@@ -24,9 +24,8 @@
 namespace df {
 
 // ln and log10 of the rate expressions by the fixed-point logarithm (the
-// dual-number versions carry the derivative d/x)
+// dual-number version carries the derivative d/x)
 __device__ __forceinline__ double fast_log(double x) { return log_rate(x); }
-__device__ __forceinline__ Dual fast_log(const Dual& x) { return Dual(log_rate(x.v), x.d / x.v); }
 __device__ __forceinline__ double fast_log10(double x) { return log10_rate(x); }
 __device__ __forceinline__ Dual fast_log10(const Dual& x) {
   return Dual(log10_rate(x.v), x.d / (x.v * 2.302585092994045684));

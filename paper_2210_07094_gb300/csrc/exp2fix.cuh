@@ -59,8 +59,9 @@ __device__ __forceinline__ double exp2_fixed(int64_t X) {
 // with up to three concentrations is a chain of integer multiplications, seven
 // instructions each where an FP64 multiplication occupies its pipe for 64 cycles.
 // The constant enters with 64 bits, each concentration with 53 at bit 62, and a
-// product drops at most two leading bits, so 57 remain after three: no rounding
-// until the number is packed.  The sign is the top bit of the concentrations'
+// product drops at most two leading bits, so 57 remain after three.  Packing truncates
+// to 53, towards zero by up to one unit in the last place, where an FP64 product rounds
+// at each multiplication, by half a unit.  The sign is the top bit of the concentrations'
 // exclusive or, carried beside.
 struct Fx {
   uint64_t m;

@@ -12,8 +12,9 @@
 // the library exp().  The kernels stage the table into shared memory (lanes
 // index it with different j).  The variant with 256 entries 2^(j/256) (|r| <=
 // ln2/512, so exp(r) - 1 needs terms only up to r^4/24, the tail r^5/120 <=
-// 3.8e-17) takes one FP64 operation fewer.  The surrogate's features use it;
-// the rate expressions use the fixed-point form of exp2fix.cuh.
+// 3.8e-17) takes one FP64 operation fewer.  The surrogate's features use the 64-entry
+// table; the 256-entry form is reached through df_probe_exp alone.  The rate
+// expressions use the fixed-point form of exp2fix.cuh.
 #pragma once
 
 #include "dev_common.cuh"  // small_int_to_double

@@ -216,13 +216,11 @@ __device__ __forceinline__ bool ros_attempt(const MechView& mv, const RosTab& tb
 // finished stages, read once per later stage in long independent runs, go to
 // local memory (about 1% of the attempt's time), and the substitutions run in
 // registers.  So do (volatile) the state and the stage state, which the evaluation
-// takes as its own copies: 40 registers that it would otherwise not have.  That leaves room for eight warps per SM, two for every FP64 pipe (the
-// registers allow no more: with 168 instead of 255 per thread a third warp per
-// pipe made 2^20 cells 22.1 instead of 19.3 ms).
-// 2^20 cells of the bimodal 9-species field: 41.6 ms with the 10 x 10 systems at
-// five warps per SM, 24.4 with 9 x 9 at eight, 21.0 with the rate products on the
-// integer pipes, 19.3 with 7 x 7, 15.9 with the exponents in groups and the states
-// in local memory.
+// takes as its own copies: 40 registers that it would otherwise not have.  That leaves room
+// for eight warps per SM, two for every FP64 pipe (the registers allow no more: a third
+// warp per pipe, at 168 instead of 255 per thread, took a seventh longer).
+// 2^20 cells of the bimodal 9-species field: 16 ms; 41.6 with 10 x 10 systems, every
+// product in FP64 and five warps per SM.
 template <int ST, class EVAL>
 __device__ __forceinline__ bool ros_attempt_gen(const MechView& mv, const RosTab& tb, double pc,
                                                 const volatile double (&y)[EVAL::kN + 1], double& h, double rtol,
