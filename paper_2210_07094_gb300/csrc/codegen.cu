@@ -1244,8 +1244,7 @@ uint64_t headers_hash(const std::string& inc) {
 
 // The tables to a module's constants.  The variant's first launch may lie inside a
 // stream capture of the caller, where the legacy stream may not be used: a stream of
-// its own that does not wait for it, and this thread in the capture mode that allows
-// calls beside the captured ones.
+// its own that does not wait for it (and RelaxedCapture).
 bool upload_tables(CUdeviceptr dst, const RosTab (&t)[2]) {
   cudaStream_t s = nullptr;
   bool ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
@@ -1254,14 +1253,6 @@ bool upload_tables(CUdeviceptr dst, const RosTab (&t)[2]) {
   if (s) cudaStreamDestroy(s);
   return ok;
 }
-
-struct RelaxedCapture {
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  bool ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
-  ~RelaxedCapture() {
-    if (ok) cudaThreadExchangeStreamCaptureMode(&mode);
-  }
-};
 
 // resolve the kernel and the table of a loaded cubin, upload the tables
 bool finish_module(Module& r, const Driver& drv, const std::vector<char>& cubin,

@@ -80,6 +80,16 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
                           int64_t nwork, cudaStream_t st, const unsigned long long* nwork_dev = nullptr,
                           int nsteps = 1, double* t_ign = nullptr);
 
+// this thread in the capture mode that allows allocations, loads and copies on other
+// streams beside a stream capture of the caller
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  bool ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+  ~RelaxedCapture() {
+    if (ok) cudaThreadExchangeStreamCaptureMode(&mode);
+  }
+};
+
 // generated thread-per-cell integrator (codegen.cu)
 struct IntegArgs;
 std::string jit_thread_source(const df_mech* m);

@@ -373,11 +373,15 @@ __global__ void k_order_scatter_list(const double* T, const int32_t* list, const
   }
 }
 
+// the cells that start at once on an SM, at most: a warp of 32 on each of its four FP64 pipes
+constexpr int ALONE_PER_SM = 128;
+
 static int ensure_order_buffers(df_mech* m, int64_t n) {
   if (m->order_cap < n) {
     if (m->order) cudaFree(m->order);
     m->order = nullptr;
     m->order_cap = 0;
+    n = std::max(n, (int64_t)ALONE_PER_SM * m->num_sms);
     int rc = cuda_check(cudaMalloc(&m->order, sizeof(int32_t) * n), "cudaMalloc order");
     if (rc) return rc;
     m->order_cap = n;
@@ -414,11 +418,20 @@ static int build_order(df_mech* m, const double* T, int64_t ncells, cudaStream_t
 // Hottest first, unless every cell starts at once on a warp that has an FP64 pipe (four
 // per SM) to itself: the longest cell then sets the time in any order, and the order's
 // four launches were a tenth of a call of 96 cells (223 -> 202 us; the sizes up to the
-// line, bimodal or not, take the same time or a little less).
+// line, bimodal or not, take the same time or a little less).  The order's scratch is
+// there from the first call on all the same, since a later one of such a size may need it
+// inside a stream capture.
 int order_unless_alone(df_mech* m, IntegArgs& a, bool order, int per_sm, int warps, int cells_per_warp,
                        cudaStream_t st) {
+  if (!order || a.ncells <= 1) return DF_OK;
   const int64_t blocks = (int64_t)m->num_sms * std::min(per_sm, 4 / warps);
-  if (!order || a.ncells <= std::max<int64_t>(1, blocks * warps * cells_per_warp)) return DF_OK;
+  if (a.ncells <= blocks * warps * cells_per_warp) {
+    if (!m->bins) {
+      const RelaxedCapture relaxed;
+      if (ensure_order_buffers(m, 1)) cudaGetLastError();  // tried again where it is needed
+    }
+    return DF_OK;
+  }
   int32_t* ord = nullptr;
   const int rc = build_order(m, a.T, a.ncells, st, &ord);
   a.order = ord;
