@@ -407,8 +407,7 @@ template <int NS, Sweep SW>
 static int launch_sweep(const df_mech* m, const AdjArgs& a, int64_t blocks, cudaStream_t st) {
   const size_t sm = sizeof(double) * adj_layout_doubles(NS, m->dims.M, SW) * ADJ_THREADS;
   if (sm > m->max_smem_optin) return set_error(DF_EUNSUPPORTED, "adjoint workspace exceeds shared memory");
-  int rc = cuda_check(cudaFuncSetAttribute(k_adjoint_thread<NS, SW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                      "set adjoint shared memory");
+  int rc = cuda_check(allow_smem(m, k_adjoint_thread<NS, SW>), "set adjoint shared memory");
   if (rc) return rc;
   k_adjoint_thread<NS, SW><<<(unsigned)blocks, ADJ_THREADS, sm, st>>>(a);
   return cuda_check(cudaGetLastError(), "adjoint kernel launch");

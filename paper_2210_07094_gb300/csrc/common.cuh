@@ -80,6 +80,14 @@ int launch_integrate_list(df_mech* m, int64_t ncells, double* T, const double* p
                           int64_t nwork, cudaStream_t st, const unsigned long long* nwork_dev = nullptr,
                           int nsteps = 1, double* t_ign = nullptr);
 
+// Launches of kernel k may take dynamic shared memory up to the device's limit.  Every
+// call sets the same value: the size of the launch at hand, which varies with the number
+// of cells, would take the room of a launch that another thread is about to make.
+template <class K>
+cudaError_t allow_smem(const df_mech* m, K k) {
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m->max_smem_optin);
+}
+
 // this thread in the capture mode that allows allocations, loads and copies on other
 // streams beside a stream capture of the caller
 struct RelaxedCapture {

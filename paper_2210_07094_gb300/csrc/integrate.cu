@@ -476,7 +476,7 @@ int eval_dispatch(const df_mech* m, int64_t ncells, const double* T, const doubl
     warps = (int)std::min<size_t>(warps, m->max_smem_optin / per_warp);
     if (warps > 0) {
       auto kf = J ? k_eval_lanes<NS, true> : k_eval_lanes<NS, false>;
-      cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per_warp * warps));
+      if (per_warp * warps > 48 * 1024) allow_smem(m, kf);
       kf<<<(unsigned)((ncells + warps - 1) / warps), 32 * warps, per_warp * warps, st>>>(a, m->csr_dev + m->occ_off, L);
       return cuda_check(cudaGetLastError(), "chemistry evaluation kernel");
     }
@@ -490,11 +490,11 @@ int eval_dispatch(const df_mech* m, int64_t ncells, const double* T, const doubl
   const int64_t blocks = (ncells + threads - 1) / threads;
   if (J) {
     auto kf = k_eval_thread<NS, true>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(m, kf);
     kf<<<(unsigned)blocks, threads, sm, st>>>(a);
   } else {
     auto kf = k_eval_thread<NS, false>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(m, kf);
     kf<<<(unsigned)blocks, threads, sm, st>>>(a);
   }
   return cuda_check(cudaGetLastError(), "chemistry evaluation kernel");
@@ -527,8 +527,7 @@ int integrate_dispatch(df_mech* m, const IntegArgs& a0, bool order, cudaStream_t
             : threads == 64  ? k_integrate_thread<NS, false, 64>
             : threads == 128 ? k_integrate_thread<NS, false, 128>
                              : k_integrate_thread<NS, false>;
-  int rc = cuda_check(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                      "set integrator shared memory");
+  int rc = cuda_check(allow_smem(m, kf), "set integrator shared memory");
   if (rc) return rc;
   int occ = 0;
   rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kf, threads, sm), "occupancy");
@@ -600,11 +599,11 @@ int eval_warp_dispatch(const df_mech* m, int64_t ncells, const double* T, const 
   const int64_t blocks = (ncells + warps - 1) / warps;
   if (J) {
     auto kf = k_eval_warp<true>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(m, kf);
     kf<<<(unsigned)blocks, 32 * warps, sm, st>>>(a, m->csr_dev, L);
   } else {
     auto kf = k_eval_warp<false>;
-    cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    allow_smem(m, kf);
     kf<<<(unsigned)blocks, 32 * warps, sm, st>>>(a, m->csr_dev, L);
   }
   return cuda_check(cudaGetLastError(), "warp evaluation kernel");
@@ -623,8 +622,7 @@ int integrate_warp_dispatch(df_mech* m, const IntegArgs& a0, bool order, cudaStr
   IntegArgs a = a0;
   a.stage_blob = stage;
   auto kf = constv ? k_integrate_warp<true> : k_integrate_warp<false>;
-  rc = cuda_check(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
-                  "set warp integrator shared memory");
+  rc = cuda_check(allow_smem(m, kf), "set warp integrator shared memory");
   if (rc) return rc;
   int occ = 0;
   rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kf, 32 * warps, sm), "occupancy");
